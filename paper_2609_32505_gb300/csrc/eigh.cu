@@ -1350,40 +1350,48 @@ static int trd_ctas_per_group(int n) {
     return std::max(1, std::min(std::min(PSVD_TRD_MINB * num_sms(), 320), n / PSVD_TRD_ROWDIV));
 }
 
-int eigh_groups(int B, int n) {
+// Matrices in flight, and workspace slots for them (the on-chip kernels take the larger number: at
+// least 4 CTAs of 32 threads per matrix).
+static int trd_groups(int B, int n) {
     const int g = trd_ctas_per_group(n);
     return std::max(1, std::min(B, (PSVD_TRD_MINB * num_sms()) / g));
+}
+int eigh_groups(int B, int n) {
+    if (n >= kTrdChipMin && n <= kTrdChipMax) return std::max(trd_groups(B, n), std::min(B, 640));
+    return trd_groups(B, n);
 }
 
 int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t st) {
     const int B = w.B, n = w.n;
     const long long ldn = w.ldn;
-    PSVD_TRY(cudaMemsetAsync(w.bar, 0, sizeof(unsigned) * (size_t)w.groups * (trd_ctas_per_group(n) + 1), st));
+    PSVD_TRY(cudaMemsetAsync(w.bar, 0, sizeof(unsigned) * (size_t)w.groups * (std::max(trd_ctas_per_group(n), 15) + 1), st));
     PSVD_TRY(cudaMemsetAsync(w.err, 0, sizeof(unsigned) * 4, st));
     PSVD_TRY(cudaMemsetAsync(w.e, 0, sizeof(double) * (size_t)B * n, st));
     PSVD_TRY(cudaMemsetAsync(w.Vh, 0, sizeof(float) * (size_t)B * w.nrp * ldn, st));
     // 1. tridiagonalization
-    {
+    const bool prof = prof_on();
+    if (prof) prof_begin(st);
+    bool on_chip = false;
+    PSVD_TRY_RC(trd_chip(Hs, w, st, &on_chip));
+    if (!on_chip) {
         TrdParams P;
         P.H = Hs; P.Aw = w.Aw; P.Vh = w.Vh; P.tau = w.tau; P.d = w.d; P.e = w.e; P.pbuf = w.pbuf;
-        P.bar = w.bar; P.err = w.err; P.B = B; P.n = n; P.groups = w.groups; P.g = trd_ctas_per_group(n); P.nrp = w.nrp;
+        P.bar = w.bar; P.err = w.err; P.B = B; P.n = n; P.groups = std::min(w.groups, trd_groups(B, n)); P.g = trd_ctas_per_group(n); P.nrp = w.nrp;
         P.ldn = ldn;
         P.spin = barrier_spin();
         const size_t smem = sizeof(float) * 3 * (size_t)ldn;
         PSVD_TRY(cudaFuncSetAttribute(sytrd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int occ = 0;
         PSVD_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sytrd_kernel, kTrdThreads, smem));
-        if (occ * num_sms() < w.groups * P.g) return cuda_fail(cudaErrorCooperativeLaunchTooLarge, __FILE__, __LINE__);
+        if (occ * num_sms() < P.groups * P.g) return cuda_fail(cudaErrorCooperativeLaunchTooLarge, __FILE__, __LINE__);
         void *args[] = {&P};
-        const bool prof = prof_on();
-        if (prof) prof_begin(st);
-        PSVD_TRY(cudaLaunchCooperativeKernel((void *)sytrd_kernel, dim3(w.groups * P.g), dim3(kTrdThreads), args,
+        PSVD_TRY(cudaLaunchCooperativeKernel((void *)sytrd_kernel, dim3(P.groups * P.g), dim3(kTrdThreads), args,
                                              smem, st));
         count_launch(1);
-        if (prof) {
-            const double j = (double)std::max(0, n - 2);   // sum_{t=1}^{n-2} 8 t^2
-            prof_end(st, 8.0 * j * (j + 1) * (2 * j + 1) / 6.0 * B, PSVD_PROF_TRD);
-        }
+    }
+    if (prof) {
+        const double j = (double)std::max(0, n - 2);   // sum_{t=1}^{n-2} 8 t^2
+        prof_end(st, 8.0 * j * (j + 1) * (2 * j + 1) / 6.0 * B, PSVD_PROF_TRD);
     }
     // 2. eigenvalues
     double *tn = reinterpret_cast<double *>(w.S2hi);   // B doubles of scratch (S2 is free until stage 4)

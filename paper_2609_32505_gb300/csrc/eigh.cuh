@@ -7,16 +7,18 @@
 namespace psvd {
 
 constexpr int kWY = 128;   // reflectors per compact-WY block in the back-transform
+constexpr int kTrdChipMin = 3, kTrdChipMax = 4096;   // sizes whose tridiagonalization runs on chip (trd.cu)
 constexpr int kBtSplit = 8; // largest K split of the back-transform's V^T Y products
 
 struct EighWS {
     int B = 0, n = 0, nblk = 0, chunk = 0, nrp = 0;   // nrp: rows of Vh, padded to kWY
-    long long ldn = 0;
+    long long ldn = 0, ll_ld = 0;
     float *Aw = nullptr;          // working copy of H (n x n per matrix)
     float *Vh = nullptr;          // Householder vectors as rows (n x ldn), v_k[k+1] = 1
     float *tau = nullptr;         // [B][n]
     double *d = nullptr, *e = nullptr, *lam = nullptr;   // tridiagonal and eigenvalues [B][n]
     float *pbuf = nullptr;        // [groups][2][n]
+    unsigned long long *ll = nullptr;   // [groups][4][ll_ld] exchange words of the on-chip tridiagonalization
     unsigned *bar = nullptr;      // [groups] barrier counters
     float *Vhi = nullptr, *Vlo = nullptr;      // Householder rows split (n x ldn)
     float *Yhi = nullptr, *Ylo = nullptr;      // Householder vectors as columns (n x ldn)
@@ -49,6 +51,9 @@ struct EighWS {
         e = cv.template take<double>(B64 * n);
         lam = cv.template take<double>(B64 * n);
         pbuf = cv.template take<float>((long long)groups * 2 * ldn);
+        ll_ld = 128;
+        while (ll_ld < n && n <= kTrdChipMax) ll_ld *= 2;
+        ll = cv.template take<unsigned long long>((long long)groups * 4 * ll_ld);
         bar = cv.template take<unsigned>((long long)groups * (2 * 160 + 1) + 1);   // release + arrival flags per group
         Vhi = cv.template take<float>(B64 * np);
         Vlo = cv.template take<float>(B64 * np);
@@ -74,6 +79,10 @@ struct EighWS {
 };
 
 int eigh_groups(int B, int n);
+
+// Tridiagonalization of the B matrices Hs (n x n) on chip where the sizes allow it (*ran tells): fills
+// w.Vh (pre-zeroed), w.tau, w.d, w.e; w.bar zeroed by the caller.
+int trd_chip(const float *Hs, EighWS &w, cudaStream_t st, bool *ran);
 
 // Eigendecomposition of the symmetric matrices Hs (B x n x n, FP32, full storage).
 // Writes eigenvalues descending to S (B x n, may be null) and V^T split into
