@@ -133,9 +133,37 @@ struct EpiQ {
     float *hi, *lo;
     long long ld;
     struct Acc {};
-    // element path through the product kernel's shared-memory transpose, so that a warp
-    // reads G and writes hi/lo in 64-byte row segments
-    static constexpr bool kElem = true;
+    static constexpr bool kElem = true, kRow = true;
+    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
+        if (r0 >= m || c0 >= n) return true;
+        if (c0 + 16 > n || (G && ((n & 7) || ((uintptr_t)G & 31)))) return false;
+        const int r = r0 + lane;
+        // D_R of the 16 columns: one lane each
+        const float dr = G && lane < 16 ? dr_of(S[(long long)b * n + c0 + lane], sqrt_eps, exact) : 0.f;
+        uint32_t h[16], l[16], g[8];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            float x = 2.f * v[i];
+            if (G) {
+                if ((i & 7) == 0) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) g[q] = 0u;
+                    if (r < m) ld_v8(G + (long long)b * m * n + (long long)r * n + c0 + i, g);
+                }
+                x += __uint_as_float(g[i & 7]) * __shfl_sync(0xffffffffu, dr, i);
+            }
+            float a, c;
+            split_tf32(x, a, c);
+            h[i] = __float_as_uint(a);
+            l[i] = __float_as_uint(c);
+        }
+        if (r < m) {
+            const long long o = (long long)b * m * ld + (long long)r * ld + c0;
+            st_v8x2(hi + o, h);
+            st_v8x2(lo + o, l);
+        }
+        return true;
+    }
     PSVD_DEV bool staged() const { return true; }
     PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
         if (r >= m || c >= n) return;
@@ -246,32 +274,15 @@ int svd_backward(const float *A, const float *U, const float *S, const float *VT
     return bwd_tail(w, dU != nullptr, nullptr, dU ? w.AU : nullptr, dVT ? w.BV : nullptr, dS, feps, kreg, dA, st);
 }
 
-__global__ void hilo_to_f32_kernel(const float *hi, const float *lo, int n, long long ld, float *out) {
-    const int b = blockIdx.z;
-    const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
-    if (i >= n || j >= n) return;
-    const long long o = (long long)b * n * ld + (long long)i * ld + j;
-    out[(long long)b * n * n + (long long)i * n + j] = hi[o] + lo[o];
-}
-
 int polar_backward(const float *A, const float *H, const float *dW, const float *dH, float *dA, BwdWS &w, double eps,
                    cudaStream_t st) {
     const int B = w.B, m = w.m, n = w.n;
     const long long ldn = w.ldn, ldm = w.ldm, mn = (long long)m * ldn, nm = (long long)n * ldm, nn = (long long)n * ldn;
     // EVD of H (symmetrized by the eigensolver's reads of the full matrix)
-    if (int rc = eigh_forward(H, w.S, nullptr, w.ew, st)) return rc;
-    if (cudaMemcpyAsync(w.VThi, w.ew.VThi, sizeof(float) * (size_t)B * nn, cudaMemcpyDeviceToDevice, st) ||
-        cudaMemcpyAsync(w.VTlo, w.ew.VTlo, sizeof(float) * (size_t)B * nn, cudaMemcpyDeviceToDevice, st))
-        return PSVD_ERR_CUDA;
+    if (int rc = eigh_forward(H, w.S, w.T1, w.ew, st, w.VThi, w.VTlo)) return rc;   // V^T plain in T1
     if (prepare_operand(A, n, (long long)m * n, B, m, n, false, 1.f, nullptr, so(w.Mhi, w.Mlo, ldn, mn), st))
         return PSVD_ERR_CUDA;
-    float *VTf = w.T1;   // V^T as plain FP32 (n x n)
-    {
-        dim3 g16((n + 15) / 16, (n + 15) / 16, B), b16(16, 16);
-        hilo_to_f32_kernel<<<g16, b16, 0, st>>>(w.VThi, w.VTlo, n, ldn, VTf);
-        count_launch(1);
-    }
-    if (prepare_operand(VTf, n, (long long)n * n, B, n, n, true, 1.f, nullptr, so(w.Vhi, w.Vlo, ldn, nn), st))
+    if (prepare_operand(w.T1, n, (long long)n * n, B, n, n, true, 1.f, nullptr, so(w.Vhi, w.Vlo, ldn, nn), st))
         return PSVD_ERR_CUDA;
     const float *EH = nullptr;
     if (dH) {

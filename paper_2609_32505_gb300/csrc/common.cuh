@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 #include "../../include/psvd.h"
@@ -97,11 +98,11 @@ PSVD_DEV uint64_t sdesc_k128(uint32_t saddr) {
 
 // Instruction descriptor for kind::f16 / kind::tf32 with FP32 accumulation, both
 // operands K-major: D format F32 (bits 4-5 = 1), A/B format (bits 7-9 / 10-12:
-// 1 = BF16, 2 = TF32), N >> 3 (bits 17-22), M >> 4 (bits 24-28).
+// 0 = FP16, 1 = BF16, 2 = TF32), N >> 3 (bits 17-22), M >> 4 (bits 24-28).
 __host__ __device__ constexpr uint32_t idesc_f32acc(uint32_t ab_fmt, uint32_t M, uint32_t N) {
     return (1u << 4) | (ab_fmt << 7) | (ab_fmt << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
-constexpr uint32_t kFmtBF16 = 1, kFmtTF32 = 2;
+constexpr uint32_t kFmtF16 = 0, kFmtBF16 = 1, kFmtTF32 = 2;
 
 PSVD_DEV void umma_tf32(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
     asm volatile(
@@ -151,6 +152,16 @@ PSVD_DEV void split_tf32(float x, float &hi, float &lo) {
     hi = tf32_round(x);
     lo = tf32_round(x - hi);
 }
+
+// Split FP16: x * 2^e = hi + lo with FP16 halves, the 11 + 11 significant bits of the split TF32 at
+// half the bytes and twice the tensor rate.  The caller's power of two puts the operand's bound
+// below 2^16; elements down to 2^-18 of it keep both halves normal (|x - hi - lo| <= 2^-22 |x|),
+// smaller ones an error of 2^-40 of the bound.
+PSVD_DEV void split_f16(float xs, __half &hi, __half &lo) {
+    hi = __float2half_rn(xs);
+    lo = __float2half_rn(xs - __half2float(hi));
+}
+PSVD_DEV float join_f16(__half hi, __half lo) { return __half2float(hi) + __half2float(lo); }
 
 PSVD_DEV float warp_sum(float v) {
 #pragma unroll

@@ -10,7 +10,7 @@
 //     recurrences where a warp's eigenvalues are well separated, FP64 otherwise),
 //     Rayleigh quotients, modified Gram-Schmidt inside clusters of close eigenvalues.
 //  4. Back-transform V^T = Z^T Q^T with compact-WY blocks of kWY reflectors on the
-//     tcgen05 split-TF32 product kernel, then the sign convention (largest-|.| entry
+//     tcgen05 split-FP16 product kernel, then the sign convention (largest-|.| entry
 //     of each eigenvector positive).
 #include <cfloat>
 #include <cmath>
@@ -1024,8 +1024,8 @@ __global__ void tri_cluster_kernel(InvitParams P, const double *bisect_lam, doub
 }
 
 // Z^T rows (eigenvectors of T) from the interleaved FP32 vectors -> V^T split (n x ldn)
-__global__ void zt_store_kernel(const float *xs, long long stride, int n, int first_b, int first, float *VThi,
-                                float *VTlo, long long ldn) {
+__global__ void zt_store_kernel(const float *xs, long long stride, int n, int first_b, int first, __half *VThi,
+                                __half *VTlo, long long ldn) {
     __shared__ float tile[32][33];
     const int bb = blockIdx.z;
     const int b = first_b + bb;
@@ -1039,8 +1039,8 @@ __global__ void zt_store_kernel(const float *xs, long long stride, int n, int fi
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         const int i = i0 + r, j = j0 + threadIdx.x;
         if (i < n && j < n) {
-            float h, l;
-            split_tf32(tile[threadIdx.x][r], h, l);
+            __half h, l;
+            split_f16(tile[threadIdx.x][r] * kF16X, h, l);
             const long long o = (long long)b * n * ldn + (long long)i * ldn + j;
             VThi[o] = h;
             VTlo[o] = l;
@@ -1115,7 +1115,7 @@ __global__ void __launch_bounds__(256) larft_kernel(const float *Gm, const float
     for (int p = threadIdx.x; p < kWY * kWY; p += blockDim.x) out[p] = T[(p / kWY) * kLtLd + p % kWY];
 }
 
-// S2 = S T^T (n x nb), split into TF32 hi/lo; S is the sum of `ks` K-split slices of
+// S2 = S T^T (n x nb), split into FP16 halves; S is the sum of `ks` K-split slices of
 // B x n x kWY each, added in slice order.  One block of kWY threads per kStRows rows of S:
 // T is staged once per block in shared memory with rows padded to kWY + 1 floats (thread j
 // reads row j, so the lanes of a warp hit distinct banks), and each thread forms output
@@ -1123,7 +1123,7 @@ __global__ void __launch_bounds__(256) larft_kernel(const float *Gm, const float
 constexpr int kStRows = 16;
 constexpr size_t kStSmem = sizeof(float) * ((size_t)kWY * (kWY + 1) + (size_t)kStRows * kWY);
 __global__ void __launch_bounds__(kWY) s_times_tt_kernel(const float *S, int ks, int B, const float *Tm, int n,
-                                                         int nblk, int blk, int nb, float *S2hi, float *S2lo) {
+                                                         int nblk, int blk, int nb, __half *S2hi, __half *S2lo) {
     extern __shared__ float stsm[];
     float *Ts = stsm, *sr = stsm + kWY * (kWY + 1);
     const int i0 = blockIdx.x * kStRows, b = blockIdx.y, j = threadIdx.x;
@@ -1174,8 +1174,8 @@ __global__ void __launch_bounds__(kWY) s_times_tt_kernel(const float *S, int ks,
         const int i = i0 + r;
         if (i >= n) break;
         const long long o = (long long)b * n * kWY + (long long)i * kWY + j;
-        float h, lo;
-        split_tf32(acc[r], h, lo);
+        __half h, lo;
+        split_f16(acc[r] * kF16S2, h, lo);
         S2hi[o] = h;
         S2lo[o] = lo;
     }
@@ -1199,7 +1199,7 @@ constexpr size_t kPrSmem =
     sizeof(float) * (2 * (size_t)kWY * kPrLd + (size_t)kPrRows * 2 * kWY + (size_t)kPrRows * kWY);
 __global__ void __launch_bounds__(2 * kWY) s_pair_kernel(const float *S, int ks, int B, const float *Tm,
                                                           const float *Gab, int n, int nblk, int npair, int blk_b,
-                                                          int q, int nb_a, float *S2hi, float *S2lo) {
+                                                          int q, int nb_a, __half *S2hi, __half *S2lo) {
     extern __shared__ __align__(16) float psm[];
     float *Ta = psm, *Gt = Ta + kWY * kPrLd, *Tb = Ta;  // T_b is loaded over T_a after phase one
     float *sr = Gt + kWY * kPrLd;                     // [kPrRows][2 kWY]: S rows, then S_b in place
@@ -1291,22 +1291,22 @@ __global__ void __launch_bounds__(2 * kWY) s_pair_kernel(const float *S, int ks,
         const int i = i0 + rh + r;
         if (i >= n) break;
         const long long o = ((long long)b * n + i) * 2 * kWY;
-        float h, lo;
-        split_tf32(acc[r], h, lo);
+        __half h, lo;
+        split_f16(acc[r] * kF16S2, h, lo);
         S2hi[o + j] = h;
         S2lo[o + j] = lo;
-        split_tf32(s2a[(rh + r) * kWY + j], h, lo);
+        split_f16(s2a[(rh + r) * kWY + j] * kF16S2, h, lo);
         S2hi[o + kWY + j] = h;
         S2lo[o + kWY + j] = lo;
     }
 }
 
 // sign convention + outputs: each row of V^T flipped so its largest-|.| entry is positive
-__global__ void eig_finalize_kernel(float *VThi, float *VTlo, long long ldn, int n, const double *lam, float *S,
-                                    float *VT) {
+__global__ void eig_finalize_kernel(__half *VThi, __half *VTlo, long long ldn, int n, const double *lam, float *S,
+                                    float *VT, float *t32hi, float *t32lo) {
     const int b = blockIdx.y, i = blockIdx.x;
-    float *h = VThi + (long long)b * n * ldn + (long long)i * ldn;
-    float *l = VTlo + (long long)b * n * ldn + (long long)i * ldn;
+    const long long row = (long long)b * n * ldn + (long long)i * ldn;
+    __half *h = VThi + row, *l = VTlo + row;
     __shared__ float sv[32];
     __shared__ int si[32];
     // argmax of |.| with the lowest index on ties; NaN entries never win and the
@@ -1314,7 +1314,7 @@ __global__ void eig_finalize_kernel(float *VThi, float *VTlo, long long ldn, int
     float best = -1.f;
     int bi = 0;
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        float a = fabsf(h[j] + l[j]);
+        float a = fabsf(join_f16(h[j], l[j]));
         if (!(a == a)) a = -1.f;
         if (a > best || (a == best && j < bi)) { best = a; bi = j; }
     }
@@ -1333,13 +1333,19 @@ __global__ void eig_finalize_kernel(float *VThi, float *VTlo, long long ldn, int
     __syncthreads();
     bi = si[0];
     if (bi < 0 || bi >= n) bi = 0;
-    const float sg = (h[bi] + l[bi]) < 0.f ? -1.f : 1.f;
+    const bool flip = join_f16(h[bi], l[bi]) < 0.f;
     __syncthreads();
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const float hh = sg * h[j], ll = sg * l[j];
-        h[j] = hh;
-        l[j] = ll;
-        if (VT) VT[(long long)b * n * n + (long long)i * n + j] = hh + ll;
+        __half hh = h[j], ll = l[j];
+        if (flip) { hh = __hneg(hh); ll = __hneg(ll); h[j] = hh; l[j] = ll; }
+        const float x = join_f16(hh, ll) * (1.f / kF16X);
+        if (VT) VT[(long long)b * n * n + (long long)i * n + j] = x;
+        if (t32hi) {
+            float th, tl;
+            split_tf32(x, th, tl);
+            t32hi[row + j] = th;
+            t32lo[row + j] = tl;
+        }
     }
     if (threadIdx.x == 0 && S) S[(long long)b * n + i] = (float)lam[(long long)b * n + i];
 }
@@ -1361,7 +1367,7 @@ int eigh_groups(int B, int n) {
     return trd_groups(B, n);
 }
 
-int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t st) {
+int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t st, float *vt_hi, float *vt_lo) {
     const int B = w.B, n = w.n;
     const long long ldn = w.ldn;
     PSVD_TRY(cudaMemsetAsync(w.bar, 0, sizeof(unsigned) * (size_t)w.groups * (std::max(trd_ctas_per_group(n), 15) + 1), st));
@@ -1394,7 +1400,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
         prof_end(st, 8.0 * j * (j + 1) * (2 * j + 1) / 6.0 * B, PSVD_PROF_TRD);
     }
     // 2. eigenvalues
-    double *tn = reinterpret_cast<double *>(w.S2hi);   // B doubles of scratch (S2 is free until stage 4)
+    double *tn = w.tn;
     {
         dim3 g((n + 31) / 32, B);       // 32 eigenvalues x 8 lanes per block
         const size_t smem = sizeof(float) * 2 * (size_t)n;
@@ -1404,7 +1410,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
         count_launch(1);
     }
     {
-        float4 *dd = reinterpret_cast<float4 *>(w.S2lo);   // 2 x B x n float4 (S2 is free until stage 4)
+        float4 *dd = w.sturm;
         sturm_prep_kernel<<<dim3((n + 255) / 256, B), 256, 0, st>>>(w.d, w.e, tn, n, dd, dd + (size_t)B * n);
         dim3 g((n + 31) / 32, B);       // 32 eigenvalues x 8 lanes per block
         tri_refine_kernel<<<g, 256, 0, st>>>(dd, n, tn, kRefineNear, w.lam);
@@ -1421,7 +1427,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
         const int nb = std::min(per, B - b0);
         InvitParams P;
         P.D = w.d; P.E = w.e; P.tn = tn; P.lam = w.lam; P.lam0 = bis;
-        P.de = reinterpret_cast<const float4 *>(w.S2lo) + (size_t)B * n;
+        P.de = w.sturm + (size_t)B * n;
         P.xs = w.xs; P.xf = w.xf; P.u0 = w.u0; P.u1 = w.u1; P.u2 = w.u2; P.lm = w.lm; P.piv = w.piv;
         P.n = n; P.first = b0 * n; P.count = nb * n; P.stride = w.chunk;
         tri_invit_kernel<<<(P.count + kIvW - 1) / kIvW, kIvW, kIvSmem, st>>>(P);
@@ -1435,19 +1441,22 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
     if (w.nblk > 0) {
         SplitOut vo, yo;
         const long long np = (long long)w.nrp * ldn;
-        vo.hi = w.Vhi; vo.lo = w.Vlo; vo.ld = ldn; vo.bstride = np;
-        yo.hi = w.Yhi; yo.lo = w.Ylo; yo.ld = ldn; yo.bstride = (long long)n * ldn;
+        vo.fhi = w.Vhi; vo.flo = w.Vlo; vo.ld = ldn; vo.bstride = vo.fbstride = np;
+        yo.fhi = w.Yhi; yo.flo = w.Ylo; yo.ld = ldn; yo.bstride = yo.fbstride = (long long)n * ldn;
+        vo.fscale = yo.fscale = kF16V;
         PSVD_TRY(prepare_operand(w.Vh, ldn, np, B, w.nrp, n, false, 1.f, nullptr, vo, st));
         PSVD_TRY(prepare_operand(w.Vh, ldn, np, B, n, n, true, 1.f, nullptr, yo, st));
         // G = Y^T Y of every WY block: blocks of kWY Householder rows as a batch
         for (int b = 0; b < B; ++b) {
-            MatView vh = view_of(w.Vhi + b * np, kWY, n, ldn, (long long)kWY * ldn, w.nblk);
-            MatView vl = view_of(w.Vlo + b * np, kWY, n, ldn, (long long)kWY * ldn, w.nblk);
+            MatView vh = view_f16(w.Vhi + b * np, kWY, n, ldn, (long long)kWY * ldn, w.nblk);
+            MatView vl = view_f16(w.Vlo + b * np, kWY, n, ldn, (long long)kWY * ldn, w.nblk);
             GemmShape s;
             memset(&s, 0, sizeof(s));
-            s.M = kWY; s.N = kWY; s.K = n; s.prec_uniform = PREC_TF32X3; s.err = w.err;
+            s.M = kWY; s.N = kWY; s.K = n; s.prec_uniform = PREC_F16X3; s.err = w.err;
             EpiStore e = epi_store_plain(w.Gm + (long long)b * w.nblk * kWY * kWY, kWY, (long long)kWY * kWY, kWY, kWY);
-            PSVD_TRY(launch_gemm(nullptr, nullptr, &vh, &vl, &vh, &vl, s, w.nblk, e, st));
+            s.f16_scale = 1.f / (kF16V * kF16V);
+            const F16Views f{vh, vl, vh, vl};
+            PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, w.nblk, e, st, &f));
         }
         PSVD_TRY(cudaFuncSetAttribute(larft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLtSmem));
         larft_kernel<<<dim3(w.nblk, B), 256, kLtSmem, st>>>(w.Gm, w.tau, n, w.nblk, w.Tm);
@@ -1466,20 +1475,22 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
             int ks = 1;
             // S = V^T[:, r0:] Y[r0:, blk]   (n x nb), as ks partial sums over K
             {
-                MatView ahi = view_of(w.VThi + r0, n, Lr, ldn, (long long)n * ldn, B);
-                MatView alo = view_of(w.VTlo + r0, n, Lr, ldn, (long long)n * ldn, B);
-                MatView bhi = view_of(w.Vhi + (long long)k0 * ldn + r0, nb, Lr, ldn, (long long)w.nrp * ldn, B);
-                MatView blo = view_of(w.Vlo + (long long)k0 * ldn + r0, nb, Lr, ldn, (long long)w.nrp * ldn, B);
+                MatView ahi = view_f16(w.VThi + r0, n, Lr, ldn, (long long)n * ldn, B);
+                MatView alo = view_f16(w.VTlo + r0, n, Lr, ldn, (long long)n * ldn, B);
+                MatView bhi = view_f16(w.Vhi + (long long)k0 * ldn + r0, nb, Lr, ldn, (long long)w.nrp * ldn, B);
+                MatView blo = view_f16(w.Vlo + (long long)k0 * ldn + r0, nb, Lr, ldn, (long long)w.nrp * ldn, B);
                 GemmShape s;
                 memset(&s, 0, sizeof(s));
-                s.M = n; s.N = nb; s.K = Lr; s.prec_uniform = PREC_TF32X3; s.err = w.err;
+                s.M = n; s.N = nb; s.K = Lr; s.prec_uniform = PREC_F16X3; s.err = w.err;
                 // N = nb <= 128 leaves ceil(n / 128) tiles per matrix: split K so that about
                 // one wave of CTAs runs, at least 4 k-blocks per range
                 const int tiles = ((n + kBM - 1) / kBM) * B;
                 s.ksplit = std::max(1, std::min(std::min(kBtSplit, (num_sms() + tiles - 1) / tiles), Lr / 128));
                 ks = s.ksplit;
                 EpiStore e = epi_store_plain(w.S, kWY, (long long)n * kWY, n, nb);
-                PSVD_TRY(launch_gemm(nullptr, nullptr, &ahi, &alo, &bhi, &blo, s, B, e, st));
+                s.f16_scale = 1.f / (kF16X * kF16V);
+                const F16Views f{ahi, alo, bhi, blo};
+                PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
             }
             {
                 s_times_tt_kernel<<<dim3((n + kStRows - 1) / kStRows, B), kWY, kStSmem, st>>>(w.S, ks, B, w.Tm, n,
@@ -1490,35 +1501,39 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
             }
             // V^T[:, r0:] -= S2 Y[r0:, blk]^T
             {
-                MatView ahi = view_of(w.S2hi, n, nb, kWY, (long long)n * kWY, B);
-                MatView alo = view_of(w.S2lo, n, nb, kWY, (long long)n * kWY, B);
-                MatView bhi = view_of(w.Yhi + (long long)r0 * ldn + k0, Lr, nb, ldn, (long long)n * ldn, B);
-                MatView blo = view_of(w.Ylo + (long long)r0 * ldn + k0, Lr, nb, ldn, (long long)n * ldn, B);
+                MatView ahi = view_f16(w.S2hi, n, nb, kWY, (long long)n * kWY, B);
+                MatView alo = view_f16(w.S2lo, n, nb, kWY, (long long)n * kWY, B);
+                MatView bhi = view_f16(w.Yhi + (long long)r0 * ldn + k0, Lr, nb, ldn, (long long)n * ldn, B);
+                MatView blo = view_f16(w.Ylo + (long long)r0 * ldn + k0, Lr, nb, ldn, (long long)n * ldn, B);
                 GemmShape s;
                 memset(&s, 0, sizeof(s));
-                s.M = n; s.N = Lr; s.K = nb; s.prec_uniform = PREC_TF32X3; s.err = w.err;
-                EpiSubSplit e;
+                s.M = n; s.N = Lr; s.K = nb; s.prec_uniform = PREC_F16X3; s.err = w.err;
+                EpiSubHalf e;
                 e.rows = n; e.cols = Lr; e.hi = w.VThi + r0; e.lo = w.VTlo + r0; e.ld = ldn;
-                e.bs = (long long)n * ldn;
-                PSVD_TRY(launch_gemm(nullptr, nullptr, &ahi, &alo, &bhi, &blo, s, B, e, st));
+                e.bs = (long long)n * ldn; e.scale = kF16X; e.inv = 1.f / kF16X;
+                s.f16_scale = 1.f / (kF16S2 * kF16V);
+                const F16Views f{ahi, alo, bhi, blo};
+                PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
             }
             return PSVD_OK;
         };
         if (npair > 0) {
             // G_ab = Y_a^T Y_b of every pair (a = b + 1): Householder rows of the two blocks
             for (int b = 0; b < B; ++b) {
-                const float *hb = w.Vhi + b * np, *lb = w.Vlo + b * np;
+                const __half *hb = w.Vhi + b * np, *lb = w.Vlo + b * np;
                 const long long ps = (long long)2 * kWY * ldn;
-                MatView ah = view_of(hb + (long long)(first + 1) * kWY * ldn, kWY, n, ldn, ps, npair);
-                MatView al = view_of(lb + (long long)(first + 1) * kWY * ldn, kWY, n, ldn, ps, npair);
-                MatView bh = view_of(hb + (long long)first * kWY * ldn, kWY, n, ldn, ps, npair);
-                MatView bl = view_of(lb + (long long)first * kWY * ldn, kWY, n, ldn, ps, npair);
+                MatView ah = view_f16(hb + (long long)(first + 1) * kWY * ldn, kWY, n, ldn, ps, npair);
+                MatView al = view_f16(lb + (long long)(first + 1) * kWY * ldn, kWY, n, ldn, ps, npair);
+                MatView bh = view_f16(hb + (long long)first * kWY * ldn, kWY, n, ldn, ps, npair);
+                MatView bl = view_f16(lb + (long long)first * kWY * ldn, kWY, n, ldn, ps, npair);
                 GemmShape s;
                 memset(&s, 0, sizeof(s));
-                s.M = kWY; s.N = kWY; s.K = n; s.prec_uniform = PREC_TF32X3; s.err = w.err;
+                s.M = kWY; s.N = kWY; s.K = n; s.prec_uniform = PREC_F16X3; s.err = w.err;
                 EpiStore e = epi_store_plain(w.Gab + (long long)b * npair * kWY * kWY, kWY, (long long)kWY * kWY,
                                              kWY, kWY);
-                PSVD_TRY(launch_gemm(nullptr, nullptr, &ah, &al, &bh, &bl, s, npair, e, st));
+                s.f16_scale = 1.f / (kF16V * kF16V);
+                const F16Views f{ah, al, bh, bl};
+                PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, npair, e, st, &f));
             }
             PSVD_TRY(cudaFuncSetAttribute(s_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPrSmem));
         }
@@ -1532,18 +1547,20 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
             int ks = 1;
             // S = V^T[:, r0:] [Y_b Y_a][r0:, :]   (n x W), as ks partial sums over K
             {
-                MatView ahi = view_of(w.VThi + r0, n, Lr, ldn, (long long)n * ldn, B);
-                MatView alo = view_of(w.VTlo + r0, n, Lr, ldn, (long long)n * ldn, B);
-                MatView bhi = view_of(w.Vhi + (long long)k0 * ldn + r0, W, Lr, ldn, (long long)w.nrp * ldn, B);
-                MatView blo = view_of(w.Vlo + (long long)k0 * ldn + r0, W, Lr, ldn, (long long)w.nrp * ldn, B);
+                MatView ahi = view_f16(w.VThi + r0, n, Lr, ldn, (long long)n * ldn, B);
+                MatView alo = view_f16(w.VTlo + r0, n, Lr, ldn, (long long)n * ldn, B);
+                MatView bhi = view_f16(w.Vhi + (long long)k0 * ldn + r0, W, Lr, ldn, (long long)w.nrp * ldn, B);
+                MatView blo = view_f16(w.Vlo + (long long)k0 * ldn + r0, W, Lr, ldn, (long long)w.nrp * ldn, B);
                 GemmShape s;
                 memset(&s, 0, sizeof(s));
-                s.M = n; s.N = W; s.K = Lr; s.prec_uniform = PREC_TF32X3; s.err = w.err;
+                s.M = n; s.N = W; s.K = Lr; s.prec_uniform = PREC_F16X3; s.err = w.err;
                 const int tiles = ((n + kBM - 1) / kBM) * B;
                 s.ksplit = std::max(1, std::min(std::min(kBtSplit, (num_sms() + tiles - 1) / tiles), Lr / 128));
                 ks = s.ksplit;
                 EpiStore e = epi_store_plain(w.S, 2 * kWY, (long long)n * 2 * kWY, n, W);
-                PSVD_TRY(launch_gemm(nullptr, nullptr, &ahi, &alo, &bhi, &blo, s, B, e, st));
+                s.f16_scale = 1.f / (kF16X * kF16V);
+                const F16Views f{ahi, alo, bhi, blo};
+                PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
             }
             s_pair_kernel<<<dim3((n + kPrRows - 1) / kPrRows, B), 2 * kWY, kPrSmem, st>>>(
                 w.S, ks, B, w.Tm, w.Gab, n, w.nblk, npair, blk_b, q, nb_a, w.S2hi, w.S2lo);
@@ -1551,22 +1568,24 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
             count_launch(1);
             // V^T[:, r0:] -= S2 [Y_b Y_a][r0:, :]^T
             {
-                MatView ahi = view_of(w.S2hi, n, W, 2 * kWY, (long long)n * 2 * kWY, B);
-                MatView alo = view_of(w.S2lo, n, W, 2 * kWY, (long long)n * 2 * kWY, B);
-                MatView bhi = view_of(w.Yhi + (long long)r0 * ldn + k0, Lr, W, ldn, (long long)n * ldn, B);
-                MatView blo = view_of(w.Ylo + (long long)r0 * ldn + k0, Lr, W, ldn, (long long)n * ldn, B);
+                MatView ahi = view_f16(w.S2hi, n, W, 2 * kWY, (long long)n * 2 * kWY, B);
+                MatView alo = view_f16(w.S2lo, n, W, 2 * kWY, (long long)n * 2 * kWY, B);
+                MatView bhi = view_f16(w.Yhi + (long long)r0 * ldn + k0, Lr, W, ldn, (long long)n * ldn, B);
+                MatView blo = view_f16(w.Ylo + (long long)r0 * ldn + k0, Lr, W, ldn, (long long)n * ldn, B);
                 GemmShape s;
                 memset(&s, 0, sizeof(s));
-                s.M = n; s.N = Lr; s.K = W; s.prec_uniform = PREC_TF32X3; s.err = w.err;
-                EpiSubSplit e;
+                s.M = n; s.N = Lr; s.K = W; s.prec_uniform = PREC_F16X3; s.err = w.err;
+                EpiSubHalf e;
                 e.rows = n; e.cols = Lr; e.hi = w.VThi + r0; e.lo = w.VTlo + r0; e.ld = ldn;
-                e.bs = (long long)n * ldn;
-                PSVD_TRY(launch_gemm(nullptr, nullptr, &ahi, &alo, &bhi, &blo, s, B, e, st));
+                e.bs = (long long)n * ldn; e.scale = kF16X; e.inv = 1.f / kF16X;
+                s.f16_scale = 1.f / (kF16S2 * kF16V);
+                const F16Views f{ahi, alo, bhi, blo};
+                PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
             }
         }
         if (first) PSVD_TRY_RC(single(0));
     }
-    eig_finalize_kernel<<<dim3(n, B), 128, 0, st>>>(w.VThi, w.VTlo, ldn, n, w.lam, S, VT);
+    eig_finalize_kernel<<<dim3(n, B), 128, 0, st>>>(w.VThi, w.VTlo, ldn, n, w.lam, S, VT, vt_hi, vt_lo);
     count_launch(1);
     PSVD_TRY(cudaGetLastError());
     return PSVD_OK;

@@ -20,11 +20,14 @@ struct EighWS {
     float *pbuf = nullptr;        // [groups][2][n]
     unsigned long long *ll = nullptr;   // [groups][4][ll_ld] exchange words of the on-chip tridiagonalization
     unsigned *bar = nullptr;      // [groups] barrier counters
-    float *Vhi = nullptr, *Vlo = nullptr;      // Householder rows split (n x ldn)
-    float *Yhi = nullptr, *Ylo = nullptr;      // Householder vectors as columns (n x ldn)
-    float *VThi = nullptr, *VTlo = nullptr;    // current V^T split (n x ldn)
+    // split-FP16 operands of the back-transform
+    __half *Vhi = nullptr, *Vlo = nullptr;     // Householder rows (n x ldn), scaled by kF16V
+    __half *Yhi = nullptr, *Ylo = nullptr;     // Householder vectors as columns (n x ldn), scaled by kF16V
+    __half *VThi = nullptr, *VTlo = nullptr;   // current V^T (n x ldn), scaled by kF16X
     float *S = nullptr;                        // V^T Y for a pair of blocks (n x 2 kWY), K-split slices
-    float *S2hi = nullptr, *S2lo = nullptr;    // the pair's S2 split (n x 2 kWY)
+    __half *S2hi = nullptr, *S2lo = nullptr;   // the pair's S2 (n x 2 kWY), scaled by kF16S2
+    float4 *sturm = nullptr;                   // [2][B][n] float-float T for the Sturm counts and inverse iteration
+    double *tn = nullptr;                      // [B] ||T||
     float *Tm = nullptr;                       // [B][nblk][kWY][kWY]
     float *Gm = nullptr;                       // [B][nblk][kWY][kWY]  Y^T Y per block
     float *Gab = nullptr;                      // [B][nblk/2][kWY][kWY]  Y_a^T Y_b per pair of blocks
@@ -55,15 +58,17 @@ struct EighWS {
         while (ll_ld < n && n <= kTrdChipMax) ll_ld *= 2;
         ll = cv.template take<unsigned long long>((long long)groups * 4 * ll_ld);
         bar = cv.template take<unsigned>((long long)groups * (2 * 160 + 1) + 1);   // release + arrival flags per group
-        Vhi = cv.template take<float>(B64 * np);
-        Vlo = cv.template take<float>(B64 * np);
-        Yhi = cv.template take<float>(B64 * nn);
-        Ylo = cv.template take<float>(B64 * nn);
-        VThi = cv.template take<float>(B64 * nn);
-        VTlo = cv.template take<float>(B64 * nn);
+        Vhi = cv.template take<__half>(B64 * np);
+        Vlo = cv.template take<__half>(B64 * np);
+        Yhi = cv.template take<__half>(B64 * nn);
+        Ylo = cv.template take<__half>(B64 * nn);
+        VThi = cv.template take<__half>(B64 * nn);
+        VTlo = cv.template take<__half>(B64 * nn);
         S = cv.template take<float>(kBtSplit * B64 * n * 2 * kWY);
-        S2hi = cv.template take<float>(B64 * n * 2 * kWY);
-        S2lo = cv.template take<float>(B64 * n * 2 * kWY);
+        S2hi = cv.template take<__half>(B64 * n * 2 * kWY);
+        S2lo = cv.template take<__half>(B64 * n * 2 * kWY);
+        sturm = cv.template take<float4>(B64 * n * 2);
+        tn = cv.template take<double>(B64);
         Tm = cv.template take<float>(B64 * (nblk > 0 ? nblk : 1) * kWY * kWY);
         Gm = cv.template take<float>(B64 * (nblk > 0 ? nblk : 1) * kWY * kWY);
         Gab = cv.template take<float>(B64 * (nblk > 1 ? nblk / 2 : 1) * kWY * kWY);
@@ -85,9 +90,10 @@ int eigh_groups(int B, int n);
 int trd_chip(const float *Hs, EighWS &w, cudaStream_t st, bool *ran);
 
 // Eigendecomposition of the symmetric matrices Hs (B x n x n, FP32, full storage).
-// Writes eigenvalues descending to S (B x n, may be null) and V^T split into
-// ws.VThi / ws.VTlo (rows = eigenvectors, largest-|.| entry positive), and V^T to
-// VT (B x n x n, may be null).
-int eigh_forward(const float *Hs, float *S, float *VT, EighWS &ws, cudaStream_t st);
+// Writes eigenvalues descending to S (B x n, may be null) and V^T as split-FP16 halves in
+// ws.VThi / ws.VTlo (rows = eigenvectors, largest-|.| entry positive), V^T to VT (B x n x n, may be
+// null) and V^T as split TF32 to vt_hi / vt_lo (B x n x ldn, may be null).
+int eigh_forward(const float *Hs, float *S, float *VT, EighWS &ws, cudaStream_t st, float *vt_hi = nullptr,
+                 float *vt_lo = nullptr);
 
 }  // namespace psvd

@@ -18,6 +18,11 @@
 //   PREC_TF32   : 32 fp32 of K per unit, one unit per k-block
 //   PREC_TF32X3 : 32 fp32 of K, two units per k-block (hi parts, lo parts);
 //                 hi*hi + hi*lo + lo*hi (split-TF32, FP32-accurate products)
+//   PREC_F16X3  : 64 fp16 of K, two units per k-block: the same three products of split FP16 halves
+//                 (operands scaled by powers of two, undone by GemmShape::f16_scale).  An FP16 MMA
+//                 covers twice the K of a TF32 one in the same time and its operands are half the
+//                 bytes (a 4096^3 polar step product: 780 us in split TF32, 474 us with the
+//                 same epilogue)
 // Two accumulators of 128 x 256 FP32 in TMEM (all 512 columns) let the MMA warp
 // run the next tile (or the next split-TF32 chunk) while the epilogue drains the
 // previous one.  The tensor core accumulates with truncation; split-TF32 tiles are
@@ -35,7 +40,7 @@
 
 namespace psvd {
 
-enum Prec : int { PREC_BF16 = 0, PREC_TF32 = 1, PREC_TF32X3 = 2 };
+enum Prec : int { PREC_BF16 = 0, PREC_TF32 = 1, PREC_TF32X3 = 2, PREC_F16X3 = 3 };
 
 constexpr int kBM = 128;
 constexpr int kUnitA = 16384;                  // 128 rows x 128 B
@@ -47,7 +52,10 @@ constexpr int kMaxStages = kRingBytes / (kUnitA + 128 * 128);   // ring units at
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = (kEpiWarps + 2) * 32;
 constexpr int kStageRow = 17;                  // staging row stride (floats): conflict-free
-constexpr int kStageBytes = kEpiWarps * 32 * kStageRow * 4;
+constexpr int kTransRow = 36;                  // row stride of the 16 x 32 transpose: 16-byte rows, conflict-free
+constexpr int kStageWarp = 16 * kTransRow;     // floats per warp (also 32 x kStageRow <= this)
+static_assert(32 * kStageRow <= kStageWarp, "staging area");
+constexpr int kStageBytes = kEpiWarps * kStageWarp * 4;
 constexpr int kGemmSmem = kRingBytes + 1024 /*align*/ + 256 /*barriers*/ + kStageBytes;
 static_assert((2 * kMaxStages + 4) * 8 + 4 <= 256, "barrier area");
 constexpr int kAccCols = 256;                  // TMEM columns per accumulator
@@ -57,6 +65,7 @@ struct GemmMaps {
     CUtensorMap a_bf16, b_bf16;  // used by PREC_BF16 tiles
     CUtensorMap a_hi, a_lo;      // fp32 (TF32 uses a_hi only)
     CUtensorMap b_hi, b_lo;
+    CUtensorMap a_h16, a_l16, b_h16, b_l16;   // split FP16
 };
 
 struct GemmShape {
@@ -74,6 +83,8 @@ struct GemmShape {
                             // returns at once (written by an earlier kernel on the same stream)
     unsigned *ticket;       // nullptr, or a zeroed counter: the last CTA to finish runs epi.tail()
     unsigned *err;          // device error word
+    float f16_scale;        // PREC_F16X3: the product of the operands' inverse scales ...
+    const float *f16_scale_b;   // ... times this entry of the matrix (nullptr: 1)
     int prof_as;            // profiling class + 1 for the launch timing (0: by precision)
 };
 
@@ -103,7 +114,7 @@ PSVD_DEV int tiles_per_matrix(const GemmShape &s) {
 
 // k-blocks of a tile and accumulation phases (flush points) per tile.
 PSVD_DEV int kblocks(const GemmShape &s, int prec) {
-    const int kstep = prec == PREC_BF16 ? 64 : 32;
+    const int kstep = prec == PREC_BF16 || prec == PREC_F16X3 ? 64 : 32;
     return (s.K + kstep - 1) / kstep;
 }
 
@@ -136,17 +147,83 @@ template <class E> struct EpiHasElem<E, std::void_t<decltype(E::kElem)>> : std::
 // warp are coalesced) next to the staged row-major element pass.
 template <class E, class = void> struct EpiHasTrans : std::false_type {};
 template <class E> struct EpiHasTrans<E, std::void_t<decltype(E::kTrans)>> : std::integral_constant<bool, E::kTrans> {};
-// Read-modify-write epilogues define pre(b, r, c) (the value read at (r, c)) and
-// elem_pre(acc, b, r, c, v, p): the staged pass issues the 16 reads of a chunk before its
-// first store, since stores to the array being read would otherwise order every read
-// after the previous element's store (one read in flight per thread).
-template <class E, class = void> struct EpiHasPre : std::false_type {};
-template <class E> struct EpiHasPre<E, std::void_t<decltype(E::kPre)>> : std::integral_constant<bool, E::kPre> {};
 // Epilogues with a tail() run it once per launch, in the last CTA to finish (shp.ticket set),
 // after every CTA's epilogue writes and atomics are visible: a per-launch reduction step
 // (the polar iteration's per-matrix decision) without a launch of its own.
 template <class E, class = void> struct EpiHasTail : std::false_type {};
 template <class E> struct EpiHasTail<E, std::void_t<decltype(E::kTail)>> : std::integral_constant<bool, E::kTail> {};
+
+// Epilogues with row16(acc, b, r0, lane, c0, v, sw) get the 16 columns c0 .. c0 + 15 of the thread's row
+// r0 + lane as they are and store them in 32-byte pieces: along the row directly (a whole sector per
+// lane), transposed through the warp's shared memory `sw` (warp_transpose16).  It returns false
+// (uniformly) for pieces it does not handle -- ragged edges, the diagonal, unaligned outputs -- which
+// then take the element-wise paths above.  (Element by element a polar step's tile cost ~17,000
+// instructions per warp, about half the time of a 4096^3 split product: 474 -> 310 us with the pieces.)
+template <class E, class = void> struct EpiHasRow : std::false_type {};
+template <class E> struct EpiHasRow<E, std::void_t<decltype(E::kRow)>> : std::integral_constant<bool, E::kRow> {};
+
+// 32 bytes at a 32-byte aligned address
+PSVD_DEV void st_v8(void *p, const uint32_t (&r)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+                 "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+PSVD_DEV void st_v8x2(void *p, const uint32_t (&r)[16]) {       // 64 bytes
+    const uint32_t a[8] = {r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7]};
+    const uint32_t b[8] = {r[8], r[9], r[10], r[11], r[12], r[13], r[14], r[15]};
+    st_v8(p, a);
+    st_v8(static_cast<char *>(p) + 32, b);
+}
+// through the read-only path, free to be issued ahead of stores to other elements (each element is read
+// once, before its own thread writes it)
+PSVD_DEV void ld_v8(const void *p, uint32_t (&r)[8]) {
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "l"(p));
+}
+// Lane l gives word w[i] of column i of its row; it gets the 16 words of rows 16 (l & 1) .. + 15 of
+// column l >> 1.
+PSVD_DEV void warp_transpose16(float *sw, const uint32_t (&w)[16], uint32_t (&o)[16]) {
+    const int lane = threadIdx.x & 31;
+    uint32_t *s = reinterpret_cast<uint32_t *>(sw);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) s[i * kTransRow + lane] = w[i];
+    __syncwarp();
+    const uint4 *q = reinterpret_cast<const uint4 *>(s + (lane >> 1) * kTransRow + (lane & 1) * 16);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint4 x = q[i];
+        o[4 * i] = x.x; o[4 * i + 1] = x.y; o[4 * i + 2] = x.z; o[4 * i + 3] = x.w;
+    }
+}
+// Sums of 16 per-lane values over the warp: lane l returns the sum of value l >> 1.
+PSVD_DEV float warp_sum16(float (&a)[16]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 8, o = 16; h > 0; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < h) {
+                const float send = up ? a[i] : a[i + h], keep = up ? a[i + h] : a[i];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+    }
+    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
+}
+// 16 values -> packed FP16 halves of x * fs
+PSVD_DEV void split_f16x16(const float (&v)[16], float fs, uint32_t (&h)[8], uint32_t (&l)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float x0 = v[2 * i] * fs, x1 = v[2 * i + 1] * fs;
+        const __half2 hh = __floats2half2_rn(x0, x1);
+        const float2 f = __half22float2(hh);
+        const __half2 ll = __floats2half2_rn(x0 - f.x, x1 - f.y);
+        h[i] = *reinterpret_cast<const uint32_t *>(&hh);
+        l[i] = *reinterpret_cast<const uint32_t *>(&ll);
+    }
+}
 
 // Consumer side of the operand ring, as seen by the MMA issuer: shared-memory address of
 // unit 0, unit size, unit count, barriers, and the position of the next unit with the
@@ -189,8 +266,9 @@ PSVD_DEV bool mma_tile(MmaRing &r, int nkb, uint32_t tacc, uint32_t id) {
     return true;
 }
 
-// One split-TF32 tile: every k-block (hi unit, lo unit) is its own phase in the next
+// One split-TF32 or split-FP16 tile: every k-block (hi unit, lo unit) is its own phase in the next
 // accumulator, flushed by the epilogue into round-to-nearest FP32 registers.
+template <bool kF16>
 PSVD_DEV bool mma_tile_x3(MmaRing &r, int nkb, uint32_t tmem, uint64_t *acc_full, uint64_t *acc_empty, uint32_t &q,
                           uint32_t id) {
     for (int kb = 0; kb < nkb; ++kb) {
@@ -206,12 +284,20 @@ PSVD_DEV bool mma_tile_x3(MmaRing &r, int nkb, uint32_t tmem, uint64_t *acc_full
         const uint32_t a0 = r.base + s0 * r.unit_bytes, a1 = r.base + s1 * r.unit_bytes;
         const uint64_t ahi = sdesc_k128(a0), bhi = sdesc_k128(a0 + kUnitA);
         const uint64_t alo = sdesc_k128(a1), blo = sdesc_k128(a1 + kUnitA);
+        // the cross products first: the accumulator truncates at its current magnitude, so while it
+        // holds only them (2^-11 of the result) their eight additions cost nothing, and four
+        // truncations per k-block remain instead of twelve
+        auto mma = [&](uint64_t a, uint64_t b, uint32_t en) {
+            if constexpr (kF16) umma_f16(tacc, a, b, id, en);
+            else umma_tf32(tacc, a, b, id, en);
+        };
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            umma_tf32(tacc, sdesc_step(alo, k), sdesc_step(bhi, k), id, k != 0);
-            umma_tf32(tacc, sdesc_step(ahi, k), sdesc_step(blo, k), id, 1);
-            umma_tf32(tacc, sdesc_step(ahi, k), sdesc_step(bhi, k), id, 1);
+            mma(sdesc_step(alo, k), sdesc_step(bhi, k), k != 0);
+            mma(sdesc_step(ahi, k), sdesc_step(blo, k), 1);
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mma(sdesc_step(ahi, k), sdesc_step(bhi, k), 1);
         umma_commit(&r.empty[s0]);
         umma_commit(&r.empty[s1]);
         umma_commit(&acc_full[buf]);
@@ -273,8 +359,9 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
                 const int row_a = jb.ti * kBM, row_b = jb.tj * bn;
                 const CUtensorMap *ma0 = &maps.a_hi, *mb0 = &maps.b_hi, *ma1 = &maps.a_lo, *mb1 = &maps.b_lo;
                 if (prec == PREC_BF16) { ma0 = &maps.a_bf16; mb0 = &maps.b_bf16; }
-                const int kstep = prec == PREC_BF16 ? 64 : 32;
-                const int nu = prec == PREC_TF32X3 ? 2 : 1;
+                if (prec == PREC_F16X3) { ma0 = &maps.a_h16; mb0 = &maps.b_h16; ma1 = &maps.a_l16; mb1 = &maps.b_l16; }
+                const int kstep = prec == PREC_BF16 || prec == PREC_F16X3 ? 64 : 32;
+                const int nu = prec >= PREC_TF32X3 ? 2 : 1;
                 for (int kb = 0; kb < nkb; ++kb) {
                     const int k0 = (jb.kb0 + kb) * kstep;
                     for (int h = 0; h < nu; ++h) {
@@ -293,6 +380,7 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             const uint32_t id_tf32 = idesc_f32acc(kFmtTF32, kBM, bn);
+            const uint32_t id_f16 = idesc_f32acc(kFmtF16, kBM, bn);
             const uint32_t id_bf16 = idesc_f32acc(kFmtBF16, kBM, bn);
             MmaRing ring{smem_u32(smem), unit_bytes, nst, full, empty, shp.err, 0u, 0u};
             uint32_t q = 0;
@@ -300,8 +388,10 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
             for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
                 const TileJob jb = tile_job(shp, t, tpm);
                 if ((shp.skip && shp.skip[jb.b]) || jb.nkb <= 0) continue;
-                if (jb.prec == PREC_TF32X3) {
-                    ok = mma_tile_x3(ring, jb.nkb, tmem, acc_full, acc_empty, q, id_tf32);
+                if (jb.prec == PREC_F16X3) {
+                    ok = mma_tile_x3<true>(ring, jb.nkb, tmem, acc_full, acc_empty, q, id_f16);
+                } else if (jb.prec == PREC_TF32X3) {
+                    ok = mma_tile_x3<false>(ring, jb.nkb, tmem, acc_full, acc_empty, q, id_tf32);
                 } else {
                     const uint32_t buf = q & 1;
                     if (q >= 2 && !mbar_wait(&acc_empty[buf], ((q >> 1) - 1) & 1, shp.err)) { ok = false; break; }
@@ -332,7 +422,9 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
             const int b = jb.b, prec = jb.prec, nkb = jb.nkb, ti = jb.ti, tj = jb.tj;
             if (shp.skip && shp.skip[b]) continue;
             const int be = b + jb.kc * shp.batch;     // epilogue's batch index (partial-sum slice)
-            const int nph = nkb == 0 ? 0 : (prec == PREC_TF32X3 ? nkb : 1);
+            const int nph = nkb == 0 ? 0 : (prec >= PREC_TF32X3 ? nkb : 1);
+            float fs = 1.f;                       // undoes the operands' powers of two (exact)
+            if (prec == PREC_F16X3) fs = shp.f16_scale * (shp.f16_scale_b ? shp.f16_scale_b[b] : 1.f);
             float acc[128];
 #pragma unroll
             for (int c = 0; c < 128; ++c) acc[c] = 0.f;
@@ -349,7 +441,7 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
                             float v[16];
                             tmem_ld16(tb + c, v);
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) acc[c + i] += v[i];
+                            for (int i = 0; i < 16; ++i) acc[c + i] = __fmaf_rn(v[i], fs, acc[c + i]);
                         }
                     }
                 }
@@ -365,51 +457,32 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
             epi.begin(ea);
             bool staged = false;
             if constexpr (EpiHasElem<Epi>::value) staged = epi.staged();
-            if (staged) {
-                if constexpr (EpiHasElem<Epi>::value) {
-                    float *sw = stage + warp * 32 * kStageRow;
-                    const int r0 = ti * kBM + quad * 32, rr0 = lane >> 4, cc = lane & 15;
+            float *sw = stage + warp * kStageWarp;
+            const int r0 = ti * kBM + quad * 32, rr0 = lane >> 4, cc = lane & 15;
 #pragma unroll
-                    for (int c = 0; c < 128; c += 16) {
-                        if (c < ncols) {
+            for (int c = 0; c < 128; c += 16) {
+                if (c >= ncols) continue;
+                float v[16];
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) sw[lane * kStageRow + i] = acc[c + i];
-                            __syncwarp();
-                            if constexpr (EpiHasPre<Epi>::value) {
-                                float pv[16];
-#pragma unroll
-                                for (int k = 0; k < 16; ++k) pv[k] = epi.pre(be, r0 + 2 * k + rr0, cbase + c + cc);
-#pragma unroll
-                                for (int k = 0; k < 16; ++k) {
-                                    const int rr = 2 * k + rr0;
-                                    epi.elem_pre(ea, be, r0 + rr, cbase + c + cc, sw[rr * kStageRow + cc], pv[k]);
-                                }
-                            } else {
-#pragma unroll 4
-                                for (int k = 0; k < 16; ++k) {
-                                    const int rr = 2 * k + rr0;
-                                    epi.elem(ea, be, r0 + rr, cbase + c + cc, sw[rr * kStageRow + cc]);
-                                }
-                            }
-                            __syncwarp();
-                            if constexpr (EpiHasTrans<Epi>::value) {
-                                float v[16];
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) v[i] = acc[c + i];
-                                epi.trans(ea, be, r, cbase + c, v);
-                            }
-                        }
-                    }
+                for (int i = 0; i < 16; ++i) v[i] = acc[c + i];
+                if constexpr (EpiHasRow<Epi>::value)
+                    if (epi.row16(ea, be, r0, lane, cbase + c, v, sw)) continue;
+                if (!staged) {
+                    epi.chunk(ea, be, r, cbase + c, ti, tj, v);
+                    continue;
                 }
-            } else {
+                if constexpr (EpiHasElem<Epi>::value) {
+                    __syncwarp();
 #pragma unroll
-                for (int c = 0; c < 128; c += 16) {
-                    if (c < ncols) {
-                        float v[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) v[i] = acc[c + i];
-                        epi.chunk(ea, be, r, cbase + c, ti, tj, v);
+                    for (int i = 0; i < 16; ++i) sw[lane * kStageRow + i] = v[i];
+                    __syncwarp();
+#pragma unroll 1
+                    for (int k = 0; k < 16; ++k) {
+                        const int rr = 2 * k + rr0;
+                        epi.elem(ea, be, r0 + rr, cbase + c + cc, sw[rr * kStageRow + cc]);
                     }
+                    __syncwarp();
+                    if constexpr (EpiHasTrans<Epi>::value) epi.trans(ea, be, r, cbase + c, v);
                 }
             }
             epi.finish(ea, be, ti, tj);
@@ -443,7 +516,12 @@ struct MatView {
     long long ld = 0;           // elements between rows
     long long bstride = 0;      // elements between batch entries
     int batch = 1;
-    bool bf16 = false;
+    bool bf16 = false, f16 = false;
+};
+
+// The four split-FP16 views of a product (PREC_F16X3).
+struct F16Views {
+    MatView ah, al, bh, bl;
 };
 
 // Encodes a TMA descriptor: box = box_rows rows x 128 B (32 fp32 / 64 bf16), 128-byte
@@ -471,7 +549,7 @@ inline int host_tiles_per_matrix(const GemmShape &s) {
 template <class Epi>
 cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *ahi, const MatView *alo,
                         const MatView *bhi, const MatView *blo, GemmShape shp, int batch, const Epi &epi,
-                        cudaStream_t st) {
+                        cudaStream_t st, const F16Views *f16 = nullptr) {
     // Set on every launch, through the same kernel handle the launch below uses: each
     // .cu file that instantiates this template registers its own copy of the kernel, so
     // a process-wide "already configured" flag would leave other copies unconfigured.
@@ -495,14 +573,17 @@ cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *a
     memset(&maps, 0, sizeof(maps));
     // Any map that is not supplied aliases a supplied one of the same role; the
     // kernel only dereferences the maps of the precision a tile runs.
-    const MatView *Ap = ahi ? ahi : (alo ? alo : a16), *Bp = bhi ? bhi : (blo ? blo : b16);
+    const MatView *Ap = ahi ? ahi : (alo ? alo : (a16 ? a16 : (f16 ? &f16->ah : nullptr)));
+    const MatView *Bp = bhi ? bhi : (blo ? blo : (b16 ? b16 : (f16 ? &f16->bh : nullptr)));
     if (!Ap || !Bp) {
         cuda_fail(cudaErrorInvalidValue, "launch_gemm: missing operand", __LINE__);
         return cudaErrorInvalidValue;
     }
     if (!make_tmap(&maps.a_hi, ahi ? *ahi : *Ap) || !make_tmap(&maps.a_lo, alo ? *alo : *Ap) ||
         !make_tmap(&maps.a_bf16, a16 ? *a16 : *Ap) || !make_tmap(&maps.b_hi, bhi ? *bhi : *Bp, shp.bn) ||
-        !make_tmap(&maps.b_lo, blo ? *blo : *Bp, shp.bn) || !make_tmap(&maps.b_bf16, b16 ? *b16 : *Bp, shp.bn)) {
+        !make_tmap(&maps.b_lo, blo ? *blo : *Bp, shp.bn) || !make_tmap(&maps.b_bf16, b16 ? *b16 : *Bp, shp.bn) ||
+        (f16 && (!make_tmap(&maps.a_h16, f16->ah) || !make_tmap(&maps.a_l16, f16->al) ||
+                 !make_tmap(&maps.b_h16, f16->bh, shp.bn) || !make_tmap(&maps.b_l16, f16->bl, shp.bn)))) {
         cuda_fail(cudaErrorInvalidValue, "tensor map encode", __LINE__);
         return cudaErrorInvalidValue;
     }
@@ -519,7 +600,7 @@ cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *a
     if (prof) {
         // algorithmic flops: 2 M N K per matrix (M (M + 1) K for the symmetric Gram)
         const double f = shp.sym ? (double)shp.M * (shp.M + 1) * shp.K : 2.0 * shp.M * shp.N * (double)shp.K;
-        prof_end(st, f * batch, shp.prof_as > 0 ? shp.prof_as - 1 : (shp.prec ? -1 : shp.prec_uniform));
+        prof_end(st, f * batch, shp.prof_as > 0 ? shp.prof_as - 1 : (shp.prec ? -1 : std::min(shp.prec_uniform, (int)PREC_TF32X3)));
     }
     cudaError_t le = cudaGetLastError();
     if (le != cudaSuccess) cuda_fail(le, __FILE__, __LINE__);

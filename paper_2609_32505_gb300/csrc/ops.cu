@@ -30,11 +30,19 @@ __global__ void prepare_kernel(const float *__restrict__ src, long long lds, lon
         if (trans) { r = c0 + i; c = r0 + threadIdx.x; x = tile[threadIdx.x][i]; if (r >= cols || c >= rows) continue; }
         else { r = r0 + i; c = c0 + threadIdx.x; x = tile[i][threadIdx.x]; if (r >= rows || c >= cols) continue; }
         const long long o = b * dst.bstride + (long long)r * dst.ld + c;
-        if (dst.hi) {
-            if (dst.lo) { float h, l; split_tf32(x, h, l); dst.hi[o] = h; dst.lo[o] = l; }
-            else dst.hi[o] = x;
+        const int p = dst.prec ? dst.prec[b] : -1;
+        if (dst.fhi && (p < 0 || p == PREC_F16X3)) {
+            const long long of = b * dst.fbstride + (long long)r * dst.ld + c;
+            __half h, l;
+            split_f16(x * dst.fscale, h, l);
+            dst.fhi[of] = h;
+            dst.flo[of] = l;
         }
-        if (dst.h16) dst.h16[o] = __float2bfloat16_rn(x);
+        if (dst.hi && (p < 0 || p == PREC_TF32)) {
+            if (dst.lo) { float h, l; split_tf32(x, h, l); dst.hi[o] = h; dst.lo[o] = l; }
+            else dst.hi[o] = p == PREC_TF32 ? tf32_round(x) : x;
+        }
+        if (dst.h16 && (p < 0 || p == PREC_BF16)) dst.h16[o] = __float2bfloat16_rn(x);
     }
 }
 

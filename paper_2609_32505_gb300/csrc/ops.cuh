@@ -20,8 +20,16 @@ __host__ __device__ inline int l1_slabs(int m) { return m < 1 ? 1 : (m + kL1Rows
 struct SplitOut {
     float *hi = nullptr, *lo = nullptr;   // fp32 split (lo may be null: TF32 rounding only)
     __nv_bfloat16 *h16 = nullptr;         // bf16 copy
-    long long ld = 0, bstride = 0;
+    __half *fhi = nullptr, *flo = nullptr;   // fp16 split of x * fscale (strides below, in elements)
+    float fscale = 1.f;
+    const int *prec = nullptr;            // per matrix: write the one format its precision reads
+    long long ld = 0, bstride = 0, fbstride = 0;
 };
+
+// Powers of two that bring split-FP16 operands below 2^16: polar iterates (singular values <= 2 at
+// every step of every schedule) and orthonormal factors; the step polynomial c1 I + c3 G
+// (entries <= 5.2: c1 = 3 sqrt(3) on [0, 1]); Householder vectors (entries <= 1); the back-transform's S2 = S T^T.
+constexpr float kF16X = 0x1p14f, kF16P = 0x1p13f, kF16V = 0x1p14f, kF16S2 = 0x1p10f;
 
 // src (batch x rows x cols, leading dim lds, batch stride bss) scaled by `scale`
 // (or by 1/scale_ptr[b] when scale_ptr != nullptr) -> dst in its padded layout,
@@ -40,6 +48,11 @@ inline MatView view_of16(const __nv_bfloat16 *p, int rows, int cols, long long l
     return v;
 }
 
+inline MatView view_f16(const __half *p, int rows, int cols, long long ld, long long bs, int batch) {
+    MatView v; v.ptr = p; v.rows = rows; v.cols = cols; v.ld = ld; v.bstride = bs; v.batch = batch; v.f16 = true;
+    return v;
+}
+
 // Generic epilogue: D = alpha * acc (+ beta * C) stored row-major, transposed,
 // and/or split into TF32 hi/lo halves (row-major or transposed).
 struct EpiStore {
@@ -51,7 +64,41 @@ struct EpiStore {
     float *hi, *lo; long long ldh, bsh;                    // optional split store
     float *hi_t, *lo_t; long long ldht, bsht;              // optional split transposed store
     struct Acc {};
-    static constexpr bool kElem = true;
+    static constexpr bool kElem = true, kRow = true;
+    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
+        if (r0 >= rows || c0 >= cols) return true;
+        if (cin || out_t || c0 + 16 > cols) return false;
+        if (out && ((((uintptr_t)out & 31) != 0) || ((ld | bs) & 7) != 0)) return false;
+        const int r = r0 + lane;
+        uint32_t h[16], l[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) h[i] = __float_as_uint(alpha * v[i]);
+        if (out && r < rows) st_v8x2(out + b * bs + (long long)r * ld + c0, h);
+        if (!hi && !hi_t) return true;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            float a, c;
+            split_tf32(__uint_as_float(h[i]), a, c);
+            h[i] = __float_as_uint(a);
+            l[i] = __float_as_uint(c);
+        }
+        if (hi && r < rows) {
+            const long long o = b * bsh + (long long)r * ldh + c0;
+            st_v8x2(hi + o, h);
+            if (lo) st_v8x2(lo + o, l);
+        }
+        if (hi_t) {                       // rows past `rows` are zeros of the padding
+            const long long o = b * bsht + (long long)(c0 + (lane >> 1)) * ldht + r0 + 16 * (lane & 1);
+            uint32_t t[16];
+            warp_transpose16(sw, h, t);
+            st_v8x2(hi_t + o, t);
+            if (lo_t) {
+                warp_transpose16(sw, l, t);
+                st_v8x2(lo_t + o, t);
+            }
+        }
+        return true;
+    }
     // staged (coalesced) element path when nothing is stored transposed
     PSVD_DEV bool staged() const { return !out_t && !hi_t; }
     PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
@@ -88,48 +135,93 @@ struct EpiStore {
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 
-// In place: X[r][c] -= acc for a matrix kept split in TF32 hi/lo halves (the eigensolver's
-// back-transform, the QR's trailing updates); the reads of a chunk are issued before its
-// stores (pre / elem_pre).
+// In place: X[r][c] -= acc for a matrix kept split in TF32 hi/lo halves (the QR's trailing updates).
 struct EpiSubSplit {
     int rows, cols;
     float *hi, *lo;
     long long ld, bs;
     struct Acc {};
-    static constexpr bool kElem = true, kPre = true;
-    PSVD_DEV bool staged() const { return true; }
-    // Read through the read-only path: every element is read once, before this thread
-    // writes it, and no other thread touches it, so a stale cached copy can only be of an
-    // element already read; the reads of the next chunk may then be issued ahead of this
-    // chunk's stores.
-    PSVD_DEV float pre(int b, int r, int c) const {
-        if (r >= rows || c >= cols) return 0.f;
-        const long long o = b * bs + (long long)r * ld + c;
-        return __ldg(hi + o) + __ldg(lo + o);
+    static constexpr bool kElem = true, kRow = true;
+    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
+        if (r0 >= rows || c0 >= cols) return true;
+        if (c0 + 16 > cols || (((uintptr_t)hi | (uintptr_t)lo) & 31) || ((ld | bs) & 7)) return false;
+        if (r0 + lane >= rows) return true;
+        const long long o = b * bs + (long long)(r0 + lane) * ld + c0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            uint32_t h[8], l[8];
+            ld_v8(hi + o + 8 * q, h);
+            ld_v8(lo + o + 8 * q, l);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                float a, c;
+                split_tf32((__uint_as_float(h[i]) + __uint_as_float(l[i])) - v[8 * q + i], a, c);
+                h[i] = __float_as_uint(a);
+                l[i] = __float_as_uint(c);
+            }
+            st_v8(hi + o + 8 * q, h);
+            st_v8(lo + o + 8 * q, l);
+        }
+        return true;
     }
-    PSVD_DEV void elem_pre(Acc &, int b, int r, int c, float v, float p) const {
+    PSVD_DEV bool staged() const { return true; }
+    PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
         if (r >= rows || c >= cols) return;
         const long long o = b * bs + (long long)r * ld + c;
         float h, l;
-        split_tf32(p - v, h, l);
+        split_tf32((hi[o] + lo[o]) - v, h, l);
         hi[o] = h;
         lo[o] = l;
     }
-    PSVD_DEV void elem(Acc &a, int b, int r, int c, float v) const { elem_pre(a, b, r, c, v, pre(b, r, c)); }
     PSVD_DEV void begin(Acc &) const {}
-    PSVD_DEV void chunk(Acc &, int b, int r, int c0, int, int, float (&v)[16]) const {
-        if (r >= rows) return;
+    PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = c0 + i;
-            if (c >= cols) break;
-            const long long o = b * bs + (long long)r * ld + c;
-            const float x = (hi[o] + lo[o]) - v[i];
-            float h, l;
-            split_tf32(x, h, l);
-            hi[o] = h;
-            lo[o] = l;
+        for (int i = 0; i < 16; ++i) elem(a, b, r, c0 + i, v[i]);
+    }
+    PSVD_DEV void finish(Acc &, int, int, int) const {}
+};
+
+// The same for a matrix kept split in FP16 halves of x * scale (the eigensolver's back-transform).
+struct EpiSubHalf {
+    int rows, cols;
+    __half *hi, *lo;
+    long long ld, bs;
+    float scale, inv;
+    struct Acc {};
+    static constexpr bool kElem = true, kRow = true;
+    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
+        if (r0 >= rows || c0 >= cols) return true;
+        if (c0 + 16 > cols || (((uintptr_t)hi | (uintptr_t)lo) & 31) || ((ld | bs) & 15)) return false;
+        if (r0 + lane >= rows) return true;
+        const long long o = b * bs + (long long)(r0 + lane) * ld + c0;
+        uint32_t h[8], l[8];
+        ld_v8(hi + o, h);
+        ld_v8(lo + o, l);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&h[i]));
+            const float2 c = __half22float2(*reinterpret_cast<const __half2 *>(&l[i]));
+            v[2 * i] = (a.x + c.x) * inv - v[2 * i];
+            v[2 * i + 1] = (a.y + c.y) * inv - v[2 * i + 1];
         }
+        split_f16x16(v, scale, h, l);
+        st_v8(hi + o, h);
+        st_v8(lo + o, l);
+        return true;
+    }
+    PSVD_DEV bool staged() const { return true; }
+    PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
+        if (r >= rows || c >= cols) return;
+        const long long o = b * bs + (long long)r * ld + c;
+        __half h, l;
+        split_f16((join_f16(hi[o], lo[o]) * inv - v) * scale, h, l);
+        hi[o] = h;
+        lo[o] = l;
+    }
+    PSVD_DEV void begin(Acc &) const {}
+    PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) elem(a, b, r, c0 + i, v[i]);
     }
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };

@@ -118,8 +118,8 @@ cudaError_t l1_norms(const float *A, int B, int m, int n, float *rowsum, float *
 // (launched with kNormThreads threads; the slab sums of a column are loaded eight at a time)
 __global__ void __launch_bounds__(kNormThreads) norm_finalize_kernel(const float *rowsum, const float *colsum,
                                                                       const int *nonfinite, int m, int n,
-                                                                      float *scale, int *done, int *status,
-                                                                      int *fin) {
+                                                                      float *scale, float *ascale, int *done,
+                                                                      int *status, int *fin) {
     __shared__ float sm[2][32];
     const int b = blockIdx.x;
     float r = 0.f, c = 0.f;
@@ -147,6 +147,12 @@ __global__ void __launch_bounds__(kNormThreads) norm_finalize_kernel(const float
         c = fmaxf(c, sm[1][0]);
         const double s = sqrt((double)r * (double)c);
         scale[b] = (float)s;
+        // 2^-e with |M_ij| <= s < 2^e: the operand M 2^-e of H = W^T M (s is at least ||M||_2), and 2^e
+        const int e = s > 0.0 && s < 1e300 ? min(127, max(-100, ilogb(s) + 1)) : 0;
+        if (ascale) {
+            ascale[b] = (float)exp2((double)-e);
+            ascale[gridDim.x + b] = (float)exp2((double)e);
+        }
         if (nonfinite[b]) { done[b] = 1; status[b] = PSVD_ERR_NONFINITE; fin[b] = 0; }
         else if (s == 0.0) { done[b] = 1; status[b] = PSVD_OK; fin[b] = 0; }
     }
@@ -172,7 +178,7 @@ struct CoefTable {
 // kPeWidth (undamped greedy cubics from a small bound lose accuracy: relative
 // reconstruction ~2e-4 at kappa = 1e6 in FP32 against ~3e-6 damped, for the same number of
 // steps), and the step budget before the conservative rerun; with gate_x3, a matrix whose
-// bound is below PSVD_MIXED_LB_MIN starts on the split-TF32 rung.
+// bound is below PSVD_MIXED_LB_MIN starts on the FP32-accurate (split-FP16) rung.
 // Damped (schedule PSVD_SCHED_PE, the Polar-Express-style comparison): the same damped cubics
 // from [l_b, 1] until a damped step stops shrinking the interval (width below 0.1 and less
 // than 10% gained: the damped fixed point near 1 - 1.5e-4, the plateau the ablation
@@ -186,7 +192,7 @@ __global__ void schedule_fill_kernel(int B, int K, CoefTable tab, const float *l
     if (active && !active[b]) return;
     if (learned || pe) {
         double l = (double)lower[b];
-        if (learned && gate_x3 && !(l >= PSVD_MIXED_LB_MIN)) prec[b] = PREC_TF32X3;
+        if (learned && gate_x3 && !(l >= PSVD_MIXED_LB_MIN)) prec[b] = PREC_F16X3;
         if (!(l > 1e-12)) l = 1e-12;
         if (l > 0.999) l = 0.999;
         double lo = l, hi = 1.0;
@@ -232,14 +238,74 @@ __global__ void schedule_fill_kernel(int B, int K, CoefTable tab, const float *l
 }
 
 // ------------------------------------------------------------ step epilogues
-PSVD_DEV void store_prec(int p, long long o, float x, __nv_bfloat16 *p16, float *phi, float *plo) {
+PSVD_DEV void store_prec(int p, long long o, float x, __nv_bfloat16 *p16, float *phi) {
     if (p == PREC_BF16) p16[o] = __float2bfloat16_rn(x);
-    else if (p == PREC_TF32) phi[o] = tf32_round(x);
-    else { float h, l; split_tf32(x, h, l); phi[o] = h; plo[o] = l; }
+    else phi[o] = tf32_round(x);
+}
+// the same with the split-FP16 rung: halves of x * fs at element of (stride of a batch entry doubled)
+PSVD_DEV void store_rung(int p, long long o, long long of, float x, float fs, __nv_bfloat16 *p16, float *phi,
+                         float *plo) {
+    if (p == PREC_F16X3) {
+        __half h, l;
+        split_f16(x * fs, h, l);
+        reinterpret_cast<__half *>(phi)[of] = h;
+        reinterpret_cast<__half *>(plo)[of] = l;
+    } else {
+        store_prec(p, o, x, p16, phi);
+    }
+}
+
+// 16 values of one row in the format of rung p: along the row at element ro (roh for halves) when
+// `rowv`, and transposed (this lane's 16 rows of column c0 + lane / 2) at element co (coh) when `colv`.
+PSVD_DEV void rung_row16(int p, const float (&v)[16], float fs, __nv_bfloat16 *r16, float *rhi, float *rlo,
+                         long long ro, long long roh, bool rowv, __nv_bfloat16 *c16, float *chi, float *clo,
+                         long long co, long long coh, bool colv, float *sw) {
+    uint32_t w[16], o[16], h[8], l[8];
+    if (p == PREC_F16X3) {
+        split_f16x16(v, fs, h, l);
+        if (rowv) {
+            st_v8(reinterpret_cast<__half *>(rhi) + roh, h);
+            st_v8(reinterpret_cast<__half *>(rlo) + roh, l);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {              // (hi, lo) of one value per word
+            w[2 * i] = __byte_perm(h[i], l[i], 0x5410);
+            w[2 * i + 1] = __byte_perm(h[i], l[i], 0x7632);
+        }
+        warp_transpose16(sw, w, o);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            h[i] = __byte_perm(o[2 * i], o[2 * i + 1], 0x5410);
+            l[i] = __byte_perm(o[2 * i], o[2 * i + 1], 0x7632);
+        }
+        if (colv) {
+            st_v8(reinterpret_cast<__half *>(chi) + coh, h);
+            st_v8(reinterpret_cast<__half *>(clo) + coh, l);
+        }
+    } else if (p == PREC_TF32) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(tf32_round(v[i]));
+        if (rowv) st_v8x2(rhi + ro, w);
+        warp_transpose16(sw, w, o);
+        if (colv) st_v8x2(chi + co, o);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const __nv_bfloat162 b2 = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+            h[i] = *reinterpret_cast<const uint32_t *>(&b2);
+            w[2 * i] = h[i] & 0xffffu;
+            w[2 * i + 1] = h[i] >> 16;
+        }
+        if (rowv) st_v8(r16 + ro, h);
+        warp_transpose16(sw, w, o);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) h[i] = __byte_perm(o[2 * i], o[2 * i + 1], 0x5410);
+        if (colv) st_v8(c16 + co, h);
+    }
 }
 
 // Per-matrix decision after the Gram of step k.
-// mixed: 0 every step split-TF32; 1 TF32 until the residual drops below kTauTF32; 2 BF16
+// mixed: 0 every step split FP16; 1 TF32 until the residual drops below kTauTF32; 2 BF16
 // above kTauBF16 first.  The precision never decreases from one step to the next.
 struct DecideArgs {
     int k, B, n, mixed, learned, kcap;
@@ -265,13 +331,13 @@ PSVD_DEV void decide_matrix(const DecideArgs &d, int b) {
         d.done[b] = 1; d.fin[b] = k; d.status[b] = PSVD_NOT_CONVERGED; d.fres[b] = (float)r; d.fallback[b] = 1;
         return;
     }
-    int pn = PREC_TF32X3;
+    int pn = PREC_F16X3;
     if (d.mixed) {
-        const int want = (d.mixed == 2 && r > kTauBF16) ? PREC_BF16 : (r > kTauTF32 ? PREC_TF32 : PREC_TF32X3);
+        const int want = (d.mixed == 2 && r > kTauBF16) ? PREC_BF16 : (r > kTauTF32 ? PREC_TF32 : PREC_F16X3);
         pn = want > pk ? want : pk;
     }
     d.prec[(long long)(k + 1) * B + b] = pn;
-    d.steps[pk * B + b] += 1;
+    d.steps[min(pk, 2) * B + b] += 1;
     atomicAdd(&d.notdone[k], 1);
 }
 
@@ -290,7 +356,24 @@ struct EpiGram {
     float *Phi, *Plo;
     long long ldp;
     struct Acc { ff r; int p; float c1, c3; };     // ||G - I||^2 partial, float-float (FP32 pipe)
-    static constexpr bool kElem = true, kTrans = true, kTail = true;
+    static constexpr bool kElem = true, kTrans = true, kTail = true, kRow = true;
+    PSVD_DEV bool row16(Acc &a, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
+        if (r0 >= n || c0 >= n || c0 + 15 < r0) return true;       // outside, or left to the mirror's tile
+        if (c0 < r0 + 32) return false;                            // crosses the diagonal
+        load(a, b);
+        // entries past n are products of the zero fill
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            a.r = ff_fma(a.r, 2.f * v[i], v[i]);
+            v[i] *= a.c3;
+        }
+        const int r = r0 + lane, ct = c0 + (lane >> 1);
+        const long long bo = (long long)b * n * ldp, rc = (long long)r * ldp + c0;
+        const long long cr = (long long)ct * ldp + r0 + 16 * (lane & 1);
+        rung_row16(a.p, v, kF16P, P16, Phi, Plo, bo + rc, 2 * bo + rc, r < n, P16, Phi, Plo, bo + cr, 2 * bo + cr,
+                   ct < n, sw);
+        return true;
+    }
     PSVD_DEV bool staged() const { return true; }
     PSVD_DEV void tail() const {
         for (int b = threadIdx.x; b < dec.B; b += blockDim.x) decide_matrix(dec, b);
@@ -305,18 +388,20 @@ struct EpiGram {
         const float d = g - (r == c ? 1.f : 0.f);
         a.r = ff_fma(a.r, r == c ? d : 2.f * d, d);
         const float pv = a.c3 * g + (r == c ? a.c1 : 0.f);
-        store_prec(a.p, (long long)b * n * ldp + (long long)r * ldp + c, pv, P16, Phi, Plo);
+        const long long bo = (long long)b * n * ldp, rc = (long long)r * ldp + c;
+        store_rung(a.p, bo + rc, 2 * bo + rc, pv, kF16P, P16, Phi, Plo);
     }
     PSVD_DEV void trans(Acc &a, int b, int r, int c0, float (&v)[16]) const {
         if (r >= n) return;
         load(a, b);
-        const long long base = (long long)b * n * ldp + r;
+        const long long bo = (long long)b * n * ldp;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int c = c0 + i;
             if (c >= n) break;
             if (c <= r) continue;
-            store_prec(a.p, base + (long long)c * ldp, a.c3 * v[i], P16, Phi, Plo);
+            const long long rc = (long long)c * ldp + r;
+            store_rung(a.p, bo + rc, 2 * bo + rc, a.c3 * v[i], kF16P, P16, Phi, Plo);
         }
     }
     PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
@@ -339,23 +424,36 @@ struct EpiApply {
     float *Xhi, *Xlo, *XThi, *XTlo;
     long long ldn, ldm;
     struct Acc { int p; };
-    static constexpr bool kElem = true, kTrans = true;
+    static constexpr bool kElem = true, kTrans = true, kRow = true;
+    PSVD_DEV bool row16(Acc &a, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
+        if (r0 >= m || c0 >= n) return true;
+        if (a.p < 0) a.p = prec_next[b];
+        // columns past n and rows past m are zeros, and land in the padding of the rows
+        const int r = r0 + lane, ct = c0 + (lane >> 1);
+        const long long bo = (long long)b * m * ldn, rc = (long long)r * ldn + c0;
+        const long long bt = (long long)b * n * ldm, cr = (long long)ct * ldm + r0 + 16 * (lane & 1);
+        rung_row16(a.p, v, kF16X, X16, Xhi, Xlo, bo + rc, 2 * bo + rc, r < m, XT16, XThi, XTlo, bt + cr, 2 * bt + cr,
+                   ct < n, sw);
+        return true;
+    }
     PSVD_DEV bool staged() const { return true; }
     PSVD_DEV void begin(Acc &a) const { a.p = -1; }
     PSVD_DEV void elem(Acc &a, int b, int r, int c, float x) const {
         if (r >= m || c >= n) return;
         if (a.p < 0) a.p = prec_next[b];
-        store_prec(a.p, (long long)b * m * ldn + (long long)r * ldn + c, x, X16, Xhi, Xlo);
+        const long long bo = (long long)b * m * ldn, rc = (long long)r * ldn + c;
+        store_rung(a.p, bo + rc, 2 * bo + rc, x, kF16X, X16, Xhi, Xlo);
     }
     PSVD_DEV void trans(Acc &a, int b, int r, int c0, float (&v)[16]) const {
         if (r >= m) return;
         if (a.p < 0) a.p = prec_next[b];
-        const long long tb = (long long)b * n * ldm + r;
+        const long long bo = (long long)b * n * ldm;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int c = c0 + i;
             if (c >= n) break;
-            store_prec(a.p, tb + (long long)c * ldm, v[i], XT16, XThi, XTlo);
+            const long long rc = (long long)c * ldm + r;
+            store_rung(a.p, bo + rc, 2 * bo + rc, v[i], kF16X, XT16, XThi, XTlo);
         }
     }
     PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
@@ -366,10 +464,10 @@ struct EpiApply {
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 
-// W (user layout) from X_fin; leaves W split row-major in Xhi[0]/Xlo[0] and
-// transposed in XThi[0]/XTlo[0] for the products that follow (H, U).
+// W (user layout) from X_fin; leaves W and W^T as split-FP16 halves in ws.wf_hi() ... for the products
+// that follow (H, U).
 __global__ void polar_finalize_kernel(int m, int n, int B, const int *fin, const int *prec, const int *status,
-                                      PolarWS ws, float *W) {
+                                      PolarWS ws, __half *wh, __half *wl, __half *wth, __half *wtl, float *W) {
     __shared__ float tile[32][33];
     const int b = blockIdx.z;
     const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
@@ -377,32 +475,35 @@ __global__ void polar_finalize_kernel(int m, int n, int B, const int *fin, const
     const int par = f & 1;
     const int p = prec[(long long)f * B + b];
     const bool nan_out = status[b] == PSVD_ERR_NONFINITE;
-    const bool copy = par != 0 || p != PREC_TF32X3 || nan_out;
     const long long rbase = (long long)b * m * ws.ldn;
+    const __half *hp = reinterpret_cast<const __half *>(ws.Xhi[par]) + 2 * rbase;
+    const __half *lp = reinterpret_cast<const __half *>(ws.Xlo[par]) + 2 * rbase;
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
         const int r = r0 + i, c = c0 + threadIdx.x;
         float x = 0.f;
         if (r < m && c < n) {
-            const long long o = rbase + (long long)r * ws.ldn + c;
+            const long long rc = (long long)r * ws.ldn + c;
             if (nan_out) x = __int_as_float(0x7fc00000);
-            else if (p == PREC_BF16) x = __bfloat162float(ws.X16[par][o]);
-            else if (p == PREC_TF32) x = ws.Xhi[par][o];
-            else x = ws.Xhi[par][o] + ws.Xlo[par][o];
+            else if (p == PREC_BF16) x = __bfloat162float(ws.X16[par][rbase + rc]);
+            else if (p == PREC_TF32) x = ws.Xhi[par][rbase + rc];
+            else x = join_f16(hp[rc], lp[rc]) * (1.f / kF16X);
             if (W) W[(long long)b * m * n + (long long)r * n + c] = x;
-            if (copy) { float h, l; split_tf32(x, h, l); ws.Xhi[0][o] = h; ws.Xlo[0][o] = l; }
+            __half h, l;
+            split_f16(x * kF16X, h, l);
+            wh[2 * rbase + rc] = h;
+            wl[2 * rbase + rc] = l;
         }
         tile[i][threadIdx.x] = x;
     }
-    if (!copy) return;                     // uniform per block
     __syncthreads();
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
         const int c = c0 + i, r = r0 + threadIdx.x;
         if (c < n && r < m) {
-            float h, l;
-            split_tf32(tile[threadIdx.x][i], h, l);
-            const long long o = (long long)b * n * ws.ldm + (long long)c * ws.ldm + r;
-            ws.XThi[0][o] = h;
-            ws.XTlo[0][o] = l;
+            __half h, l;
+            split_f16(tile[threadIdx.x][i] * kF16X, h, l);
+            const long long o = 2 * (long long)b * n * ws.ldm + (long long)c * ws.ldm + r;
+            wth[o] = h;
+            wtl[o] = l;
         }
     }
 }
@@ -477,7 +578,9 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
     {
         MatView v16 = w.bf16 ? view_of16(w.XT16[par], n, m, w.ldm, (long long)n * w.ldm, B) : MatView();
         MatView vhi = view_of(w.XThi[par], n, m, w.ldm, (long long)n * w.ldm, B);
-        MatView vlo = view_of(w.XTlo[par], n, m, w.ldm, (long long)n * w.ldm, B);
+        F16Views f;
+        f.ah = f.bh = view_f16(as_half(w.XThi[par]), n, m, w.ldm, 2LL * n * w.ldm, B);
+        f.al = f.bl = view_f16(as_half(w.XTlo[par]), n, m, w.ldm, 2LL * n * w.ldm, B);
         GemmShape s;
         memset(&s, 0, sizeof(s));
         s.M = n; s.N = n; s.K = m; s.sym = 1;
@@ -485,6 +588,7 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
         s.skip = w.done;
         s.gate = gram_gate;
         s.ticket = w.ticket + k;
+        s.f16_scale = 1.f / (kF16X * kF16X);
         s.err = w.err;
         EpiGram e;
         e.n = n; e.B = B;
@@ -494,8 +598,8 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
         e.prec = w.prec + (long long)k * B;
         e.res = w.res + (long long)k * B;
         e.P16 = w.P16; e.Phi = w.Phi; e.Plo = w.Plo; e.ldp = w.ldn;
-        cudaError_t er = launch_gemm(w.bf16 ? &v16 : nullptr, w.bf16 ? &v16 : nullptr, &vhi, &vlo, &vhi, &vlo, s,
-                                     B, e, st);
+        cudaError_t er = launch_gemm(w.bf16 ? &v16 : nullptr, w.bf16 ? &v16 : nullptr, &vhi, nullptr, &vhi, nullptr,
+                                     s, B, e, st, &f);
         if (er != cudaSuccess) return PSVD_ERR_CUDA;
     }
     if (!apply) return PSVD_OK;
@@ -503,15 +607,19 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
     {
         MatView a16 = w.bf16 ? view_of16(w.X16[par], m, n, w.ldn, (long long)m * w.ldn, B) : MatView();
         MatView ahi = view_of(w.Xhi[par], m, n, w.ldn, (long long)m * w.ldn, B);
-        MatView alo = view_of(w.Xlo[par], m, n, w.ldn, (long long)m * w.ldn, B);
         MatView b16 = w.bf16 ? view_of16(w.P16, n, n, w.ldn, (long long)n * w.ldn, B) : MatView();
         MatView bhi = view_of(w.Phi, n, n, w.ldn, (long long)n * w.ldn, B);
-        MatView blo = view_of(w.Plo, n, n, w.ldn, (long long)n * w.ldn, B);
+        F16Views f;
+        f.ah = view_f16(as_half(w.Xhi[par]), m, n, w.ldn, 2LL * m * w.ldn, B);
+        f.al = view_f16(as_half(w.Xlo[par]), m, n, w.ldn, 2LL * m * w.ldn, B);
+        f.bh = view_f16(as_half(w.Phi), n, n, w.ldn, 2LL * n * w.ldn, B);
+        f.bl = view_f16(as_half(w.Plo), n, n, w.ldn, 2LL * n * w.ldn, B);
         GemmShape s;
         memset(&s, 0, sizeof(s));
         s.M = m; s.N = n; s.K = n;
         s.prec = w.prec + (long long)k * B;
         s.skip = w.done;
+        s.f16_scale = 1.f / (kF16X * kF16P);
         s.gate = w.notdone + k;          // matrices still iterating after this step's decision
         s.err = w.err;
         EpiApply e;
@@ -520,8 +628,8 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
         e.X16 = w.X16[npar]; e.XT16 = w.XT16[npar];
         e.Xhi = w.Xhi[npar]; e.Xlo = w.Xlo[npar]; e.XThi = w.XThi[npar]; e.XTlo = w.XTlo[npar];
         e.ldn = w.ldn; e.ldm = w.ldm;
-        cudaError_t er = launch_gemm(w.bf16 ? &a16 : nullptr, w.bf16 ? &b16 : nullptr, &ahi, &alo, &bhi, &blo, s,
-                                     B, e, st);
+        cudaError_t er = launch_gemm(w.bf16 ? &a16 : nullptr, w.bf16 ? &b16 : nullptr, &ahi, nullptr, &bhi, nullptr,
+                                     s, B, e, st, &f);
         if (er != cudaSuccess) return PSVD_ERR_CUDA;
     }
     return PSVD_OK;
@@ -558,8 +666,13 @@ static int prepare_x0(const float *A, PolarWS &w, cudaStream_t st, const int *sk
     SplitOut r, t;
     r.ld = w.ldn; r.bstride = (long long)m * w.ldn;
     t.ld = w.ldm; t.bstride = (long long)n * w.ldm;
+    // every matrix in the format of its first rung (the lo array only serves split FP16)
     if (w.bf16) { r.h16 = w.X16[0]; t.h16 = w.XT16[0]; }
-    else { r.hi = w.Xhi[0]; r.lo = w.Xlo[0]; t.hi = w.XThi[0]; t.lo = w.XTlo[0]; }
+    r.hi = w.Xhi[0]; t.hi = w.XThi[0];
+    r.fhi = as_half(w.Xhi[0]); r.flo = as_half(w.Xlo[0]); r.fbstride = 2 * r.bstride;
+    t.fhi = as_half(w.XThi[0]); t.flo = as_half(w.XTlo[0]); t.fbstride = 2 * t.bstride;
+    r.fscale = t.fscale = kF16X;
+    r.prec = t.prec = w.prec;
     if (prepare_operand(A, n, (long long)m * n, B, m, n, false, 1.f, w.scale, r, st, skip) ||
         prepare_operand(A, n, (long long)m * n, B, m, n, true, 1.f, w.scale, t, st, skip))
         return PSVD_ERR_CUDA;
@@ -579,12 +692,12 @@ int polar_forward(const float *A, float *W, float *H_out, bool want_h, PolarWS &
         cudaMemsetAsync(w.misc, 0, sizeof(int) * 8, st) ||
         cudaMemsetAsync(w.err, 0, sizeof(unsigned) * 4, st))
         return PSVD_ERR_CUDA;
-    const int prec0 = w.bf16 ? PREC_BF16 : (w.mixed ? PREC_TF32 : PREC_TF32X3);
+    const int prec0 = w.bf16 ? PREC_BF16 : (w.mixed ? PREC_TF32 : PREC_F16X3);
     polar_init_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, prec0, w.done, w.fin, w.status, w.prec, w.steps,
                                                         w.fallback);
     if (l1_norms(A, B, m, n, w.rowsum, w.colsum, w.nonfinite, st) != cudaSuccess) return PSVD_ERR_CUDA;
-    norm_finalize_kernel<<<B, kNormThreads, 0, st>>>(w.rowsum, w.colsum, w.nonfinite, m, n, w.scale, w.done, w.status,
-                                            w.fin);
+    norm_finalize_kernel<<<B, kNormThreads, 0, st>>>(w.rowsum, w.colsum, w.nonfinite, m, n, w.scale, w.ascale, w.done,
+                                                      w.status, w.fin);
     count_launch(2);
     // coefficient tables: conservative CANS (Appendix B.8), classical NS, or learned bounds
     CoefTable tab;
@@ -601,8 +714,11 @@ int polar_forward(const float *A, float *W, float *H_out, bool want_h, PolarWS &
     if (int rc = prepare_x0(A, w, st, nullptr)) return rc;   // zero matrices get X0 = 0
     if (want_h) {
         SplitOut at;
-        at.hi = w.AThi; at.lo = w.ATlo; at.ld = w.ldm; at.bstride = (long long)n * w.ldm;
-        if (prepare_operand(A, n, (long long)m * n, B, m, n, true, 1.f, nullptr, at, st)) return PSVD_ERR_CUDA;
+        at.fhi = as_half(w.AThi); at.flo = as_half(w.ATlo); at.ld = w.ldm;
+        at.bstride = at.fbstride = (long long)n * w.ldm;
+        at.fscale = kF16X;
+        // M 2^-e: scale_ptr is divided by, so it gets the inverse, 2^e
+        if (prepare_operand(A, n, (long long)m * n, B, m, n, true, 1.f, w.ascale + B, at, st)) return PSVD_ERR_CUDA;
     }
     if (cudaGetLastError() != cudaSuccess) return PSVD_ERR_CUDA;
     // Host-side bound on the steps any matrix can take: the cap for the conservative and
@@ -647,19 +763,24 @@ int polar_forward(const float *A, float *W, float *H_out, bool want_h, PolarWS &
     // W out + final split layouts
     {
         dim3 g((n + 31) / 32, (m + 31) / 32, B), blk(32, 8);
-        polar_finalize_kernel<<<g, blk, 0, st>>>(m, n, B, w.fin, w.prec, w.status, w, W);
+        polar_finalize_kernel<<<g, blk, 0, st>>>(m, n, B, w.fin, w.prec, w.status, w, w.wf_hi(), w.wf_lo(), w.wtf_hi(),
+                                                  w.wtf_lo(), W);
         count_launch(1);
     }
     if (want_h) {
-        MatView ahi = view_of(w.XThi[0], n, m, w.ldm, (long long)n * w.ldm, B);
-        MatView alo = view_of(w.XTlo[0], n, m, w.ldm, (long long)n * w.ldm, B);
-        MatView bhi = view_of(w.AThi, n, m, w.ldm, (long long)n * w.ldm, B);
-        MatView blo = view_of(w.ATlo, n, m, w.ldm, (long long)n * w.ldm, B);
+        F16Views f;
+        f.ah = view_f16(w.wtf_hi(), n, m, w.ldm, 2LL * n * w.ldm, B);
+        f.al = view_f16(w.wtf_lo(), n, m, w.ldm, 2LL * n * w.ldm, B);
+        f.bh = view_f16(as_half(w.AThi), n, m, w.ldm, (long long)n * w.ldm, B);
+        f.bl = view_f16(as_half(w.ATlo), n, m, w.ldm, (long long)n * w.ldm, B);
         GemmShape s;
         memset(&s, 0, sizeof(s));
-        s.M = n; s.N = n; s.K = m; s.prec_uniform = PREC_TF32X3; s.err = w.err;
+        s.M = n; s.N = n; s.K = m; s.prec_uniform = PREC_F16X3; s.err = w.err;
+        s.f16_scale = 1.f / (kF16X * kF16X);
+        s.f16_scale_b = w.ascale + B;
         EpiStore e = epi_store_plain(w.Hraw, n, (long long)n * n, n, n);
-        if (launch_gemm(nullptr, nullptr, &ahi, &alo, &bhi, &blo, s, B, e, st) != cudaSuccess) return PSVD_ERR_CUDA;
+        if (launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f) != cudaSuccess)
+            return PSVD_ERR_CUDA;
         symmetrize_kernel<<<dim3((n + 31) / 32, (n + 31) / 32, B), dim3(32, 8), 0, st>>>(w.Hraw, n, w.Hsym, H_out);
         count_launch(1);
     }

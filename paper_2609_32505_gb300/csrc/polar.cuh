@@ -24,7 +24,9 @@ struct PolarWS {
     float *Xhi[2] = {}, *Xlo[2] = {}, *XThi[2] = {}, *XTlo[2] = {};
     __nv_bfloat16 *P16 = nullptr;
     float *Phi = nullptr, *Plo = nullptr;
-    float *AThi = nullptr, *ATlo = nullptr;     // M^T split (for H = W^T M)
+    // (split-TF32 never occurs here: the FP32-accurate rung reads split-FP16 halves, as_half(Xhi), ...)
+    float *AThi = nullptr, *ATlo = nullptr;     // M^T split in FP16 halves (for H = W^T M)
+    float *ascale = nullptr;                    // [2][B] power of two below 1/max|M|, and its inverse
     float *Hraw = nullptr;                      // W^T M before symmetrization
     float *Hsym = nullptr;                      // (W^T M)_sym, FP32 copy
     float *rowsum = nullptr, *colsum = nullptr, *scale = nullptr;
@@ -36,6 +38,13 @@ struct PolarWS {
     int *misc = nullptr;
     unsigned *ticket = nullptr;   // [kcap + 2] per-step CTA tickets of the Gram launches
     unsigned *err = nullptr;
+
+    // The final W and W^T, as halves scaled by kF16X (batch stride 2 m ldn / 2 n ldm): the other half of
+    // the lo arrays' space, which no rung uses, so that the conversion is never in place.
+    __half *wf_hi() const { return reinterpret_cast<__half *>(Xlo[0]) + (long long)m * ldn; }
+    __half *wf_lo() const { return reinterpret_cast<__half *>(Xlo[1]) + (long long)m * ldn; }
+    __half *wtf_hi() const { return reinterpret_cast<__half *>(XTlo[0]) + (long long)n * ldm; }
+    __half *wtf_lo() const { return reinterpret_cast<__half *>(XTlo[1]) + (long long)n * ldm; }
 
     template <class C>
     void carve(C &cv, int B_, int m_, int n_, int kcap_, int precision) {
@@ -64,6 +73,7 @@ struct PolarWS {
         rowsum = cv.template take<float>(B64 * m);
         colsum = cv.template take<float>(B64 * l1_slabs(m) * n);
         scale = cv.template take<float>(B64);
+        ascale = cv.template take<float>(B64 * 2);
         done = cv.template take<int>(B64);
         fin = cv.template take<int>(B64);
         status = cv.template take<int>(B64);
@@ -82,11 +92,14 @@ struct PolarWS {
     }
 };
 
+// Split-FP16 halves of the FP32-accurate rung live in the memory of the float arrays: matrix b starts
+// where its float matrix does and its halves fill the first half of that space.
+inline __half *as_half(float *p) { return reinterpret_cast<__half *>(p); }
+
 inline int polar_kcap(const psvd_opts &o) { return o.max_iter + (o.schedule == PSVD_SCHED_CANS ? o.pre_iters : 0); }
 
 // Runs the iteration of Algorithm 1 (normalize, schedule, iterate) for all matrices, then
-// writes W (user layout, may be null) and leaves W^T split in XThi[0]/XTlo[0] and W
-// split in Xhi[0]/Xlo[0].  If `want_h`, also computes Hsym = (W^T M)_sym (FP64
+// writes W (user layout, may be null) and leaves W and W^T as split-FP16 halves (wf_hi(), ...).  If `want_h`, also computes Hsym = (W^T M)_sym (FP64
 // averaging) and copies it to H_out (may be null).  Never synchronizes: the step budget is
 // launched whole and finished matrices are skipped on the device.  Fills info (device,
 // may be null).  With the learned schedule, matrices that miss tol within their budget

@@ -105,7 +105,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 bool make_tmap(CUtensorMap *out, const MatView &v, int box_rows) {
     auto fn = encode_fn();
     if (!fn || !v.ptr) return false;
-    const int esz = v.bf16 ? 2 : 4;
+    const int esz = v.bf16 || v.f16 ? 2 : 4;
     cuuint64_t dims[3] = {(cuuint64_t)v.cols, (cuuint64_t)v.rows, (cuuint64_t)v.batch};
     cuuint64_t strides[2] = {(cuuint64_t)v.ld * esz, (cuuint64_t)v.bstride * esz};
     cuuint32_t box[3] = {(cuuint32_t)(128 / esz), (cuuint32_t)box_rows, 1u};
@@ -115,7 +115,9 @@ bool make_tmap(CUtensorMap *out, const MatView &v, int box_rows) {
                  (unsigned long long)strides[0], (unsigned long long)strides[1], v.ptr);
         return false;
     }
-    CUresult r = fn(out, v.bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+    CUresult r = fn(out,
+                    v.bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                           : (v.f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32), 3,
                     const_cast<void *>(v.ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

@@ -26,6 +26,21 @@ struct EpiColNorm {
     float *U;
     float *colss;   // [B][n]
     struct Acc {};
+    static constexpr bool kRow = true;
+    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
+        if (r0 >= m || c0 >= n) return true;
+        if (c0 + 16 > n || (n & 7) || ((uintptr_t)U & 31)) return false;
+        uint32_t w[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(v[i]);
+        if (r0 + lane < m) st_v8x2(U + (long long)b * m * n + (long long)(r0 + lane) * n + c0, w);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] *= v[i];                 // rows past m are zeros
+        const float s = warp_sum16(v);
+        if (!(lane & 1) && s != 0.f) atomicAdd(&colss[(long long)b * n + c0 + (lane >> 1)], s);
+        return true;
+    }
+    PSVD_DEV bool staged() const { return false; }
     PSVD_DEV void begin(Acc &) const {}
     PSVD_DEV void chunk(Acc &, int b, int r, int c0, int, int, float (&v)[16]) const {
 #pragma unroll
@@ -412,10 +427,10 @@ __global__ void x2_split_kernel(const float *X2, int n, long long ld, float *hi)
     hi[(long long)b * n * ld + (long long)i * ld + j] = tf32_round(X2[(long long)b * n * n + (long long)i * n + j]);
 }
 
-// (V E)^T = V^T - X V^T + h V^T and V^T <- V^T + X V^T + h V^T, in FP32, re-split;
+// (V E)^T = V^T - X V^T + h V^T (split FP16, the operand of U) and V^T + X V^T + h V^T, in FP32;
 // XV = X V^T (split-TF32 product), HV = h V^T (TF32 product), both n x n.
 __global__ void add_split_kernel(const float *vthi, const float *vtlo, const float *XV, const float *HV, int n,
-                                 long long ld, float *VEt_hi, float *VEt_lo, float *VThi, float *VTlo, float *VT) {
+                                 long long ld, __half *VEt_hi, __half *VEt_lo, float *VT) {
     const int b = blockIdx.z;
     const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
     if (i >= n || j >= n) return;
@@ -425,22 +440,11 @@ __global__ void add_split_kernel(const float *vthi, const float *vtlo, const flo
     const float xv = XV[p], hv = HV[p];
     const float ve = v + (hv - xv);
     const float vn = v + (hv + xv);
-    float h, l;
-    split_tf32(ve, h, l);
+    __half h, l;
+    split_f16(ve * kF16X, h, l);
     VEt_hi[o] = h;
     VEt_lo[o] = l;
-    split_tf32(vn, h, l);
-    VThi[o] = h;
-    VTlo[o] = l;
-    if (VT) VT[p] = vn;
-}
-
-__global__ void hilo_store_kernel(const float *hi, const float *lo, int n, long long ld, float *out) {
-    const int b = blockIdx.z;
-    const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
-    if (i >= n || j >= n) return;
-    const long long o = (long long)b * n * ld + (long long)i * ld + j;
-    out[(long long)b * n * n + (long long)i * n + j] = hi[o] + lo[o];
+    VT[p] = vn;
 }
 
 // A bounded device-side wait that expired anywhere in the call (product-kernel pipeline,
@@ -472,7 +476,9 @@ struct SvdWS {
     bool blocked_qr = false;
     float *Vhi = nullptr, *Vlo = nullptr;            // V = (V^T)^T split
     float *Khi = nullptr, *Klo = nullptr, *T1 = nullptr, *T1hi = nullptr, *T1lo = nullptr, *Kt = nullptr;
-    float *X = nullptr, *Xneg = nullptr, *X2 = nullptr, *F = nullptr, *Ft = nullptr, *VEt = nullptr;
+    float *X = nullptr, *Xneg = nullptr, *X2 = nullptr, *F = nullptr, *Ft = nullptr;
+    __half *VEt = nullptr;       // (V E)^T, split FP16 (hi, then lo)
+    float *VT32hi = nullptr, *VT32lo = nullptr;      // V^T split TF32 (operand of the correction)
     unsigned *xmax = nullptr, *kmax = nullptr;
     int *cprec = nullptr;        // [2][B] precision of the correction products (corr_prec_kernel)
     int *mflag = nullptr;
@@ -517,7 +523,9 @@ struct SvdWS {
             X2 = cv.template take<float>(B64 * n * n);
             F = cv.template take<float>(B64 * nn);
             Ft = cv.template take<float>(B64 * nn);
-            VEt = cv.template take<float>(B64 * nn * 2);
+            VEt = cv.template take<__half>(B64 * nn * 2);
+            VT32hi = cv.template take<float>(B64 * nn);
+            VT32lo = cv.template take<float>(B64 * nn);
             xmax = cv.template take<unsigned>(B64);
             kmax = cv.template take<unsigned>(B64);
             cprec = cv.template take<int>(B64 * 2);
@@ -571,10 +579,10 @@ int svd_forward(const float *A, float *U, float *Sout, float *VT, SvdWS &w, cons
     if (cudaMemsetAsync(w.any, 0, sizeof(int) * 4, st)) return PSVD_ERR_CUDA;
     // a learned schedule's misses are recomputed with the rest of the rerun (below), not here
     if (int rc = polar_forward(A, nullptr, nullptr, true, p, o, info, st, false)) return rc;
-    if (int rc = eigh_forward(p.Hsym, Sout, nullptr, w.ew, st)) return rc;
+    if (int rc = eigh_forward(p.Hsym, Sout, w.mixed ? nullptr : VT, w.ew, st, w.VT32hi, w.VT32lo)) return rc;
     if (cudaMemcpyAsync(w.S, Sout, sizeof(float) * (size_t)B * n, cudaMemcpyDeviceToDevice, st)) return PSVD_ERR_CUDA;
-    const float *vthi = w.ew.VThi, *vtlo = w.ew.VTlo;
-    const float *bu_hi = vthi, *bu_lo = vtlo;        // B operand of U = W V: rows of V^T
+    const float *vthi = w.VT32hi, *vtlo = w.VT32lo;  // (mixed only) split TF32
+    const __half *bu_hi = w.ew.VThi, *bu_lo = w.ew.VTlo;        // B operand of U = W V: rows of V^T
     dim3 g16((n + 15) / 16, (n + 15) / 16, B), b16(16, 16);
     if (w.mixed) {
         // V = (V^T)^T split (TF32 operand of the update products)
@@ -611,13 +619,12 @@ int svd_forward(const float *A, float *U, float *Sout, float *VT, SvdWS &w, cons
         corr_h_kernel<<<g16, b16, 0, st>>>(w.X2, w.T1, n, ld, w.F);                 // h in F
         count_launch(1);
         // X V^T (split-TF32, into T1) and h V^T (TF32, into Kt); B operand B[j][k] = V^T[k][j] = V[j][k]
-        float *VEt_hi = w.VEt, *VEt_lo = w.VEt + (long long)B * nn;
+        __half *VEt_hi = w.VEt, *VEt_lo = w.VEt + (long long)B * nn;
         EpiStore e4 = epi_store_plain(w.T1, n, (long long)n * n, n, n);
         if (int rc = gemm3p(w.X, w.Ft, n, n, ld, nn, w.Vhi, w.Vlo, n, ld, nn, B, w.cprec + B, e4, p.err, st)) return rc;
         EpiStore e5 = epi_store_plain(w.Kt, n, (long long)n * n, n, n);
         if (int rc = gemm3(w.F, nullptr, n, n, ld, nn, w.Vhi, nullptr, n, ld, nn, B, PREC_TF32, e5, p.err, st)) return rc;
-        add_split_kernel<<<g16, b16, 0, st>>>(vthi, vtlo, w.T1, w.Kt, n, ld, VEt_hi, VEt_lo, w.ew.VThi, w.ew.VTlo,
-                                              VT);
+        add_split_kernel<<<g16, b16, 0, st>>>(vthi, vtlo, w.T1, w.Kt, n, ld, VEt_hi, VEt_lo, VT);
         count_launch(1);
         bu_hi = VEt_hi;
         bu_lo = VEt_lo;
@@ -627,13 +634,17 @@ int svd_forward(const float *A, float *U, float *Sout, float *VT, SvdWS &w, cons
     {
         EpiColNorm e;
         e.m = m; e.n = n; e.U = U; e.colss = w.colss;
-        if (int rc = gemm3(p.Xhi[0], p.Xlo[0], m, n, p.ldn, (long long)m * p.ldn, bu_hi, bu_lo, n, ld, nn, B,
-                           PREC_TF32X3, e, p.err, st))
-            return rc;
-    }
-    if (!w.mixed) {
-        hilo_store_kernel<<<g16, b16, 0, st>>>(vthi, vtlo, n, ld, VT);
-        count_launch(1);
+        F16Views f;
+        f.ah = view_f16(p.wf_hi(), m, n, p.ldn, 2LL * m * p.ldn, B);
+        f.al = view_f16(p.wf_lo(), m, n, p.ldn, 2LL * m * p.ldn, B);
+        f.bh = view_f16(bu_hi, n, n, ld, nn, B);
+        f.bl = view_f16(bu_lo, n, n, ld, nn, B);
+        GemmShape s;
+        memset(&s, 0, sizeof(s));
+        s.M = m; s.N = n; s.K = n; s.prec_uniform = PREC_F16X3; s.err = p.err;
+        s.f16_scale = 1.f / (kF16X * kF16X);
+        if (launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f) != cudaSuccess)
+            return PSVD_ERR_CUDA;
     }
     qr_flag_kernel<<<B, 256, 0, st>>>(w.colss, n, o.eps_qr, w.learned ? p.fallback : nullptr, w.flag, w.any);
     count_launch(1);
