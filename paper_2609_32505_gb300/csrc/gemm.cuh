@@ -309,6 +309,10 @@ PSVD_DEV bool mma_tile_x3(MmaRing &r, int nkb, uint32_t tmem, uint64_t *acc_full
 template <class Epi>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi epi) {
+    // Launched ahead of its predecessor's end (programmatic dependent launch): let the next launch
+    // come, then wait until everything before this one has completed and is visible.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // A gated launch with nothing left to do returns before any allocation (uniform: every
     // thread reads the same word, final since the kernel that wrote it has completed).
     if (shp.gate && *shp.gate == 0) return;
@@ -333,10 +337,6 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
         s_abort = 0;
     }
     if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
-    if (warp == kEpiWarps && lane == 0) {
-        tma_prefetch(&maps.a_hi); tma_prefetch(&maps.b_hi);
-        tma_prefetch(&maps.a_bf16); tma_prefetch(&maps.b_bf16);
-    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -571,17 +571,14 @@ cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *a
     }
     GemmMaps maps;
     memset(&maps, 0, sizeof(maps));
-    // Any map that is not supplied aliases a supplied one of the same role; the
-    // kernel only dereferences the maps of the precision a tile runs.
-    const MatView *Ap = ahi ? ahi : (alo ? alo : (a16 ? a16 : (f16 ? &f16->ah : nullptr)));
-    const MatView *Bp = bhi ? bhi : (blo ? blo : (b16 ? b16 : (f16 ? &f16->bh : nullptr)));
-    if (!Ap || !Bp) {
+    // A map that is not supplied stays zero; the kernel only reads those of the precisions its tiles have.
+    auto encode = [&](CUtensorMap *m, const MatView *v, int rows) { return !v || make_tmap(m, *v, rows); };
+    if (!(ahi && bhi) && !(a16 && b16) && !f16) {
         cuda_fail(cudaErrorInvalidValue, "launch_gemm: missing operand", __LINE__);
         return cudaErrorInvalidValue;
     }
-    if (!make_tmap(&maps.a_hi, ahi ? *ahi : *Ap) || !make_tmap(&maps.a_lo, alo ? *alo : *Ap) ||
-        !make_tmap(&maps.a_bf16, a16 ? *a16 : *Ap) || !make_tmap(&maps.b_hi, bhi ? *bhi : *Bp, shp.bn) ||
-        !make_tmap(&maps.b_lo, blo ? *blo : *Bp, shp.bn) || !make_tmap(&maps.b_bf16, b16 ? *b16 : *Bp, shp.bn) ||
+    if (!encode(&maps.a_hi, ahi, kBM) || !encode(&maps.a_lo, alo, kBM) || !encode(&maps.a_bf16, a16, kBM) ||
+        !encode(&maps.b_hi, bhi, shp.bn) || !encode(&maps.b_lo, blo, shp.bn) || !encode(&maps.b_bf16, b16, shp.bn) ||
         (f16 && (!make_tmap(&maps.a_h16, f16->ah) || !make_tmap(&maps.a_l16, f16->al) ||
                  !make_tmap(&maps.b_h16, f16->bh, shp.bn) || !make_tmap(&maps.b_l16, f16->bl, shp.bn)))) {
         cuda_fail(cudaErrorInvalidValue, "tensor map encode", __LINE__);
@@ -595,7 +592,24 @@ cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *a
     const int grid = (int)std::min<long long>(total, num_sms());
     const bool prof = prof_on();
     if (prof) prof_begin(st);
-    gemm_tn_kernel<Epi><<<grid, kGemmThreads, kGemmSmem, st>>>(maps, shp, epi);
+    // Programmatic dependent launch: the grid is set up while the kernel before it still runs (its
+    // CTAs wait at their first instruction), which takes the launch latency out of the chains of
+    // short products of small matrices and of the polar steps that find nothing to do.
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.dynamicSmemBytes = kGemmSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    {
+        cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_tn_kernel<Epi>, maps, shp, epi);
+        if (e != cudaSuccess) { cuda_fail(e, __FILE__, __LINE__); return e; }
+    }
     count_launch();
     if (prof) {
         // algorithmic flops: 2 M N K per matrix (M (M + 1) K for the symmetric Gram)

@@ -598,8 +598,9 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
         e.prec = w.prec + (long long)k * B;
         e.res = w.res + (long long)k * B;
         e.P16 = w.P16; e.Phi = w.Phi; e.Plo = w.Plo; e.ldp = w.ldn;
-        cudaError_t er = launch_gemm(w.bf16 ? &v16 : nullptr, w.bf16 ? &v16 : nullptr, &vhi, nullptr, &vhi, nullptr,
-                                     s, B, e, st, &f);
+        const MatView *t = w.mixed ? &vhi : nullptr;
+        cudaError_t er = launch_gemm(w.bf16 ? &v16 : nullptr, w.bf16 ? &v16 : nullptr, t, nullptr, t, nullptr, s, B, e,
+                                     st, &f);
         if (er != cudaSuccess) return PSVD_ERR_CUDA;
     }
     if (!apply) return PSVD_OK;
@@ -628,8 +629,8 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
         e.X16 = w.X16[npar]; e.XT16 = w.XT16[npar];
         e.Xhi = w.Xhi[npar]; e.Xlo = w.Xlo[npar]; e.XThi = w.XThi[npar]; e.XTlo = w.XTlo[npar];
         e.ldn = w.ldn; e.ldm = w.ldm;
-        cudaError_t er = launch_gemm(w.bf16 ? &a16 : nullptr, w.bf16 ? &b16 : nullptr, &ahi, nullptr, &bhi, nullptr,
-                                     s, B, e, st, &f);
+        cudaError_t er = launch_gemm(w.bf16 ? &a16 : nullptr, w.bf16 ? &b16 : nullptr, w.mixed ? &ahi : nullptr, nullptr,
+                                     w.mixed ? &bhi : nullptr, nullptr, s, B, e, st, &f);
         if (er != cudaSuccess) return PSVD_ERR_CUDA;
     }
     return PSVD_OK;
