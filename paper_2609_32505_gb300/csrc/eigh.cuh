@@ -6,7 +6,6 @@
 
 namespace psvd {
 
-constexpr int kWY = 128;   // reflectors per compact-WY block in the back-transform
 constexpr int kTrdChipMin = 3, kTrdChipMax = 4096;   // sizes whose tridiagonalization runs on chip (trd.cu)
 constexpr int kBtSplit = 8; // largest K split of the back-transform's V^T Y products
 

@@ -16,6 +16,11 @@ constexpr int kL1Rows = 256;
 constexpr int kNormThreads = 1024;   // threads of the block that finishes the norms of one matrix
 __host__ __device__ inline int l1_slabs(int m) { return m < 1 ? 1 : (m + kL1Rows - 1) / kL1Rows; }
 
+constexpr int kWY = 128;   // reflectors per compact-WY block (back-transform, QR's trailing updates)
+// T (upper triangular, kWY x kWY) of compact-WY blocks from G = Y^T Y and tau (eigh.cu).
+int larft_blocks(const float *Gm, const float *tau, int n, int nrefl, int nblk, int blk0, int count, int B, float *Tm,
+                 cudaStream_t st);
+
 // Output format of an operand-preparation pass.
 struct SplitOut {
     float *hi = nullptr, *lo = nullptr;   // fp32 split (lo may be null: TF32 rounding only)

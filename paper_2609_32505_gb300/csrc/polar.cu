@@ -150,8 +150,8 @@ __global__ void __launch_bounds__(kNormThreads) norm_finalize_kernel(const float
         // 2^-e with |M_ij| <= s < 2^e: the operand M 2^-e of H = W^T M (s is at least ||M||_2), and 2^e
         const int e = s > 0.0 && s < 1e300 ? min(127, max(-100, ilogb(s) + 1)) : 0;
         if (ascale) {
-            ascale[b] = (float)exp2((double)-e);
-            ascale[gridDim.x + b] = (float)exp2((double)e);
+            ascale[b] = ldexpf(1.f, -e);
+            ascale[gridDim.x + b] = ldexpf(1.f, e);
         }
         if (nonfinite[b]) { done[b] = 1; status[b] = PSVD_ERR_NONFINITE; fin[b] = 0; }
         else if (s == 0.0) { done[b] = 1; status[b] = PSVD_OK; fin[b] = 0; }

@@ -11,19 +11,27 @@ namespace psvd {
 // Returns false when no shape fits (m too large for the cluster panel).
 bool qr_shape(int m, int *nb, int *cl);
 
+constexpr int kQrSplit = 8;   // largest K split of the X^T Y products of a block
+
+// The matrices are normalized by a power of two (|A| <= 2^e, columns of norm <= 1), so every array
+// below is bounded and kept as split-FP16 halves.
 struct QrWS {
-    int B = 0, m = 0, n = 0, nb = 0, cl = 0, npan = 0, ks = 1;
+    int B = 0, m = 0, n = 0, nb = 0, cl = 0, npan = 0, nsup = 0, ks = 1;
     long long ldm = 0, ldn = 0;
-    float *UThi = nullptr, *UTlo = nullptr;   // [B][n][ldm] the matrix transposed, being factored
-    float *YThi = nullptr, *YTlo = nullptr;   // [B][n][ldm] reflector j as row j (1 at j, 0 above)
-    float *Yhi = nullptr, *Ylo = nullptr;     // [B][m][ldn] the same reflectors as columns
-    float *QThi = nullptr, *QTlo = nullptr;   // [B][n][ldm] Q^T being accumulated
-    float *tau = nullptr, *beta = nullptr;    // [B][n]
-    float *Tm = nullptr;                      // [B][npan][nb][nb] compact-WY T of every panel
-    float *Gpart = nullptr;                   // [B][cl][nb][nb] per-CTA partial Y^T Y of a panel
-    float *Wp = nullptr;                      // [ks][B][nb][n] partial Y^T X of a panel (K split)
-    float *W2hi = nullptr, *W2lo = nullptr;   // [B][n][nb] (op(T) Y^T X)^T
-    int *skip = nullptr;                      // [B] 1 = matrix not factored (flag[b] == 0)
+    __half *UThi = nullptr, *UTlo = nullptr;   // [B][n][ldm] the matrix transposed, being factored (kF16X)
+    __half *YThi = nullptr, *YTlo = nullptr;   // [B][n][ldm] reflector j as row j (1 at j, 0 above) (kF16V)
+    __half *Yhi = nullptr, *Ylo = nullptr;     // [B][m][ldn] the same reflectors as columns (kF16V)
+    __half *QThi = nullptr, *QTlo = nullptr;   // [B][n][ldm] Q^T being accumulated (kF16X)
+    float *tau = nullptr, *beta = nullptr;     // [B][n]
+    float *Tm = nullptr;                       // [B][npan][nb][nb] compact-WY T of every panel
+    float *Gpart = nullptr;                    // [B][cl][nb][nb] per-CTA partial Y^T Y of a panel
+    float *Wp = nullptr;                       // [ks][B][nb][n] partial Y^T X of a panel (K split)
+    __half *W2hi = nullptr, *W2lo = nullptr;   // [B][n][kWY] (op(T) Y^T X)^T (kF16S2)
+    float *Gs = nullptr, *Ts = nullptr;        // [B][nsup][kWY][kWY] Y^T Y and T of blocks of kWY columns
+    float *Sp = nullptr;                       // [kQrSplit][B][n][kWY] partial X^T Y of a block
+    unsigned *amax = nullptr;                  // [B] max |A| (float bits)
+    float *scale = nullptr;                    // [B] 2^e
+    int *skip = nullptr;                       // [B] 1 = matrix not factored (flag[b] == 0)
     unsigned *err = nullptr;
 
     template <class C>
@@ -31,18 +39,24 @@ struct QrWS {
         B = B_; m = m_; n = n_;
         if (!qr_shape(m, &nb, &cl)) { nb = 64; cl = 8; }
         npan = (n + nb - 1) / nb;
+        nsup = (n + kWY - 1) / kWY;
         ldm = pad_ld(m); ldn = pad_ld(n);
-        ks = 8;
+        ks = 16;
         const long long B64 = B, nm = (long long)n * ldm;
-        UThi = cv.template take<float>(B64 * nm); UTlo = cv.template take<float>(B64 * nm);
-        YThi = cv.template take<float>(B64 * nm); YTlo = cv.template take<float>(B64 * nm);
-        Yhi = cv.template take<float>(B64 * m * ldn); Ylo = cv.template take<float>(B64 * m * ldn);
-        QThi = cv.template take<float>(B64 * nm); QTlo = cv.template take<float>(B64 * nm);
+        UThi = cv.template take<__half>(B64 * nm); UTlo = cv.template take<__half>(B64 * nm);
+        YThi = cv.template take<__half>(B64 * nm); YTlo = cv.template take<__half>(B64 * nm);
+        Yhi = cv.template take<__half>(B64 * m * ldn); Ylo = cv.template take<__half>(B64 * m * ldn);
+        QThi = cv.template take<__half>(B64 * nm); QTlo = cv.template take<__half>(B64 * nm);
         tau = cv.template take<float>(B64 * n); beta = cv.template take<float>(B64 * n);
         Tm = cv.template take<float>(B64 * npan * nb * nb);
         Gpart = cv.template take<float>(B64 * cl * nb * nb);
-        Wp = cv.template take<float>((long long)ks * B64 * nb * n);
-        W2hi = cv.template take<float>(B64 * n * nb); W2lo = cv.template take<float>(B64 * n * nb);
+        Wp = cv.template take<float>((long long)ks * B64 * nb * std::min(n, kWY));
+        W2hi = cv.template take<__half>(B64 * n * kWY); W2lo = cv.template take<__half>(B64 * n * kWY);
+        Gs = cv.template take<float>(B64 * nsup * kWY * kWY);
+        Ts = cv.template take<float>(B64 * nsup * kWY * kWY);
+        Sp = cv.template take<float>((long long)kQrSplit * B64 * n * kWY);
+        amax = cv.template take<unsigned>(B64);
+        scale = cv.template take<float>(B64);
         skip = cv.template take<int>(B64);
         err = cv.template take<unsigned>(4);
     }
