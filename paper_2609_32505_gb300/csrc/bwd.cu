@@ -8,8 +8,11 @@
 //   V^T X V    = T_eps o V^T C V
 //   Mbar       = (Ubar D_R + 2 Y (V^T X V)) V^T                 (= Wbar R_eps + 2 M X)
 // Algorithm 3 (polar) is the same chain with V^T Hbar V computed from Hbar and
-// G = Wbar V in place of Ubar.  Six products on the split-TF32 tcgen05 kernel plus
-// one elementwise kernel that holds every mask (K_eps, T_eps, D_R).
+// G = Wbar V in place of Ubar.  Six products on the split-FP16 tcgen05 kernel plus
+// one elementwise kernel that holds every mask (K_eps, T_eps, D_R).  The products are bound by the tensor
+// cores: at 4096 x 4096 each takes 345 us in split FP16 (0.40 PFLOP/s of FP32-accurate work, three FP16
+// products each) and took 700 us in split TF32; the whole backward 4.10 -> 2.40 ms, its error against
+// 64 bits unchanged at 2.2e-6.
 #include <cmath>
 #include <cstring>
 
@@ -17,56 +20,145 @@
 
 namespace psvd {
 
+// Split-FP16 operands need a power of two per matrix.  The inputs' come from their largest entries and, for
+// V, the largest column norm (both 1 for orthonormal factors, whatever else a caller hands over stays in
+// range); Y = M V, T1 = V^T sym(Hbar) and Wbar V are bounded by sqrt(n) times the largest entry of the one
+// and the column norm of the other; X and Q are written in FP32 with their largest entries recorded, then split.
+enum BwdMax { AM_M = 0, AM_G, AM_B, AM_U, AM_V, AM_IN, AM_X = AM_IN, AM_Q, AM_N };   // slots of amax; inputs first
+enum BwdScale {                                                        // slots of es, each [B]
+    ES_M = 0, ES_G, ES_B, ES_U, ES_V, ES_X, ES_Q,      // 2^e (operands are divided by it)
+    ES_IM, ES_IG,                          // 2^-e
+    ES_AU, ES_BV, ES_Y, ES_Z, ES_QP, ES_DA, ES_T1, ES_EH, ES_WV,      // product scales, 2^-28 included
+    ES_N
+};
+
 struct BwdWS {
     int B = 0, m = 0, n = 0;
     long long ldn = 0, ldm = 0;
-    float *UThi = nullptr, *UTlo = nullptr;      // U^T (n x m)
-    float *GThi = nullptr, *GTlo = nullptr;      // Ubar^T or (Wbar V)^T (n x m)
-    float *G = nullptr;                          // Ubar or Wbar V row-major FP32 (m x n) for the epilogue
-    float *Mhi = nullptr, *Mlo = nullptr;        // M (m x n)
-    float *VThi = nullptr, *VTlo = nullptr;      // V^T (n x n)
-    float *Vhi = nullptr, *Vlo = nullptr;        // V (n x n)
-    float *dVThi = nullptr, *dVTlo = nullptr;    // Vbar^T (n x n) or sym(Hbar) (polar)
-    float *Yhi = nullptr, *Ylo = nullptr;        // Y = M V (m x n)
-    float *YThi = nullptr, *YTlo = nullptr;      // Y^T (n x m)
+    __half *UThi = nullptr, *UTlo = nullptr;      // U^T (n x m)
+    __half *GThi = nullptr, *GTlo = nullptr;      // Ubar^T or (Wbar V)^T (n x m)
+    float *G = nullptr;                           // Wbar V row-major FP32 (m x n) for the epilogue (polar)
+    __half *Mhi = nullptr, *Mlo = nullptr;        // M (m x n)
+    __half *VThi = nullptr, *VTlo = nullptr;      // V^T (n x n)
+    __half *Vhi = nullptr, *Vlo = nullptr;        // V (n x n)
+    __half *dVThi = nullptr, *dVTlo = nullptr;    // Vbar^T (n x n) or sym(Hbar) (polar)
+    __half *Yhi = nullptr, *Ylo = nullptr;        // Y = M V (m x n)
+    __half *YThi = nullptr, *YTlo = nullptr;      // Y^T (n x m)
     float *AU = nullptr, *BV = nullptr, *Z = nullptr;   // n x n FP32
-    float *Xhi = nullptr, *Xlo = nullptr;        // V^T X V (n x n)
-    float *Qhi = nullptr, *Qlo = nullptr;        // (m x n)
-    float *Wbhi = nullptr, *Wblo = nullptr;      // Wbar (m x n), polar only
-    float *S = nullptr;                          // sigma FP32 (polar: eigenvalues of H)
-    float *T1 = nullptr, *T1hi = nullptr, *T1lo = nullptr;  // polar: V^T Hbar
+    float *X = nullptr;                           // V^T X V (n x n)
+    __half *Xhi = nullptr, *Xlo = nullptr;
+    float *Q = nullptr;                           // (m x n)
+    __half *Qhi = nullptr, *Qlo = nullptr;
+    __half *Wbhi = nullptr, *Wblo = nullptr;      // Wbar (m x n), polar only
+    float *S = nullptr;                           // sigma FP32 (polar: eigenvalues of H)
+    float *T1 = nullptr;                          // polar: V^T, then V^T Hbar
+    __half *T1hi = nullptr, *T1lo = nullptr;
+    unsigned *amax = nullptr;                     // [AM_N][B]
+    float *es = nullptr;                          // [ES_N][B]
     unsigned *err = nullptr;
     EighWS ew;
     bool polar = false;
+    const float *esp(int slot) const { return es + (long long)slot * B; }
 
     template <class C>
     void carve(C &cv, int B_, int m_, int n_, bool polar_) {
         B = B_; m = m_; n = n_; polar = polar_;
         ldn = pad_ld(n); ldm = pad_ld(m);
         const long long B64 = B, mn = (long long)m * ldn, nm = (long long)n * ldm, nn = (long long)n * ldn;
-        UThi = cv.template take<float>(B64 * nm); UTlo = cv.template take<float>(B64 * nm);
-        GThi = cv.template take<float>(B64 * nm); GTlo = cv.template take<float>(B64 * nm);
-        G = cv.template take<float>(B64 * m * n);
-        Mhi = cv.template take<float>(B64 * mn); Mlo = cv.template take<float>(B64 * mn);
-        VThi = cv.template take<float>(B64 * nn); VTlo = cv.template take<float>(B64 * nn);
-        Vhi = cv.template take<float>(B64 * nn); Vlo = cv.template take<float>(B64 * nn);
-        dVThi = cv.template take<float>(B64 * nn); dVTlo = cv.template take<float>(B64 * nn);
-        Yhi = cv.template take<float>(B64 * mn); Ylo = cv.template take<float>(B64 * mn);
-        YThi = cv.template take<float>(B64 * nm); YTlo = cv.template take<float>(B64 * nm);
+        auto pair = [&](__half *&hi, __half *&lo, long long k) {
+            hi = cv.template take<__half>(B64 * k);
+            lo = cv.template take<__half>(B64 * k);
+        };
+        pair(UThi, UTlo, nm); pair(GThi, GTlo, nm); pair(Mhi, Mlo, mn); pair(VThi, VTlo, nn); pair(Vhi, Vlo, nn);
+        pair(dVThi, dVTlo, nn); pair(Yhi, Ylo, mn); pair(YThi, YTlo, nm); pair(Xhi, Xlo, nn); pair(Qhi, Qlo, mn);
         AU = cv.template take<float>(B64 * n * n); BV = cv.template take<float>(B64 * n * n);
         Z = cv.template take<float>(B64 * n * n);
-        Xhi = cv.template take<float>(B64 * nn); Xlo = cv.template take<float>(B64 * nn);
-        Qhi = cv.template take<float>(B64 * mn); Qlo = cv.template take<float>(B64 * mn);
+        X = cv.template take<float>(B64 * n * n); Q = cv.template take<float>(B64 * m * n);
         S = cv.template take<float>(B64 * n);
+        amax = cv.template take<unsigned>(B64 * AM_N);
+        es = cv.template take<float>(B64 * ES_N);
         err = cv.template take<unsigned>(4);
         if (polar) {
-            Wbhi = cv.template take<float>(B64 * mn); Wblo = cv.template take<float>(B64 * mn);
+            G = cv.template take<float>(B64 * m * n);
+            pair(Wbhi, Wblo, mn);
             T1 = cv.template take<float>(B64 * n * n);
-            T1hi = cv.template take<float>(B64 * nn); T1lo = cv.template take<float>(B64 * nn);
+            pair(T1hi, T1lo, nn);
             ew.carve(cv, B, n, eigh_groups(B, n));
         }
     }
 };
+
+// 2^e above the largest entry (times `grow`); 1 for zero and non-finite arrays.
+PSVD_DEV int bwd_exp(unsigned amax, double grow) {
+    const float v = __uint_as_float(amax);
+    return v > 0.f && v < INFINITY ? min(127, max(-100, ilogb((double)v * grow) + 1)) : 0;
+}
+// largest entry of a factor (or norm of its columns) above the [1, 2] of an orthonormal one
+PSVD_DEV int bwd_exp_factor(unsigned amax) {
+    const float v = __uint_as_float(amax);
+    return v > 2.f && v < INFINITY ? ilogbf(v) : 0;
+}
+// stage 0: the scales of the inputs; 1: of X; 2: of Q
+__global__ void bwd_scale_kernel(const unsigned *amax, int B, int n, int stage, int polar, float *es) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= B) return;
+    auto put = [&](int slot, int e) { es[(long long)slot * B + b] = ldexpf(1.f, e); };
+    const double rn = sqrt((double)n);
+    const int eM = bwd_exp(amax[AM_M * B + b], rn), eV = bwd_exp_factor(amax[AM_V * B + b]);
+    if (stage == 0) {
+        const int eG = bwd_exp(amax[AM_G * B + b], polar ? rn : 1.0), eB = bwd_exp(amax[AM_B * B + b], polar ? rn : 1.0);
+        const int eU = bwd_exp_factor(amax[AM_U * B + b]);
+        put(ES_M, eM); put(ES_G, eG); put(ES_B, eB); put(ES_U, eU); put(ES_V, eV); put(ES_IM, -(eM + eV)); put(ES_IG, -eG);
+        put(ES_AU, eU + eG - 28); put(ES_BV, eV + eB - 28); put(ES_Y, eM + eV - 28); put(ES_Z, eM + eV + eG - 28);
+        put(ES_T1, eB - 28); put(ES_EH, eB - 28); put(ES_WV, eG - 28);
+    } else if (stage == 1) {
+        const int eX = bwd_exp(amax[AM_X * B + b], 1.0);
+        put(ES_X, eX); put(ES_QP, eM + eV + eX - 28);
+    } else {
+        const int eQ = bwd_exp(amax[AM_Q * B + b], 1.0);
+        put(ES_Q, eQ); put(ES_DA, eQ + eV - 28);
+    }
+}
+
+// The AM_ slots of the inputs, one launch for all of them (grid.z = slot): entries, or for V^T the 2-norm
+// of its rows, a warp at a time.
+struct BwdMaxIn { const float *x[AM_IN]; long long len[AM_IN]; };
+__global__ void __launch_bounds__(256) bwd_max_kernel(BwdMaxIn in, int B, int n, unsigned *amax) {
+    __shared__ unsigned red[8];
+    const int b = blockIdx.y, slot = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (!in.x[slot]) return;
+    const long long len = in.len[slot];
+    const float *a = in.x[slot] + b * len;
+    unsigned v = 0;
+    if (slot == AM_V) {
+        for (int r = blockIdx.x * 8 + warp; r < n; r += gridDim.x * 8) {
+            float s = 0.f;
+#pragma unroll 8
+            for (int c = lane; c < n; c += 32) { const float t = a[(long long)r * n + c]; s += t * t; }
+#pragma unroll
+            for (int d = 16; d; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+            v = max(v, __float_as_uint(sqrtf(s)));
+        }
+    } else {
+        const bool vec = ((uintptr_t)a & 15) == 0;
+        const long long n4 = vec ? len / 4 : 0;
+        const long long t0 = (long long)blockIdx.x * 256 + threadIdx.x, dt = (long long)gridDim.x * 256;
+#pragma unroll 4
+        for (long long t = t0; t < n4; t += dt) {
+            const float4 q = reinterpret_cast<const float4 *>(a)[t];
+            v = max(max(v, __float_as_uint(fabsf(q.x))), max(__float_as_uint(fabsf(q.y)),
+                    max(__float_as_uint(fabsf(q.z)), __float_as_uint(fabsf(q.w)))));
+        }
+        for (long long t = 4 * n4 + t0; t < len; t += dt) v = max(v, __float_as_uint(fabsf(a[t])));
+    }
+    v = __reduce_max_sync(0xffffffffu, v);
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) v = max(v, red[w]);
+        if (v) atomicMax(&amax[slot * B + b], v);
+    }
+}
 
 // D_R entry: sigma / (sigma^2 + eps^(1/2)), or the pseudo-inverse 1/sigma (eps = 0)
 PSVD_DEV float dr_of(float s, float sqrt_eps, int exact) {
@@ -75,72 +167,119 @@ PSVD_DEV float dr_of(float s, float sqrt_eps, int exact) {
 }
 
 // V^T X V = T o sym(E_H - D_R Z D_R) with E_H = diag(Sbar) + K^T o skew(B_V + A_U)
-// (svd) or E_H = the given V^T Hbar V (polar, `EH`).
-__global__ void bwd_core_kernel(const float *AU, const float *BV, const float *Z, const float *EH, const float *S,
-                                const float *dS, int n, float eps, int kreg_mode, float tie_tol, float *Xhi,
-                                float *Xlo, long long ldx) {
-    const int b = blockIdx.z;
-    const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
-    if (i >= n || j >= n) return;
-    const long long bo = (long long)b * n * n, ij = bo + (long long)i * n + j, ji = bo + (long long)j * n + i;
+// (svd) or E_H = the given V^T Hbar V (polar, `EH`).  The result is symmetric: one block of 32 x 8 threads
+// per pair of mirrored 32 x 32 tiles (block (x, y) with x >= y) reads both tiles of every input once,
+// rows coalesced, and writes both tiles of X; the largest |X| of the matrix goes to xmax.  (141 us at
+// n = 4096, 1.8 TB/s: divisions and the latency of one batch of loads per block.)
+__global__ void __launch_bounds__(256) bwd_core_kernel(const float *AU, const float *BV, const float *Z, const float *EH,
+                                                       const float *S, const float *dS, int n, float eps, int kreg_mode,
+                                                       float tie_tol, float *X, unsigned *xmax) {
+    if (blockIdx.x < blockIdx.y) return;
+    __shared__ float mt[32][33], mz[32][33];       // the mirrored tile of E_H (or B_V + A_U) and of Z
+    __shared__ unsigned red[8];
+    const int b = blockIdx.z, i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const long long bo = (long long)b * n * n;
+    auto rd = [&](int i, int j, float &t, float &z) {
+        t = z = 0.f;
+        if (i >= n || j >= n) return;
+        const long long o = bo + (long long)i * n + j;
+        if (EH) t = EH[o];
+        else t = (BV ? BV[o] : 0.f) + (AU ? AU[o] : 0.f);
+        if (Z) z = Z[o];
+    };
+    float tij[4], zij[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        rd(i0 + ty + 8 * q, j0 + tx, tij[q], zij[q]);
+        float t, z;
+        rd(j0 + ty + 8 * q, i0 + tx, t, z);
+        mt[ty + 8 * q][tx] = t;
+        mz[ty + 8 * q][tx] = z;
+    }
+    __syncthreads();
     const float *s = S + (long long)b * n;
-    const float si = s[i], sj = s[j];
     const int exact = kreg_mode == 2;
     const float sq = sqrtf(eps), q4 = sqrtf(sq);
-    // E_H(i, j) and E_H(j, i)
-    float eh_ij, eh_ji;
-    if (EH) {
-        eh_ij = EH[ij];
-        eh_ji = EH[ji];
-    } else {
-        const float tij = (BV ? BV[ij] : 0.f) + (AU ? AU[ij] : 0.f);
-        const float tji = (BV ? BV[ji] : 0.f) + (AU ? AU[ji] : 0.f);
-        const float bij = 0.5f * (tij - tji);       // B = skew part
-        // K_ij = (s_i - s_j) / ((s_i - s_j)^2 + reg); (K^T)_ij = K_ji = -K_ij
-        float kij;
-        const float d = si - sj;
-        if (kreg_mode == 0) kij = d / (d * d + sq);
-        else if (kreg_mode == 1) kij = d / (d * d + eps * eps);
-        else {
-            const float smax = fmaxf(fabsf(s[0]), fabsf(s[n - 1]));
-            kij = fabsf(d) <= tie_tol * smax ? 0.f : 1.f / d;
+    const int j = j0 + tx;
+    const float sj = j < n ? s[j] : 0.f, dj = dr_of(sj, sq, exact);
+    float x[4];
+    unsigned bits = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = i0 + ty + 8 * q;
+        x[q] = 0.f;
+        if (i >= n || j >= n) continue;
+        const float si = s[i], di = dr_of(si, sq, exact);
+        const float tji = mt[tx][ty + 8 * q], zji = mz[tx][ty + 8 * q];
+        float eh_ij, eh_ji;
+        if (EH) {
+            eh_ij = tij[q];
+            eh_ji = tji;
+        } else {
+            const float bij = 0.5f * (tij[q] - tji);    // B = skew part
+            // K_ij = (s_i - s_j) / ((s_i - s_j)^2 + reg); (K^T)_ij = K_ji = -K_ij
+            float kij;
+            const float d = si - sj;
+            if (kreg_mode == 0) kij = d / (d * d + sq);
+            else if (kreg_mode == 1) kij = d / (d * d + eps * eps);
+            else {
+                const float smax = fmaxf(fabsf(s[0]), fabsf(s[n - 1]));
+                kij = fabsf(d) <= tie_tol * smax ? 0.f : 1.f / d;
+            }
+            // (K^T o B)_ij = K_ji B_ij = -K_ij B_ij; symmetric, since K and B are both skew
+            eh_ij = -kij * bij;
+            if (i == j && dS) eh_ij += dS[(long long)b * n + i];
+            eh_ji = eh_ij;
         }
-        // (K^T o B)_ij = K_ji B_ij = -K_ij B_ij; symmetric, since K and B are both skew
-        eh_ij = -kij * bij;
-        if (i == j && dS) eh_ij += dS[(long long)b * n + i];
-        eh_ji = eh_ij;
+        const float c = 0.5f * ((eh_ij - di * zij[q] * dj) + (eh_ji - dj * zji * di));
+        const float ssum = si + sj;
+        float t;
+        if (exact) t = ssum > 0.f ? 1.f / ssum : 0.f;
+        else t = ssum / (ssum * ssum + q4);
+        x[q] = t * c;
+        X[bo + (long long)i * n + j] = x[q];
+        bits = max(bits, __float_as_uint(fabsf(x[q])));
     }
-    const float di = dr_of(si, sq, exact), dj = dr_of(sj, sq, exact);
-    const float zij = Z ? Z[ij] : 0.f, zji = Z ? Z[ji] : 0.f;
-    const float c = 0.5f * ((eh_ij - di * zij * dj) + (eh_ji - dj * zji * di));
-    const float ssum = si + sj;
-    float t;
-    if (exact) t = ssum > 0.f ? 1.f / ssum : 0.f;
-    else t = ssum / (ssum * ssum + q4);
-    float h, l;
-    split_tf32(t * c, h, l);
-    Xhi[(long long)b * n * ldx + (long long)i * ldx + j] = h;
-    Xlo[(long long)b * n * ldx + (long long)i * ldx + j] = l;
+    __syncthreads();                               // the mirrored tile has been read
+    if (i0 != j0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mt[ty + 8 * q][tx] = x[q];
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = j0 + ty + 8 * q, c = i0 + tx;
+            if (r < n && c < n) X[bo + (long long)r * n + c] = mt[tx][ty + 8 * q];
+        }
+    }
+    bits = __reduce_max_sync(0xffffffffu, bits);
+    if (tx == 0) red[ty] = bits;
+    __syncthreads();
+    if (tx == 0 && ty == 0) {
+        for (int w = 1; w < 8; ++w) bits = max(bits, red[w]);
+        atomicMax(&xmax[b], bits);
+    }
 }
 
-// Q = G D_R + 2 acc (acc = Y (V^T X V)), split row-major
+// Q = G D_R + 2 acc (acc = Y (V^T X V)), row-major FP32, its largest |entry| recorded per matrix
 struct EpiQ {
     int m, n;
     const float *G;      // m x n FP32 (nullable = zero)
     const float *S;
     float sqrt_eps;
     int exact;
-    float *hi, *lo;
-    long long ld;
-    struct Acc {};
-    static constexpr bool kElem = true, kRow = true;
-    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
+    float *Q;
+    unsigned *qmax;
+    struct Acc { unsigned mx; };
+    static constexpr bool kRow = true;
+    PSVD_DEV bool row16(Acc &a, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
         if (r0 >= m || c0 >= n) return true;
-        if (c0 + 16 > n || (G && ((n & 7) || ((uintptr_t)G & 31)))) return false;
+        if (c0 + 16 > n || (n & 7) || ((uintptr_t)Q & 31) || (G && ((uintptr_t)G & 31))) return false;
         const int r = r0 + lane;
         // D_R of the 16 columns: one lane each
         const float dr = G && lane < 16 ? dr_of(S[(long long)b * n + c0 + lane], sqrt_eps, exact) : 0.f;
-        uint32_t h[16], l[16], g[8];
+        const long long o = (long long)b * m * n + (long long)r * n + c0;
+        uint32_t w[16], g[8];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             float x = 2.f * v[i];
@@ -148,52 +287,51 @@ struct EpiQ {
                 if ((i & 7) == 0) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q) g[q] = 0u;
-                    if (r < m) ld_v8(G + (long long)b * m * n + (long long)r * n + c0 + i, g);
+                    if (r < m) ld_v8(G + o + i, g);
                 }
                 x += __uint_as_float(g[i & 7]) * __shfl_sync(0xffffffffu, dr, i);
             }
-            float a, c;
-            split_tf32(x, a, c);
-            h[i] = __float_as_uint(a);
-            l[i] = __float_as_uint(c);
+            w[i] = __float_as_uint(x);
+            if (r < m) a.mx = max(a.mx, __float_as_uint(fabsf(x)));
         }
-        if (r < m) {
-            const long long o = (long long)b * m * ld + (long long)r * ld + c0;
-            st_v8x2(hi + o, h);
-            st_v8x2(lo + o, l);
-        }
+        if (r < m) st_v8x2(Q + o, w);
         return true;
     }
-    PSVD_DEV bool staged() const { return true; }
-    PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
-        if (r >= m || c >= n) return;
-        float x = 2.f * v;
-        if (G) x += G[(long long)b * m * n + (long long)r * n + c] * dr_of(S[(long long)b * n + c], sqrt_eps, exact);
-        float h, l;
-        split_tf32(x, h, l);
-        const long long o = (long long)b * m * ld + (long long)r * ld + c;
-        hi[o] = h;
-        lo[o] = l;
-    }
-    PSVD_DEV void begin(Acc &) const {}
+    PSVD_DEV bool staged() const { return false; }
+    PSVD_DEV void begin(Acc &a) const { a.mx = 0u; }
     PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
+        if (r >= m) return;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) elem(a, b, r, c0 + i, v[i]);
+        for (int i = 0; i < 16; ++i) {
+            const int c = c0 + i;
+            if (c >= n) break;
+            const long long o = (long long)b * m * n + (long long)r * n + c;
+            float x = 2.f * v[i];
+            if (G) x += G[o] * dr_of(S[(long long)b * n + c], sqrt_eps, exact);
+            Q[o] = x;
+            a.mx = max(a.mx, __float_as_uint(fabsf(x)));
+        }
     }
-    PSVD_DEV void finish(Acc &, int, int, int) const {}
+    PSVD_DEV void finish(Acc &a, int b, int, int) const {
+        const unsigned v = __reduce_max_sync(0xffffffffu, a.mx);
+        if ((threadIdx.x & 31) == 0 && v) atomicMax(&qmax[b], v);
+    }
 };
 
-__global__ void sym_split_kernel(const float *H, int n, float *hi, float *lo, long long ld) {
+// sym(H) / scale as FP16 halves
+__global__ void sym_split_kernel(const float *H, const float *scale, int n, __half *hi, __half *lo, long long ld) {
     const int b = blockIdx.z;
     const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
     if (i >= n || j >= n) return;
     const float *h = H + (long long)b * n * n;
-    float x = 0.5f * (h[(long long)i * n + j] + h[(long long)j * n + i]), a, c;
-    split_tf32(x, a, c);
+    const float x = 0.5f * (h[(long long)i * n + j] + h[(long long)j * n + i]);
+    __half a, c;
+    split_f16(x / scale[b] * kF16X, a, c);
     hi[(long long)b * n * ld + (long long)i * ld + j] = a;
     lo[(long long)b * n * ld + (long long)i * ld + j] = c;
 }
 
+// split TF32 (the EVD backward, whose factors E and Z have no bound known in advance)
 template <class Epi>
 static int g3(const float *ahi, const float *alo, int M, int K, long long lda, long long bsa, const float *bhi,
               const float *blo, int N, long long ldb, long long bsb, int B, const Epi &e, unsigned *err,
@@ -205,43 +343,86 @@ static int g3(const float *ahi, const float *alo, int M, int K, long long lda, l
     s.M = M; s.N = N; s.K = K; s.prec_uniform = PREC_TF32X3; s.err = err;
     return launch_gemm(nullptr, nullptr, &vah, &val, &vbh, &vbl, s, B, e, st) == cudaSuccess ? PSVD_OK : PSVD_ERR_CUDA;
 }
+// split FP16, scaled by scale[b]
+template <class Epi>
+static int g16(const __half *ahi, const __half *alo, int M, int K, long long lda, long long bsa, const __half *bhi,
+               const __half *blo, int N, long long ldb, long long bsb, int B, const float *scale, const Epi &e,
+               unsigned *err, cudaStream_t st) {
+    F16Views f;
+    f.ah = view_f16(ahi, M, K, lda, bsa, B);
+    f.al = view_f16(alo, M, K, lda, bsa, B);
+    f.bh = view_f16(bhi, N, K, ldb, bsb, B);
+    f.bl = view_f16(blo, N, K, ldb, bsb, B);
+    GemmShape s;
+    memset(&s, 0, sizeof(s));
+    s.M = M; s.N = N; s.K = K; s.prec_uniform = PREC_F16X3; s.err = err;
+    s.f16_scale = 1.f;
+    s.f16_scale_b = scale;
+    return launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f) == cudaSuccess
+               ? PSVD_OK : PSVD_ERR_CUDA;
+}
 
 static SplitOut so(float *hi, float *lo, long long ld, long long bs) {
     SplitOut s;
     s.hi = hi; s.lo = lo; s.ld = ld; s.bstride = bs;
     return s;
 }
+static SplitOut so16(__half *hi, __half *lo, long long ld, long long bs) {
+    SplitOut s;
+    s.fhi = hi; s.flo = lo; s.fscale = kF16X; s.ld = ld; s.bstride = s.fbstride = bs;
+    return s;
+}
 
-// Shared tail: Y = M V (row-major + transposed), Z = Y^T G, core, Q, dA = Q V^T.
-static int bwd_tail(BwdWS &w, bool have_g, const float *EH, const float *AU, const float *BV, const float *dS,
+// Largest entries of the inputs (null: none) and the scales that follow from them.
+static int bwd_scales(BwdWS &w, const float *A, const float *G, const float *Bm, const float *U, const float *VT,
+                      cudaStream_t st) {
+    const int B = w.B, m = w.m, n = w.n;
+    const long long mn = (long long)m * n, nn = (long long)n * n;
+    PSVD_TRY(cudaMemsetAsync(w.amax, 0, sizeof(unsigned) * (size_t)B * AM_N, st));
+    const BwdMaxIn in = {{A, G, Bm, U, VT}, {mn, mn, nn, mn, nn}};
+    const long long per = std::max(1, 8 * num_sms() / std::min(B, 8));
+    bwd_max_kernel<<<dim3((unsigned)std::min<long long>((mn + 4095) / 4096, per), B, AM_IN), 256, 0, st>>>(in, B, n, w.amax);
+    bwd_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, n, 0, w.polar ? 1 : 0, w.es);
+    count_launch(2);
+    PSVD_TRY(cudaGetLastError());
+    return PSVD_OK;
+}
+
+// Shared tail: Y = M V (row-major + transposed), Z = Y^T G, core, Q, dA = Q V^T.  G: Ubar or Wbar V, FP32 (null: zero).
+static int bwd_tail(BwdWS &w, const float *G, const float *EH, const float *AU, const float *BV, const float *dS,
                     float eps, int kreg, float *dA, cudaStream_t st) {
     const int B = w.B, m = w.m, n = w.n;
     const long long ldn = w.ldn, ldm = w.ldm, mn = (long long)m * ldn, nm = (long long)n * ldm, nn = (long long)n * ldn;
     {   // Y = M V : B operand B[j][k] = V[k][j] = V^T[j][k]
-        EpiStore e;
+        EpiHalf e;
         memset(&e, 0, sizeof(e));
-        e.rows = m; e.cols = n; e.alpha = 1.f;
+        e.rows = m; e.cols = n; e.inv = w.esp(ES_IM);
         e.hi = w.Yhi; e.lo = w.Ylo; e.ldh = ldn; e.bsh = mn;
         e.hi_t = w.YThi; e.lo_t = w.YTlo; e.ldht = ldm; e.bsht = nm;
-        if (int rc = g3(w.Mhi, w.Mlo, m, n, ldn, mn, w.VThi, w.VTlo, n, ldn, nn, B, e, w.err, st)) return rc;
+        PSVD_TRY_RC(g16(w.Mhi, w.Mlo, m, n, ldn, mn, w.VThi, w.VTlo, n, ldn, nn, B, w.esp(ES_Y), e, w.err, st));
     }
-    if (have_g) {   // Z = Y^T G
+    if (G) {   // Z = Y^T G
         EpiStore e = epi_store_plain(w.Z, n, (long long)n * n, n, n);
-        if (int rc = g3(w.YThi, w.YTlo, n, m, ldm, nm, w.GThi, w.GTlo, n, ldm, nm, B, e, w.err, st)) return rc;
+        PSVD_TRY_RC(g16(w.YThi, w.YTlo, n, m, ldm, nm, w.GThi, w.GTlo, n, ldm, nm, B, w.esp(ES_Z), e, w.err, st));
     }
-    dim3 g16((n + 15) / 16, (n + 15) / 16, B), b16(16, 16);
-    bwd_core_kernel<<<g16, b16, 0, st>>>(AU, BV, have_g ? w.Z : nullptr, EH, w.S, dS, n, eps, kreg, 1e-6f, w.Xhi,
-                                         w.Xlo, ldn);
-    count_launch(1);
+    const unsigned nt = (n + 31) / 32;
+    bwd_core_kernel<<<dim3(nt, nt, B), dim3(32, 8), 0, st>>>(AU, BV, G ? w.Z : nullptr, EH, w.S, dS, n, eps, kreg, 1e-6f,
+                                                            w.X, w.amax + AM_X * B);
+    bwd_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, n, 1, 0, w.es);
+    count_launch(2);
+    PSVD_TRY(prepare_operand(w.X, n, (long long)n * n, B, n, n, false, 1.f, w.esp(ES_X), so16(w.Xhi, w.Xlo, ldn, nn), st));
     {   // Q = G D_R + 2 Y (V^T X V)  (B operand = V^T X V, symmetric)
         EpiQ e;
-        e.m = m; e.n = n; e.G = have_g ? w.G : nullptr; e.S = w.S; e.sqrt_eps = sqrtf(eps); e.exact = kreg == 2;
-        e.hi = w.Qhi; e.lo = w.Qlo; e.ld = ldn;
-        if (int rc = g3(w.Yhi, w.Ylo, m, n, ldn, mn, w.Xhi, w.Xlo, n, ldn, nn, B, e, w.err, st)) return rc;
+        e.m = m; e.n = n; e.G = G; e.S = w.S; e.sqrt_eps = sqrtf(eps); e.exact = kreg == 2;
+        e.Q = w.Q; e.qmax = w.amax + AM_Q * B;
+        PSVD_TRY_RC(g16(w.Yhi, w.Ylo, m, n, ldn, mn, w.Xhi, w.Xlo, n, ldn, nn, B, w.esp(ES_QP), e, w.err, st));
     }
+    bwd_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, n, 2, 0, w.es);
+    count_launch(1);
+    PSVD_TRY(prepare_operand(w.Q, n, (long long)m * n, B, m, n, false, 1.f, w.esp(ES_Q), so16(w.Qhi, w.Qlo, ldn, mn), st));
     {   // dA = Q V^T : B operand B[j][k] = V^T[k][j] = V[j][k]
         EpiStore e = epi_store_plain(dA, n, (long long)m * n, m, n);
-        if (int rc = g3(w.Qhi, w.Qlo, m, n, ldn, mn, w.Vhi, w.Vlo, n, ldn, nn, B, e, w.err, st)) return rc;
+        PSVD_TRY_RC(g16(w.Qhi, w.Qlo, m, n, ldn, mn, w.Vhi, w.Vlo, n, ldn, nn, B, w.esp(ES_DA), e, w.err, st));
     }
     return cudaGetLastError() == cudaSuccess ? PSVD_OK : PSVD_ERR_CUDA;
 }
@@ -250,70 +431,64 @@ int svd_backward(const float *A, const float *U, const float *S, const float *VT
                  const float *dVT, float *dA, BwdWS &w, double eps, int kreg, cudaStream_t st) {
     const int B = w.B, m = w.m, n = w.n;
     const long long ldn = w.ldn, ldm = w.ldm, mn = (long long)m * ldn, nm = (long long)n * ldm, nn = (long long)n * ldn;
+    const long long umn = (long long)m * n, unn = (long long)n * n;
     const float feps = kreg == 2 ? 0.f : (float)eps;
-    if (cudaMemcpyAsync(w.S, S, sizeof(float) * (size_t)B * n, cudaMemcpyDeviceToDevice, st)) return PSVD_ERR_CUDA;
-    if (prepare_operand(A, n, (long long)m * n, B, m, n, false, 1.f, nullptr, so(w.Mhi, w.Mlo, ldn, mn), st) ||
-        prepare_operand(VT, n, (long long)n * n, B, n, n, false, 1.f, nullptr, so(w.VThi, w.VTlo, ldn, nn), st) ||
-        prepare_operand(VT, n, (long long)n * n, B, n, n, true, 1.f, nullptr, so(w.Vhi, w.Vlo, ldn, nn), st))
-        return PSVD_ERR_CUDA;
+    PSVD_TRY(cudaMemcpyAsync(w.S, S, sizeof(float) * (size_t)B * n, cudaMemcpyDeviceToDevice, st));
+    PSVD_TRY_RC(bwd_scales(w, A, dU, dVT, dU ? U : nullptr, VT, st));
+    PSVD_TRY(prepare_operand(A, n, umn, B, m, n, false, 1.f, w.esp(ES_M), so16(w.Mhi, w.Mlo, ldn, mn), st));
+    PSVD_TRY(prepare_operand(VT, n, unn, B, n, n, false, 1.f, w.esp(ES_V), so16(w.VThi, w.VTlo, ldn, nn), st));
+    PSVD_TRY(prepare_operand(VT, n, unn, B, n, n, true, 1.f, w.esp(ES_V), so16(w.Vhi, w.Vlo, ldn, nn), st));
     if (dU) {
-        if (prepare_operand(U, n, (long long)m * n, B, m, n, true, 1.f, nullptr, so(w.UThi, w.UTlo, ldm, nm), st) ||
-            prepare_operand(dU, n, (long long)m * n, B, m, n, true, 1.f, nullptr, so(w.GThi, w.GTlo, ldm, nm), st))
-            return PSVD_ERR_CUDA;
-        if (cudaMemcpyAsync(w.G, dU, sizeof(float) * (size_t)B * m * n, cudaMemcpyDeviceToDevice, st))
-            return PSVD_ERR_CUDA;
-        EpiStore e = epi_store_plain(w.AU, n, (long long)n * n, n, n);       // A_U = U^T Ubar
-        if (int rc = g3(w.UThi, w.UTlo, n, m, ldm, nm, w.GThi, w.GTlo, n, ldm, nm, B, e, w.err, st)) return rc;
+        PSVD_TRY(prepare_operand(U, n, umn, B, m, n, true, 1.f, w.esp(ES_U), so16(w.UThi, w.UTlo, ldm, nm), st));
+        PSVD_TRY(prepare_operand(dU, n, umn, B, m, n, true, 1.f, w.esp(ES_G), so16(w.GThi, w.GTlo, ldm, nm), st));
+        EpiStore e = epi_store_plain(w.AU, n, unn, n, n);       // A_U = U^T Ubar
+        PSVD_TRY_RC(g16(w.UThi, w.UTlo, n, m, ldm, nm, w.GThi, w.GTlo, n, ldm, nm, B, w.esp(ES_AU), e, w.err, st));
     }
     if (dVT) {
-        if (prepare_operand(dVT, n, (long long)n * n, B, n, n, false, 1.f, nullptr, so(w.dVThi, w.dVTlo, ldn, nn), st))
-            return PSVD_ERR_CUDA;
-        EpiStore e = epi_store_plain(w.BV, n, (long long)n * n, n, n);       // B_V = V^T Vbar
-        if (int rc = g3(w.VThi, w.VTlo, n, n, ldn, nn, w.dVThi, w.dVTlo, n, ldn, nn, B, e, w.err, st)) return rc;
+        PSVD_TRY(prepare_operand(dVT, n, unn, B, n, n, false, 1.f, w.esp(ES_B), so16(w.dVThi, w.dVTlo, ldn, nn), st));
+        EpiStore e = epi_store_plain(w.BV, n, unn, n, n);       // B_V = V^T Vbar
+        PSVD_TRY_RC(g16(w.VThi, w.VTlo, n, n, ldn, nn, w.dVThi, w.dVTlo, n, ldn, nn, B, w.esp(ES_BV), e, w.err, st));
     }
-    return bwd_tail(w, dU != nullptr, nullptr, dU ? w.AU : nullptr, dVT ? w.BV : nullptr, dS, feps, kreg, dA, st);
+    return bwd_tail(w, dU, nullptr, dU ? w.AU : nullptr, dVT ? w.BV : nullptr, dS, feps, kreg, dA, st);
 }
 
 int polar_backward(const float *A, const float *H, const float *dW, const float *dH, float *dA, BwdWS &w, double eps,
                    cudaStream_t st) {
     const int B = w.B, m = w.m, n = w.n;
     const long long ldn = w.ldn, ldm = w.ldm, mn = (long long)m * ldn, nm = (long long)n * ldm, nn = (long long)n * ldn;
-    // EVD of H (symmetrized by the eigensolver's reads of the full matrix)
-    if (int rc = eigh_forward(H, w.S, w.T1, w.ew, st, w.VThi, w.VTlo)) return rc;   // V^T plain in T1
-    if (prepare_operand(A, n, (long long)m * n, B, m, n, false, 1.f, nullptr, so(w.Mhi, w.Mlo, ldn, mn), st))
-        return PSVD_ERR_CUDA;
-    if (prepare_operand(w.T1, n, (long long)n * n, B, n, n, true, 1.f, nullptr, so(w.Vhi, w.Vlo, ldn, nn), st))
-        return PSVD_ERR_CUDA;
-    const float *EH = nullptr;
+    const long long umn = (long long)m * n, unn = (long long)n * n;
+    // EVD of H (symmetrized by the eigensolver's reads of the full matrix); V^T plain in T1
+    PSVD_TRY_RC(eigh_forward(H, w.S, w.T1, w.ew, st));
+    PSVD_TRY_RC(bwd_scales(w, A, dW, dH, nullptr, nullptr, st));
+    PSVD_TRY(prepare_operand(A, n, umn, B, m, n, false, 1.f, w.esp(ES_M), so16(w.Mhi, w.Mlo, ldn, mn), st));
+    PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, false, 1.f, nullptr, so16(w.VThi, w.VTlo, ldn, nn), st));
+    PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, true, 1.f, nullptr, so16(w.Vhi, w.Vlo, ldn, nn), st));
+    const float *EH = w.BV;
     if (dH) {
-        dim3 g16((n + 15) / 16, (n + 15) / 16, B), b16(16, 16);
-        sym_split_kernel<<<g16, b16, 0, st>>>(dH, n, w.dVThi, w.dVTlo, ldn);    // sym(Hbar)
+        dim3 g16x((n + 15) / 16, (n + 15) / 16, B), b16(16, 16);
+        sym_split_kernel<<<g16x, b16, 0, st>>>(dH, w.esp(ES_B), n, w.dVThi, w.dVTlo, ldn);    // sym(Hbar)
         count_launch(1);
         // T1 = V^T sym(Hbar)  (B operand B[j][k] = Hs[k][j] = Hs[j][k])
-        EpiStore e = epi_store_plain(w.T1, n, (long long)n * n, n, n);
-        if (int rc = g3(w.VThi, w.VTlo, n, n, ldn, nn, w.dVThi, w.dVTlo, n, ldn, nn, B, e, w.err, st)) return rc;
-        if (prepare_operand(w.T1, n, (long long)n * n, B, n, n, false, 1.f, nullptr, so(w.T1hi, w.T1lo, ldn, nn), st))
-            return PSVD_ERR_CUDA;
+        EpiStore e = epi_store_plain(w.T1, n, unn, n, n);
+        PSVD_TRY_RC(g16(w.VThi, w.VTlo, n, n, ldn, nn, w.dVThi, w.dVTlo, n, ldn, nn, B, w.esp(ES_T1), e, w.err, st));
+        PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, false, 1.f, w.esp(ES_B), so16(w.T1hi, w.T1lo, ldn, nn), st));
         // E_H = T1 V  (B operand B[j][k] = V[k][j] = V^T[j][k])
-        EpiStore e2 = epi_store_plain(w.BV, n, (long long)n * n, n, n);
-        if (int rc = g3(w.T1hi, w.T1lo, n, n, ldn, nn, w.VThi, w.VTlo, n, ldn, nn, B, e2, w.err, st)) return rc;
-        EH = w.BV;
+        EpiStore e2 = epi_store_plain(w.BV, n, unn, n, n);
+        PSVD_TRY_RC(g16(w.T1hi, w.T1lo, n, n, ldn, nn, w.VThi, w.VTlo, n, ldn, nn, B, w.esp(ES_EH), e2, w.err, st));
     } else {
-        if (cudaMemsetAsync(w.BV, 0, sizeof(float) * (size_t)B * n * n, st)) return PSVD_ERR_CUDA;
-        EH = w.BV;
+        PSVD_TRY(cudaMemsetAsync(w.BV, 0, sizeof(float) * (size_t)B * n * n, st));
     }
     if (dW) {
-        // G = Wbar V (row-major FP32 for the epilogue, and transposed split for Z)
-        if (prepare_operand(dW, n, (long long)m * n, B, m, n, false, 1.f, nullptr, so(w.Wbhi, w.Wblo, ldn, mn), st))
-            return PSVD_ERR_CUDA;
-        EpiStore e;
+        // G = Wbar V (row-major FP32 for the epilogue, and transposed halves for Z)
+        PSVD_TRY(prepare_operand(dW, n, umn, B, m, n, false, 1.f, w.esp(ES_G), so16(w.Wbhi, w.Wblo, ldn, mn), st));
+        EpiHalf e;
         memset(&e, 0, sizeof(e));
-        e.rows = m; e.cols = n; e.alpha = 1.f;
-        e.out = w.G; e.ld = n; e.bs = (long long)m * n;
+        e.rows = m; e.cols = n; e.inv = w.esp(ES_IG);
+        e.out = w.G; e.ld = n; e.bs = umn;
         e.hi_t = w.GThi; e.lo_t = w.GTlo; e.ldht = ldm; e.bsht = nm;
-        if (int rc = g3(w.Wbhi, w.Wblo, m, n, ldn, mn, w.VThi, w.VTlo, n, ldn, nn, B, e, w.err, st)) return rc;
+        PSVD_TRY_RC(g16(w.Wbhi, w.Wblo, m, n, ldn, mn, w.VThi, w.VTlo, n, ldn, nn, B, w.esp(ES_WV), e, w.err, st));
     }
-    return bwd_tail(w, dW != nullptr, EH, nullptr, nullptr, nullptr, (float)eps, eps == 0.0 ? 2 : 0, dA, st);
+    return bwd_tail(w, dW ? w.G : nullptr, EH, nullptr, nullptr, nullptr, (float)eps, eps == 0.0 ? 2 : 0, dA, st);
 }
 
 

@@ -231,6 +231,81 @@ struct EpiSubHalf {
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 
+// 16 values of one row as split-FP16 halves of v * fs: along the row at rhi / rlo when `rowv`, transposed
+// (this lane's 16 rows of column c0 + lane / 2) at chi / clo when `colv`; all lanes call it.
+PSVD_DEV void f16_row16(const float (&v)[16], float fs, __half *rhi, __half *rlo, bool rowv, __half *chi, __half *clo,
+                        bool colv, float *sw) {
+    uint32_t w[16], o[16], h[8], l[8];
+    split_f16x16(v, fs, h, l);
+    if (rowv) {
+        st_v8(rhi, h);
+        st_v8(rlo, l);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {                  // (hi, lo) of one value per word
+        w[2 * i] = __byte_perm(h[i], l[i], 0x5410);
+        w[2 * i + 1] = __byte_perm(h[i], l[i], 0x7632);
+    }
+    warp_transpose16(sw, w, o);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        h[i] = __byte_perm(o[2 * i], o[2 * i + 1], 0x5410);
+        l[i] = __byte_perm(o[2 * i], o[2 * i + 1], 0x7632);
+    }
+    if (colv) {
+        st_v8(chi, h);
+        st_v8(clo, l);
+    }
+}
+
+// Split-FP16 output of v * inv[b] * kF16X, row-major (hi, may be null) and transposed (hi_t), optionally with
+// the plain values (out).
+struct EpiHalf {
+    int rows, cols;
+    const float *inv;
+    float *out;
+    long long ld, bs;
+    __half *hi, *lo;
+    long long ldh, bsh;
+    __half *hi_t, *lo_t;
+    long long ldht, bsht;
+    struct Acc {};
+    static constexpr bool kRow = true;
+    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
+        if (r0 >= rows || c0 >= cols) return true;
+        if (c0 + 16 > cols || (out && ((((uintptr_t)out & 31) != 0) || ((ld | bs) & 7) != 0))) return false;
+        const int r = r0 + lane, ct = c0 + (lane >> 1);
+        if (out && r < rows) {
+            uint32_t w[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(v[i]);
+            st_v8x2(out + b * bs + (long long)r * ld + c0, w);
+        }
+        const long long o = b * bsh + (long long)r * ldh + c0;
+        const long long t = b * bsht + (long long)ct * ldht + r0 + 16 * (lane & 1);    // (padding past `rows`: zeros)
+        f16_row16(v, inv[b] * kF16X, hi + o, lo + o, hi && r < rows, hi_t + t, lo_t + t, true, sw);
+        return true;
+    }
+    PSVD_DEV void begin(Acc &) const {}
+    PSVD_DEV void chunk(Acc &, int b, int r, int c0, int, int, float (&v)[16]) const {
+        if (r >= rows) return;
+        const float fs = inv[b] * kF16X;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int c = c0 + i;
+            if (c >= cols) break;
+            if (out) out[b * bs + (long long)r * ld + c] = v[i];
+            __half h, l;
+            split_f16(v[i] * fs, h, l);
+            if (hi) { hi[b * bsh + (long long)r * ldh + c] = h; lo[b * bsh + (long long)r * ldh + c] = l; }
+            hi_t[b * bsht + (long long)c * ldht + r] = h;
+            lo_t[b * bsht + (long long)c * ldht + r] = l;
+        }
+    }
+    PSVD_DEV bool staged() const { return false; }
+    PSVD_DEV void finish(Acc &, int, int, int) const {}
+};
+
 inline EpiStore epi_store_plain(float *out, long long ld, long long bs, int rows, int cols) {
     EpiStore e;
     memset(&e, 0, sizeof(e));

@@ -260,28 +260,10 @@ PSVD_DEV void store_rung(int p, long long o, long long of, float x, float fs, __
 PSVD_DEV void rung_row16(int p, const float (&v)[16], float fs, __nv_bfloat16 *r16, float *rhi, float *rlo,
                          long long ro, long long roh, bool rowv, __nv_bfloat16 *c16, float *chi, float *clo,
                          long long co, long long coh, bool colv, float *sw) {
-    uint32_t w[16], o[16], h[8], l[8];
+    uint32_t w[16], o[16], h[8];
     if (p == PREC_F16X3) {
-        split_f16x16(v, fs, h, l);
-        if (rowv) {
-            st_v8(reinterpret_cast<__half *>(rhi) + roh, h);
-            st_v8(reinterpret_cast<__half *>(rlo) + roh, l);
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {              // (hi, lo) of one value per word
-            w[2 * i] = __byte_perm(h[i], l[i], 0x5410);
-            w[2 * i + 1] = __byte_perm(h[i], l[i], 0x7632);
-        }
-        warp_transpose16(sw, w, o);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            h[i] = __byte_perm(o[2 * i], o[2 * i + 1], 0x5410);
-            l[i] = __byte_perm(o[2 * i], o[2 * i + 1], 0x7632);
-        }
-        if (colv) {
-            st_v8(reinterpret_cast<__half *>(chi) + coh, h);
-            st_v8(reinterpret_cast<__half *>(clo) + coh, l);
-        }
+        f16_row16(v, fs, reinterpret_cast<__half *>(rhi) + roh, reinterpret_cast<__half *>(rlo) + roh, rowv,
+                  reinterpret_cast<__half *>(chi) + coh, reinterpret_cast<__half *>(clo) + coh, colv, sw);
     } else if (p == PREC_TF32) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(tf32_round(v[i]));

@@ -66,3 +66,32 @@ def test_product_rows_off_alignment(M, N, K, precision):
         tol = {0: 2.0 ** -8, 1: 2.0 ** -10, 2: 2.0 ** -19}[precision]   # operand rounding, with a factor 2
         bound = (a.double().abs() @ b.double().abs().transpose(1, 2))
         assert ((d - ref).abs() <= tol * bound + 1e-30).all()
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (40, 7), (70, 33), (129, 64), (300, 257)])
+@pytest.mark.parametrize("sa,su,sv,sg", [(1.0, 1.0, 1.0, 1.0), (1e6, 1.0, 1.0, 1e-12), (1e-6, 1.0, 1.0, 1e12),
+                                         (1.0, 1e3, 24.0, 1.0)])
+def test_backward_edges_and_ranges(m, n, sa, su, sv, sg):
+    """The formula of the backward in FP64 on the same FP32 inputs, also with inputs far from 1 and with factors
+    that are not orthonormal.  Bound: a product errs by about 3 * 2^-22 of the size of its terms, and the
+    divided differences of an evenly spaced spectrum raise the largest term over the mean by less than 25:
+    25 * 3 * 2^-22 < 2e-5."""
+    import paper_2609_32505_gb300 as P
+    s = W.linear_spectrum(n) if n > 1 else np.ones(1)
+    a, q1, q2 = W.constructed(61, m, n, s)
+    gu, gs, gv = W.loss_weights(62, m, n)
+    f32 = lambda x: np.ascontiguousarray(x).astype(np.float32)
+    A, U, S, VT = f32(sa * a), f32(su * q1), f32(sa * s), f32(sv * q2.T)
+    dU, dS, dVT = f32(sg * gu), f32(sg / sa * gs), f32(sg * gv.T)
+    t = lambda x: torch.from_numpy(x).cuda()
+    da = P.svd_bwd(t(A), t(U), t(S), t(VT), t(dU), t(dS), t(dVT), 0.0, 2).cpu().double().numpy()
+    A, U, S, VT, dU, dS, dVT = [x.astype(np.float64) for x in (A, U, S, VT, dU, dS, dVT)]
+    B = U.T @ dU + VT @ dVT.T
+    d = S[:, None] - S[None, :]
+    K = np.divide(1.0, d, out=np.zeros_like(d), where=np.abs(d) > 1e-6 * S.max())
+    Y = A @ VT.T
+    D = 1.0 / S
+    E = np.diag(dS) - K * (B - B.T) / 2 - D[:, None] * (Y.T @ dU) * D[None, :]
+    X = (E + E.T) / 2 / (S[:, None] + S[None, :])
+    ref = (dU * D[None, :] + 2 * Y @ X) @ VT
+    assert _rel(da, ref) <= 2e-5
