@@ -1,13 +1,13 @@
 // Symmetric eigendecomposition H = V Sigma V^T (the EVD of Algorithm 1), in four stages:
-//  1. Householder tridiagonalization Q^T H Q = T (FP32, persistent cooperative kernel,
-//     one group barrier per reflector; the row that the next reflector is built from
-//     is left un-updated and corrected on the fly, so the rank-2 update of step k and
+//  1. Householder tridiagonalization Q^T H Q = T in FP32: on chip (trd.cu) for 3 <= n <= 4096, otherwise the
+//     persistent cooperative kernel below (one group barrier per reflector; the row that the next reflector
+//     is built from is left un-updated and corrected on the fly, so the rank-2 update of step k and
 //     the matrix-vector product of step k+1 touch only rows owned by the same warp).
 //  2. Eigenvalues of T by Sturm-count multisection (FP32, on T scaled to unit norm);
 //     eigenvalues with close neighbours refined by multisection with float-float counts.
-//  3. Eigenvectors of T by inverse iteration (one thread per eigenvalue, partially
-//     pivoted tridiagonal LU, operands streamed through shared memory; float-float
-//     recurrences where a warp's eigenvalues are well separated, FP64 otherwise),
+//  3. Eigenvectors of T by inverse iteration (two lanes per eigenvalue, tridiagonal LU with row
+//     interchanges from both ends, operands streamed through shared memory; float-float
+//     arithmetic where a warp's eigenvalues are well separated, FP64 otherwise),
 //     Rayleigh quotients, modified Gram-Schmidt inside clusters of close eigenvalues.
 //  4. Back-transform V^T = Z^T Q^T with compact-WY blocks of kWY reflectors on the
 //     tcgen05 split-FP16 product kernel, then the sign convention (largest-|.| entry
@@ -443,21 +443,31 @@ PSVD_DEV int sturm_count_ff(const float4 *__restrict__ dd, int n, ff x, float pi
     return c;
 }
 
-// dd[b][t] = {split(d_t / tn), split(e_{t-1}^2 / tn^2)} for the float-float Sturm counts, and
-// de[b][t] = {split(d_t / tn), split(e_t / tn)} (e_{n-1} = 0) for float-float inverse iteration.
-__global__ void sturm_prep_kernel(const double *D, const double *E, const double *tnorm, int n, float4 *dd,
-                                  float4 *de) {
+// dd[b][t] = {split(d_t / tn), split(e_{t-1}^2 / tn^2)} for the float-float Sturm counts, and the tables of
+// inverse iteration: tabf / tabd[b][k][0] = {d_k, e_k} / tn and [b][k][1] = {d_{n-1-k}, e_{n-2-k}} / tn.
+__global__ void sturm_prep_kernel(const double *D, const double *E, const double *tnorm, int n, int rows, float4 *dd,
+                                  float4 *tabf, double2 *tabd) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    if (t >= n) return;
     const double tn = tnorm[b], inv = tn > 0.0 ? 1.0 / tn : 0.0;
-    const double dv = D[(long long)b * n + t] * inv;
-    const double ev = t > 0 ? E[(long long)b * n + t - 1] * inv : 0.0;
-    const double e2 = ev * ev;
-    const float dh = (float)dv, eh = (float)e2;
-    dd[(long long)b * n + t] = make_float4(dh, (float)(dv - (double)dh), eh, (float)(e2 - (double)eh));
-    const double en = t + 1 < n ? E[(long long)b * n + t] * inv : 0.0;
-    const float enh = (float)en;
-    de[(long long)b * n + t] = make_float4(dh, (float)(dv - (double)dh), enh, (float)(en - (double)enh));
+    const double *d = D + (long long)b * n, *e = E + (long long)b * n;
+    auto split4 = [](double x, double y) {
+        const float xh = (float)x, yh = (float)y;
+        return make_float4(xh, (float)(x - (double)xh), yh, (float)(y - (double)yh));
+    };
+    if (t < n) {
+        const double ev = t > 0 ? e[t - 1] * inv : 0.0;
+        dd[(long long)b * n + t] = split4(d[t] * inv, ev * ev);
+    }
+    if (t < rows) {
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            const int j = side ? n - 1 - t : t, je = side ? j - 1 : j;
+            const double dv = j >= 0 && j < n ? d[j] * inv : 0.0, ev = je >= 0 && je < n - 1 ? e[je] * inv : 0.0;
+            const long long o = ((long long)b * rows + t) * 2 + side;
+            tabf[o] = split4(dv, ev);
+            tabd[o] = make_double2(dv, ev);
+        }
+    }
 }
 
 // 1/a by the hardware's approximate reciprocal refined with two Newton-Raphson steps
@@ -540,7 +550,7 @@ __global__ void tri_refine_kernel(const float4 *DD, int n, const double *tnorm, 
     if (refined && l == 0) lb[i] = 0.5 * (lo + hi);
 }
 
-// ------------------------------------------------------------ inverse iteration (FP64)
+// ------------------------------------------------------------ inverse iteration
 PSVD_DEV double hash_unit(unsigned a, unsigned b) {
     unsigned h = a * 0x9E3779B1u ^ (b + 0x7F4A7C15u) * 0x85EBCA77u;
     h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
@@ -552,377 +562,348 @@ PSVD_DEV double hash_unit(unsigned a, unsigned b) {
 constexpr double kRefineNear = 1e-5;
 constexpr double kClusterTol = 1e-11;
 
+// Inverse iteration of one matrix's eigenvectors, 16 to a warp: lanes 0-15 work from the first row down,
+// lanes 16-31 on the same vectors from the last row up, and the two meet in a 2 x 2 system in the middle,
+// so the chain of dependent steps is half as long.  "Row k" of a lane is component k of the one or
+// n - 1 - k of the other; both run the same code on a table that holds T in both orders.
 struct InvitParams {
     const double *D, *E, *tn;
-    const float4 *de;        // [b][j] = {d_j / tn, e_j / tn} as float-float pairs (e_{n-1} = 0)
+    const float4 *tabf;      // [b][rows][2] T / tn: {d, e} as float-float pairs, in row order and reversed
+    const double2 *tabd;     // the same in FP64
     const double *lam0;      // the eigenvalues before inverse iteration (for the gaps)
     double *lam;
-    double *xs, *u0, *u1, *u2, *lm;
-    float *xf;               // the normalized eigenvectors, interleaved [n][stride] like xs
-    unsigned *piv;           // pivot flags, bit (j % 32) of word [j / 32][t]
-    int n, first, count;     // vectors [first, first + count) of the flattened (b, i) index
+    double *x, *l, *u;       // per warp: [rows][32] vectors and multipliers, [rows][3][32] pivot rows
+    float *xf;               // the normalized eigenvectors, interleaved [n][stride]
+    int n, rows, first, count;   // vectors [first, first + count) of the flattened (b, i) index
     long long stride;        // = chunk
 };
 
-// Each thread owns one eigenvector and walks its length-n recurrences in order.  The
-// operands of every pass are streamed through a per-warp shared-memory ring with
-// cp.async (kIvR stages of kIvJ rows, up to kIvNA arrays), so a warp keeps about
-// (kIvR - 1) kIvJ rows of loads in flight instead of waiting on each one.  (Measured at
-// n = 4096: 8 or 16 vectors per warp instead of 32 leave the time unchanged, each vector's
-// chain of dependent operations sets it; plain loads prefetched 2, 4 or 8 steps ahead into
-// registers instead of the ring make eigh ~11 ms slower.)
-constexpr int kIvJ = 16, kIvR = 4, kIvNA = 4, kIvW = 32;
-constexpr int kIvStage = kIvNA * kIvJ * kIvW;                     // doubles per stage
-constexpr size_t kIvSmem = sizeof(double) * kIvR * kIvStage;      // 64 KB per warp
+// Each lane walks its recurrences in order, and the chain of dependent operations of a step is what
+// bounds the kernel as long as there are few warps per SM; so a warp takes 16 vectors although that
+// doubles the warps, and what is not on the chain is kept cheap: every pass reads its operands through a
+// shared-memory ring of kIvR stages of kIvJ rows, which lie in memory as they lie in the ring, so a stage
+// is a few 16-byte cp.async per lane (one 8-byte copy, pointer and range check per value before).  At
+// n = 4096 (256 warps) 1.03 ms, where one thread per vector from the first row to the last took 3.9 ms;
+// 64 matrices of 512 3.2 -> 1.4 ms; 4 matrices of 4096, most of them in FP64, 42 -> 8 ms, there also because
+// they run at the same time.  (Three stages of 8 rows against four: 64 x 512 1.36 against 1.49 ms, 8 x 1024
+// 0.31 against 0.33, others the same; stages of 4 or 16 rows are up to 20% slower at 4096.)
+constexpr int kIvR = 3, kIvW = 32, kIvV = 16;
+constexpr int kIvRow = 8 * kIvW;                                  // bytes of one value per lane
+constexpr int kIvStage = 4 * kIvJ * kIvRow;
+constexpr size_t kIvSmem = (size_t)kIvR * kIvStage;               // 24 KB per warp
 
-PSVD_DEV void cp_async8(double *sdst, const double *gsrc) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(sdst)), "l"(gsrc) : "memory");
+PSVD_DEV void cp_async16(unsigned char *sdst, const unsigned char *gsrc) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(sdst)), "l"(gsrc) : "memory");
 }
 PSVD_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 PSVD_DEV void cp_async_wait_ring() { asm volatile("cp.async.wait_group %0;" ::"n"(kIvR - 2) : "memory"); }
 
-// One streamed operand: row k lives at p + k * stride (p already at row 0; stride may be
-// negative), rows k in [kmin, kmax) exist, the others are not fetched (their slots are
-// left as they are and the body does not read them).
-struct IvArr {
-    const double *p;
-    long long stride;
-    int kmin, kmax;
-};
-
-// Streams `nsteps` rows of NA operands through the ring; body(k, ring slot pointer) consumes
-// them in order, slot(a) = p + a*kIvJ*32.  The issuing walks one pointer per operand, so a
-// row costs an add, a copy and a shared address per operand.
-template <int NA, class Body>
-PSVD_DEV void iv_stream(double *ring, int nsteps, const IvArr (&arr)[NA], Body body) {
-    const int lane = threadIdx.x & 31;
-    const int nst = (nsteps + kIvJ - 1) / kIvJ;
-    const double *next[NA];
+// Streams stages 0 .. nst - 1 (descending if kDesc) of two operands with N0 and N1 bytes per stage through
+// the ring; body(k, stage buffer, row in the stage) for every row k < cnt of this lane.  The first `full`
+// stages hold rows of every lane (no check per row).  All lanes of the warp call it.
+template <bool kDesc, int N0, int N1, class Body>
+PSVD_DEV void iv_stream(unsigned char *ring, int nst, int full, int cnt, const void *g0, const void *g1, Body body) {
+    static_assert(N0 + N1 <= kIvStage && N0 % 16 == 0 && N1 % 16 == 0, "stage size");
+    const int at = (threadIdx.x & 31) * 16;
+    const unsigned char *p0 = static_cast<const unsigned char *>(g0) + at, *p1 = static_cast<const unsigned char *>(g1) + at;
+    auto issue = [&](int i) {
+        if (i < nst) {
+            unsigned char *buf = ring + (i % kIvR) * kIvStage + at;
+            const long long s = kDesc ? nst - 1 - i : i;
 #pragma unroll
-    for (int a = 0; a < NA; ++a) next[a] = arr[a].p;
-    int kn = 0;                                    // row the pointers stand at
-    auto issue = [&](int st) {
-        if (st < nst) {
-            double *buf = ring + (st % kIvR) * kIvStage + lane;
-            for (int jj = 0; jj < kIvJ && kn < nsteps; ++jj, ++kn) {
+            for (int o = 0; o < N0; o += 512)
+                if (o + 512 <= N0 || at < N0 - o) cp_async16(buf + o, p0 + s * N0 + o);
 #pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    if (kn >= arr[a].kmin && kn < arr[a].kmax) cp_async8(buf + (a * kIvJ + jj) * kIvW, next[a]);
-                    next[a] += arr[a].stride;
-                }
-            }
+            for (int o = 0; o < N1; o += 512)
+                if (o + 512 <= N1 || at < N1 - o) cp_async16(buf + N0 + o, p1 + s * N1 + o);
         }
         cp_async_commit();
     };
-    for (int st = 0; st < kIvR - 1; ++st) issue(st);
-    for (int st = 0; st < nst; ++st) {
+    for (int i = 0; i < kIvR - 1; ++i) issue(i);
+    for (int i = 0; i < nst; ++i) {
         cp_async_wait_ring();
-        const double *buf = ring + (st % kIvR) * kIvStage + lane;
+        __syncwarp();                              // every lane's copies are in, and stage i - 1 has been read
+        issue(i + kIvR - 1);
+        const unsigned char *buf = ring + (i % kIvR) * kIvStage;
+        const int s = kDesc ? nst - 1 - i : i;
+        if (s < full) {
 #pragma unroll 4
-        for (int jj = 0; jj < kIvJ; ++jj) {
-            const int k = st * kIvJ + jj;
-            if (k >= nsteps) break;
-            body(k, buf + jj * kIvW);
+            for (int jj = 0; jj < kIvJ; ++jj) {
+                const int r = kDesc ? kIvJ - 1 - jj : jj;
+                body(s * kIvJ + r, buf, r);
+            }
+        } else {
+#pragma unroll 1
+            for (int jj = 0; jj < kIvJ; ++jj) {
+                const int r = kDesc ? kIvJ - 1 - jj : jj;
+                if (s * kIvJ + r < cnt) body(s * kIvJ + r, buf, r);
+            }
         }
-        issue(st + kIvR - 1);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    __threadfence_block();   // this pass's stores before the next pass's async reads
-}
-#define IV_SLOT(p, a) (p)[(a) * kIvJ * kIvW]
-
-PSVD_DEV double iv_start(int i, int j) { return hash_unit((unsigned)i, (unsigned)j) + 0.0625; }
-
-// Factor T - mu I = P L U (U with two superdiagonals, reciprocal pivots in u0).
-PSVD_DEV void iv_factor(const InvitParams &P, double *ring, const double *D, const double *E, int n, double mu,
-                        double tiny, int t) {
-    const long long s = P.stride;
-    double a = D[0] - mu;
-    double bsup = E[0];
-    unsigned word = 0;
-    const IvArr arr[3] = {{D + 1, 1, 0, n - 1}, {E, 1, 0, n - 1}, {E + 1, 1, 0, n - 2}};
-    iv_stream(ring, n - 1, arr,
-              [&](int j, const double *p) {
-                  const double c = IV_SLOT(p, 1);
-                  const double dn = IV_SLOT(p, 0) - mu;
-                  const double en = j + 1 < n - 1 ? IV_SLOT(p, 2) : 0.0;
-                  const long long o = (long long)j * s + t;
-                  if (fabs(a) >= fabs(c)) {
-                      if (fabs(a) < tiny) a = a < 0 ? -tiny : tiny;
-                      const double ra = recip64(a);
-                      const double m = c * ra;
-                      P.u0[o] = ra; P.u1[o] = bsup; P.u2[o] = 0.0; P.lm[o] = m;
-                      a = dn - m * bsup;
-                      bsup = en;
-                  } else {
-                      const double rc = recip64(c);
-                      const double m = a * rc;
-                      P.u0[o] = rc; P.u1[o] = dn; P.u2[o] = en; P.lm[o] = m;
-                      word |= 1u << (j & 31);
-                      a = bsup - m * dn;
-                      bsup = -m * en;
-                  }
-                  if ((j & 31) == 31 || j == n - 2) { P.piv[(long long)(j >> 5) * s + t] = word; word = 0; }
-              });
-    if (fabs(a) < tiny) a = a < 0 ? -tiny : tiny;
-    P.u0[(long long)(n - 1) * s + t] = recip64(a);
+    __threadfence_block();                         // this pass's stores before the next pass's copies
+    __syncwarp();
 }
 
-// Forward part of one solve: x <- P-and-L applied to b, where b = scale * x, or the
-// start vector when `first`.
-PSVD_DEV void iv_forward(const InvitParams &P, double *ring, int n, int t, int i, bool first, double scale) {
-    const long long s = P.stride;
-    double *x = P.xs;
-    double carry = first ? iv_start(i, 0) : x[t] * scale;
-    unsigned pword = 0;
-    unsigned pnext = P.piv[t];
-    const IvArr arr[2] = {{x + s + t, s, 0, first ? 0 : n - 1}, {P.lm + t, s, 0, n - 1}};
-    iv_stream(ring, n - 1, arr,
-              [&](int j, const double *p) {
-                  if ((j & 31) == 0) {
-                      pword = pnext;
-                      const long long nw = (long long)((j >> 5) + 1);
-                      if ((nw << 5) < n - 1) pnext = P.piv[nw * s + t];
-                  }
-                  double a = carry;
-                  double b = first ? iv_start(i, j + 1) : IV_SLOT(p, 0) * scale;
-                  if ((pword >> (j & 31)) & 1u) { const double tmp = a; a = b; b = tmp; }
-                  x[(long long)j * s + t] = a;
-                  carry = b - IV_SLOT(p, 1) * a;
-              });
-    x[(long long)(n - 1) * s + t] = carry;
-}
-
-// Backward part: U x = y in place; returns ||x||^2.
-PSVD_DEV double iv_backward(const InvitParams &P, double *ring, int n, int t) {
-    const long long s = P.stride;
-    double *x = P.xs;
-    const long long last = (long long)(n - 1) * s + t;
-    double x1 = x[last] * P.u0[last], x2 = 0.0;
-    x[last] = x1;
-    double nrm = x1 * x1;
-    const long long o0 = (long long)(n - 2) * s + t;     // row n - 2 - k at step k
-    const IvArr arr[4] = {{x + o0, -s, 0, n - 1}, {P.u0 + o0, -s, 0, n - 1}, {P.u1 + o0, -s, 0, n - 1},
-                          {P.u2 + o0, -s, 0, n - 1}};
-    iv_stream(ring, n - 1, arr,
-              [&](int k, const double *p) {
-                  const double v = (IV_SLOT(p, 0) - IV_SLOT(p, 2) * x1 - IV_SLOT(p, 3) * x2) * IV_SLOT(p, 1);
-                  x[(long long)(n - 2 - k) * s + t] = v;
-                  x2 = x1;
-                  x1 = v;
-                  nrm += v * v;
-              });
-    return nrm;
-}
-
-// xf <- scale * x (rounded to FP32) and the Rayleigh quotient x^T T x of the scaled vector.
-PSVD_DEV double iv_finish(const InvitParams &P, double *ring, const double *D, const double *E, int n, int t,
-                          double scale) {
-    const long long s = P.stride;
-    double *x = P.xs;
-    double r = 0.0, prev = 0.0;
-    const IvArr arr[3] = {{x + t, s, 0, n}, {D, 1, 0, n}, {E - 1, 1, 1, n}};   // E[j - 1] from j = 1 on
-    iv_stream(ring, n, arr,
-              [&](int j, const double *p) {
-                  const double xj = IV_SLOT(p, 0) * scale;
-                  P.xf[(long long)j * s + t] = (float)xj;
-                  r += IV_SLOT(p, 1) * xj * xj;
-                  if (j > 0) r += 2.0 * IV_SLOT(p, 2) * prev * xj;
-                  prev = xj;
-              });
-    return r;
-}
-
-// ------------------------------------------------ inverse iteration in float-float
-// The same factorization and solves on T / tn with two-float values on the FP32 pipe, for
-// vectors whose eigenvalue is at least kIvFFGap ||T|| from its neighbours.  The factors
-// and the vectors between passes are stored as (hi, lo) pairs in the 8-byte slots of the
-// FP64 arrays.  A factorization in ~2^-46 arithmetic is exact for a matrix within a few
-// 2^-46 ||T|| of T, so these vectors are off by ~1e-13 ||T|| / gap <= 1e-7; closer
-// eigenvalues keep the FP64 recurrences above.  Rounding the right-hand sides (the stored
-// vectors) perturbs nothing but the start of each solve.
+// Float-float arithmetic on T / tn, for vectors whose eigenvalue is at least kIvFFGap ||T|| from its
+// neighbours.  A factorization in ~2^-45 arithmetic is exact for a matrix within a few 2^-45 ||T|| of T, so
+// these vectors are off by ~1e-13 ||T|| / gap <= 1e-7; closer eigenvalues take the FP64 arithmetic below.
+// Rounding the right-hand sides (the stored vectors) perturbs nothing but the start of each solve.
 constexpr double kIvFFGap = 1e-6;
-constexpr float kIvFFTiny = 0x1p-44f;          // pivot floor on T / tn
-
-PSVD_DEV ff ff_sel(bool c, ff a, ff b) { return ff{c ? a.hi : b.hi, c ? a.lo : b.lo}; }
-PSVD_DEV ff ff_ld(const double *slot) {
-    const float2 v = *reinterpret_cast<const float2 *>(slot);
-    return ff{v.x, v.y};
-}
-PSVD_DEV void ff_st(double *slot, ff v) { *reinterpret_cast<float2 *>(slot) = make_float2(v.hi, v.lo); }
-PSVD_DEV float iv_start_f(int i, int j) {
-    unsigned h = (unsigned)i * 0x9E3779B1u ^ ((unsigned)j + 0x7F4A7C15u) * 0x85EBCA77u;
-    h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
-    return __fmaf_rn((float)(h >> 8), 0x1p-23f, -0.9375f);          // in [-0.9375, 1.0625)
-}
-
-// Factor T/tn - mu I = P L U as iv_factor does; stored per row: u0 = 1 / pivot, u1 u0 and
-// u2 u0 (the superdiagonals pre-scaled, so that each back-substitution step is one
-// dependent multiply-add), and the multiplier.  The pivot choice and both row orders are
-// evaluated with selects (no divergence inside the warp).
-PSVD_DEV void ivf_factor(const InvitParams &P, double *ring, const float4 *de, int n, ff mu, int t) {
-    const long long s = P.stride;
-    const float4 r0 = de[0];
-    ff a = ff_add(ff{r0.x, r0.y}, ff_neg(mu));
-    ff bs = ff{r0.z, r0.w};
-    unsigned word = 0;
-    const double *dd = reinterpret_cast<const double *>(de);     // (d, e) pairs: 2 slots per row
-    const IvArr arr[3] = {{dd + 2, 2, 0, n - 1}, {dd + 1, 2, 0, n - 1}, {dd + 3, 2, 0, n - 1}};
-    iv_stream(ring, n - 1, arr,
-              [&](int j, const double *p) {
-                  const ff dn = ff_add(ff_ld(&IV_SLOT(p, 0)), ff_neg(mu));
-                  const ff c = ff_ld(&IV_SLOT(p, 1));
-                  const ff en = ff_ld(&IV_SLOT(p, 2));
-                  const bool pv = fabsf(a.hi) < fabsf(c.hi);
-                  ff den = ff_sel(pv, c, a);
-                  if (fabsf(den.hi) < kIvFFTiny) den = ff{den.hi < 0.f ? -kIvFFTiny : kIvFFTiny, 0.f};
-                  const ff m = ff_div(ff_sel(pv, a, c), den);
-                  const ff rp = ff_div(ff{1.f, 0.f}, den);
-                  const ff y = ff_sel(pv, dn, bs);
-                  a = ff_add(ff_sel(pv, bs, dn), ff_neg(ff_mul(m, y)));
-                  const ff me = ff_mul(m, en);
-                  const ff u2 = pv ? en : ff{0.f, 0.f};
-                  bs = ff_sel(pv, ff_neg(me), en);
-                  const long long o = (long long)j * s + t;
-                  ff_st(P.u0 + o, rp);
-                  ff_st(P.u1 + o, ff_mul(y, rp));
-                  ff_st(P.u2 + o, ff_mul(u2, rp));
-                  ff_st(P.lm + o, m);
-                  word |= (unsigned)pv << (j & 31);
-                  if ((j & 31) == 31 || j == n - 2) { P.piv[(long long)(j >> 5) * s + t] = word; word = 0; }
-              });
-    if (fabsf(a.hi) < kIvFFTiny) a = ff{a.hi < 0.f ? -kIvFFTiny : kIvFFTiny, 0.f};
-    ff_st(P.u0 + (long long)(n - 1) * s + t, ff_div(ff{1.f, 0.f}, a));
-}
-
-// Forward part of one solve (the pivots and L), right-hand side scale * x or the start vector.
-PSVD_DEV void ivf_forward(const InvitParams &P, double *ring, int n, int t, int i, bool first, float scale) {
-    const long long s = P.stride;
-    double *x = P.xs;
-    ff carry = first ? ff{iv_start_f(i, 0), 0.f} : ff_mulf(ff_ld(x + t), scale);
-    unsigned pword = 0;
-    unsigned pnext = P.piv[t];
-    const IvArr arr[2] = {{x + s + t, s, 0, first ? 0 : n - 1}, {P.lm + t, s, 0, n - 1}};
-    iv_stream(ring, n - 1, arr,
-              [&](int j, const double *p) {
-                  if ((j & 31) == 0) {
-                      pword = pnext;
-                      const long long nw = (long long)((j >> 5) + 1);
-                      if ((nw << 5) < n - 1) pnext = P.piv[nw * s + t];
-                  }
-                  const ff bn = first ? ff{iv_start_f(i, j + 1), 0.f} : ff_mulf(ff_ld(&IV_SLOT(p, 0)), scale);
-                  const bool sw = (pword >> (j & 31)) & 1u;
-                  const ff a = ff_sel(sw, bn, carry);
-                  const ff b = ff_sel(sw, carry, bn);
-                  ff_st(x + (long long)j * s + t, a);
-                  carry = ff_add(b, ff_neg(ff_mul(ff_ld(&IV_SLOT(p, 1)), a)));
-              });
-    ff_st(x + (long long)(n - 1) * s + t, carry);
-}
-
-// Backward part: U x = y in place; returns ||x||^2 (float-float).
-PSVD_DEV ff ivf_backward(const InvitParams &P, double *ring, int n, int t) {
-    const long long s = P.stride;
-    double *x = P.xs;
-    const long long last = (long long)(n - 1) * s + t;
-    ff x1 = ff_mul(ff_ld(x + last), ff_ld(P.u0 + last)), x2 = ff{0.f, 0.f};
-    ff_st(x + last, x1);
-    ff nrm = ff_fma(ff_zero(), x1.hi, x1.hi);
-    const long long o0 = (long long)(n - 2) * s + t;     // row n - 2 - k at step k
-    const IvArr arr[4] = {{x + o0, -s, 0, n - 1}, {P.u0 + o0, -s, 0, n - 1}, {P.u1 + o0, -s, 0, n - 1},
-                          {P.u2 + o0, -s, 0, n - 1}};
-    iv_stream(ring, n - 1, arr,
-              [&](int k, const double *p) {
-                  ff r = ff_mul(ff_ld(&IV_SLOT(p, 0)), ff_ld(&IV_SLOT(p, 1)));
-                  r = ff_add(r, ff_neg(ff_mul(ff_ld(&IV_SLOT(p, 3)), x2)));
-                  const ff v = ff_add(r, ff_neg(ff_mul(ff_ld(&IV_SLOT(p, 2)), x1)));
-                  ff_st(x + (long long)(n - 2 - k) * s + t, v);
-                  x2 = x1;
-                  x1 = v;
-                  nrm = ff_fma(nrm, v.hi, v.hi);
-              });
-    return nrm;
-}
-
-// xf <- scale * x (FP32) and the Rayleigh quotient x^T (T/tn) x / x^T x of that vector.
-PSVD_DEV double ivf_finish(const InvitParams &P, double *ring, const float4 *de, int n, int t, float scale) {
-    const long long s = P.stride;
-    const double *x = P.xs;
-    const double *dd = reinterpret_cast<const double *>(de);
-    ff num = ff_zero(), den = ff_zero();
-    float prev = 0.f;
-    const IvArr arr[3] = {{x + t, s, 0, n}, {dd, 2, 0, n}, {dd - 1, 2, 1, n}};   // e_{j-1} from j = 1 on
-    iv_stream(ring, n, arr,
-              [&](int j, const double *p) {
-                  const float xj = __fmul_rn(__fadd_rn(ff_ld(&IV_SLOT(p, 0)).hi, ff_ld(&IV_SLOT(p, 0)).lo), scale);
-                  P.xf[(long long)j * s + t] = xj;
-                  // x_j (d_j x_j + 2 e_{j-1} x_{j-1})
-                  ff q = ff_mulf(ff_ld(&IV_SLOT(p, 1)), xj);
-                  if (j > 0) q = ff_add(q, ff_mulf(ff_ld(&IV_SLOT(p, 2)), __fmul_rn(2.f, prev)));
-                  num = ff_add(num, ff_mulf(q, xj));
-                  den = ff_fma(den, xj, xj);
-                  prev = xj;
-              });
-    return ((double)num.hi + (double)num.lo) / ((double)den.hi + (double)den.lo);
-}
-
-// One warp per block: 32 eigenvectors, each by inverse iteration from a fixed
-// pseudo-random start.  The bisection shift is accurate to ~1e-7 ||T||: three solves
-// reduce the other components by (shift error / gap)^3.  A warp whose 32 eigenvalues are
-// all at least kIvFFGap ||T|| from their neighbours runs the float-float recurrences, the
-// others the FP64 ones (the choice is per warp, so no warp runs both).
-__global__ void __launch_bounds__(kIvW) tri_invit_kernel(InvitParams P) {
-    extern __shared__ __align__(16) double ivring[];
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = P.n;
-    const long long gi = (long long)P.first + t;
-    const int b = (int)(gi / n), i = (int)(gi % n);
-    bool ffok = true;
-    double tn = 0.0;
-    if (t < P.count) {
-        tn = P.tn[b];
-        const double *lb = P.lam0 + (long long)b * n;
-        double g = 1e300;
-        if (i > 0) g = fmin(g, lb[i - 1] - lb[i]);
-        if (i + 1 < n) g = fmin(g, lb[i] - lb[i + 1]);
-        ffok = n > 1 && tn > 0.0 && g >= kIvFFGap * tn;
+struct IvFF {
+    using V = ff;
+    using S = float;
+    static PSVD_DEV V of(double v) { const float h = (float)v; return ff{h, (float)(v - (double)h)}; }
+    static PSVD_DEV V ld(const void *p) { const float2 v = *static_cast<const float2 *>(p); return ff{v.x, v.y}; }
+    static PSVD_DEV void st(void *p, V v) { *static_cast<float2 *>(p) = make_float2(v.hi, v.lo); }
+    static PSVD_DEV void row(const void *p, V &d, V &e) {
+        const float4 v = *static_cast<const float4 *>(p);
+        d = ff{v.x, v.y};
+        e = ff{v.z, v.w};
     }
-    const bool use_ff = __all_sync(0xffffffffu, ffok);
-    if (t >= P.count) return;
-    const long long s = P.stride;
-    const double mu = P.lam[gi];
-    if (use_ff) {
-        const float4 *de = P.de + (long long)b * n;
-        const double ms = mu / tn;
-        const float mh = (float)ms;
-        ivf_factor(P, ivring, de, n, ff{mh, (float)(ms - (double)mh)}, t);
-        float scale = 1.f;
-        for (int it = 0; it < 3; ++it) {
-            ivf_forward(P, ivring, n, t, i, it == 0, scale);
-            const ff nrm = ivf_backward(P, ivring, n, t);
-            const double nv = (double)nrm.hi + (double)nrm.lo;
-            scale = nv > 0.0 ? (float)(1.0 / sqrt(nv)) : 0.f;
-        }
-        P.lam[gi] = ivf_finish(P, ivring, de, n, t, scale) * tn;
-        return;
+    static PSVD_DEV V start(int i, int j) {
+        unsigned h = (unsigned)i * 0x9E3779B1u ^ ((unsigned)j + 0x7F4A7C15u) * 0x85EBCA77u;
+        h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
+        return ff{__fmaf_rn((float)(h >> 8), 0x1p-23f, -0.9375f), 0.f};          // in [-0.9375, 1.0625)
     }
-    const double *D = P.D + (long long)b * n, *E = P.E + (long long)b * n;
-    if (n == 1) { P.xf[t] = 1.f; return; }
-    if (!(tn > 0.0)) {
-        // T = 0: every vector is an eigenvector; take the unit vectors
-        for (int j = 0; j < n; ++j) P.xf[j * s + t] = j == i ? 1.f : 0.f;
-        P.lam[gi] = 0.0;
-        return;
+    static PSVD_DEV V sel(bool c, V a, V b) { return ff{c ? a.hi : b.hi, c ? a.lo : b.lo}; }
+    static PSVD_DEV V neg(V a) { return ff_neg(a); }
+    static PSVD_DEV V sub(V a, V b) { return ff_add(a, ff_neg(b)); }
+    static PSVD_DEV V mul(V a, V b) { return ff_mul(a, b); }
+    static PSVD_DEV V muls(V a, S s) { return ff_mulf(a, s); }
+    static PSVD_DEV V nfma(V a, V x, V y) { return ff_add(a, ff_neg(ff_mul(x, y))); }       // a - x y
+    static PSVD_DEV V sq(V s, V v) { return ff_fma(s, v.hi, v.hi); }                        // s + v^2
+    static PSVD_DEV bool less(V a, V b) { return fabsf(a.hi) < fabsf(b.hi); }
+    static PSVD_DEV V pivot(V a) {                                                         // floor 2^-44
+        const bool small = fabsf(a.hi) < 0x1p-44f;
+        return ff{small ? copysignf(0x1p-44f, a.hi) : a.hi, small ? 0.f : a.lo};
     }
-    const double tiny = fmax(tn * 2.2e-16, 1e-280);
-    iv_factor(P, ivring, D, E, n, mu, tiny, t);
-    double scale = 1.0;
+    static PSVD_DEV S rcp0(V den) {
+        float r;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(den.hi));
+        return r;
+    }
+    // a / den from r0 ~ 1 / den: the quotient of the leading words and one correction from its residual
+    static PSVD_DEV V div(V a, V den, S r0) {
+        const float r = __fmul_rn(a.hi, r0);
+        const float res = __fadd_rn(__fmaf_rn(-r, den.lo, __fmaf_rn(-r, den.hi, a.hi)), a.lo);
+        const float r2 = __fmul_rn(res, r0);
+        const float h = __fadd_rn(r, r2);
+        return ff{h, __fsub_rn(r2, __fsub_rn(h, r))};
+    }
+    static PSVD_DEV V inv(V den, S r0) { return div(ff{1.f, 0.f}, den, r0); }
+    // one flag in the last bit of a value
+    static PSVD_DEV V flag(V v, bool f) {
+        return ff{v.hi, __uint_as_float((__float_as_uint(v.lo) & ~1u) | (f ? 1u : 0u))};
+    }
+    static PSVD_DEV bool flagged(V v) { return __float_as_uint(v.lo) & 1u; }
+    static PSVD_DEV V other(V v) {
+        return ff{__shfl_xor_sync(0xffffffffu, v.hi, 16), __shfl_xor_sync(0xffffffffu, v.lo, 16)};
+    }
+    static PSVD_DEV double d(V v) { return (double)v.hi + (double)v.lo; }
+    static PSVD_DEV S scaled(V v, S s) { return __fmul_rn(__fadd_rn(v.hi, v.lo), s); }
+    // d x^2 + 2 e x prev for FP32 x
+    static PSVD_DEV V quad(V d, V e, S x, S prev) {
+        return ff_mulf(ff_add(ff_mulf(d, x), ff_mulf(e, __fmul_rn(2.f, prev))), x);
+    }
+    static PSVD_DEV V add(V a, V b) { return ff_add(a, b); }
+    static PSVD_DEV V sqs(V s, S x) { return ff_fma(s, x, x); }
+    static PSVD_DEV V zero() { return ff{0.f, 0.f}; }
+};
+struct IvD {
+    using V = double;
+    using S = double;
+    static PSVD_DEV V of(double v) { return v; }
+    static PSVD_DEV V ld(const void *p) { return *static_cast<const double *>(p); }
+    static PSVD_DEV void st(void *p, V v) { *static_cast<double *>(p) = v; }
+    static PSVD_DEV void row(const void *p, V &d, V &e) {
+        const double2 v = *static_cast<const double2 *>(p);
+        d = v.x;
+        e = v.y;
+    }
+    static PSVD_DEV V start(int i, int j) { return hash_unit((unsigned)i, (unsigned)j) + 0.0625; }
+    static PSVD_DEV V sel(bool c, V a, V b) { return c ? a : b; }
+    static PSVD_DEV V neg(V a) { return -a; }
+    static PSVD_DEV V sub(V a, V b) { return a - b; }
+    static PSVD_DEV V mul(V a, V b) { return a * b; }
+    static PSVD_DEV V muls(V a, S s) { return a * s; }
+    static PSVD_DEV V nfma(V a, V x, V y) { return fma(-x, y, a); }
+    static PSVD_DEV V sq(V s, V v) { return fma(v, v, s); }
+    static PSVD_DEV bool less(V a, V b) { return fabs(a) < fabs(b); }
+    static PSVD_DEV V pivot(V a) { return fabs(a) < 2.2e-16 ? copysign(2.2e-16, a) : a; }
+    static PSVD_DEV S rcp0(V den) { return recip64(den); }
+    static PSVD_DEV V div(V a, V, S r0) { return a * r0; }
+    static PSVD_DEV V inv(V, S r0) { return r0; }
+    static PSVD_DEV V flag(V v, bool f) {
+        return __longlong_as_double((__double_as_longlong(v) & ~1LL) | (f ? 1LL : 0LL));
+    }
+    static PSVD_DEV bool flagged(V v) { return __double_as_longlong(v) & 1LL; }
+    static PSVD_DEV V other(V v) { return __shfl_xor_sync(0xffffffffu, v, 16); }
+    static PSVD_DEV double d(V v) { return v; }
+    static PSVD_DEV S scaled(V v, S s) { return v * s; }
+    static PSVD_DEV V quad(V d, V e, S x, S prev) { return fma(2.0 * e, prev, d * x) * x; }
+    static PSVD_DEV V add(V a, V b) { return a + b; }
+    static PSVD_DEV V sqs(V s, S x) { return fma(x, x, s); }
+    static PSVD_DEV V zero() { return 0.0; }
+};
+
+// The vector of eigenvalue mu tn of matrix b (n >= 2): factorization of T / tn - mu I with row interchanges
+// from both ends, three solves from a fixed pseudo-random start (the first right-hand side goes along with
+// the factorization), normalization.  Stored per eliminated row: 1 / pivot, the two superdiagonals over
+// the pivot (so that a back-substitution step is one dependent multiply-add) and the multiplier, whose
+// last bit tells whether the rows were interchanged.  Returns the Rayleigh quotient over tn; the vector
+// goes to column `col` of xf if `live`.  All lanes of the warp call it.
+template <class A>
+PSVD_DEV double iv_vector(const InvitParams &P, unsigned char *ring, const void *table, int i, double mu, bool live,
+                          long long col) {
+    using V = typename A::V;
+    using S = typename A::S;
+    const int n = P.n, lane = threadIdx.x & 31, side = lane >> 4, at = 8 * lane;
+    const int p = (n - 1) / 2, q = (n - 2) / 2, cnt = side ? q : p;    // rows eliminated from each end
+    const long long blk = (long long)blockIdx.y * gridDim.x + blockIdx.x;
+    unsigned char *X = reinterpret_cast<unsigned char *>(P.x + blk * P.rows * kIvW);
+    unsigned char *L = reinterpret_cast<unsigned char *>(P.l + blk * P.rows * kIvW);
+    unsigned char *U = reinterpret_cast<unsigned char *>(P.u + blk * P.rows * 3 * kIvW);
+    const unsigned char *T = static_cast<const unsigned char *>(table);
+    const int nst = (p + kIvJ - 1) / kIvJ, full = q / kIvJ;
+    constexpr int kXB = kIvJ * kIvRow, kTB = kIvJ * 32;
+    auto comp = [&](int k) { return side ? n - 1 - k : k; };
+
+    const V m0 = A::of(mu);
+    V a, bs, d0, ep;
+    A::row(T + 16 * side, d0, ep);
+    a = A::sub(d0, m0);
+    bs = ep;
+    V carry = A::start(i, comp(0));
+    iv_stream<false, kTB, 0>(ring, nst, full, cnt, T + 32, T, [&](int k, const unsigned char *buf, int r) {
+        V dn, en;
+        A::row(buf + r * 32 + 16 * side, dn, en);
+        dn = A::sub(dn, m0);
+        const V c = ep;
+        const bool pv = A::less(a, c);
+        const V den = A::pivot(A::sel(pv, c, a));
+        const S r0 = A::rcp0(den);
+        const V m = A::flag(A::div(A::sel(pv, a, c), den, r0), pv);
+        const V rp = A::inv(den, r0);
+        const V y = A::sel(pv, dn, bs);
+        a = A::nfma(A::sel(pv, bs, dn), m, y);
+        bs = A::sel(pv, A::neg(A::mul(m, en)), en);
+        ep = en;
+        A::st(U + (long long)k * 3 * kIvRow + at, rp);
+        A::st(U + (long long)k * 3 * kIvRow + kIvRow + at, A::mul(y, rp));
+        A::st(U + (long long)k * 3 * kIvRow + 2 * kIvRow + at, A::mul(A::sel(pv, en, A::zero()), rp));
+        A::st(L + (long long)k * kIvRow + at, m);
+        const V b = A::start(i, comp(k + 1));
+        const V ar = A::sel(pv, b, carry);
+        A::st(X + (long long)k * kIvRow + at, ar);
+        carry = A::nfma(A::sel(pv, carry, b), m, ar);
+    });
+    // the middle: [a bs; bs' a'] (x, x') = (carry, carry'), the same elimination in both halves
+    V m11 = a, m12 = bs, m21 = A::other(bs), m22 = A::other(a);
+    if (side) {
+        V t = m11; m11 = m22; m22 = t;
+        t = m12; m12 = m21; m21 = t;
+    }
+    const bool pv = A::less(m11, m21);
+    if (pv) {
+        V t = m11; m11 = m21; m21 = t;
+        t = m12; m12 = m22; m22 = t;
+    }
+    m11 = A::pivot(m11);
+    const S r11 = A::rcp0(m11);
+    const V ml = A::div(m21, m11, r11);
+    m22 = A::pivot(A::nfma(m22, ml, m12));
+    const S r22 = A::rcp0(m22);
+    S scale = (S)1;
     for (int it = 0; it < 3; ++it) {
-        iv_forward(P, ivring, n, t, i, it == 0, scale);
-        const double nrm = iv_backward(P, ivring, n, t);
-        scale = nrm > 0 ? 1.0 / sqrt(nrm) : 0.0;
+        if (it > 0) {
+            carry = A::muls(A::ld(X + at), scale);
+            iv_stream<false, kXB, kXB>(ring, nst, full, cnt, X + kIvRow, L, [&](int k, const unsigned char *buf, int r) {
+                const V b = A::muls(A::ld(buf + r * kIvRow + at), scale);
+                const V m = A::ld(buf + kXB + r * kIvRow + at);
+                const bool sw = A::flagged(m);
+                const V ar = A::sel(sw, b, carry);
+                A::st(X + (long long)k * kIvRow + at, ar);
+                carry = A::nfma(A::sel(sw, carry, b), m, ar);
+            });
+        }
+        V x1, x2;
+        {
+            const V o = A::other(carry);
+            const V rt = A::sel(side, o, carry), rb = A::sel(side, carry, o);
+            const V r1 = A::sel(pv, rb, rt), r2 = A::sel(pv, rt, rb);
+            const V xb = A::div(A::nfma(r2, ml, r1), m22, r22);
+            const V xt = A::div(A::nfma(r1, m12, xb), m11, r11);
+            x1 = A::sel(side, xb, xt);
+            x2 = A::sel(side, xt, xb);
+        }
+        A::st(X + (long long)cnt * kIvRow + at, x1);
+        V nrm = A::sq(A::zero(), x1);
+        iv_stream<true, kXB, 3 * kXB>(ring, nst, full, cnt, X, U, [&](int k, const unsigned char *buf, int r) {
+            const unsigned char *u = buf + kXB + r * 3 * kIvRow + at;
+            V v = A::mul(A::ld(buf + r * kIvRow + at), A::ld(u));
+            v = A::nfma(v, A::ld(u + 2 * kIvRow), x2);
+            v = A::nfma(v, A::ld(u + kIvRow), x1);
+            A::st(X + (long long)k * kIvRow + at, v);
+            x2 = x1;
+            x1 = v;
+            nrm = A::sq(nrm, v);
+        });
+        nrm = A::add(nrm, A::other(nrm));
+        const double nv = A::d(nrm);
+        scale = nv > 0.0 ? (S)(1.0 / sqrt(nv)) : (S)0;
     }
-    P.lam[gi] = iv_finish(P, ivring, D, E, n, t, scale);
+    // the vector (rounded to FP32) and x^T (T / tn) x / x^T x
+    V num = A::zero(), den = A::zero(), e1 = A::zero();
+    S prev = (S)0;
+    float *xf = P.xf + col;
+    iv_stream<false, kXB, kTB>(ring, (p + kIvJ) / kIvJ, (q + 1) / kIvJ, cnt + 1, X, T,
+                              [&](int k, const unsigned char *buf, int r) {
+        const S x = A::scaled(A::ld(buf + r * kIvRow + at), scale);
+        V d, e;
+        A::row(buf + kXB + r * 32 + 16 * side, d, e);
+        if (live) xf[(long long)comp(k) * P.stride] = (float)x;
+        num = A::add(num, A::quad(d, e1, x, prev));
+        den = A::sqs(den, x);
+        prev = x;
+        e1 = e;
+    });
+    const S xo = __shfl_xor_sync(0xffffffffu, prev, 16);
+    if (!side) num = A::add(num, A::quad(A::zero(), e1, prev, xo));      // the coupling of the two middle rows
+    num = A::add(num, A::other(num));
+    den = A::add(den, A::other(den));
+    return A::d(num) / A::d(den);
+}
+
+// One warp per block, 16 eigenvectors of matrix blockIdx.y of the chunk.  The shift of close eigenvalues is
+// accurate to ~6e-14 ||T||, that of others to ~1e-7 ||T||: three solves reduce the other components by
+// (shift error / gap)^3.  A warp whose eigenvalues are all at least kIvFFGap ||T|| from their neighbours
+// runs in float-float, the others in FP64 (the choice is per warp, so no warp runs both).
+__global__ void __launch_bounds__(kIvW) tri_invit_kernel(InvitParams P) {
+    extern __shared__ __align__(16) unsigned char ivring[];
+    const int n = P.n, lane = threadIdx.x & 31;
+    const int b = P.first / n + blockIdx.y, t = blockIdx.x * kIvV + (lane & 15);
+    const bool live = t < n;
+    const int i = live ? t : n - 1;
+    const long long gi = (long long)b * n + i, col = (long long)blockIdx.y * n + i;
+    const double tn = P.tn[b];
+    if (n == 1 || !(tn > 0.0)) {                   // T = 0: every vector is an eigenvector; take the unit vectors
+        if (!live) return;
+        for (int j = lane >> 4; j < n; j += 2) P.xf[j * P.stride + col] = j == i ? 1.f : 0.f;
+        if (n > 1 && lane < 16) P.lam[gi] = 0.0;
+        return;
+    }
+    const double *lb = P.lam0 + (long long)b * n;
+    double g = 1e300;
+    if (i > 0) g = fmin(g, lb[i - 1] - lb[i]);
+    if (i + 1 < n) g = fmin(g, lb[i] - lb[i + 1]);
+    const double mu = P.lam[gi] / tn;
+    double r;
+    if (__all_sync(0xffffffffu, g >= kIvFFGap * tn))
+        r = iv_vector<IvFF>(P, ivring, P.tabf + (long long)b * P.rows * 2, i, mu, live, col);
+    else
+        r = iv_vector<IvD>(P, ivring, P.tabd + (long long)b * P.rows * 2, i, mu, live, col);
+    if (live && lane < 16) P.lam[gi] = r * tn;
 }
 
 // Modified Gram-Schmidt inside clusters of eigenvalues closer than ctol * ||T||,
@@ -1422,7 +1403,9 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
     }
     {
         float4 *dd = w.sturm;
-        sturm_prep_kernel<<<dim3((n + 255) / 256, B), 256, 0, st>>>(w.d, w.e, tn, n, dd, dd + (size_t)B * n);
+        const int rows = iv_rows(n);
+        sturm_prep_kernel<<<dim3((std::max(n, rows) + 255) / 256, B), 256, 0, st>>>(w.d, w.e, tn, n, rows, dd, w.tabf,
+                                                                                   w.tabd);
         dim3 g((n + 31) / 32, B);       // 32 eigenvalues x 8 lanes per block
         tri_refine_kernel<<<g, 256, 0, st>>>(dd, n, tn, kRefineNear, w.lam);
         PSVD_TRY(cudaGetLastError());
@@ -1438,10 +1421,10 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
         const int nb = std::min(per, B - b0);
         InvitParams P;
         P.D = w.d; P.E = w.e; P.tn = tn; P.lam = w.lam; P.lam0 = bis;
-        P.de = w.sturm + (size_t)B * n;
-        P.xs = w.xs; P.xf = w.xf; P.u0 = w.u0; P.u1 = w.u1; P.u2 = w.u2; P.lm = w.lm; P.piv = w.piv;
-        P.n = n; P.first = b0 * n; P.count = nb * n; P.stride = w.chunk;
-        tri_invit_kernel<<<(P.count + kIvW - 1) / kIvW, kIvW, kIvSmem, st>>>(P);
+        P.tabf = w.tabf; P.tabd = w.tabd;
+        P.x = w.xs; P.l = w.lm; P.u = w.u; P.xf = w.xf;
+        P.n = n; P.rows = iv_rows(n); P.first = b0 * n; P.count = nb * n; P.stride = w.chunk;
+        tri_invit_kernel<<<dim3((n + kIvV - 1) / kIvV, nb), kIvW, kIvSmem, st>>>(P);
         tri_cluster_kernel<<<nb, 256, 0, st>>>(P, bis, kClusterTol);
         dim3 g((n + 31) / 32, (n + 31) / 32, nb), blk(32, 8);
         zt_store_kernel<<<g, blk, 0, st>>>(w.xf, w.chunk, n, b0, b0 * n, w.VThi, w.VTlo, ldn);

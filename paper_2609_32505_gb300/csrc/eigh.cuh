@@ -9,6 +9,10 @@ namespace psvd {
 constexpr int kTrdChipMin = 3, kTrdChipMax = 4096;   // sizes whose tridiagonalization runs on chip (trd.cu)
 constexpr int kBtSplit = 8; // largest K split of the back-transform's V^T Y products
 
+constexpr int kIvJ = 8;     // rows per stage of inverse iteration's ring
+// rows of its arrays: half the matrix from either end, and what the last stage reads past it
+inline int iv_rows(int n) { return (int)round_up((n - 1) / 2 + kIvJ + 1, 2); }
+
 struct EighWS {
     int B = 0, n = 0, nblk = 0, chunk = 0, nrp = 0;   // nrp: rows of Vh, padded to kWY
     long long ldn = 0, ll_ld = 0;
@@ -25,15 +29,15 @@ struct EighWS {
     __half *VThi = nullptr, *VTlo = nullptr;   // current V^T (n x ldn), scaled by kF16X
     float *S = nullptr;                        // V^T Y for a pair of blocks (n x 2 kWY), K-split slices
     __half *S2hi = nullptr, *S2lo = nullptr;   // the pair's S2 (n x 2 kWY), scaled by kF16S2
-    float4 *sturm = nullptr;                   // [2][B][n] float-float T for the Sturm counts and inverse iteration
+    float4 *sturm = nullptr;                   // [B][n] float-float T for the Sturm counts
+    float4 *tabf = nullptr;                    // [B][iv_rows][2] T for inverse iteration, float-float
+    double2 *tabd = nullptr;                   // the same in FP64
     double *tn = nullptr;                      // [B] ||T||
     float *Tm = nullptr;                       // [B][nblk][kWY][kWY]
     float *Gm = nullptr;                       // [B][nblk][kWY][kWY]  Y^T Y per block
     float *Gab = nullptr;                      // [B][nblk/2][kWY][kWY]  Y_a^T Y_b per pair of blocks
-    double *xs = nullptr;                      // inverse-iteration vectors, interleaved [n][chunk]
+    double *xs = nullptr, *lm = nullptr, *u = nullptr;   // inverse-iteration vectors, multipliers, pivot rows
     float *xf = nullptr;                       // the normalized eigenvectors of T, interleaved [n][chunk]
-    double *u0 = nullptr, *u1 = nullptr, *u2 = nullptr, *lm = nullptr;
-    unsigned *piv = nullptr;            // pivot bits, [ceil(n/32)][chunk]
     unsigned *err = nullptr;
     int groups = 0;
 
@@ -44,8 +48,9 @@ struct EighWS {
         nblk = n > 2 ? (n - 2 + kWY - 1) / kWY : 0;
         nrp = (int)round_up(n < 1 ? 1 : n, kWY);
         const long long B64 = B, nn = (long long)n * ldn, np = (long long)nrp * ldn;
-        // inverse-iteration scratch holds whole matrices: n vectors x n entries each
-        chunk = n * (int)std::max<long long>(1, std::min<long long>(B64, (1LL << 24) / ((long long)n * n)));
+        // inverse-iteration scratch holds whole matrices: n vectors x n entries each, 44 bytes an entry; 2.9 GB
+        // at most (matrices of 4096 in fours; one at a time leaves most of the chip idle)
+        chunk = n * (int)std::max<long long>(1, std::min<long long>(B64, (1LL << 26) / ((long long)n * n)));
         Aw = cv.template take<float>(B64 * n * ldn);
         Vh = cv.template take<float>(B64 * np);
         tau = cv.template take<float>(B64 * n);
@@ -66,18 +71,18 @@ struct EighWS {
         S = cv.template take<float>(kBtSplit * B64 * n * 2 * kWY);
         S2hi = cv.template take<__half>(B64 * n * 2 * kWY);
         S2lo = cv.template take<__half>(B64 * n * 2 * kWY);
-        sturm = cv.template take<float4>(B64 * n * 2);
+        sturm = cv.template take<float4>(B64 * n);
+        tabf = cv.template take<float4>(B64 * iv_rows(n) * 2);
+        tabd = cv.template take<double2>(B64 * iv_rows(n) * 2);
         tn = cv.template take<double>(B64);
         Tm = cv.template take<float>(B64 * (nblk > 0 ? nblk : 1) * kWY * kWY);
         Gm = cv.template take<float>(B64 * (nblk > 0 ? nblk : 1) * kWY * kWY);
         Gab = cv.template take<float>(B64 * (nblk > 1 ? nblk / 2 : 1) * kWY * kWY);
-        xs = cv.template take<double>((long long)n * chunk);
         xf = cv.template take<float>((long long)n * chunk);
-        u0 = cv.template take<double>((long long)n * chunk);
-        u1 = cv.template take<double>((long long)n * chunk);
-        u2 = cv.template take<double>((long long)n * chunk);
-        lm = cv.template take<double>((long long)n * chunk);
-        piv = cv.template take<unsigned>((long long)((n + 31) / 32) * chunk);
+        const long long iv = (long long)(chunk / n) * ((n + 15) / 16) * iv_rows(n) * 32;   // 16 vectors per warp
+        xs = cv.template take<double>(iv);
+        lm = cv.template take<double>(iv);
+        u = cv.template take<double>(3 * iv);
         err = cv.template take<unsigned>(4);
     }
 };

@@ -57,3 +57,20 @@ def test_vanishing_reflectors(n):
     t = d + torch.diag(torch.full((n - 1,), 0.25), 1) + torch.diag(torch.full((n - 1,), 0.25), -1)
     u = torch.ones(n, 1) / n ** 0.5
     _check(torch.stack([d, t, torch.zeros(n, n), u @ u.T, 1e-12 * (u @ u.T)]).cuda())
+
+
+@pytest.mark.parametrize("n", [2, 3, 4, 15, 16, 17, 18, 31, 32, 33, 34, 35, 48, 49, 255, 256, 257, 258])
+@pytest.mark.parametrize("gap", [1e-2, 1e-7])
+def test_inverse_iteration_halves(n, gap):
+    """Inverse iteration works from both ends of T towards the middle, 8 rows to a stage, 16 vectors to a
+    warp: odd and even sizes around those, with all eigenvalues apart (float-float) and in pairs
+    1e-7 apart (FP64)."""
+    g = torch.Generator()
+    g.manual_seed(n)
+    q = torch.linalg.qr(torch.randn(n, n, generator=g, dtype=torch.float64))[0]
+    lam = torch.linspace(1.0, -1.0, n, dtype=torch.float64) if gap > 1e-3 else \
+        torch.linspace(1.0, -1.0, (n + 1) // 2, dtype=torch.float64).repeat_interleave(2)[:n]
+    if gap < 1e-3:
+        lam = lam + gap * (torch.arange(n, dtype=torch.float64) % 2)
+    h = (q * lam) @ q.T
+    _check(torch.stack([h, -3.0 * h]).float().cuda())
