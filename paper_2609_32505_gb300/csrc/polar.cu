@@ -832,8 +832,8 @@ struct PolarPreqr {
 };
 
 static bool polar_use_preqr(const psvd_opts &o, int64_t m, int64_t n) {
-    int nb = 0, cl = 0;
-    return o.preqr == 1 && m > n && qr_shape((int)m, &nb, &cl);
+    int nb = 0;
+    return o.preqr == 1 && m > n && qr_shape((int)m, &nb);
 }
 
 extern "C" size_t psvd_polar_workspace_bytes(int64_t batch, int64_t m, int64_t n, const psvd_opts *opts) {

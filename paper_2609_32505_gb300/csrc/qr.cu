@@ -25,211 +25,272 @@ namespace psvd {
 
 namespace cg = cooperative_groups;
 
-constexpr int kQrThreads = 512;
-constexpr size_t kQrSlabMax = 180 * 1024;   // shared memory for one CTA's slab of the panel
+constexpr int kQrWarps = 16, kQrThreads = 32 * kQrWarps;
+constexpr int kQrMaxCl = 16;
+constexpr int kQrRows8 = 2048;            // panels of 64 columns up to here: 256 rows per CTA
 
-// Slab column stride: odd, so that the lanes of a warp (consecutive columns, same row) fall
-// in distinct shared-memory banks.
-__host__ __device__ inline int qr_slab_stride(int S) { return (S & 1) ? S : S + 1; }
-
-static size_t qr_panel_smem(int m, int nb, int cl) {
-    const int S = qr_slab_stride((m + cl - 1) / cl);
-    const size_t slab = std::max<size_t>((size_t)S * nb, (size_t)2 * nb * (nb + 1)) * sizeof(float);
-    const size_t red = sizeof(float) * (size_t)kQrThreads;
-    return sizeof(double) * ((size_t)2 * cl * 2 * nb + 5 * nb) + red + slab;
-}
-
-bool qr_shape(int m, int *nb, int *cl) {
-    const int nbs[2] = {64, 32}, cls[2] = {8, 16};
-    for (int a = 0; a < 2; ++a)
-        for (int c = 0; c < 2; ++c) {
-            const int S = qr_slab_stride((m + cls[c] - 1) / cls[c]);
-            if ((size_t)S * nbs[a] * sizeof(float) <= kQrSlabMax) { *nb = nbs[a]; *cl = cls[c]; return true; }
-        }
-    return false;
+// The panel is 64 columns wide up to 8192 rows and 32 above, so that a CTA's rows fit its registers with
+// at most 16 CTAs per matrix; 23024 rows at most.
+bool qr_shape(int m, int *nb) {
+    *nb = m <= 8192 ? 64 : 32;
+    return m <= 23024;
 }
 
 struct PanelArgs {
     __half *UThi, *UTlo, *YThi, *YTlo, *Yhi, *Ylo;
-    float *tau, *beta, *Tm, *Gpart;
+    float *tau, *beta, *Tm;
     const int *skip;
-    int m, n, j0, pw, panel, npan, nb, cl;
+    int m, n, j0, pw, panel, npan, cl;
     long long ldm, ldn;
 };
 
-// One cluster per matrix factors columns j0 .. j0 + pw - 1 (rows j0 .. m - 1).  CTA q of the
-// cluster owns rows [j0 + q S, j0 + (q + 1) S), S = ceil((m - j0) / cl), column-major in
-// shared memory.  For column j every CTA contributes, over its rows r > j, the partial sums
-// P_c' = sum x_r y_c',r (c' = j: the squared norm below the diagonal) and, from the owner of
-// row j, the row-j values; each CTA writes its vector into a slot of every CTA of the cluster,
-// and after the barrier every CTA adds the slots in rank order (so all get the same totals,
-// bit for bit) and builds the reflector redundantly: beta = -sign(alpha) sqrt(alpha^2 + s2),
-// tau = (beta - alpha) / beta, v = [1; x / (alpha - beta)].  Slots are double-buffered by
-// column parity, which makes one barrier per column enough.  The slots and their sums are
-// FP32, like the partial sums they hold (FP64 sums of the cluster's 8 or 16 partials took
-// ~40% of a column's time on the narrow FP64 pipe, measured, and added no accuracy that
-// the FP32 partial sums had).
+// Shared memory of the panel kernel: NB columns of S = 32 RPL rows per CTA.
+template <int RPL, int C>
+struct PanelSmem {
+    static constexpr int S = 32 * RPL, NB = kQrWarps * C;
+    static constexpr int kSlot = NB + 4;              // a slot's stride: spreads the CTAs' slots over the banks
+    alignas(16) float x[2][S];                        // column c, rows above and at the diagonal zeroed
+    float slot[2][kQrMaxCl][kSlot];                   // every CTA's partial sums of the column
+    float row[2][kSlot];                              // the row-j entries, from CTA 0
+    float G[NB][NB + 1];                              // Y^T Y above its diagonal
+    float tau[NB];
+    float slab[NB][S + 1];                            // the factored panel, for the outputs
+};
+
+// One cluster of cl CTAs per matrix factors columns j0 .. j0 + pw - 1 (rows j0 .. m - 1).  CTA q owns rows
+// [j0 + q S, j0 + (q + 1) S), in registers: lane l of warp w holds rows 4 l + 128 i + (0..3) of columns
+// w, w + 16, ..., so a column's update and its dot products touch nothing but registers and the one
+// column x = column c that its warp has put into shared memory.  For column c every warp forms, over
+// its rows r > j, the sums P_k = sum x_r a_r,k of its C columns (of column c itself: the squared norm below the
+// diagonal; of the finished ones: what Y^T Y needs) and writes them into a slot of every CTA of the
+// cluster, CTA 0, which holds all diagonal rows, also the row-j entries a_j,k; after the cluster's barrier
+// every warp adds the slots of its columns (the same order everywhere, so all get the same totals bit
+// for bit) and builds the reflector redundantly: beta = -sign(alpha) sqrt(alpha^2 + s2), tau = (beta -
+// alpha) / beta, v = [1; x / (alpha - beta)].  With g_k = a_j,k + scal P_k a later column takes
+// -= tau g_k v, and g_k of an earlier one is (Y^T Y)_kc.  The warp of column c + 1 then writes it out.  Slots
+// and columns are double-buffered by column parity, which makes one cluster barrier and one block
+// barrier per column enough.
+//
+// A panel is a chain of pw such columns, so its time is latency: with the panel in shared memory (5 block
+// barriers per column, every multiply-add fed from shared memory, the Gram matrix and T formed
+// afterwards) a column took 2.9 us at 256 rows, 6.2 at 4096 (8 matrices) and 7.4 at 14336 (4 matrices); it
+// takes 1.4, 2.6 and 3.0 us, everything included.
+template <int RPL, int C>
 __global__ void __launch_bounds__(kQrThreads, 1) qr_panel_kernel(PanelArgs P) {
+    using Sm = PanelSmem<RPL, C>;
+    constexpr int S = Sm::S, NB = Sm::NB, Q = RPL / 4;
+    constexpr bool kKeepX = RPL <= 16;               // x stays in registers between its two uses
     cg::cluster_group cluster = cg::this_cluster();
-    const int CL = P.cl, rank = (int)cluster.block_rank();
+    const int CL = P.cl, rank = CL > 1 ? (int)cluster.block_rank() : 0;
     const int b = blockIdx.x / CL;
     if (P.skip[b]) return;                       // uniform across the cluster
-    extern __shared__ __align__(16) double qsm[];
-    const int nb = P.nb, pw = P.pw, j0 = P.j0, m = P.m, n = P.n;
-    float *xch = reinterpret_cast<float *>(qsm); // [2][CL][2 nb] slots, double-buffered by column parity
-    double *part = qsm + 2 * CL * 2 * nb;        // [2 nb] doubles of room
-    float *vec = reinterpret_cast<float *>(part); // [2 nb] this CTA's vector of the column
-    float *coef = reinterpret_cast<float *>(part + 4 * nb);   // [nb] f_c' of this column, then [2] scal, beta
-    float *scal_s = coef + nb;
-    float *red = reinterpret_cast<float *>(part + 5 * nb);    // [kQrThreads] row-block partial sums
-    float *slab = red + kQrThreads;                           // [pw][Sp] column-major, Sp odd
-    const int S = (m - j0 + CL - 1) / CL;
-    const int Sp = qr_slab_stride(S);
-    const int r0 = j0 + rank * S;
-    const int nr = max(0, min(m, r0 + S) - r0);
-    const int tid = threadIdx.x;
+    extern __shared__ __align__(16) unsigned char qsm[];
+    Sm &sm = *reinterpret_cast<Sm *>(qsm);
+    const int pw = P.pw, j0 = P.j0, m = P.m, n = P.n;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int r0 = j0 + rank * S;                    // multiple of 4
     const long long ubase = (long long)b * n * P.ldm;
-    // thread -> (column cc, row block rb): the lanes of a warp share rb and hold consecutive columns
-    const int nrb = kQrThreads / nb, cc = tid % nb, rb = tid / nb;
-    const int rbs = (nr + nrb - 1) / nrb;
-    const int rlo = rb * rbs, rhi = min(nr, rlo + rbs);
 
-    for (int c = 0; c < pw; ++c) {
-        const __half *hi = P.UThi + ubase + (long long)(j0 + c) * P.ldm + r0;
-        const __half *lo = P.UTlo + ubase + (long long)(j0 + c) * P.ldm + r0;
-        for (int rr = tid; rr < nr; rr += blockDim.x) slab[c * Sp + rr] = join_f16(hi[rr], lo[rr]) * (1.f / kF16X);
-    }
-    __syncthreads();
+    float a[C][RPL];
+#pragma unroll
+    for (int k = 0; k < C; ++k)
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const int c = k * kQrWarps + w, r = r0 + 128 * i + 4 * lane;
+            __align__(8) __half h[4], l[4];
+            *reinterpret_cast<uint2 *>(h) = *reinterpret_cast<uint2 *>(l) = make_uint2(0u, 0u);
+            if (c < pw && r < m) {                   // (the padding of a row takes part as zeros)
+                const long long o = ubase + (long long)(j0 + c) * P.ldm + r;
+                *reinterpret_cast<uint2 *>(h) = *reinterpret_cast<const uint2 *>(P.UThi + o);
+                *reinterpret_cast<uint2 *>(l) = *reinterpret_cast<const uint2 *>(P.UTlo + o);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a[k][4 * i + e] = r + e < m ? join_f16(h[e], l[e]) * (1.f / kF16X) : 0.f;
+        }
+    // column c (this warp's index k) to shared memory, zero in rows <= c of CTA 0
+    auto publish = [&](const float (&col)[RPL], int c) {
+        float *x = sm.x[c & 1];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            float4 v = make_float4(col[4 * i], col[4 * i + 1], col[4 * i + 2], col[4 * i + 3]);
+            if (i == 0 && rank == 0) {
+                const int r = 4 * lane;
+                if (r <= c) v.x = 0.f;
+                if (r + 1 <= c) v.y = 0.f;
+                if (r + 2 <= c) v.z = 0.f;
+                if (r + 3 <= c) v.w = 0.f;
+            }
+            *reinterpret_cast<float4 *>(x + 128 * i + 4 * lane) = v;
+        }
+    };
+    if (w == 0) publish(a[0], 0);
+    if (CL > 1) cluster.sync();                      // every CTA runs before its shared memory is written to
+    else __syncthreads();
 
-    for (int c = 0; c < pw; ++c) {
-        const int j = j0 + c, par = c & 1;
-        const int jl = j - r0;
-        const bool own = jl >= 0 && jl < nr;
-        const int start = max(0, jl + 1);
-        const int live = pw - c;                 // entries c .. pw-1 of the vectors are needed
-        const float *x = slab + c * Sp;
-        // partial dot products of column c with columns cc >= c over rows r > j of this block
-        if (cc >= c && cc < pw) {
-            const float *y = slab + cc * Sp;
-            float a0 = 0.f, a1 = 0.f;
-            int rr = max(rlo, start);
-            for (; rr + 1 < rhi; rr += 2) {
-                a0 = fmaf(x[rr], y[rr], a0);
-                a1 = fmaf(x[rr + 1], y[rr + 1], a1);
+#pragma unroll
+    for (int kc = 0; kc < C; ++kc) {
+#pragma unroll 1
+        for (int wc = 0; wc < kQrWarps; ++wc) {
+            const int c = kc * kQrWarps + wc, par = c & 1;
+            if (c >= pw) break;
+            const float *xs = sm.x[par] + 4 * lane;
+            // the sums of this warp's columns
+            float x[kKeepX ? RPL : 1];
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const float4 v = *reinterpret_cast<const float4 *>(xs + 128 * i);
+                if constexpr (kKeepX) { x[4 * i] = v.x; x[4 * i + 1] = v.y; x[4 * i + 2] = v.z; x[4 * i + 3] = v.w; }
+#pragma unroll
+                for (int k = 0; k < C; ++k) {
+                    s[k] = fmaf(v.x, a[k][4 * i], s[k]);
+                    s[k] = fmaf(v.y, a[k][4 * i + 1], s[k]);
+                    s[k] = fmaf(v.z, a[k][4 * i + 2], s[k]);
+                    s[k] = fmaf(v.w, a[k][4 * i + 3], s[k]);
+                }
             }
-            if (rr < rhi) a0 = fmaf(x[rr], y[rr], a0);
-            red[rb * nb + cc] = a0 + a1;
-        }
-        // the previous column becomes its reflector (v below the diagonal, beta on it); no
-        // thread reads it in this phase (the dot products above start at column c)
-        if (c > 0) {
-            const int jlp = j - 1 - r0;
-            float *xp = slab + (c - 1) * Sp;
-            const float fsp = scal_s[0];
-            for (int rr = max(0, jlp + 1) + tid; rr < nr; rr += blockDim.x) xp[rr] *= fsp;
-            if (jlp >= 0 && jlp < nr && tid == 0) xp[jlp] = scal_s[1];
-        }
-        __syncthreads();
-        // this CTA's vector (sum over the row blocks; the row-j values from its owner), formed
-        // once in shared memory, then copied into a slot of every CTA of the cluster
-        for (int k = tid; k < 2 * live; k += blockDim.x) {
-            if (k < live) {
-                const int e = c + k;
-                float sum = 0.f;
-                for (int q = 0; q < nrb; ++q) sum += red[q * nb + e];
-                vec[e] = sum;
-            } else {
-                const int e = nb + c + (k - live);
-                vec[e] = own ? slab[(e - nb) * Sp + jl] : 0.f;
+            // lanes 8 v .. 8 v + 7 get the sum of column index v over the warp
+            const bool up = lane & 16, up8 = lane & 8;
+            float t0 = (up ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, up ? s[0] : s[2], 16);
+            float t1 = (up ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, up ? s[1] : s[3], 16);
+            float t = (up8 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, up8 ? t0 : t1, 8);
+            t += __shfl_xor_sync(0xffffffffu, t, 4);
+            t += __shfl_xor_sync(0xffffffffu, t, 2);
+            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            const int v = lane >> 3, q = lane & 7, e = v * kQrWarps + w;
+            float rv = 0.f;
+            if (rank == 0) {                         // row j = local row c, in lane c / 4
+                const int ce = c & 3, cl4 = c >> 2;
+#pragma unroll
+                for (int k = 0; k < C; ++k) {
+                    const float y = ce == 0 ? a[k][0] : (ce == 1 ? a[k][1] : (ce == 2 ? a[k][2] : a[k][3]));
+                    const float z = __shfl_sync(0xffffffffu, y, cl4);
+                    if (k == v) rv = z;
+                }
             }
-        }
-        __syncthreads();
-        // the row-j values are nonzero only in the CTA that owns row j: only it sends them,
-        // and the readers take them from its slot
-        const int nsend = own ? 2 * live : live;
-        for (int t = tid; t < CL * nsend; t += blockDim.x) {
-            const int peer = t / nsend, k = t - peer * nsend;
-            const int e = k < live ? c + k : nb + c + (k - live);
-            float *dst = cluster.map_shared_rank(xch + ((long long)par * CL + rank) * 2 * nb, peer);
-            dst[e] = vec[e];
-        }
-        cluster.sync();
-        // warp 0: the cluster totals, the reflector (FP32, as single-precision Householder QR
-        // computes it) and the coefficient f_c' = tau (v^T y_c') = tau (y_c',j + scal P_c')
-        if (tid < 32) {
-            const int lane = tid;
-            const float *slots = xch + (long long)par * CL * 2 * nb;
-            const float *oslot = slots + (long long)((j - j0) / S) * 2 * nb;   // the owner of row j
-            float s2 = 0.f;
-            for (int q = 0; q < CL; ++q) s2 += slots[q * 2 * nb + c];
-            const float alpha = oslot[nb + c];
-            const float fa = alpha, f2 = s2;
+            if (v < C) {
+                if (CL == 1) {
+                    if (q == 0) { sm.slot[par][0][e] = t; sm.row[par][e] = rv; }
+                } else {
+                    for (int peer = q; peer < CL; peer += 8) {
+                        *cluster.map_shared_rank(&sm.slot[par][rank][e], peer) = t;
+                        if (rank == 0) *cluster.map_shared_rank(&sm.row[par][e], peer) = rv;
+                    }
+                }
+            }
+            if (CL == 1) __syncthreads();
+            else cluster.sync();
+            // totals of this warp's columns (lanes 8 v ..) and of column c
+            float pt = 0.f, s2 = 0.f;
+            for (int p = q; p < CL; p += 8) {
+                if (v < C) pt += sm.slot[par][p][e];
+                s2 += sm.slot[par][p][c];
+            }
+#pragma unroll
+            for (int d = 4; d; d >>= 1) {
+                pt += __shfl_xor_sync(0xffffffffu, pt, d);
+                s2 += __shfl_xor_sync(0xffffffffu, s2, d);
+            }
+            const float fa = sm.row[par][c];
             float beta, tau, scal;
-            if (f2 == 0.f) { beta = fa; tau = 0.f; scal = 0.f; }
+            if (s2 == 0.f) { beta = fa; tau = 0.f; scal = 0.f; }
             else {
-                beta = -copysignf(sqrtf(fmaf(fa, fa, f2)), fa);
+                beta = -copysignf(sqrtf(fmaf(fa, fa, s2)), fa);
                 tau = (beta - fa) / beta;
                 scal = 1.f / (fa - beta);
             }
-            for (int k = c + 1 + lane; k < pw; k += 32) {
-                float pc = 0.f;
-                for (int q = 0; q < CL; ++q) pc += slots[q * 2 * nb + k];
-                coef[k] = tau * (oslot[nb + k] + pc * scal);
-            }
-            if (lane == 0) {
-                scal_s[0] = scal;
-                scal_s[1] = beta;
-                if (rank == 0) {
-                    P.tau[(long long)b * n + j] = tau;
-                    P.beta[(long long)b * n + j] = beta;
+            const float g = v < C ? fmaf(pt, scal, sm.row[par][e]) : 0.f;
+            if (rank == 0) {
+                if (q == 0 && v < C && e < c) sm.G[e][c] = g;
+                if (tid == 0) {
+                    sm.tau[c] = tau;
+                    P.tau[(long long)b * n + j0 + c] = tau;
+                    P.beta[(long long)b * n + j0 + c] = beta;
                 }
             }
+            // y -= f v for the later columns, v = [1; x scal]; column c becomes its reflector
+#pragma unroll
+            for (int k = kc; k < C; ++k) {
+                const float f = tau * __shfl_sync(0xffffffffu, g, 8 * k);
+                if (k > kc || w > wc) {
+                    const float fs = f * scal;
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) {
+                        float4 xv;
+                        if constexpr (kKeepX) xv = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+                        else xv = *reinterpret_cast<const float4 *>(xs + 128 * i);
+                        a[k][4 * i] = fmaf(-fs, xv.x, a[k][4 * i]);
+                        a[k][4 * i + 1] = fmaf(-fs, xv.y, a[k][4 * i + 1]);
+                        a[k][4 * i + 2] = fmaf(-fs, xv.z, a[k][4 * i + 2]);
+                        a[k][4 * i + 3] = fmaf(-fs, xv.w, a[k][4 * i + 3]);
+                    }
+                    if (rank == 0 && lane == c >> 2) {
+#pragma unroll
+                        for (int ee = 0; ee < 4; ++ee)
+                            if ((c & 3) == ee) a[k][ee] -= f;
+                    }
+                } else if (w == wc) {
+#pragma unroll
+                    for (int i = 0; i < RPL; ++i) {
+                        const int r = rank * S + 128 * (i / 4) + 4 * lane + (i & 3);      // row - j0
+                        a[k][i] = r > c ? a[k][i] * scal : (r == c ? beta : a[k][i]);
+                    }
+                }
+            }
+            if (wc + 1 < kQrWarps) {
+                if (w == wc + 1) publish(a[kc], c + 1);
+            } else if (kc + 1 < C) {
+                if (w == 0) publish(a[kc + 1 < C ? kc + 1 : kc], c + 1);
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        // y -= f_c' v for the later panel columns, v = [1; x * scal]
-        if (cc > c && cc < pw) {
-            float *y = slab + cc * Sp;
-            const float f = coef[cc] * scal_s[0];
-            for (int rr = max(rlo, start); rr < rhi; ++rr) y[rr] = fmaf(-f, x[rr], y[rr]);
-            if (own && jl >= rlo && jl < rhi) y[jl] -= coef[cc];
-        }
-        __syncthreads();
-    }
-    if (pw > 0) {                                // the last column's reflector
-        const int jlp = j0 + pw - 1 - r0;
-        float *xp = slab + (pw - 1) * Sp;
-        const float fsp = scal_s[0];
-        for (int rr = max(0, jlp + 1) + tid; rr < nr; rr += blockDim.x) xp[rr] *= fsp;
-        if (jlp >= 0 && jlp < nr && tid == 0) xp[jlp] = scal_s[1];
-        __syncthreads();
     }
 
-    // the factored panel back to UT (R entries above the diagonal, beta on it, v below);
-    // the reflectors also as clean rows (YT: 0 above, 1 on the diagonal) and columns (Y)
-    for (int c = 0; c < pw; ++c) {
-        const int j = j0 + c;
-        const long long o = ubase + (long long)j * P.ldm + r0;
-        for (int rr = tid; rr < nr; rr += blockDim.x) {
-            const int r = r0 + rr;
-            const float v = slab[c * Sp + rr];
-            __half h, l;
-            split_f16(v * kF16X, h, l);
-            P.UThi[o + rr] = h;
-            P.UTlo[o + rr] = l;
-            split_f16((r < j ? 0.f : (r == j ? 1.f : v)) * kF16V, h, l);
-            P.YThi[o + rr] = h;
-            P.YTlo[o + rr] = l;
+    // the factored panel back to UT (R entries above the diagonal, beta on it, v below); the
+    // reflectors also as clean rows (YT: 0 above, 1 on the diagonal) and columns (Y)
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+        const int c = k * kQrWarps + w;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const int rl = 128 * i + 4 * lane, r = r0 + rl;
+            __align__(8) __half uh[4], ul[4], yh[4], yl[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float v = a[k][4 * i + e];
+                const int d = r + e - (j0 + c);
+                const float y = d < 0 ? 0.f : (d == 0 ? 1.f : v);
+                split_f16(v * kF16X, uh[e], ul[e]);
+                split_f16(y * kF16V, yh[e], yl[e]);
+                sm.slab[c][rl + e] = y;
+            }
+            if (c < pw && r < m) {                   // rows of UT and YT are padded to multiples of 32
+                const long long o = ubase + (long long)(j0 + c) * P.ldm + r;
+                *reinterpret_cast<uint2 *>(P.UThi + o) = *reinterpret_cast<const uint2 *>(uh);
+                *reinterpret_cast<uint2 *>(P.UTlo + o) = *reinterpret_cast<const uint2 *>(ul);
+                *reinterpret_cast<uint2 *>(P.YThi + o) = *reinterpret_cast<const uint2 *>(yh);
+                *reinterpret_cast<uint2 *>(P.YTlo + o) = *reinterpret_cast<const uint2 *>(yl);
+            }
         }
     }
-    const long long ybase = (long long)b * m * P.ldn;
-    for (int t = tid; t < nr * pw; t += blockDim.x) {
-        const int rr = t / pw, c = t - rr * pw;
-        const int r = r0 + rr, j = j0 + c;
-        const float v = slab[c * Sp + rr];
-        __half h, l;
-        split_f16((r < j ? 0.f : (r == j ? 1.f : v)) * kF16V, h, l);
-        P.Yhi[ybase + (long long)r * P.ldn + j] = h;
-        P.Ylo[ybase + (long long)r * P.ldn + j] = l;
+    __syncthreads();
+    const long long ybase = (long long)b * m * P.ldn + j0;
+    {
+        const int c = 2 * (tid % (NB / 2)), nr = min(S, m - r0);
+        for (int rl = tid / (NB / 2); rl < nr; rl += kQrThreads / (NB / 2)) {
+            if (c >= pw) continue;
+            __half h0, l0, h1, l1;
+            split_f16(sm.slab[c][rl] * kF16V, h0, l0);
+            split_f16(sm.slab[c + 1][rl] * kF16V, h1, l1);
+            const long long o = ybase + (long long)(r0 + rl) * P.ldn + c;
+            if (c + 1 < pw) {
+                *reinterpret_cast<__half2 *>(P.Yhi + o) = __halves2half2(h0, h1);
+                *reinterpret_cast<__half2 *>(P.Ylo + o) = __halves2half2(l0, l1);
+            } else {
+                P.Yhi[o] = h0;
+                P.Ylo[o] = l0;
+            }
+        }
     }
     // zeros above the panel's first row, down from the first row of its block (the block's products read them)
     const int s0 = j0 - j0 % kWY;
@@ -237,57 +298,68 @@ __global__ void __launch_bounds__(kQrThreads, 1) qr_panel_kernel(PanelArgs P) {
         for (int t = tid; t < (j0 - s0) * pw; t += blockDim.x) {
             const int rr = t / pw, c = t - rr * pw;
             const __half z = __float2half_rn(0.f);
-            P.Yhi[ybase + (long long)(s0 + rr) * P.ldn + j0 + c] = z;
-            P.Ylo[ybase + (long long)(s0 + rr) * P.ldn + j0 + c] = z;
+            P.Yhi[ybase + (long long)(s0 + rr) * P.ldn + c] = z;
+            P.Ylo[ybase + (long long)(s0 + rr) * P.ldn + c] = z;
             const long long o = ubase + (long long)(j0 + c) * P.ldm + s0 + rr;
             P.YThi[o] = z;
             P.YTlo[o] = z;
         }
-    // partial G = Y^T Y over this CTA's rows (upper triangle), summed by CTA 0 into T
-    float *gp = P.Gpart + ((long long)b * CL + rank) * nb * nb;
-    for (int t = tid; t < pw * pw; t += blockDim.x) {
-        const int i = t / pw, k = t - i * pw;
-        if (k < i) continue;
-        const int ji = j0 + i, jk = j0 + k;
-        float acc = 0.f;
-        for (int rr = max(0, jk - r0); rr < nr; ++rr) {      // Y_r,k = 0 above its diagonal (jk >= ji)
-            const int r = r0 + rr;
-            const float yi = r == ji ? 1.f : slab[i * Sp + rr];
-            const float yk = r == jk ? 1.f : slab[k * Sp + rr];
-            acc = fmaf(yi, yk, acc);
+    if (rank != 0 || 4 * w >= NB) return;
+    // T[c][c] = tau_c, T[:c, c] = -tau_c T[:c, :c] G[:c, c].  Row i needs nothing of the other rows: 8 lanes
+    // per row, lane q with entries q, q + 8, ...
+    const int i = 4 * w + (lane >> 3), q = lane & 7;
+    float *out = P.Tm + ((long long)b * P.npan + P.panel) * NB * NB + (long long)i * NB;
+    float tr[NB / 8];
+#pragma unroll
+    for (int cb = 0; cb < NB / 8; ++cb) tr[cb] = 0.f;
+#pragma unroll
+    for (int cb = 0; cb < NB / 8; ++cb)
+#pragma unroll 1
+        for (int cq = 0; cq < 8; ++cq) {
+            const int c = 8 * cb + cq;
+            float v = 0.f;
+            if (c < pw) {
+#pragma unroll
+                for (int lb = 0; lb <= cb; ++lb)
+                    if (8 * lb + q < c) v = fmaf(tr[lb], sm.G[8 * lb + q][c], v);
+#pragma unroll
+                for (int d = 4; d; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+                const float tc = sm.tau[c];
+                v = i < c ? -tc * v : (i == c ? tc : 0.f);
+                if (q == cq) tr[cb] = v;
+            }
         }
-        gp[i * nb + k] = acc;
-    }
-    __threadfence();
-    cluster.sync();
-    if (rank != 0) return;
-    const int ldt = nb + 1;                          // padded rows: conflict-free column access
-    float *G = slab, *T = slab + nb * ldt;           // the slab is no longer needed
-    __syncthreads();
-    for (int t = tid; t < pw * pw; t += blockDim.x) {
-        const int i = t / pw, k = t - i * pw;
-        float s = 0.f;
-        if (k >= i)
-            for (int q = 0; q < CL; ++q) s += P.Gpart[((long long)b * CL + q) * nb * nb + i * nb + k];
-        G[i * ldt + k] = s;
-        T[i * ldt + k] = 0.f;
-    }
-    __syncthreads();
-    // T[c][c] = tau_c, T[:c, c] = -tau_c T[:c, :c] G[:c, c]  (G upper triangle)
-    const float *tb = P.tau + (long long)b * n + j0;
-    if (tid == 0) T[0] = tb[0];
-    __syncthreads();
-    for (int c = 1; c < pw; ++c) {
-        float v = 0.f;
-        if (tid < c)
-            for (int l = tid; l < c; ++l) v += T[tid * ldt + l] * G[l * ldt + c];
-        __syncthreads();
-        if (tid < c) T[tid * ldt + c] = -tb[c] * v;
-        if (tid == 0) T[c * ldt + c] = tb[c];
-        __syncthreads();
-    }
-    float *out = P.Tm + ((long long)b * P.npan + P.panel) * nb * nb;
-    for (int t = tid; t < nb * nb; t += blockDim.x) out[t] = t / nb < pw && t % nb < pw ? T[(t / nb) * ldt + t % nb] : 0.f;
+#pragma unroll
+    for (int cb = 0; cb < NB / 8; ++cb) out[8 * cb + q] = i < pw ? tr[cb] : 0.f;
+}
+
+// Launch of one panel: the fewest CTAs whose registers hold its m - j0 rows, 256 rows each as far as 8 CTAs
+// reach (64 columns), else 512; 1024 or 1536 for panels of 32 columns.
+template <int RPL, int C>
+static int qr_launch_panel(PanelArgs &a, int B, cudaStream_t st) {
+    using Sm = PanelSmem<RPL, C>;
+    a.cl = (a.m - a.j0 + Sm::S - 1) / Sm::S;
+    if (a.cl > kQrMaxCl || a.pw > Sm::NB) return PSVD_ERR_ARG;
+    static_assert(sizeof(Sm) <= 227 * 1024, "panel too large");
+    PSVD_TRY(cudaFuncSetAttribute(qr_panel_kernel<RPL, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sm)));
+    if (a.cl > 8)
+        PSVD_TRY(cudaFuncSetAttribute(qr_panel_kernel<RPL, C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(B * a.cl));
+    cfg.blockDim = dim3(kQrThreads);
+    cfg.dynamicSmemBytes = sizeof(Sm);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = a.cl;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    PSVD_TRY(cudaLaunchKernelEx(&cfg, qr_panel_kernel<RPL, C>, a));
+    count_launch(1);
+    return PSVD_OK;
 }
 
 // W2^T[c][i] = sum_l T^T[i][l] W[l][c], W = sum of the ks K-split slices of Y^T X, for the ncol <= 96
@@ -561,7 +633,7 @@ static int qr_apply_block(QrWS &w, int j0, int ws, int sup, int c0, int ncol, __
 }
 
 int qr_factor(const float *A, float *Q, float *R, const int *flag, QrWS &w, cudaStream_t st) {
-    const int B = w.B, m = w.m, n = w.n, nb = w.nb, CL = w.cl;
+    const int B = w.B, m = w.m, n = w.n, nb = w.nb;
     const long long nm = (long long)n * w.ldm;
     qr_skip_kernel<<<(B + 127) / 128, 128, 0, st>>>(flag, B, w.skip);
     PSVD_TRY(cudaMemsetAsync(w.amax, 0, sizeof(unsigned) * (size_t)B, st));
@@ -575,33 +647,18 @@ int qr_factor(const float *A, float *Q, float *R, const int *flag, QrWS &w, cuda
         t.fhi = w.UThi; t.flo = w.UTlo; t.ld = w.ldm; t.bstride = t.fbstride = nm; t.fscale = kF16X;
         PSVD_TRY(prepare_operand(A, n, mn, B, m, n, true, 1.f, w.scale, t, st, w.skip));
     }
-    const size_t smem = qr_panel_smem(m, nb, CL);
-    PSVD_TRY(cudaFuncSetAttribute(qr_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (CL > 8) PSVD_TRY(cudaFuncSetAttribute(qr_panel_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)(B * CL));
-    cfg.blockDim = dim3(kQrThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     for (int sp = 0; sp < w.nsup; ++sp) {
         const int s0 = sp * kWY, s1 = std::min(n, s0 + kWY);
         for (int j0 = s0; j0 < s1; j0 += nb) {
             const int pw = std::min(nb, s1 - j0), p = j0 / nb;
             PanelArgs a;
             a.UThi = w.UThi; a.UTlo = w.UTlo; a.YThi = w.YThi; a.YTlo = w.YTlo; a.Yhi = w.Yhi; a.Ylo = w.Ylo;
-            a.tau = w.tau; a.beta = w.beta; a.Tm = w.Tm; a.Gpart = w.Gpart; a.skip = w.skip;
-            a.m = m; a.n = n; a.j0 = j0; a.pw = pw; a.panel = p; a.npan = w.npan; a.nb = nb; a.cl = CL;
+            a.tau = w.tau; a.beta = w.beta; a.Tm = w.Tm; a.skip = w.skip;
+            a.m = m; a.n = n; a.j0 = j0; a.pw = pw; a.panel = p; a.npan = w.npan;
             a.ldm = w.ldm; a.ldn = w.ldn;
-            PSVD_TRY(cudaLaunchKernelEx(&cfg, qr_panel_kernel, a));
-            count_launch(1);
+            const int rows = m - j0;
+            if (nb == 64) PSVD_TRY_RC(rows <= kQrRows8 ? (qr_launch_panel<8, 4>(a, B, st)) : (qr_launch_panel<16, 4>(a, B, st)));
+            else PSVD_TRY_RC(rows <= 16384 ? (qr_launch_panel<32, 2>(a, B, st)) : (qr_launch_panel<48, 2>(a, B, st)));
             if (j0 + pw < s1) PSVD_TRY_RC(qr_apply_panel(w, j0, pw, p, j0 + pw, s1 - j0 - pw, st));
         }
         PSVD_TRY_RC(qr_block_t(w, s0, s1 - s0, sp, st));
@@ -640,10 +697,10 @@ extern "C" size_t psvd_qr_workspace_bytes(int64_t batch, int64_t m, int64_t n) {
 
 extern "C" int psvd_qr(const float *A, float *Q, float *R, int64_t batch, int64_t m, int64_t n, void *ws,
                        size_t ws_bytes, void *stream) {
-    int nb = 0, cl = 0;
+    int nb = 0;
     if (!A || !Q || batch <= 0 || n <= 0 || m < n || batch > 65535 || n > 16384 || (long long)m * n > (1LL << 31))
         return PSVD_ERR_ARG;
-    if (!qr_shape((int)m, &nb, &cl))
+    if (!qr_shape((int)m, &nb))
         return fail_msg(PSVD_ERR_ARG, "psvd_qr: m = %lld rows exceed the cluster panel", (long long)m);
     if (int e = check_device()) return e;
     if (ws_bytes < psvd_qr_workspace_bytes(batch, m, n)) return PSVD_ERR_WORKSPACE;

@@ -6,17 +6,15 @@
 
 namespace psvd {
 
-// Panel shape for m rows: panel width nb (64 or 32) and cluster size cl (8 or 16 CTAs per
-// matrix) such that each CTA's slab of ceil(m / cl) rows x nb columns fits in shared memory.
-// Returns false when no shape fits (m too large for the cluster panel).
-bool qr_shape(int m, int *nb, int *cl);
+// Panel width nb (64 or 32) for m rows; false when m is too large for the cluster panel.
+bool qr_shape(int m, int *nb);
 
 constexpr int kQrSplit = 8;   // largest K split of the X^T Y products of a block
 
 // The matrices are normalized by a power of two (|A| <= 2^e, columns of norm <= 1), so every array
 // below is bounded and kept as split-FP16 halves.
 struct QrWS {
-    int B = 0, m = 0, n = 0, nb = 0, cl = 0, npan = 0, nsup = 0, ks = 1;
+    int B = 0, m = 0, n = 0, nb = 0, npan = 0, nsup = 0, ks = 1;
     long long ldm = 0, ldn = 0;
     __half *UThi = nullptr, *UTlo = nullptr;   // [B][n][ldm] the matrix transposed, being factored (kF16X)
     __half *YThi = nullptr, *YTlo = nullptr;   // [B][n][ldm] reflector j as row j (1 at j, 0 above) (kF16V)
@@ -24,7 +22,6 @@ struct QrWS {
     __half *QThi = nullptr, *QTlo = nullptr;   // [B][n][ldm] Q^T being accumulated (kF16X)
     float *tau = nullptr, *beta = nullptr;     // [B][n]
     float *Tm = nullptr;                       // [B][npan][nb][nb] compact-WY T of every panel
-    float *Gpart = nullptr;                    // [B][cl][nb][nb] per-CTA partial Y^T Y of a panel
     float *Wp = nullptr;                       // [ks][B][nb][n] partial Y^T X of a panel (K split)
     __half *W2hi = nullptr, *W2lo = nullptr;   // [B][n][kWY] (op(T) Y^T X)^T (kF16S2)
     float *Gs = nullptr, *Ts = nullptr;        // [B][nsup][kWY][kWY] Y^T Y and T of blocks of kWY columns
@@ -37,7 +34,7 @@ struct QrWS {
     template <class C>
     void carve(C &cv, int B_, int m_, int n_) {
         B = B_; m = m_; n = n_;
-        if (!qr_shape(m, &nb, &cl)) { nb = 64; cl = 8; }
+        if (!qr_shape(m, &nb)) nb = 64;
         npan = (n + nb - 1) / nb;
         nsup = (n + kWY - 1) / kWY;
         ldm = pad_ld(m); ldn = pad_ld(n);
@@ -49,7 +46,6 @@ struct QrWS {
         QThi = cv.template take<__half>(B64 * nm); QTlo = cv.template take<__half>(B64 * nm);
         tau = cv.template take<float>(B64 * n); beta = cv.template take<float>(B64 * n);
         Tm = cv.template take<float>(B64 * npan * nb * nb);
-        Gpart = cv.template take<float>(B64 * cl * nb * nb);
         Wp = cv.template take<float>((long long)ks * B64 * nb * std::min(n, kWY));
         W2hi = cv.template take<__half>(B64 * n * kWY); W2lo = cv.template take<__half>(B64 * n * kWY);
         Gs = cv.template take<float>(B64 * nsup * kWY * kWY);

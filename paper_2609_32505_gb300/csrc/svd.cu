@@ -497,8 +497,8 @@ struct SvdWS {
         colss = cv.template take<float>(B64 * n);
         flag = cv.template take<int>(B64);
         any = cv.template take<int>(4);
-        int qnb = 0, qcl = 0;
-        blocked_qr = qr_shape(m, &qnb, &qcl);
+        int qnb = 0;
+        blocked_qr = qr_shape(m, &qnb);
         if (blocked_qr) {
             qw.carve(cv, B, m, n);
         } else {
@@ -863,8 +863,8 @@ static psvd_opts square_opts(const psvd_opts &o) {
 }
 
 static bool use_preqr(const psvd_opts &o, int64_t m, int64_t n) {
-    int nb = 0, cl = 0;
-    return o.preqr && m > n && qr_shape((int)m, &nb, &cl);
+    int nb = 0;
+    return o.preqr && m > n && qr_shape((int)m, &nb);
 }
 
 extern "C" size_t psvd_svd_workspace_bytes(int64_t batch, int64_t m, int64_t n, const psvd_opts *opts) {

@@ -95,3 +95,25 @@ def test_backward_edges_and_ranges(m, n, sa, su, sv, sg):
     X = (E + E.T) / 2 / (S[:, None] + S[None, :])
     ref = (dU * D[None, :] + 2 * Y @ X) @ VT
     assert _rel(da, ref) <= 2e-5
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (3, 2), (33, 17), (65, 64), (255, 63), (257, 65), (260, 130), (513, 70),
+                                 (2048, 66), (2049, 66), (2300, 40), (4100, 33), (8192, 65), (8193, 65), (16385, 33),
+                                 (23024, 34)])
+def test_qr_panel_shapes(m, n):
+    """The panel's launch shapes: one to sixteen CTAs per matrix, 256, 512, 1024 and 1536 rows each, panels of 64 and
+    32 columns, with remainders in rows and columns; the last matrix has dependent columns (a zero
+    reflector).  The rounding errors of a column of m entries add up to about sqrt(m) 2^-24, those of the split
+    products to a few 2^-22: 4 sqrt(m) 2^-24 + 2^-19."""
+    import paper_2609_32505_gb300 as P
+    g = torch.Generator()
+    g.manual_seed(m + n)
+    a = torch.randn(2, m, n, generator=g)
+    a[1, :, n // 2:] = 0.0
+    q, r = P.qr(a.cuda())
+    a, q, r = a.double(), q.cpu().double(), r.cpu().double()
+    tol = 4 * m ** 0.5 * 2.0 ** -24 + 2.0 ** -19
+    for b in range(2):
+        assert torch.linalg.matrix_norm(q[b] @ r[b] - a[b]) <= tol * torch.linalg.matrix_norm(a[b])
+        assert (q[b].T @ q[b] - torch.eye(n, dtype=torch.float64)).abs().max() <= tol
+        assert torch.equal(r[b], torch.triu(r[b])) and torch.all(torch.diagonal(r[b]) >= 0)
