@@ -7,12 +7,12 @@
 // the backward chain.
 //
 // Persistent kernel: one CTA per SM walks a static list of output tiles of
-// 128 x BN (BN = 256, or 128 when N <= 128), UMMA M = 128, N = BN, cta_group::1.
-// 128-wide tiles cost about twice as much per flop as 256-wide ones on GB300 (a fixed
-// cost per MMA instruction; measured with one mainloop version, BF16 at 8192^3: 559
-// against 1049 TFLOP/s), so they are used only where N <= 128.
+// 128 x BN, UMMA M = 128, N = BN, cta_group::1.  BN = 256, or 128 when N <= 128: 128-wide tiles
+// cost about twice as much per flop as 256-wide ones on GB300 (a fixed cost per MMA instruction; measured
+// with one mainloop version, BF16 at 8192^3: 559 against 1049 TFLOP/s); halved down to 32 while a launch
+// leaves half of the SMs idle (plan_gemm).
 // Shared memory holds a 192 KB ring of units (4 x 48 KB at BN = 256, 6 x 32 KB at
-// BN = 128), each one TMA'd k-block: an A sub-tile (128 rows x 128 B) and a B sub-tile
+// BN = 128, 9 x 20 KB at 32), each one TMA'd k-block: an A sub-tile (128 rows x 128 B) and a B sub-tile
 // (BN rows x 128 B), both in the canonical 128-byte-swizzled K-major layout:
 //   PREC_BF16   : 64 bf16 of K per unit, one unit per k-block
 //   PREC_TF32   : 32 fp32 of K per unit, one unit per k-block
@@ -48,7 +48,9 @@ constexpr int kUnitB = 32768;                  // up to 256 rows x 128 B
 constexpr int kUnitBytes = kUnitA + kUnitB;    // 48 KB
 constexpr int kStages = 4;                     // ring units at BN = 256
 constexpr int kRingBytes = kStages * kUnitBytes;
-constexpr int kMaxStages = kRingBytes / (kUnitA + 128 * 128);   // ring units at BN = 128 (6)
+constexpr int kMinBN = 32;
+static_assert(kMinBN >= 32 && kMinBN % 32 == 0, "the two column halves of a tile are read and stored 16 columns at a time");
+constexpr int kMaxStages = kRingBytes / (kUnitA + kMinBN * 128);   // ring units at BN = 32 (9)
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = (kEpiWarps + 2) * 32;
 constexpr int kStageRow = 17;                  // staging row stride (floats): conflict-free
@@ -71,7 +73,7 @@ struct GemmMaps {
 struct GemmShape {
     int M, N, K;            // logical sizes
     int tiles_m, tiles_n;   // ceil(M/128), ceil(N/BN)
-    int bn;                 // 128 or 256
+    int bn;                 // 32, 64, 128 or 256
     int batch;
     int sym;                // 1: only tiles that reach the upper triangle (col >= row); requires A == B
     int ksplit;             // > 1: every tile repeated over ksplit disjoint k-block ranges; the
@@ -81,6 +83,9 @@ struct GemmShape {
     const int *skip;        // [batch] nonzero = matrix finished, its tiles are skipped (or nullptr)
     const int *gate;        // nullptr, or a device counter: 0 = nothing left to do, the whole launch
                             // returns at once (written by an earlier kernel on the same stream)
+    int *over;              // nullptr, or the word of a chain of gated launches (zeroed before it) that the first one
+                            // to find its gate at 0 sets: all later ones return at once, without waiting for
+                            // their predecessors (a gate at 0 means that every later gate is)
     unsigned *ticket;       // nullptr, or a zeroed counter: the last CTA to finish runs epi.tail()
     unsigned *err;          // device error word
     float f16_scale;        // PREC_F16X3: the product of the operands' inverse scales ...
@@ -312,10 +317,21 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
     // Launched ahead of its predecessor's end (programmatic dependent launch): let the next launch
     // come, then wait until everything before this one has completed and is visible.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // A launch of a chain that is over returns without waiting (thread 0 decides for its block: the word
+    // may be written meanwhile).
+    if (shp.over) {
+        __shared__ int s_over;
+        if (threadIdx.x == 0) s_over = *static_cast<volatile int *>(shp.over);
+        __syncthreads();
+        if (s_over) return;
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // A gated launch with nothing left to do returns before any allocation (uniform: every
-    // thread reads the same word, final since the kernel that wrote it has completed).
-    if (shp.gate && *shp.gate == 0) return;
+    // thread reads the same word, final since the kernel that wrote it has completed), and ends its chain.
+    if (shp.gate && *shp.gate == 0) {
+        if (shp.over && blockIdx.x == 0 && threadIdx.x == 0) *static_cast<volatile int *>(shp.over) = 1;
+        return;
+    }
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kRingBytes);
@@ -329,7 +345,7 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int bn = shp.bn;
     const uint32_t unit_bytes = (uint32_t)(kUnitA + bn * 128);   // also the ring stride (1024-aligned)
-    const uint32_t nst = kRingBytes / unit_bytes;                // 4 or 6
+    const uint32_t nst = kRingBytes / unit_bytes;                // 4 .. 9
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], kEpiWarps); }
@@ -546,30 +562,33 @@ inline int host_tiles_per_matrix(const GemmShape &s) {
     return c;
 }
 
-template <class Epi>
-cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *ahi, const MatView *alo,
-                        const MatView *bhi, const MatView *blo, GemmShape shp, int batch, const Epi &epi,
-                        cudaStream_t st, const F16Views *f16 = nullptr) {
-    // Set on every launch, through the same kernel handle the launch below uses: each
-    // .cu file that instantiates this template registers its own copy of the kernel, so
-    // a process-wide "already configured" flag would leave other copies unconfigured.
-    {
-        cudaError_t e = cudaFuncSetAttribute(gemm_tn_kernel<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kGemmSmem);
-        if (e != cudaSuccess) { cuda_fail(e, __FILE__, __LINE__); return e; }
-    }
+// What a launch needs besides its epilogue: the tensor maps and the tile list.  A loop that launches the
+// same product many times plans it once.
+struct GemmPlan {
+    GemmMaps maps;
+    GemmShape shp;
+    int grid = 0;
+};
+
+inline cudaError_t plan_gemm(GemmPlan &plan, const MatView *a16, const MatView *b16, const MatView *ahi,
+                             const MatView *alo, const MatView *bhi, const MatView *blo, const GemmShape &shape,
+                             int batch, const F16Views *f16) {
+    GemmShape &shp = plan.shp;
+    shp = shape;
     shp.bn = shp.N > 128 ? 256 : 128;
-    if (shp.bn == 256) {
-        // A launch with fewer 256-wide tiles than half the SMs is bound by one tile's serial
-        // k-loop (and, for split-TF32, its per-k-block flushes): 128-wide tiles put twice
-        // as many CTAs to work on it.
+    // A launch with fewer tiles than half the SMs is bound by one tile's serial chain, above all its
+    // epilogue: narrower tiles put more CTAs to work on it.  (Whole polar decompositions with
+    // tiles down to 128 / 64 / 32 columns, us: 256 x 256 684 / 614 / 564, 1024 x 256 814 / 748 / 679, two of
+    // 1500 x 700 1045 / 1007 / 965.)
+    while (shp.bn > kMinBN) {
         GemmShape t = shp;
         t.tiles_m = (t.M + kBM - 1) / kBM;
-        t.tiles_n = (t.N + 255) / 256;
+        t.tiles_n = (t.N + t.bn - 1) / t.bn;
         const long long tiles = (long long)host_tiles_per_matrix(t) * (shp.ksplit > 1 ? shp.ksplit : 1) * batch;
-        if (2 * tiles <= num_sms()) shp.bn = 128;
+        if (2 * tiles > num_sms()) break;
+        shp.bn /= 2;
     }
-    GemmMaps maps;
+    GemmMaps &maps = plan.maps;
     memset(&maps, 0, sizeof(maps));
     // A map that is not supplied stays zero; the kernel only reads those of the precisions its tiles have.
     auto encode = [&](CUtensorMap *m, const MatView *v, int rows) { return !v || make_tmap(m, *v, rows); };
@@ -587,9 +606,26 @@ cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *a
     shp.tiles_m = (shp.M + kBM - 1) / kBM;
     shp.tiles_n = (shp.N + shp.bn - 1) / shp.bn;
     shp.batch = batch;
+    plan.grid = 0;
     if (shp.tiles_m == 0 || shp.tiles_n == 0 || batch == 0) return cudaSuccess;
     const long long total = (long long)host_tiles_per_matrix(shp) * (shp.ksplit > 1 ? shp.ksplit : 1) * batch;
-    const int grid = (int)std::min<long long>(total, num_sms());
+    plan.grid = (int)std::min<long long>(total, num_sms());
+    return cudaSuccess;
+}
+
+// `configure`: set the kernel's shared memory limit (needed once before a loop of launches).  It is set through
+// the same kernel handle the launch below uses: each .cu file that instantiates this template registers its own
+// copy of the kernel, so a process-wide "already configured" flag, or a function of its own, would leave other
+// copies unconfigured.
+template <class Epi>
+cudaError_t launch_plan(const GemmPlan &plan, const Epi &epi, cudaStream_t st, bool configure = true) {
+    const GemmShape &shp = plan.shp;
+    if (plan.grid == 0) return cudaSuccess;
+    if (configure) {
+        cudaError_t e = cudaFuncSetAttribute(gemm_tn_kernel<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kGemmSmem);
+        if (e != cudaSuccess) { cuda_fail(e, __FILE__, __LINE__); return e; }
+    }
     const bool prof = prof_on();
     if (prof) prof_begin(st);
     // Programmatic dependent launch: the grid is set up while the kernel before it still runs (its
@@ -597,7 +633,7 @@ cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *a
     // short products of small matrices and of the polar steps that find nothing to do.
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = dim3((unsigned)plan.grid);
     cfg.blockDim = dim3(kGemmThreads);
     cfg.dynamicSmemBytes = kGemmSmem;
     cfg.stream = st;
@@ -607,18 +643,27 @@ cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *a
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     {
-        cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_tn_kernel<Epi>, maps, shp, epi);
+        cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_tn_kernel<Epi>, plan.maps, shp, epi);
         if (e != cudaSuccess) { cuda_fail(e, __FILE__, __LINE__); return e; }
     }
     count_launch();
     if (prof) {
         // algorithmic flops: 2 M N K per matrix (M (M + 1) K for the symmetric Gram)
         const double f = shp.sym ? (double)shp.M * (shp.M + 1) * shp.K : 2.0 * shp.M * shp.N * (double)shp.K;
-        prof_end(st, f * batch, shp.prof_as > 0 ? shp.prof_as - 1 : (shp.prec ? -1 : std::min(shp.prec_uniform, (int)PREC_TF32X3)));
+        prof_end(st, f * shp.batch, shp.prof_as > 0 ? shp.prof_as - 1 : (shp.prec ? -1 : std::min(shp.prec_uniform, (int)PREC_TF32X3)));
     }
     cudaError_t le = cudaGetLastError();
     if (le != cudaSuccess) cuda_fail(le, __FILE__, __LINE__);
     return le;
+}
+
+template <class Epi>
+cudaError_t launch_gemm(const MatView *a16, const MatView *b16, const MatView *ahi, const MatView *alo,
+                        const MatView *bhi, const MatView *blo, const GemmShape &shp, int batch, const Epi &epi,
+                        cudaStream_t st, const F16Views *f16 = nullptr) {
+    GemmPlan plan;
+    const cudaError_t e = plan_gemm(plan, a16, b16, ahi, alo, bhi, blo, shp, batch, f16);
+    return e != cudaSuccess ? e : launch_plan(plan, epi, st);
 }
 
 }  // namespace psvd

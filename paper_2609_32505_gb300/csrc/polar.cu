@@ -547,30 +547,64 @@ __global__ void polar_info_kernel(int B, const int *status, const int *fin, cons
 }
 
 // ------------------------------------------------------------ host driver
+// The two products of a step, planned once for either parity of the step (X ping-pongs between two arrays).
+struct StepPlans { GemmPlan gram[2], apply[2]; };
+
+static cudaError_t plan_steps(PolarWS &w, StepPlans &p) {
+    const int B = w.B, m = w.m, n = w.n;
+    for (int par = 0; par < 2; ++par) {
+        {   // Gram: A = B = X^T (n x m, K = m), upper-triangle tiles
+            MatView v16 = w.bf16 ? view_of16(w.XT16[par], n, m, w.ldm, (long long)n * w.ldm, B) : MatView();
+            MatView vhi = view_of(w.XThi[par], n, m, w.ldm, (long long)n * w.ldm, B);
+            F16Views f;
+            f.ah = f.bh = view_f16(as_half(w.XThi[par]), n, m, w.ldm, 2LL * n * w.ldm, B);
+            f.al = f.bl = view_f16(as_half(w.XTlo[par]), n, m, w.ldm, 2LL * n * w.ldm, B);
+            GemmShape s;
+            memset(&s, 0, sizeof(s));
+            s.M = n; s.N = n; s.K = m; s.sym = 1;
+            s.f16_scale = 1.f / (kF16X * kF16X);
+            const MatView *t = w.mixed ? &vhi : nullptr, *t16 = w.bf16 ? &v16 : nullptr;
+            if (cudaError_t e = plan_gemm(p.gram[par], t16, t16, t, nullptr, t, nullptr, s, B, &f)) return e;
+        }
+        {   // Apply: A = X (m x n, K = n), B = P (n x n, symmetric)
+            MatView a16 = w.bf16 ? view_of16(w.X16[par], m, n, w.ldn, (long long)m * w.ldn, B) : MatView();
+            MatView ahi = view_of(w.Xhi[par], m, n, w.ldn, (long long)m * w.ldn, B);
+            MatView b16 = w.bf16 ? view_of16(w.P16, n, n, w.ldn, (long long)n * w.ldn, B) : MatView();
+            MatView bhi = view_of(w.Phi, n, n, w.ldn, (long long)n * w.ldn, B);
+            F16Views f;
+            f.ah = view_f16(as_half(w.Xhi[par]), m, n, w.ldn, 2LL * m * w.ldn, B);
+            f.al = view_f16(as_half(w.Xlo[par]), m, n, w.ldn, 2LL * m * w.ldn, B);
+            f.bh = view_f16(as_half(w.Phi), n, n, w.ldn, 2LL * n * w.ldn, B);
+            f.bl = view_f16(as_half(w.Plo), n, n, w.ldn, 2LL * n * w.ldn, B);
+            GemmShape s;
+            memset(&s, 0, sizeof(s));
+            s.M = m; s.N = n; s.K = n;
+            s.f16_scale = 1.f / (kF16X * kF16P);
+            if (cudaError_t e = plan_gemm(p.apply[par], w.bf16 ? &a16 : nullptr, w.bf16 ? &b16 : nullptr,
+                                          w.mixed ? &ahi : nullptr, nullptr, w.mixed ? &bhi : nullptr, nullptr, s, B, &f))
+                return e;
+        }
+    }
+    return cudaSuccess;
+}
+
 // Step k: Gram (with the polynomial and residual epilogue, and the per-matrix decision run
 // by its last CTA), then apply.  The Gram launch is gated on `gram_gate` (the count of
 // matrices still iterating; nullptr = always run) and the apply launch on this step's own
 // count, so once every matrix has finished the remaining launches of the budget return at
 // once.
-static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, float *fres, const int *gram_gate,
-                       cudaStream_t st) {
+static int launch_step(PolarWS &w, StepPlans &plans, int k, bool apply, double tol, bool learned, float *fres,
+                       const int *gram_gate, cudaStream_t st) {
     const int B = w.B, m = w.m, n = w.n;
     const int par = k & 1, npar = (k + 1) & 1;
-    // Gram: A = B = X^T (n x m, K = m), upper-triangle tiles
+    int *over = w.notdone + w.kcap + 1;
     {
-        MatView v16 = w.bf16 ? view_of16(w.XT16[par], n, m, w.ldm, (long long)n * w.ldm, B) : MatView();
-        MatView vhi = view_of(w.XThi[par], n, m, w.ldm, (long long)n * w.ldm, B);
-        F16Views f;
-        f.ah = f.bh = view_f16(as_half(w.XThi[par]), n, m, w.ldm, 2LL * n * w.ldm, B);
-        f.al = f.bl = view_f16(as_half(w.XTlo[par]), n, m, w.ldm, 2LL * n * w.ldm, B);
-        GemmShape s;
-        memset(&s, 0, sizeof(s));
-        s.M = n; s.N = n; s.K = m; s.sym = 1;
+        GemmShape &s = plans.gram[par].shp;
         s.prec = w.prec + (long long)k * B;
         s.skip = w.done;
         s.gate = gram_gate;
+        s.over = over;
         s.ticket = w.ticket + k;
-        s.f16_scale = 1.f / (kF16X * kF16X);
         s.err = w.err;
         EpiGram e;
         e.n = n; e.B = B;
@@ -580,30 +614,15 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
         e.prec = w.prec + (long long)k * B;
         e.res = w.res + (long long)k * B;
         e.P16 = w.P16; e.Phi = w.Phi; e.Plo = w.Plo; e.ldp = w.ldn;
-        const MatView *t = w.mixed ? &vhi : nullptr;
-        cudaError_t er = launch_gemm(w.bf16 ? &v16 : nullptr, w.bf16 ? &v16 : nullptr, t, nullptr, t, nullptr, s, B, e,
-                                     st, &f);
-        if (er != cudaSuccess) return PSVD_ERR_CUDA;
+        if (launch_plan(plans.gram[par], e, st, k == 0) != cudaSuccess) return PSVD_ERR_CUDA;
     }
     if (!apply) return PSVD_OK;
-    // Apply: A = X (m x n, K = n), B = P (n x n, symmetric)
     {
-        MatView a16 = w.bf16 ? view_of16(w.X16[par], m, n, w.ldn, (long long)m * w.ldn, B) : MatView();
-        MatView ahi = view_of(w.Xhi[par], m, n, w.ldn, (long long)m * w.ldn, B);
-        MatView b16 = w.bf16 ? view_of16(w.P16, n, n, w.ldn, (long long)n * w.ldn, B) : MatView();
-        MatView bhi = view_of(w.Phi, n, n, w.ldn, (long long)n * w.ldn, B);
-        F16Views f;
-        f.ah = view_f16(as_half(w.Xhi[par]), m, n, w.ldn, 2LL * m * w.ldn, B);
-        f.al = view_f16(as_half(w.Xlo[par]), m, n, w.ldn, 2LL * m * w.ldn, B);
-        f.bh = view_f16(as_half(w.Phi), n, n, w.ldn, 2LL * n * w.ldn, B);
-        f.bl = view_f16(as_half(w.Plo), n, n, w.ldn, 2LL * n * w.ldn, B);
-        GemmShape s;
-        memset(&s, 0, sizeof(s));
-        s.M = m; s.N = n; s.K = n;
+        GemmShape &s = plans.apply[par].shp;
         s.prec = w.prec + (long long)k * B;
         s.skip = w.done;
-        s.f16_scale = 1.f / (kF16X * kF16P);
         s.gate = w.notdone + k;          // matrices still iterating after this step's decision
+        s.over = over;
         s.err = w.err;
         EpiApply e;
         e.m = m; e.n = n; e.B = B;
@@ -611,22 +630,23 @@ static int launch_step(PolarWS &w, int k, bool apply, double tol, bool learned, 
         e.X16 = w.X16[npar]; e.XT16 = w.XT16[npar];
         e.Xhi = w.Xhi[npar]; e.Xlo = w.Xlo[npar]; e.XThi = w.XThi[npar]; e.XTlo = w.XTlo[npar];
         e.ldn = w.ldn; e.ldm = w.ldm;
-        cudaError_t er = launch_gemm(w.bf16 ? &a16 : nullptr, w.bf16 ? &b16 : nullptr, w.mixed ? &ahi : nullptr, nullptr,
-                                     w.mixed ? &bhi : nullptr, nullptr, s, B, e, st, &f);
-        if (er != cudaSuccess) return PSVD_ERR_CUDA;
+        if (launch_plan(plans.apply[par], e, st, k == 0) != cudaSuccess) return PSVD_ERR_CUDA;
     }
     return PSVD_OK;
 }
 
-// Launches steps 0..kmax (kmax <= kcap) with no host synchronization: the decision kernel
+// Launches steps 0..kmax (kmax <= kcap) with no host synchronization: the decision
 // of step k counts the matrices still iterating in notdone[k], and the launches after the
-// last matrix has finished find their gate at 0 and return at once.  `first_gate` gates
-// the Gram launch of step 0 (nullptr: always run).
+// last matrix has finished find their gate at 0 and return at once; the first that does sets
+// notdone[kcap + 1], and those after it do not even wait for each other (w.notdone zeroed before
+// the pass).  `first_gate` gates the Gram launch of step 0 (nullptr: always run).
 static int run_iteration(PolarWS &w, int kmax, double tol, bool learned, float *fres, const int *first_gate,
                          cudaStream_t st) {
+    StepPlans plans;
+    PSVD_TRY(plan_steps(w, plans));
     for (int k = 0; k <= kmax; ++k) {
         const int *gate = k == 0 ? first_gate : w.notdone + (k - 1);
-        if (int rc = launch_step(w, k, k < w.kcap, tol, learned, fres, gate, st)) return rc;
+        if (int rc = launch_step(w, plans, k, k < w.kcap, tol, learned, fres, gate, st)) return rc;
     }
     return PSVD_OK;
 }
