@@ -339,6 +339,20 @@ PSVD_DEV int sturm_count(const float *d, const float *e2, int n, float x, float 
     return c;
 }
 
+// Lanes per eigenvalue of the two multisections: L lanes cut the interval into L + 1 parts with one count
+// each, so more lanes mean fewer rounds, each a chain of n dependent steps, and fewer lanes mean less work.
+// The most lanes that keep the chip at no more than 16 warps per SM, where the warps' chains still hide each
+// other.  Against 8 lanes for all sizes, bisection / refinement in us: 1 x 256 (32 lanes) 83 -> 55 / 199 -> 112,
+// 1 x 1999 (32) 558 -> 420 / -, 1 x 4096 (16) 918 -> 973 / -, 64 x 512 (2) 525 -> 337 / 1926 -> 939, 4 x 4096 (4) about
+// 2900 -> 1960 / 9000 -> 5400; 8 x 1024 keeps its 8 (4 would take 317 against 290 / 804 against 584).
+// (Refinement: part of it from the cheaper division.)
+static int section_lanes(long long eigenvalues) {
+    int L = 32;
+    while (L > 2 && eigenvalues * L > 16LL * 32 * num_sms()) L /= 2;
+    return L;
+}
+
+template <int L>
 __global__ void tri_bisect_kernel(const double *D, const double *E, int n, double *lam, double *tnorm_out) {
     extern __shared__ float s[];
     float *d = s, *e2 = s + n;
@@ -374,30 +388,31 @@ __global__ void tri_bisect_kernel(const double *D, const double *E, int n, doubl
     glo = FLT_MAX; ghi = -FLT_MAX;
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { glo = fminf(glo, sh_lo[i]); ghi = fmaxf(ghi, sh_hi[i]); }
     if (blockIdx.x == 0 && threadIdx.x == 0 && tnorm_out) tnorm_out[b] = tn;
-    // 9-way multisection: the 8 lanes of a group evaluate the Sturm count at the 8
+    // Multisection: the L lanes of a group evaluate the Sturm count at the L
     // interior points of [lo, hi]; the counts are non-decreasing in x, so the lanes whose
     // count is <= j form a prefix and its length selects the next interval.
-    const int grp = threadIdx.x >> 3, l = threadIdx.x & 7;
-    const int i = blockIdx.x * (blockDim.x >> 3) + grp;   // descending index
+    constexpr unsigned kMask = L == 32 ? 0xffffffffu : (1u << L) - 1u;
+    const int grp = threadIdx.x / L, l = threadIdx.x % L;
+    const int i = blockIdx.x * (blockDim.x / L) + grp;    // descending index
     const bool valid = i < n;
     const int j = n - 1 - i;
     const float pivmin = 1e-30f;
     const float pad = 4.f * FLT_EPSILON * n + 1e-30f;
     float lo = glo - pad, hi = ghi + pad;
-    const unsigned gshift = (threadIdx.x & 31) & ~7u;
+    const unsigned gshift = (threadIdx.x & 31) & ~(L - 1u);
     bool stalled = false;
-    for (int round = 0; round < 24; ++round) {
+    for (int round = 0; round < 64; ++round) {
         const bool active = valid && tn > 0.0 && !stalled &&
                             hi - lo > 2.f * FLT_EPSILON * fmaxf(fabsf(lo), fabsf(hi)) + 2e-30f;
         if (!__any_sync(0xffffffffu, active)) break;
         const float w = hi - lo;
-        const float x = lo + w * ((float)(l + 1) * (1.f / 9.f));
+        const float x = lo + w * ((float)(l + 1) * (1.f / (L + 1)));
         const bool le = active && sturm_count(d, e2, n, x, pivmin) <= j;
-        const unsigned bits = (__ballot_sync(0xffffffffu, le) >> gshift) & 0xFFu;
+        const unsigned bits = (__ballot_sync(0xffffffffu, le) >> gshift) & kMask;
         if (active) {
             const int k = __popc(bits);
-            const float nlo = k > 0 ? lo + w * ((float)k * (1.f / 9.f)) : lo;
-            const float nhi = k < 8 ? lo + w * ((float)(k + 1) * (1.f / 9.f)) : hi;
+            const float nlo = k > 0 ? lo + w * ((float)k * (1.f / (L + 1))) : lo;
+            const float nhi = k < L ? lo + w * ((float)(k + 1) * (1.f / (L + 1))) : hi;
             if (nlo <= lo && nhi >= hi) stalled = true;   // no progress at float resolution
             else { lo = nlo; hi = nhi; }
         }
@@ -408,15 +423,17 @@ __global__ void tri_bisect_kernel(const double *D, const double *E, int n, doubl
 }
 
 // ------------------------------------------------------------ refinement (float-float)
-// Float-float quotient a / b (a, b two-float values, b.hi != 0): the FP32 quotient of the
-// leading words, then one correction from the exact residual a - r b, so that the result
-// carries ~2^-44 relative accuracy on the FP32 pipe.
-PSVD_DEV ff ff_div(ff a, ff b) {
-    const float r = __fdividef(a.hi, b.hi);
-    const float p = __fmul_rn(r, b.hi);
-    const float pe = __fmaf_rn(r, b.hi, -p);                  // r b.hi = p + pe exactly
-    const float res = __fadd_rn(__fsub_rn(__fsub_rn(a.hi, p), pe), __fsub_rn(a.lo, __fmul_rn(r, b.lo)));
-    const float r2 = __fdividef(res, b.hi);
+// Float-float quotient a / b from r0 ~ 1 / b.hi: the quotient of the leading words and one correction from its
+// residual (formed by FMAs), ~2^-45 relative on the FP32 pipe.
+PSVD_DEV float ff_rcp0(ff b) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b.hi));
+    return r;
+}
+PSVD_DEV ff ff_div(ff a, ff b, float r0) {
+    const float r = __fmul_rn(a.hi, r0);
+    const float res = __fadd_rn(__fmaf_rn(-r, b.lo, __fmaf_rn(-r, b.hi, a.hi)), a.lo);
+    const float r2 = __fmul_rn(res, r0);
     const float h = __fadd_rn(r, r2);
     return ff{h, __fsub_rn(r2, __fsub_rn(h, r))};
 }
@@ -435,7 +452,7 @@ PSVD_DEV int sturm_count_ff(const float4 *__restrict__ dd, int n, ff x, float pi
     for (int t = 1; t < n; ++t) {
         v = dd[t];
         const ff a = ff_add(ff{v.x, v.y}, ff{-x.hi, -x.lo});
-        const ff r = ff_div(ff{v.z, v.w}, q);
+        const ff r = ff_div(ff{v.z, v.w}, q, ff_rcp0(q));
         q = ff_add(a, ff{-r.hi, -r.lo});
         if (fabsf(q.hi) < pivmin) q = ff{-pivmin, 0.f};
         c += q.hi < 0.f;
@@ -482,16 +499,18 @@ PSVD_DEV double recip64(double a) {
     return fma(y, e, y);
 }
 
-// Eigenvalues whose FP32 neighbours are closer than `near` * ||T|| are refined by 9-way
-// multisection (8 lanes per eigenvalue) from a bracket around the FP32 value, with
+// Eigenvalues whose FP32 neighbours are closer than `near` * ||T|| are refined by
+// multisection (section_lanes lanes per eigenvalue) from a bracket around the FP32 value, with
 // float-float Sturm counts, down to 16 * 2^-48 ||T|| (~6e-14 ||T||; the FP64 counts that
 // reached 4 u_64 ||T|| kept the narrow FP64 pipe busy for ~30 ms on graded spectra at n = 4096).
 // With such shifts three inverse-iteration solves separate gaps down to ~1e-11 ||T|| by
 // themselves; closer groups get the Gram-Schmidt of tri_cluster_kernel.
+template <int L>
 __global__ void tri_refine_kernel(const float4 *DD, int n, const double *tnorm, double near, double *lam) {
     const int b = blockIdx.y;
-    const int grp = threadIdx.x >> 3, l = threadIdx.x & 7;
-    const int i = blockIdx.x * (blockDim.x >> 3) + grp;     // descending index
+    constexpr unsigned kMask = L == 32 ? 0xffffffffu : (1u << L) - 1u;
+    const int grp = threadIdx.x / L, l = threadIdx.x % L;
+    const int i = blockIdx.x * (blockDim.x / L) + grp;       // descending index
     const float4 *dd = DD + (long long)b * n;
     double *lb = lam + (long long)b * n;
     const double tn = tnorm[b];
@@ -516,33 +535,29 @@ __global__ void tri_refine_kernel(const float4 *DD, int n, const double *tnorm, 
     };
     double w = 64.0 * FLT_EPSILON * tn;
     double lo = mid - w, hi = mid + w;
-    const unsigned gshift = (threadIdx.x & 31) & ~7u;
+    const unsigned gshift = (threadIdx.x & 31) & ~(L - 1u);
     // a bracket with count(lo) <= j < count(hi), widened if the FP32 value was off
     for (int tries = 0; tries < 6; ++tries) {
-        bool need = false;
-        if (active) {
-            const double x = l == 0 ? lo : hi;
-            const int c = l < 2 ? count(x) : 0;
-            const bool ok = l == 0 ? c <= j : (l == 1 ? c > j : true);
-            const unsigned bad = (__ballot_sync(0xffffffffu, !ok) >> gshift) & 0x3u;
-            need = bad != 0;
-        } else {
-            __ballot_sync(0xffffffffu, false);
+        bool ok = true;
+        if (active && l < 2) {
+            const int c = count(l == 0 ? lo : hi);
+            ok = l == 0 ? c <= j : c > j;
         }
+        const bool need = ((__ballot_sync(0xffffffffu, !ok) >> gshift) & kMask) != 0;
         if (!__any_sync(0xffffffffu, need)) break;
         if (need) { w *= 16.0; lo = mid - w; hi = mid + w; }
     }
-    for (int round = 0; round < 24; ++round) {
+    for (int round = 0; round < 64; ++round) {
         const bool go = active && hi - lo > stop;
         if (!__any_sync(0xffffffffu, go)) break;
         const double width = hi - lo;
-        const double x = lo + width * ((double)(l + 1) / 9.0);
+        const double x = lo + width * ((double)(l + 1) / (L + 1));
         const bool le = go && count(x) <= j;
-        const unsigned bits = (__ballot_sync(0xffffffffu, le) >> gshift) & 0xFFu;
+        const unsigned bits = (__ballot_sync(0xffffffffu, le) >> gshift) & kMask;
         if (go) {
             const int k = __popc(bits);
-            const double nlo = k > 0 ? lo + width * ((double)k / 9.0) : lo;
-            const double nhi = k < 8 ? lo + width * ((double)(k + 1) / 9.0) : hi;
+            const double nlo = k > 0 ? lo + width * ((double)k / (L + 1)) : lo;
+            const double nhi = k < L ? lo + width * ((double)(k + 1) / (L + 1)) : hi;
             if (nlo <= lo && nhi >= hi) active = false;
             else { lo = nlo; hi = nhi; }
         }
@@ -678,19 +693,8 @@ struct IvFF {
         const bool small = fabsf(a.hi) < 0x1p-44f;
         return ff{small ? copysignf(0x1p-44f, a.hi) : a.hi, small ? 0.f : a.lo};
     }
-    static PSVD_DEV S rcp0(V den) {
-        float r;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(den.hi));
-        return r;
-    }
-    // a / den from r0 ~ 1 / den: the quotient of the leading words and one correction from its residual
-    static PSVD_DEV V div(V a, V den, S r0) {
-        const float r = __fmul_rn(a.hi, r0);
-        const float res = __fadd_rn(__fmaf_rn(-r, den.lo, __fmaf_rn(-r, den.hi, a.hi)), a.lo);
-        const float r2 = __fmul_rn(res, r0);
-        const float h = __fadd_rn(r, r2);
-        return ff{h, __fsub_rn(r2, __fsub_rn(h, r))};
-    }
+    static PSVD_DEV S rcp0(V den) { return ff_rcp0(den); }
+    static PSVD_DEV V div(V a, V den, S r0) { return ff_div(a, den, r0); }
     static PSVD_DEV V inv(V den, S r0) { return div(ff{1.f, 0.f}, den, r0); }
     // one flag in the last bit of a value
     static PSVD_DEV V flag(V v, bool f) {
@@ -1394,22 +1398,24 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
     // 2. eigenvalues
     double *tn = w.tn;
     {
-        dim3 g((n + 31) / 32, B);       // 32 eigenvalues x 8 lanes per block
+        const int L = section_lanes((long long)B * n);
+        const dim3 g((n + 256 / L - 1) / (256 / L), B);         // 256 / L eigenvalues per block
         const size_t smem = sizeof(float) * 2 * (size_t)n;
-        PSVD_TRY(cudaFuncSetAttribute(tri_bisect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        tri_bisect_kernel<<<g, 256, smem, st>>>(w.d, w.e, n, w.lam, tn);
-        PSVD_TRY(cudaGetLastError());
-        count_launch(1);
-    }
-    {
-        float4 *dd = w.sturm;
         const int rows = iv_rows(n);
-        sturm_prep_kernel<<<dim3((std::max(n, rows) + 255) / 256, B), 256, 0, st>>>(w.d, w.e, tn, n, rows, dd, w.tabf,
-                                                                                   w.tabd);
-        dim3 g((n + 31) / 32, B);       // 32 eigenvalues x 8 lanes per block
-        tri_refine_kernel<<<g, 256, 0, st>>>(dd, n, tn, kRefineNear, w.lam);
-        PSVD_TRY(cudaGetLastError());
-        count_launch(2);
+        auto run = [&](auto lanes) -> cudaError_t {
+            constexpr int kL = decltype(lanes)::value;
+            cudaError_t e = cudaFuncSetAttribute(tri_bisect_kernel<kL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            tri_bisect_kernel<kL><<<g, 256, smem, st>>>(w.d, w.e, n, w.lam, tn);
+            sturm_prep_kernel<<<dim3((std::max(n, rows) + 255) / 256, B), 256, 0, st>>>(w.d, w.e, tn, n, rows, w.sturm,
+                                                                                       w.tabf, w.tabd);
+            tri_refine_kernel<kL><<<g, 256, 0, st>>>(w.sturm, n, tn, kRefineNear, w.lam);
+            return cudaGetLastError();
+        };
+        PSVD_TRY(L == 2 ? run(std::integral_constant<int, 2>{}) : L == 4 ? run(std::integral_constant<int, 4>{})
+                 : L == 8 ? run(std::integral_constant<int, 8>{}) : L == 16 ? run(std::integral_constant<int, 16>{})
+                 : run(std::integral_constant<int, 32>{}));
+        count_launch(3);
     }
     // keep the eigenvalues for cluster detection
     double *bis = reinterpret_cast<double *>(w.S);   // B*n doubles (S holds B*n*kWY floats)

@@ -74,3 +74,21 @@ def test_inverse_iteration_halves(n, gap):
         lam = lam + gap * (torch.arange(n, dtype=torch.float64) % 2)
     h = (q * lam) @ q.T
     _check(torch.stack([h, -3.0 * h]).float().cuda())
+
+
+@pytest.mark.parametrize("batch,n", [(1, 255), (10, 511), (20, 500), (37, 512), (75, 512), (150, 520)])
+def test_multisection_lanes(batch, n):
+    # 32, 16, 8, 4 and 2 lanes per eigenvalue, blocks with a remainder, eigenvalues apart and in pairs (refined)
+    g = torch.Generator()
+    g.manual_seed(n)
+    q = torch.linalg.qr(torch.randn(n, n, generator=g, dtype=torch.float64))[0]
+    lam = torch.linspace(1.0, -1.0, n, dtype=torch.float64)
+    pairs = lam[::2].repeat_interleave(2)[:n] + 1e-7 * (torch.arange(n, dtype=torch.float64) % 2)
+    h = torch.stack([(q * lam) @ q.T, (q * pairs) @ q.T]).float().cuda()
+    h = h.repeat((batch + 1) // 2, 1, 1)[:batch].contiguous()
+    _check(h)
+    import paper_2609_32505_gb300 as P
+    s = P.eigh(h)[0].double()
+    for b in range(min(2, batch)):
+        w = torch.linalg.eigvalsh(h[b].double()).flip(-1)
+        assert (s[b::2] - w).abs().max() <= 2e-6 * max(1.0, n ** 0.5 / 8)
