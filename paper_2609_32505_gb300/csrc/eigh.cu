@@ -1044,17 +1044,22 @@ __global__ void zt_store_kernel(const float *xs, long long stride, int n, int fi
 static_assert(kWY % 32 == 0 && (kWY & (kWY - 1)) == 0 && kWY / 32 <= 8, "larft halving assumes 32 x 2^j reflectors");
 constexpr int kLtLd = kWY + 1;                  // padded row stride of G and T in shared memory
 constexpr size_t kLtSmem = sizeof(float) * ((size_t)2 * kWY * kLtLd + (kWY / 2) * (kWY / 2) + kWY);
-__global__ void __launch_bounds__(256) larft_kernel(const float *Gm, const float *tau, int n, int nrefl, int nblk,
-                                                    int blk0, float *Tm) {
+__global__ void __launch_bounds__(256) larft_kernel(const float *Gm, int ks, long long gbs, const float *tau,
+                                                    int n, int nrefl, int nblk, int blk0, float *Tm) {
     extern __shared__ float sm2[];
     float *G = sm2, *T = G + kWY * kLtLd, *W = T + kWY * kLtLd, *ts = W + (kWY / 2) * (kWY / 2);
     const int blk = blk0 + blockIdx.x, b = blockIdx.y;
     const int k0 = blk * kWY;
     const int nb = min(kWY, nrefl - k0);
-    const float *Gb = Gm + ((long long)b * nblk + blk) * kWY * kWY;
+    // G of block blk0 + x: matrix x of Gm + b gbs, the sum of ks K-split slices
+    const float *Gb = Gm + b * gbs + (long long)blockIdx.x * kWY * kWY;
+    const long long gs = gridDim.y * gbs;
     for (int p = threadIdx.x; p < kWY * kWY; p += blockDim.x) {
         const int r = p / kWY, c = p % kWY;
-        G[r * kLtLd + c] = r < nb && c < nb ? Gb[p] : 0.f;
+        float g = 0.f;
+        if (r < nb && c < nb)
+            for (int k = 0; k < ks; ++k) g += Gb[k * gs + p];
+        G[r * kLtLd + c] = g;
         T[r * kLtLd + c] = 0.f;
     }
     for (int c = threadIdx.x; c < kWY; c += blockDim.x) ts[c] = c < nb ? tau[(long long)b * n + k0 + c] : 0.f;
@@ -1102,10 +1107,10 @@ __global__ void __launch_bounds__(256) larft_kernel(const float *Gm, const float
 }
 
 // T of blocks blk0 .. blk0 + count - 1 (of nblk per matrix) of nrefl reflectors, tau with stride n.
-int larft_blocks(const float *Gm, const float *tau, int n, int nrefl, int nblk, int blk0, int count, int B, float *Tm,
-                 cudaStream_t st) {
+int larft_blocks(const float *Gm, int ks, long long gbs, const float *tau, int n, int nrefl, int nblk, int blk0,
+                 int count, int B, float *Tm, cudaStream_t st) {
     PSVD_TRY(cudaFuncSetAttribute(larft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLtSmem));
-    larft_kernel<<<dim3(count, B), 256, kLtSmem, st>>>(Gm, tau, n, nrefl, nblk, blk0, Tm);
+    larft_kernel<<<dim3(count, B), 256, kLtSmem, st>>>(Gm, ks, gbs, tau, n, nrefl, nblk, blk0, Tm);
     count_launch(1);
     PSVD_TRY(cudaGetLastError());
     return PSVD_OK;
@@ -1458,7 +1463,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
             const F16Views f{vh, vl, vh, vl};
             PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, w.nblk, e, st, &f));
         }
-        PSVD_TRY_RC(larft_blocks(w.Gm, w.tau, n, n - 2, w.nblk, 0, w.nblk, B, w.Tm, st));
+        PSVD_TRY_RC(larft_blocks(w.Gm, 1, (long long)w.nblk * kWY * kWY, w.tau, n, n - 2, w.nblk, 0, w.nblk, B, w.Tm, st));
         PSVD_TRY(cudaFuncSetAttribute(s_times_tt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStSmem));
         // The blocks are applied in pairs (s_pair_kernel): one V^T Y product of width 2 kWY and
         // one update with K = 2 kWY per pair halve the read-modify-write passes over V^T.

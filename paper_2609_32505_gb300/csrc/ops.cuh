@@ -18,8 +18,8 @@ __host__ __device__ inline int l1_slabs(int m) { return m < 1 ? 1 : (m + kL1Rows
 
 constexpr int kWY = 128;   // reflectors per compact-WY block (back-transform, QR's trailing updates)
 // T (upper triangular, kWY x kWY) of compact-WY blocks from G = Y^T Y and tau (eigh.cu).
-int larft_blocks(const float *Gm, const float *tau, int n, int nrefl, int nblk, int blk0, int count, int B, float *Tm,
-                 cudaStream_t st);
+int larft_blocks(const float *Gm, int ks, long long gbs, const float *tau, int n, int nrefl, int nblk, int blk0,
+                 int count, int B, float *Tm, cudaStream_t st);
 
 // Output format of an operand-preparation pass.
 struct SplitOut {
@@ -140,53 +140,8 @@ struct EpiStore {
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 
-// In place: X[r][c] -= acc for a matrix kept split in TF32 hi/lo halves (the QR's trailing updates).
-struct EpiSubSplit {
-    int rows, cols;
-    float *hi, *lo;
-    long long ld, bs;
-    struct Acc {};
-    static constexpr bool kElem = true, kRow = true;
-    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
-        if (r0 >= rows || c0 >= cols) return true;
-        if (c0 + 16 > cols || (((uintptr_t)hi | (uintptr_t)lo) & 31) || ((ld | bs) & 7)) return false;
-        if (r0 + lane >= rows) return true;
-        const long long o = b * bs + (long long)(r0 + lane) * ld + c0;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            uint32_t h[8], l[8];
-            ld_v8(hi + o + 8 * q, h);
-            ld_v8(lo + o + 8 * q, l);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                float a, c;
-                split_tf32((__uint_as_float(h[i]) + __uint_as_float(l[i])) - v[8 * q + i], a, c);
-                h[i] = __float_as_uint(a);
-                l[i] = __float_as_uint(c);
-            }
-            st_v8(hi + o + 8 * q, h);
-            st_v8(lo + o + 8 * q, l);
-        }
-        return true;
-    }
-    PSVD_DEV bool staged() const { return true; }
-    PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
-        if (r >= rows || c >= cols) return;
-        const long long o = b * bs + (long long)r * ld + c;
-        float h, l;
-        split_tf32((hi[o] + lo[o]) - v, h, l);
-        hi[o] = h;
-        lo[o] = l;
-    }
-    PSVD_DEV void begin(Acc &) const {}
-    PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) elem(a, b, r, c0 + i, v[i]);
-    }
-    PSVD_DEV void finish(Acc &, int, int, int) const {}
-};
-
-// The same for a matrix kept split in FP16 halves of x * scale (the eigensolver's back-transform).
+// In place: X[r][c] -= acc for a matrix kept as FP16 halves of x * scale (the eigensolver's back-transform,
+// the QR's trailing updates).
 struct EpiSubHalf {
     int rows, cols;
     __half *hi, *lo;
@@ -305,6 +260,8 @@ struct EpiHalf {
     PSVD_DEV bool staged() const { return false; }
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
+
+int orth_product(Carver &cv, const float *Q, const float *X, float *out, int B, int M, int N, cudaStream_t st);
 
 inline EpiStore epi_store_plain(float *out, long long ld, long long bs, int rows, int cols) {
     EpiStore e;

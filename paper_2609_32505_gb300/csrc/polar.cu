@@ -844,7 +844,7 @@ struct PolarPreqr {
         QrWS qw;
         qw.carve(q, (int)B, (int)m, (int)n);
         const long long ld = pad_ld(n);
-        const size_t ops = (size_t)(2 * B * m * ld + 2 * B * n * ld) * sizeof(float) + 1024;
+        const size_t ops = (size_t)(2 * B * m * ld + 2 * B * n * ld) * sizeof(__half) + 2048;
         need = head + std::max(std::max(q.used + 256, polar_direct_bytes(B, n, n, o)), ops);
         rest = ws ? static_cast<char *>(ws) + head : nullptr;
         rest_bytes = ws_bytes > head ? ws_bytes - head : 0;
@@ -900,26 +900,8 @@ extern "C" int psvd_polar_fwd(const float *A, float *W, float *H, int64_t batch,
         if (cv.overflow) return PSVD_ERR_WORKSPACE;
         PSVD_TRY_RC(polar_forward(l.R, l.WR, H, H != nullptr, w, o, info, st));
     }
-    // W = Q W_R: B operand B[k][j] = W_R[j][k] (W_R transposed)
     Carver cv(l.rest, l.rest_bytes);
-    const long long ld = pad_ld(N);
-    float *qhi = cv.take<float>((size_t)B * M * ld), *qlo = cv.take<float>((size_t)B * M * ld);
-    float *whi = cv.take<float>((size_t)B * N * ld), *wlo = cv.take<float>((size_t)B * N * ld);
-    unsigned *err = cv.take<unsigned>(4);
-    if (cv.overflow) return PSVD_ERR_WORKSPACE;
-    SplitOut a, bt;
-    a.hi = qhi; a.lo = qlo; a.ld = ld; a.bstride = (long long)M * ld;
-    bt.hi = whi; bt.lo = wlo; bt.ld = ld; bt.bstride = (long long)N * ld;
-    PSVD_TRY(prepare_operand(l.Q, N, (long long)M * N, B, M, N, false, 1.f, nullptr, a, st));
-    PSVD_TRY(prepare_operand(l.WR, N, (long long)N * N, B, N, N, true, 1.f, nullptr, bt, st));
-    MatView ah = view_of(qhi, M, N, ld, (long long)M * ld, B), al = view_of(qlo, M, N, ld, (long long)M * ld, B);
-    MatView bh = view_of(whi, N, N, ld, (long long)N * ld, B), bl = view_of(wlo, N, N, ld, (long long)N * ld, B);
-    GemmShape s;
-    memset(&s, 0, sizeof(s));
-    s.M = M; s.N = N; s.K = N; s.prec_uniform = PREC_TF32X3; s.err = err;
-    EpiStore e = epi_store_plain(W, N, (long long)M * N, M, N);
-    PSVD_TRY(launch_gemm(nullptr, nullptr, &ah, &al, &bh, &bl, s, B, e, st));
-    return PSVD_OK;
+    return orth_product(cv, l.Q, l.WR, W, B, M, N, st);     // W = Q W_R
 }
 
 // ------------------------------------------------------------ allocation-free variant

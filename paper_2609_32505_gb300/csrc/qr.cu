@@ -592,7 +592,7 @@ static int qr_apply_panel(QrWS &w, int j0, int pw, int panel, int c0, int ncol, 
 // T of the block of ws <= kWY columns from j0 on.
 static int qr_block_t(QrWS &w, int j0, int ws, int sup, cudaStream_t st) {
     const int B = w.B, K = w.m - j0;
-    const long long nm = (long long)w.n * w.ldm, ts = (long long)w.nsup * kWY * kWY;
+    const long long nm = (long long)w.n * w.ldm, gbs = (long long)w.n * kWY;
     F16Views f;
     f.ah = f.bh = view_f16(w.YThi + (long long)j0 * w.ldm + j0, ws, K, w.ldm, nm, B);
     f.al = f.bl = view_f16(w.YTlo + (long long)j0 * w.ldm + j0, ws, K, w.ldm, nm, B);
@@ -600,9 +600,11 @@ static int qr_block_t(QrWS &w, int j0, int ws, int sup, cudaStream_t st) {
     memset(&s, 0, sizeof(s));
     s.M = ws; s.N = ws; s.K = K; s.prec_uniform = PREC_F16X3; s.skip = w.skip; s.err = w.err;
     s.f16_scale = 1.f / (kF16V * kF16V);
-    EpiStore e = epi_store_plain(w.Gs + (long long)sup * kWY * kWY, kWY, ts, ws, ws);
+    // one tile with all of K: split (4 matrices of 14336 rows 185 -> 29 us, and 38 -> 64 in the T kernel that adds the slices)
+    s.ksplit = std::max(1, std::min(kQrSplit, (K + 255) / 256));
+    EpiStore e = epi_store_plain(w.Sp, kWY, gbs, ws, ws);
     PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
-    return larft_blocks(w.Gs, w.tau, w.n, w.n, w.nsup, sup, 1, B, w.Ts, st);
+    return larft_blocks(w.Sp, s.ksplit, gbs, w.tau, w.n, w.n, w.nsup, sup, 1, B, w.Ts, st);
 }
 
 // The reflectors of a whole block on rows c0 .. c0 + ncol - 1 of X^T: trans = 0 in the factorization

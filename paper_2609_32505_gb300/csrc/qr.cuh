@@ -24,8 +24,8 @@ struct QrWS {
     float *Tm = nullptr;                       // [B][npan][nb][nb] compact-WY T of every panel
     float *Wp = nullptr;                       // [ks][B][nb][n] partial Y^T X of a panel (K split)
     __half *W2hi = nullptr, *W2lo = nullptr;   // [B][n][kWY] (op(T) Y^T X)^T (kF16S2)
-    float *Gs = nullptr, *Ts = nullptr;        // [B][nsup][kWY][kWY] Y^T Y and T of blocks of kWY columns
-    float *Sp = nullptr;                       // [kQrSplit][B][n][kWY] partial X^T Y of a block
+    float *Ts = nullptr;                       // [B][nsup][kWY][kWY] T of blocks of kWY columns
+    float *Sp = nullptr;                       // [kQrSplit][B][n][kWY] partial X^T Y, or Y^T Y, of a block
     unsigned *amax = nullptr;                  // [B] max |A| (float bits)
     float *scale = nullptr;                    // [B] 2^e
     int *skip = nullptr;                       // [B] 1 = matrix not factored (flag[b] == 0)
@@ -48,7 +48,6 @@ struct QrWS {
         Tm = cv.template take<float>(B64 * npan * nb * nb);
         Wp = cv.template take<float>((long long)ks * B64 * nb * std::min(n, kWY));
         W2hi = cv.template take<__half>(B64 * n * kWY); W2lo = cv.template take<__half>(B64 * n * kWY);
-        Gs = cv.template take<float>(B64 * nsup * kWY * kWY);
         Ts = cv.template take<float>(B64 * nsup * kWY * kWY);
         Sp = cv.template take<float>((long long)kQrSplit * B64 * n * kWY);
         amax = cv.template take<unsigned>(B64);

@@ -543,20 +543,16 @@ static int num_sms_svd() {
 }
 
 template <class Epi>
-static int gemm3(const float *ahi, const float *alo, int M, int K, long long lda, long long bsa, const float *bhi,
-                 const float *blo, int N, long long ldb, long long bsb, int B, int prec, const Epi &e, unsigned *err,
-                 cudaStream_t st) {
-    MatView vah = view_of(ahi, M, K, lda, bsa, B), val = view_of(alo ? alo : ahi, M, K, lda, bsa, B);
-    MatView vbh = view_of(bhi, N, K, ldb, bsb, B), vbl = view_of(blo ? blo : bhi, N, K, ldb, bsb, B);
+static int gemm1(const float *a, int M, int K, long long lda, long long bsa, const float *b, int N, long long ldb,
+                 long long bsb, int B, const Epi &e, unsigned *err, cudaStream_t st) {
+    MatView va = view_of(a, M, K, lda, bsa, B), vb = view_of(b, N, K, ldb, bsb, B);
     GemmShape s;
     memset(&s, 0, sizeof(s));
-    s.M = M; s.N = N; s.K = K; s.prec_uniform = prec; s.err = err;
-    cudaError_t r = prec == PREC_TF32X3 ? launch_gemm(nullptr, nullptr, &vah, &val, &vbh, &vbl, s, B, e, st)
-                                        : launch_gemm(nullptr, nullptr, &vah, nullptr, &vbh, nullptr, s, B, e, st);
-    return r == cudaSuccess ? PSVD_OK : PSVD_ERR_CUDA;
+    s.M = M; s.N = N; s.K = K; s.prec_uniform = PREC_TF32; s.err = err;
+    return launch_gemm(nullptr, nullptr, &va, nullptr, &vb, nullptr, s, B, e, st) == cudaSuccess ? PSVD_OK : PSVD_ERR_CUDA;
 }
 
-// As gemm3, with the precision of each matrix read on the device from prec[B] (TF32 or
+// The same with the precision of each matrix read on the device from prec[B] (TF32 or
 // split-TF32; both operand splits supplied).
 template <class Epi>
 static int gemm3p(const float *ahi, const float *alo, int M, int K, long long lda, long long bsa, const float *bhi,
@@ -610,12 +606,12 @@ int svd_forward(const float *A, float *U, float *Sout, float *VT, SvdWS &w, cons
         count_launch(3);
         // X^2 = X X   (B operand B[j][k] = X[k][j] = -X[j][k])
         EpiStore e3 = epi_store_plain(w.X2, n, (long long)n * n, n, n);
-        if (int rc = gemm3(w.X, nullptr, n, n, ld, nn, w.Xneg, nullptr, n, ld, nn, B, PREC_TF32, e3, p.err, st)) return rc;
+        if (int rc = gemm1(w.X, n, n, ld, nn, w.Xneg, n, ld, nn, B, e3, p.err, st)) return rc;
         // X^4 = X^2 X^2 (X^2 symmetric), kept in T1
         x2_split_kernel<<<g16, b16, 0, st>>>(w.X2, n, ld, w.T1hi);
         count_launch(1);
         EpiStore e3b = epi_store_plain(w.T1, n, (long long)n * n, n, n);
-        if (int rc = gemm3(w.T1hi, nullptr, n, n, ld, nn, w.T1hi, nullptr, n, ld, nn, B, PREC_TF32, e3b, p.err, st)) return rc;
+        if (int rc = gemm1(w.T1hi, n, n, ld, nn, w.T1hi, n, ld, nn, B, e3b, p.err, st)) return rc;
         corr_h_kernel<<<g16, b16, 0, st>>>(w.X2, w.T1, n, ld, w.F);                 // h in F
         count_launch(1);
         // X V^T (split-TF32, into T1) and h V^T (TF32, into Kt); B operand B[j][k] = V^T[k][j] = V[j][k]
@@ -623,7 +619,7 @@ int svd_forward(const float *A, float *U, float *Sout, float *VT, SvdWS &w, cons
         EpiStore e4 = epi_store_plain(w.T1, n, (long long)n * n, n, n);
         if (int rc = gemm3p(w.X, w.Ft, n, n, ld, nn, w.Vhi, w.Vlo, n, ld, nn, B, w.cprec + B, e4, p.err, st)) return rc;
         EpiStore e5 = epi_store_plain(w.Kt, n, (long long)n * n, n, n);
-        if (int rc = gemm3(w.F, nullptr, n, n, ld, nn, w.Vhi, nullptr, n, ld, nn, B, PREC_TF32, e5, p.err, st)) return rc;
+        if (int rc = gemm1(w.F, n, n, ld, nn, w.Vhi, n, ld, nn, B, e5, p.err, st)) return rc;
         add_split_kernel<<<g16, b16, 0, st>>>(vthi, vtlo, w.T1, w.Kt, n, ld, VEt_hi, VEt_lo, VT);
         count_launch(1);
         bu_hi = VEt_hi;
@@ -848,7 +844,7 @@ struct PreqrLayout {
         QrWS qw;
         qw.carve(q, (int)B, (int)m, (int)n);
         const long long ld = pad_ld(n);
-        const size_t ops = (size_t)(2 * B * m * ld + 2 * B * n * ld) * sizeof(float) + 1024;
+        const size_t ops = (size_t)(2 * B * m * ld + 2 * B * n * ld) * sizeof(__half) + 2048;
         const size_t region = std::max(std::max(q.used + 256, svd_direct_bytes(B, n, n, sq)), ops);
         need = head + region;
         rest = ws ? static_cast<char *>(ws) + head : nullptr;
@@ -905,20 +901,6 @@ extern "C" int psvd_svd_fwd(const float *A, float *U, float *S, float *VT, int64
         PSVD_TRY_RC(qr_factor(A, l.Q, l.R, nullptr, qw, st));
     }
     PSVD_TRY_RC(svd_direct(l.R, l.UR, S, VT, B, N, N, sq, l.rest, l.rest_bytes, info, st));
-    // U = Q U_R: B operand B[k][j] = U_R[j][k] (U_R transposed)
     Carver cv(l.rest, l.rest_bytes);
-    const long long ld = pad_ld(N);
-    float *qhi = cv.take<float>((size_t)B * M * ld), *qlo = cv.take<float>((size_t)B * M * ld);
-    float *uhi = cv.take<float>((size_t)B * N * ld), *ulo = cv.take<float>((size_t)B * N * ld);
-    if (cv.overflow) return PSVD_ERR_WORKSPACE;
-    SplitOut a, bt;
-    a.hi = qhi; a.lo = qlo; a.ld = ld; a.bstride = (long long)M * ld;
-    bt.hi = uhi; bt.lo = ulo; bt.ld = ld; bt.bstride = (long long)N * ld;
-    PSVD_TRY(prepare_operand(l.Q, N, (long long)M * N, B, M, N, false, 1.f, nullptr, a, st));
-    PSVD_TRY(prepare_operand(l.UR, N, (long long)N * N, B, N, N, true, 1.f, nullptr, bt, st));
-    unsigned *err = reinterpret_cast<unsigned *>(cv.take<unsigned>(4));
-    if (cv.overflow) return PSVD_ERR_WORKSPACE;
-    EpiStore e = epi_store_plain(U, N, (long long)M * N, M, N);
-    return gemm3(qhi, qlo, M, N, ld, (long long)M * ld, uhi, ulo, N, ld, (long long)N * ld, B, PREC_TF32X3, e, err,
-                 st);
+    return orth_product(cv, l.Q, l.UR, U, B, M, N, st);     // U = Q U_R
 }
