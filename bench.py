@@ -3,8 +3,8 @@ geometric spectrum, the square-matrix setting of Section 4.1 / Tables 1-2), FP32
 
 One step = psvd_svd_fwd (Algorithm 1) + psvd_svd_bwd (Algorithm 4, eps = 1e-8) of the
 loss <G_U, U> + <g_S, sigma> + <G_V, V> with seeded N(0,1) weights.  The headline
-`value` is the mixed-precision path (BF16 -> TF32 -> split-TF32 polish, eigenbasis
-correction); the plain FP32-accurate path (split-TF32 throughout) is timed beside it.
+`value` is the mixed-precision path (BF16 -> TF32 -> split-FP16 polish, eigenbasis
+correction); the plain FP32-accurate path (split FP16 throughout) is timed beside it.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -33,10 +33,6 @@ N = 4096
 KAPPA = 10.0
 EPS = 1e-8
 METRIC = "SVD fwd+bwd ms at 4096^2, f32-accurate: mixed vs plain path; % tensor-core peak"
-# DRAM bytes (read + written) of one sytrd_kernel launch at n = 4096, from an ncu capture of
-# the current kernel (dram__bytes.sum.per_second x gpu__time_duration.sum = 148.13 GB/s x
-# 39.116 ms); valid while the kernel is unchanged
-TRD_DRAM_BYTES = 5794092046
 WORKLOAD = (f"SVD fwd+bwd of one {N}x{N} fp32 matrix A = Q1 diag(s) Q2^T, s_i = {KAPPA:g}^((n-i)/(n-1)), "
             f"eps=1e-8, kreg Algorithm 4")
 
@@ -339,10 +335,8 @@ def main():
     def cls(arr, c):
         return {"launches": int(arr[4 * c]), "ms": arr[4 * c + 1], "work": arr[4 * c + 2], "max_ms": arr[4 * c + 3]}
 
-    hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     bf16_burst = float(peaks.get("bf16_tflops", 1900.0))
     bf16_peak = float(peaks.get("bf16_tflops_sustained", bf16_burst))
-    tf32_peak = bf16_peak * (1.1 / 2.25)
     l2_gbs = l2_rmw_gbs(dev)
     trd = cls(prof_m, 4)
     trd_gbs = trd["work"] / (trd["ms"] * 1e-3) / 1e9 if trd["ms"] > 0 else 0.0
@@ -353,7 +347,7 @@ def main():
     st = [info_m["steps_bf16"], info_m["steps_tf32"], info_m["steps_3xtf32"]]
 
     def weighted(bf16):
-        pk = [bf16, bf16 * 1.1 / 2.25, bf16 * 1.1 / 2.25 / 3.0]
+        pk = [bf16, bf16 * 1.1 / 2.25, bf16 / 3.0]
         return sum(st) / sum(k / p for k, p in zip(st, pk)) if sum(st) else bf16
 
     # Algorithmic flops of the chain from the steps the matrix actually took: K steps of a
@@ -363,26 +357,29 @@ def main():
     k_steps = sum(st)
     chain_flops = (k_steps + 1) * N * (N + 1) * N + k_steps * 2.0 * N * N * N
     chain_tf = chain_flops / (mix["ms"] * 1e-3) / 1e12 if mix["ms"] > 0 else 0.0
-    roofline = {"bound": "l2", "achieved": trd_gbs, "peak": l2_gbs, "unit": "GB/s", "frac": trd_gbs / l2_gbs,
-                "traffic": TRD_DRAM_BYTES if N == 4096 else None,
-                "kernel": "sytrd_kernel (Householder tridiagonalization of H, eigensolver stage 1; one launch)",
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    smem_gbs = sms * 128 * 2.07                        # shared-memory port, 128 B per clock and SM at 2.07 GHz
+    roofline = {"bound": "on-chip", "achieved": trd_gbs, "peak": smem_gbs, "unit": "GB/s", "frac": trd_gbs / smem_gbs,
+                "traffic": None,
+                "kernel": "trd_chip_kernel (Householder tridiagonalization of H, eigensolver stage 1; all its launches)",
                 "algorithmic_bytes": trd["work"], "ms": trd["ms"], "share_of_step": trd["ms"] / ms_mixed,
-                "peak_src": "measured in this run: read-modify-write of a 48 MB L2-resident buffer",
-                "note": (f"every step reads and writes the trailing matrix, 8 sum (n-k-2)^2 bytes, served from "
-                         f"L2 (DRAM sees the traffic above); against the measured HBM copy ({hbm_peak:.0f} GB/s) "
-                         f"that is {trd_gbs / hbm_peak:.2f}; in flops (4/3 n^3) "
-                         f"{trd_flops / (trd['ms'] * 1e-3) / 1e12 if trd['ms'] > 0 else 0:.2f} TFLOP/s; the "
-                         f"kernel waits on one grid barrier per reflector"),
+                "peak_src": "SMs x 128 B/clock x 2.07 GHz (shared memory)",
+                "l2_peak": l2_gbs,
+                "note": (f"every step reads and writes the trailing matrix, 8 sum (n-k-2)^2 bytes, held in the SMs' "
+                         f"registers, shared and tensor memory; streamed through L2 the measured read-modify-write "
+                         f"peak would be {l2_gbs:.0f} GB/s; in flops (4/3 n^3) "
+                         f"{trd_flops / (trd['ms'] * 1e-3) / 1e12 if trd['ms'] > 0 else 0:.2f} TFLOP/s; one exchange "
+                         f"between all SMs per reflector (~1.5 us) is the other half of the time"),
                 "polar_chain": {"bound": "tensor", "achieved": chain_tf, "unit": "TFLOP/s",
                                 "peak_sustained": weighted(bf16_peak), "frac_sustained": chain_tf / weighted(bf16_peak),
                                 "peak_burst": weighted(bf16_burst), "frac_burst": chain_tf / weighted(bf16_burst),
                                 "steps": st, "launches": mix["launches"], "ms": mix["ms"],
                                 "peak_src": f"{peak_src} bf16 {bf16_burst:.0f} burst / {bf16_peak:.0f} sustained, "
-                                            f"TF32 x1.1/2.25, split-TF32 /3, weighted by the steps taken"}}
+                                            f"TF32 x1.1/2.25, split FP16 /3, weighted by the steps taken"}}
     x3 = cls(prof_p, 2)
     plain_tf = x3["work"] / (x3["ms"] * 1e-3) / 1e12 if x3["ms"] > 0 else 0.0
-    tensor = {"split_tf32_all_plain": {"achieved": plain_tf, "peak": tf32_peak / 3.0, "unit": "TFLOP/s",
-                                       "frac": plain_tf / (tf32_peak / 3.0), "launches": x3["launches"],
+    tensor = {"split_all_plain": {"achieved": plain_tf, "peak": bf16_peak / 3.0, "unit": "TFLOP/s",
+                                       "frac": plain_tf / (bf16_peak / 3.0), "launches": x3["launches"],
                                        "ms": x3["ms"]},
               "product_kernel_ms_share_mixed": sum(cls(prof_m, c)["ms"] for c in range(4)) / ms_mixed}
 
@@ -538,8 +535,8 @@ def main():
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
                 "config": {"workload": WORKLOAD,
                            "path": "mixed: learned lower bound (sketch + MLP kernels) -> greedy cubics, TF32 steps "
-                                   "-> split-TF32 polish, eigenbasis correction; plain: conservative CANS "
-                                   "(delta=0.99), split-TF32 throughout",
+                                   "-> split-FP16 polish, eigenbasis correction; plain: conservative CANS "
+                                   "(delta=0.99), split FP16 throughout",
                            "schedule_mixed": sched_m,
                            "bf16_ladder": bf16_report,
                            "plain_ms": ms_plain, "speedup_mixed_vs_plain": ms_plain / ms_mixed,

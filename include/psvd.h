@@ -50,11 +50,12 @@ extern "C" {
 #define PSVD_ERR_UNSUPPORTED   -6   /* device is not sm_103 / sm_100 class            */
 
 /* ---- options ----------------------------------------------------------- */
-#define PSVD_PREC_FP32       0   /* every product FP32-accurate (split hi+lo TF32, "3xTF32") */
-#define PSVD_PREC_MIXED      1   /* TF32 steps -> 3xTF32 polish, switched per matrix from the
+#define PSVD_PREC_FP32       0   /* every product FP32-accurate (operands split into FP16
+                                    halves hi + lo and scaled by powers of two, three products) */
+#define PSVD_PREC_MIXED      1   /* TF32 steps -> FP32-accurate polish, switched per matrix from the
                                     measured orthogonality residual; with the learned
-                                    schedule, bounds below PSVD_MIXED_LB_MIN start at 3xTF32 */
-#define PSVD_PREC_MIXED_BF16 2   /* BF16 early steps -> TF32 -> 3xTF32 polish; the BF16
+                                    schedule, bounds below PSVD_MIXED_LB_MIN start there */
+#define PSVD_PREC_MIXED_BF16 2   /* BF16 early steps -> TF32 -> the same polish; the BF16
                                     rounding leaves a rotation that the eigenbasis correction
                                     undoes only to first order (reconstruction ~1e-5 at
                                     n = 4096, kappa = 10)                                    */
@@ -136,7 +137,7 @@ typedef struct psvd_info {
 
 /* PSVD_PREC_MIXED with the learned schedule: a matrix whose lower bound (opts.lower_bound,
  * in units of X0 = M / sqrt(||M||_1 ||M||_inf)) is below PSVD_MIXED_LB_MIN starts on the
- * 3xTF32 rung.  TF32 steps at such small singular values leave corrections above
+ * FP32-accurate rung.  TF32 steps at such small singular values leave corrections above
  * PSVD_MIXED_CORR_MAX, and the matrix would be recomputed anyway (measured at n = 4096:
  * kappa = 1e2 keeps its TF32 result, kappa = 1e3 and above fall back).  steps_tf32 = 0
  * in psvd_info shows that the gate applied. */
@@ -302,9 +303,9 @@ int psvd_mlp_calibrate(const float *params, const float *F, const float *target,
 /* ---- QR (Appendix A.2's fallback; Section 4.1's preprocessing) ------------------
  * psvd_qr -- thin QR A = Q R of a batch of m x n matrices (m >= n), diag(R) >= 0, by blocked
  *   Householder: panels of 64 (or 32) columns factored by one thread-block cluster per
- *   matrix, trailing updates and the accumulation of Q in compact-WY form on the split-TF32
- *   tcgen05 product kernel.  A: batch x m x n (read); Q: batch x m x n out (may alias A);
- *   R: batch x n x n out, upper triangular (may be NULL).  m <= 23040. */
+ *   matrix, trailing updates and the accumulation of Q in compact-WY form on the tcgen05
+ *   product kernel (split FP16, the matrix scaled by a power of two).  A: batch x m x n (read); Q: batch x m x n out (may alias A);
+ *   R: batch x n x n out, upper triangular (may be NULL).  m <= 23024. */
 size_t psvd_qr_workspace_bytes(int64_t batch, int64_t m, int64_t n);
 int psvd_qr(const float *A, float *Q, float *R, int64_t batch, int64_t m, int64_t n, void *ws,
             size_t ws_bytes, void *stream);
@@ -347,7 +348,7 @@ int psvd_debug_set_barrier_spin(uint32_t polls);
  * pointer; synchronizes on the recorded events. */
 #define PSVD_PROF_BF16     0   /* product kernel, BF16 operands        */
 #define PSVD_PROF_TF32     1   /* product kernel, TF32 operands        */
-#define PSVD_PROF_TF32X3   2   /* product kernel, split-TF32 operands  */
+#define PSVD_PROF_TF32X3   2   /* product kernel, split operands (TF32 or FP16)  */
 #define PSVD_PROF_MIXED    3   /* product kernel, per-matrix precision */
 #define PSVD_PROF_TRD      4   /* tridiagonalization (eigh stage 1)    */
 #define PSVD_PROF_CLASSES  5

@@ -24,8 +24,8 @@
 //                 bytes (a 4096^3 polar step product: 780 us in split TF32, 474 us with the
 //                 same epilogue)
 // Two accumulators of 128 x 256 FP32 in TMEM (all 512 columns) let the MMA warp
-// run the next tile (or the next split-TF32 chunk) while the epilogue drains the
-// previous one.  The tensor core accumulates with truncation; split-TF32 tiles are
+// run the next tile (or the next k-block of a split one) while the epilogue drains the
+// previous one.  The tensor core accumulates with truncation; split tiles are
 // therefore flushed into round-to-nearest FP32 registers after every k-block.
 // Warp roles: warps 0-7 epilogue (warp w reads TMEM lanes 32 (w % 4) .. + 31 and
 // the column half w / 4), warp 8 TMA producer, warp 9 MMA issuer.  The precision is

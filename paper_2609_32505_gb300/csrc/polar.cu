@@ -4,9 +4,9 @@
 //   step k:  G_k = X_k^T X_k,  r_k = ||G_k - I||_F / sqrt(n)   (stop if r_k <= tol)
 //            P_k = c1_k I + c3_k G_k,  X_{k+1} = X_k P_k         (degree-3 CANS / NS step)
 //   H = (W^T M)_sym with W = X_final                           (FP64 averaging)
-// Each step is three launches: the Gram product (upper-triangle tiles, with the
-// polynomial and the residual fused in its epilogue), a per-matrix decision
-// kernel (stop / precision of the next step), and the apply product X_k P_k
+// Each step is two launches: the Gram product (upper-triangle tiles, with the
+// polynomial and the residual fused in its epilogue; its last CTA takes the per-matrix
+// decision, stop / precision of the next step), and the apply product X_k P_k
 // whose epilogue writes X_{k+1} both row-major and transposed in the precision
 // the next step uses.  Matrices that finished are skipped by every later CTA.
 #include <algorithm>

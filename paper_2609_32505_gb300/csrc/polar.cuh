@@ -12,7 +12,7 @@ namespace psvd {
 #define PSVD_TAU_TF32 2e-3
 #endif
 constexpr double kTauBF16 = PSVD_TAU_BF16;   // mixed path: leave BF16 once the residual is below this
-constexpr double kTauTF32 = PSVD_TAU_TF32;   // ... and TF32 once below this (3xTF32 polish afterwards)
+constexpr double kTauTF32 = PSVD_TAU_TF32;   // ... and TF32 once below this (split-FP16 polish afterwards)
 
 struct PolarWS {
     int B = 0, m = 0, n = 0, kcap = 0;

@@ -3,7 +3,7 @@
 //
 // The matrix is scaled by a power of two to columns of norm <= 1 and kept transposed and split into
 // FP16 hi/lo halves (UT: row j = column j).  Panels of nb columns are factored by one thread-block
-// cluster per matrix: each of the cl CTAs holds a slab of the panel's rows in shared memory, and the
+// cluster per matrix: each of its CTAs holds a slab of the panel's rows in registers, and the
 // per-column dot products (the norm below the diagonal and the projections of the later panel
 // columns) are summed across the cluster through distributed shared memory -- one cluster barrier
 // per column, where the unblocked kernel needed three grid barriers.
