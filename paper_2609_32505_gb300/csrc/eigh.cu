@@ -1199,8 +1199,8 @@ static_assert(kPrRows % 2 == 0, "two halves of the rows");
 constexpr size_t kPrSmem =
     sizeof(float) * (2 * (size_t)kWY * kPrLd + (size_t)kPrRows * 2 * kWY + (size_t)kPrRows * kWY);
 __global__ void __launch_bounds__(2 * kWY) s_pair_kernel(const float *S, int ks, int B, const float *Tm,
-                                                          const float *Gab, int n, int nblk, int npair, int blk_b,
-                                                          int q, int nb_a, __half *S2hi, __half *S2lo) {
+                                                          const float *Gab, int n, int nblk, int nbp, int blk_b,
+                                                          int nb_a, __half *S2hi, __half *S2lo) {
     extern __shared__ __align__(16) float psm[];
     float *Ta = psm, *Gt = Ta + kWY * kPrLd, *Tb = Ta;  // T_b is loaded over T_a after phase one
     float *sr = Gt + kWY * kPrLd;                     // [kPrRows][2 kWY]: S rows, then S_b in place
@@ -1233,7 +1233,7 @@ __global__ void __launch_bounds__(2 * kWY) s_pair_kernel(const float *S, int ks,
         }
     };
     stage(Tm + ((long long)b * nblk + blk_b + 1) * kWY * kWY, Ta, false);
-    stage(Gab + ((long long)b * npair + q) * kWY * kWY, Gt, true);
+    stage(Gab + ((long long)b * nbp + blk_b) * kWY * kWY, Gt, true);
     const long long slice = (long long)B * n * 2 * kWY;
 #pragma unroll
     for (int r = 0; r < kPrRows; ++r) {
@@ -1451,19 +1451,27 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
         vo.fscale = yo.fscale = kF16V;
         PSVD_TRY(prepare_operand(w.Vh, ldn, np, B, w.nrp, n, false, 1.f, nullptr, vo, st));
         PSVD_TRY(prepare_operand(w.Vh, ldn, np, B, n, n, true, 1.f, nullptr, yo, st));
-        // G = Y^T Y of every WY block: blocks of kWY Householder rows as a batch
-        for (int b = 0; b < B; ++b) {
-            MatView vh = view_f16(w.Vhi + b * np, kWY, n, ldn, (long long)kWY * ldn, w.nblk);
-            MatView vl = view_f16(w.Vlo + b * np, kWY, n, ldn, (long long)kWY * ldn, w.nblk);
+        // G = Y^T Y of every WY block: the blocks of kWY Householder rows of all matrices as one batch (the
+        // rows are padded to whole blocks, zero past the last reflector).  One launch per matrix
+        // took two thirds of the launches of 64 x 512.
+        const int nbp = w.nrp / kWY;
+        const long long bb = (long long)kWY * kWY;
+        auto block_product = [&](int shift, int count, float *out) -> cudaError_t {   // block i + shift times block i
+            const long long bs = (long long)kWY * ldn;
+            F16Views f;
+            f.ah = view_f16(w.Vhi + shift * bs, kWY, n, ldn, bs, count);
+            f.al = view_f16(w.Vlo + shift * bs, kWY, n, ldn, bs, count);
+            f.bh = view_f16(w.Vhi, kWY, n, ldn, bs, count);
+            f.bl = view_f16(w.Vlo, kWY, n, ldn, bs, count);
             GemmShape s;
             memset(&s, 0, sizeof(s));
             s.M = kWY; s.N = kWY; s.K = n; s.prec_uniform = PREC_F16X3; s.err = w.err;
-            EpiStore e = epi_store_plain(w.Gm + (long long)b * w.nblk * kWY * kWY, kWY, (long long)kWY * kWY, kWY, kWY);
             s.f16_scale = 1.f / (kF16V * kF16V);
-            const F16Views f{vh, vl, vh, vl};
-            PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, w.nblk, e, st, &f));
-        }
-        PSVD_TRY_RC(larft_blocks(w.Gm, 1, (long long)w.nblk * kWY * kWY, w.tau, n, n - 2, w.nblk, 0, w.nblk, B, w.Tm, st));
+            EpiStore e = epi_store_plain(out, kWY, bb, kWY, kWY);
+            return launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, count, e, st, &f);
+        };
+        PSVD_TRY(block_product(0, B * nbp, w.Gm));
+        PSVD_TRY_RC(larft_blocks(w.Gm, 1, nbp * bb, w.tau, n, n - 2, w.nblk, 0, w.nblk, B, w.Tm, st));
         PSVD_TRY(cudaFuncSetAttribute(s_times_tt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStSmem));
         // The blocks are applied in pairs (s_pair_kernel): one V^T Y product of width 2 kWY and
         // one update with K = 2 kWY per pair halve the read-modify-write passes over V^T.
@@ -1520,23 +1528,8 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
             return PSVD_OK;
         };
         if (npair > 0) {
-            // G_ab = Y_a^T Y_b of every pair (a = b + 1): Householder rows of the two blocks
-            for (int b = 0; b < B; ++b) {
-                const __half *hb = w.Vhi + b * np, *lb = w.Vlo + b * np;
-                const long long ps = (long long)2 * kWY * ldn;
-                MatView ah = view_f16(hb + (long long)(first + 1) * kWY * ldn, kWY, n, ldn, ps, npair);
-                MatView al = view_f16(lb + (long long)(first + 1) * kWY * ldn, kWY, n, ldn, ps, npair);
-                MatView bh = view_f16(hb + (long long)first * kWY * ldn, kWY, n, ldn, ps, npair);
-                MatView bl = view_f16(lb + (long long)first * kWY * ldn, kWY, n, ldn, ps, npair);
-                GemmShape s;
-                memset(&s, 0, sizeof(s));
-                s.M = kWY; s.N = kWY; s.K = n; s.prec_uniform = PREC_F16X3; s.err = w.err;
-                EpiStore e = epi_store_plain(w.Gab + (long long)b * npair * kWY * kWY, kWY, (long long)kWY * kWY,
-                                             kWY, kWY);
-                s.f16_scale = 1.f / (kF16V * kF16V);
-                const F16Views f{ah, al, bh, bl};
-                PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, npair, e, st, &f));
-            }
+            // G_ab = Y_a^T Y_b (a = b + 1) of all neighbouring blocks, of which the pairs use every other one
+            PSVD_TRY(block_product(1, B * nbp - 1, w.Gab));
             PSVD_TRY(cudaFuncSetAttribute(s_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPrSmem));
         }
         for (int q = npair - 1; q >= 0; --q) {
@@ -1565,7 +1558,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
                 PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
             }
             s_pair_kernel<<<dim3((n + kPrRows - 1) / kPrRows, B), 2 * kWY, kPrSmem, st>>>(
-                w.S, ks, B, w.Tm, w.Gab, n, w.nblk, npair, blk_b, q, nb_a, w.S2hi, w.S2lo);
+                w.S, ks, B, w.Tm, w.Gab, n, w.nblk, nbp, blk_b, nb_a, w.S2hi, w.S2lo);
             PSVD_TRY(cudaGetLastError());
             count_launch(1);
             // V^T[:, r0:] -= S2 [Y_b Y_a][r0:, :]^T

@@ -34,8 +34,8 @@ struct EighWS {
     double2 *tabd = nullptr;                   // the same in FP64
     double *tn = nullptr;                      // [B] ||T||
     float *Tm = nullptr;                       // [B][nblk][kWY][kWY]
-    float *Gm = nullptr;                       // [B][nblk][kWY][kWY]  Y^T Y per block
-    float *Gab = nullptr;                      // [B][nblk/2][kWY][kWY]  Y_a^T Y_b per pair of blocks
+    float *Gm = nullptr;                       // [B][nrp / kWY][kWY][kWY]  Y^T Y per block
+    float *Gab = nullptr;                      // the same for neighbouring blocks, Y_{a+1}^T Y_a
     double *xs = nullptr, *lm = nullptr, *u = nullptr;   // inverse-iteration vectors, multipliers, pivot rows
     float *xf = nullptr;                       // the normalized eigenvectors of T, interleaved [n][chunk]
     unsigned *err = nullptr;
@@ -76,8 +76,8 @@ struct EighWS {
         tabd = cv.template take<double2>(B64 * iv_rows(n) * 2);
         tn = cv.template take<double>(B64);
         Tm = cv.template take<float>(B64 * (nblk > 0 ? nblk : 1) * kWY * kWY);
-        Gm = cv.template take<float>(B64 * (nblk > 0 ? nblk : 1) * kWY * kWY);
-        Gab = cv.template take<float>(B64 * (nblk > 1 ? nblk / 2 : 1) * kWY * kWY);
+        Gm = cv.template take<float>(B64 * nrp * kWY);
+        Gab = cv.template take<float>(B64 * nrp * kWY);
         xf = cv.template take<float>((long long)n * chunk);
         const long long iv = (long long)(chunk / n) * ((n + 15) / 16) * iv_rows(n) * 32;   // 16 vectors per warp
         xs = cv.template take<double>(iv);
