@@ -83,9 +83,6 @@ struct GemmShape {
     const int *skip;        // [batch] nonzero = matrix finished, its tiles are skipped (or nullptr)
     const int *gate;        // nullptr, or a device counter: 0 = nothing left to do, the whole launch
                             // returns at once (written by an earlier kernel on the same stream)
-    int *over;              // nullptr, or the word of a chain of gated launches (zeroed before it) that the first one
-                            // to find its gate at 0 sets: all later ones return at once, without waiting for
-                            // their predecessors (a gate at 0 means that every later gate is)
     unsigned *ticket;       // nullptr, or a zeroed counter: the last CTA to finish runs epi.tail()
     unsigned *err;          // device error word
     float f16_scale;        // PREC_F16X3: the product of the operands' inverse scales ...
@@ -315,23 +312,15 @@ template <class Epi>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi epi) {
     // Launched ahead of its predecessor's end (programmatic dependent launch): let the next launch
-    // come, then wait until everything before this one has completed and is visible.
+    // come, then wait until everything before this one has completed and is visible.  Every thread of every
+    // launch waits, also of one with nothing to do: only then does the completion of a launch stand for that of
+    // all before it, which whatever follows relies on (a reset of the counters, a graph's next node, a reuse of
+    // the workspace).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // A launch of a chain that is over returns without waiting (thread 0 decides for its block: the word
-    // may be written meanwhile).
-    if (shp.over) {
-        __shared__ int s_over;
-        if (threadIdx.x == 0) s_over = *static_cast<volatile int *>(shp.over);
-        __syncthreads();
-        if (s_over) return;
-    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // A gated launch with nothing left to do returns before any allocation (uniform: every
-    // thread reads the same word, final since the kernel that wrote it has completed), and ends its chain.
-    if (shp.gate && *shp.gate == 0) {
-        if (shp.over && blockIdx.x == 0 && threadIdx.x == 0) *static_cast<volatile int *>(shp.over) = 1;
-        return;
-    }
+    // thread reads the same word, final since the kernel that wrote it has completed).
+    if (shp.gate && *shp.gate == 0) return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kRingBytes);

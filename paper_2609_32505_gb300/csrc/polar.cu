@@ -597,13 +597,11 @@ static int launch_step(PolarWS &w, StepPlans &plans, int k, bool apply, double t
                        const int *gram_gate, cudaStream_t st) {
     const int B = w.B, m = w.m, n = w.n;
     const int par = k & 1, npar = (k + 1) & 1;
-    int *over = w.notdone + w.kcap + 1;
     {
         GemmShape &s = plans.gram[par].shp;
         s.prec = w.prec + (long long)k * B;
         s.skip = w.done;
         s.gate = gram_gate;
-        s.over = over;
         s.ticket = w.ticket + k;
         s.err = w.err;
         EpiGram e;
@@ -622,7 +620,6 @@ static int launch_step(PolarWS &w, StepPlans &plans, int k, bool apply, double t
         s.prec = w.prec + (long long)k * B;
         s.skip = w.done;
         s.gate = w.notdone + k;          // matrices still iterating after this step's decision
-        s.over = over;
         s.err = w.err;
         EpiApply e;
         e.m = m; e.n = n; e.B = B;
@@ -637,9 +634,8 @@ static int launch_step(PolarWS &w, StepPlans &plans, int k, bool apply, double t
 
 // Launches steps 0..kmax (kmax <= kcap) with no host synchronization: the decision
 // of step k counts the matrices still iterating in notdone[k], and the launches after the
-// last matrix has finished find their gate at 0 and return at once; the first that does sets
-// notdone[kcap + 1], and those after it do not even wait for each other (w.notdone zeroed before
-// the pass).  `first_gate` gates the Gram launch of step 0 (nullptr: always run).
+// last matrix has finished find their gate at 0 and return at once.  `first_gate` gates
+// the Gram launch of step 0 (nullptr: always run).
 static int run_iteration(PolarWS &w, int kmax, double tol, bool learned, float *fres, const int *first_gate,
                          cudaStream_t st) {
     StepPlans plans;
