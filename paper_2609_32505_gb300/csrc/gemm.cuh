@@ -176,12 +176,12 @@ PSVD_DEV void st_v8x2(void *p, const uint32_t (&r)[16]) {       // 64 bytes
     st_v8(p, a);
     st_v8(static_cast<char *>(p) + 32, b);
 }
-// through the read-only path, free to be issued ahead of stores to other elements (each element is read
-// once, before its own thread writes it)
+// (an ordinary load: the in-place epilogues write what they read, which the read-only path does not allow)
 PSVD_DEV void ld_v8(const void *p, uint32_t (&r)[8]) {
-    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-        : "l"(p));
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "l"(p)
+                 : "memory");
 }
 // Lane l gives word w[i] of column i of its row; it gets the 16 words of rows 16 (l & 1) .. + 15 of
 // column l >> 1.

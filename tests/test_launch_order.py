@@ -28,6 +28,14 @@ def test_every_path_waits_for_the_launch_before():
     assert seen > 0
 
 
+def test_epilogues_do_not_read_through_the_read_only_path():
+    # the in-place epilogues of the product kernel overwrite what they read; the non-coherent path is only for
+    # memory that nothing writes while the kernel runs
+    for name in ("gemm.cuh", "ops.cuh"):
+        text = _code(os.path.join(CSRC, name))
+        assert "global.nc" not in text and "__ldg" not in text, name
+
+
 @pytest.mark.gpu
 def test_captured_rerun_matches_stream():
     # a learned schedule whose bounds are far off for one matrix: its rerun resets the counters that the
