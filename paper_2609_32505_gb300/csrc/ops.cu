@@ -21,7 +21,12 @@ __global__ void prepare_kernel(const float *__restrict__ src, long long lds, lon
     const float *S = src + b * bss;
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
         const int r = r0 + i, c = c0 + threadIdx.x;
-        tile[i][threadIdx.x] = (r < rows && c < cols) ? S[(long long)r * lds + c] * sc : 0.f;
+        float x = 0.f;
+        if (r < rows && c < cols) {
+            x = S[(long long)r * lds + c] * sc;
+            if (dst.colscale) x *= dst.colscale[(long long)b * cols + c];
+        }
+        tile[i][threadIdx.x] = x;
     }
     __syncthreads();
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
@@ -119,6 +124,7 @@ __global__ void __launch_bounds__(256) prepare_vec_kernel(const float *__restric
     if constexpr (kTrans) {
         const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 32;
         const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        if (dst.colscale && c0 + lane < cols) sc *= dst.colscale[(long long)b * cols + c0 + lane];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int r = r0 + w + 8 * i, c = c0 + lane;
@@ -145,6 +151,11 @@ __global__ void __launch_bounds__(256) prepare_vec_kernel(const float *__restric
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i) x[i] *= sc;
+        if (dst.colscale) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < nv) x[i] *= dst.colscale[(long long)b * cols + c + i];
+        }
         prepare_store8(dst, p, b, r, c, nv, x);
     }
 }

@@ -27,6 +27,7 @@ struct SplitOut {
     __nv_bfloat16 *h16 = nullptr;         // bf16 copy
     __half *fhi = nullptr, *flo = nullptr;   // fp16 split of x * fscale (strides below, in elements)
     float fscale = 1.f;
+    const float *colscale = nullptr;      // factors of the source's columns [batch][cols], or null
     const int *prec = nullptr;            // per matrix: write the one format its precision reads
     long long ld = 0, bstride = 0, fbstride = 0;
 };

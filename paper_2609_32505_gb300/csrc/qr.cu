@@ -1,8 +1,9 @@
 // Blocked Householder QR (m >= n, diag(R) >= 0) for the QR fallback of Algorithm 1
 // (Appendix A.2) and the QR preprocessing of rectangular inputs (Section 4.1).
 //
-// The matrix is scaled by a power of two to columns of norm <= 1 and kept transposed and split into
-// FP16 hi/lo halves (UT: row j = column j).  Panels of nb columns are factored by one thread-block
+// Every column is scaled by its own power of two to a norm <= 1 (A D = Q (R D), exactly, so the scales only come
+// back on R's columns, and a small column beside large ones keeps its accuracy) and the matrix kept transposed
+// and split into FP16 hi/lo halves (UT: row j = column j).  Panels of nb columns are factored by one thread-block
 // cluster per matrix: each of its CTAs holds a slab of the panel's rows in registers, and the
 // per-column dot products (the norm below the diagonal and the projections of the later panel
 // columns) are summed across the cluster through distributed shared memory -- one cluster barrier
@@ -457,30 +458,37 @@ __global__ void __launch_bounds__(2 * kWY) qr_stapply_kernel(const float *Sp, in
     }
 }
 
-// max |A| of every factored matrix (float bits; a NaN compares above every finite value)
-__global__ void qr_absmax_kernel(const float *A, long long mn, const int *skip, unsigned *amax) {
-    __shared__ unsigned red[8];
-    const int b = blockIdx.y;
+// max |a| of every column of the factored matrices (float bits; a NaN compares above every finite value): one
+// block of 32 x 8 threads per 32 columns and kCmRows rows
+constexpr int kCmRows = 512;
+__global__ void __launch_bounds__(256) qr_colmax_kernel(const float *A, int m, int n, const int *skip, unsigned *amax) {
+    __shared__ unsigned red[8][32];
+    const int b = blockIdx.z, tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c = blockIdx.x * 32 + tx;
     if (skip[b]) return;
-    const float *a = A + b * mn;
     unsigned v = 0;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < mn; t += (long long)gridDim.x * blockDim.x)
-        v = max(v, __float_as_uint(fabsf(a[t])));
-    v = __reduce_max_sync(0xffffffffu, v);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    if (c < n) {
+        const float *a = A + (long long)b * m * n + c;
+        const int r1 = min(m, ((int)blockIdx.y + 1) * kCmRows);
+#pragma unroll 8
+        for (int r = blockIdx.y * kCmRows + ty; r < r1; r += 8) v = max(v, __float_as_uint(fabsf(a[(long long)r * n])));
+    }
+    red[ty][tx] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) v = max(v, red[w]);
-        atomicMax(&amax[b], v);
+    if (ty == 0 && c < n) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) v = max(v, red[w][tx]);
+        atomicMax(&amax[(long long)b * n + c], v);
     }
 }
-// 2^e >= sqrt(m) max |A| >= every column norm (1 where there is none: a zero or non-finite matrix)
-__global__ void qr_scale_kernel(const unsigned *amax, int B, int m, float *scale) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const float v = __uint_as_float(amax[b]);
+// 2^e >= sqrt(m) max |a| >= the norm of column c (1 where there is none: a zero or non-finite column), and 2^-e
+__global__ void qr_scale_kernel(const unsigned *amax, long long cols, int m, float *scale, float *iscale) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= cols) return;
+    const float v = __uint_as_float(amax[c]);
     const bool ok = v > 0.f && v < INFINITY;
-    scale[b] = ok ? ldexpf(1.f, min(127, max(-100, ilogb((double)v * sqrt((double)m)) + 1))) : 1.f;
+    const int e = ok ? min(126, max(-100, ilogb((double)v * sqrt((double)m)) + 1)) : 0;
+    scale[c] = ldexpf(1.f, e);
+    iscale[c] = ldexpf(1.f, -e);
 }
 
 __global__ void qr_skip_kernel(const int *flag, int B, int *skip) {
@@ -500,7 +508,7 @@ __global__ void qr_qinit_kernel(int n, int m, long long ldm, const int *skip, __
 }
 
 // Q[r][c] = sign(beta_c) Q^T[c][r] (transposed through a shared tile) and, if R is given,
-// R[r][c] = 2^e sign(beta_r) (r < c ? UT[c][r] : r == c ? beta_c : 0).
+// R[r][c] = 2^e_c sign(beta_r) (r < c ? UT[c][r] : r == c ? beta_c : 0).
 __global__ void qr_store_kernel(const __half *QThi, const __half *QTlo, const __half *UThi, const __half *UTlo,
                                 const float *beta, const float *scale, int m, int n, long long ldm, const int *skip,
                                 float *Q, float *R) {
@@ -533,7 +541,7 @@ __global__ void qr_store_kernel(const __half *QThi, const __half *QTlo, const __
             const long long o = ((long long)b * n + c) * ldm + r;
             v = r < c ? join_f16(UThi[o], UTlo[o]) * (1.f / kF16X) : (r == c ? fabsf(bb[c]) : 0.f);
             if (r < c && bb[r] < 0.f) v = -v;
-            v *= scale[b];
+            v *= scale[(long long)b * n + c];
         }
         tile[i][threadIdx.x] = v;
     }
@@ -638,16 +646,16 @@ int qr_factor(const float *A, float *Q, float *R, const int *flag, QrWS &w, cuda
     const int B = w.B, m = w.m, n = w.n, nb = w.nb;
     const long long nm = (long long)n * w.ldm;
     qr_skip_kernel<<<(B + 127) / 128, 128, 0, st>>>(flag, B, w.skip);
-    PSVD_TRY(cudaMemsetAsync(w.amax, 0, sizeof(unsigned) * (size_t)B, st));
-    const long long mn = (long long)m * n;
-    qr_absmax_kernel<<<dim3((unsigned)std::min<long long>((mn + 2047) / 2048, 8 * num_sms()), B), 256, 0, st>>>(
-        A, mn, w.skip, w.amax);
-    qr_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, m, w.scale);
+    const long long mn = (long long)m * n, bn = (long long)B * n;
+    PSVD_TRY(cudaMemsetAsync(w.amax, 0, sizeof(unsigned) * (size_t)bn, st));
+    qr_colmax_kernel<<<dim3((n + 31) / 32, (m + kCmRows - 1) / kCmRows, B), 256, 0, st>>>(A, m, n, w.skip, w.amax);
+    qr_scale_kernel<<<(unsigned)((bn + 127) / 128), 128, 0, st>>>(w.amax, bn, m, w.scale, w.iscale);
     count_launch(3);
     {
         SplitOut t;
         t.fhi = w.UThi; t.flo = w.UTlo; t.ld = w.ldm; t.bstride = t.fbstride = nm; t.fscale = kF16X;
-        PSVD_TRY(prepare_operand(A, n, mn, B, m, n, true, 1.f, w.scale, t, st, w.skip));
+        t.colscale = w.iscale;
+        PSVD_TRY(prepare_operand(A, n, mn, B, m, n, true, 1.f, nullptr, t, st, w.skip));
     }
     for (int sp = 0; sp < w.nsup; ++sp) {
         const int s0 = sp * kWY, s1 = std::min(n, s0 + kWY);

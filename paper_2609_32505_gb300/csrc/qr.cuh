@@ -11,8 +11,8 @@ bool qr_shape(int m, int *nb);
 
 constexpr int kQrSplit = 8;   // largest K split of the X^T Y products of a block
 
-// The matrices are normalized by a power of two (|A| <= 2^e, columns of norm <= 1), so every array
-// below is bounded and kept as split-FP16 halves.
+// The columns are normalized by powers of two (norms <= 1), so every array below is bounded and kept as
+// split-FP16 halves.
 struct QrWS {
     int B = 0, m = 0, n = 0, nb = 0, npan = 0, nsup = 0, ks = 1;
     long long ldm = 0, ldn = 0;
@@ -26,8 +26,8 @@ struct QrWS {
     __half *W2hi = nullptr, *W2lo = nullptr;   // [B][n][kWY] (op(T) Y^T X)^T (kF16S2)
     float *Ts = nullptr;                       // [B][nsup][kWY][kWY] T of blocks of kWY columns
     float *Sp = nullptr;                       // [kQrSplit][B][n][kWY] partial X^T Y, or Y^T Y, of a block
-    unsigned *amax = nullptr;                  // [B] max |A| (float bits)
-    float *scale = nullptr;                    // [B] 2^e
+    unsigned *amax = nullptr;                  // [B][n] max |a| of every column (float bits)
+    float *scale = nullptr, *iscale = nullptr; // [B][n] 2^e and 2^-e of every column
     int *skip = nullptr;                       // [B] 1 = matrix not factored (flag[b] == 0)
     unsigned *err = nullptr;
 
@@ -50,8 +50,9 @@ struct QrWS {
         W2hi = cv.template take<__half>(B64 * n * kWY); W2lo = cv.template take<__half>(B64 * n * kWY);
         Ts = cv.template take<float>(B64 * nsup * kWY * kWY);
         Sp = cv.template take<float>((long long)kQrSplit * B64 * n * kWY);
-        amax = cv.template take<unsigned>(B64);
-        scale = cv.template take<float>(B64);
+        amax = cv.template take<unsigned>(B64 * n);
+        scale = cv.template take<float>(B64 * n);
+        iscale = cv.template take<float>(B64 * n);
         skip = cv.template take<int>(B64);
         err = cv.template take<unsigned>(4);
     }
