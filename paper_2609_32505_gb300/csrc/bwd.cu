@@ -104,16 +104,17 @@ __global__ void bwd_scale_kernel(const unsigned *amax, int B, int n, int stage, 
     if (b >= B) return;
     auto put = [&](int slot, int e) { es[(long long)slot * B + b] = ldexpf(1.f, e); };
     const double rn = sqrt((double)n);
-    const int eM = bwd_exp(amax[AM_M * B + b], rn), eV = bwd_exp_factor(amax[AM_V * B + b]);
+    const int eM = bwd_exp(amax[AM_M * B + b], 1.0), eV = bwd_exp_factor(amax[AM_V * B + b]);
+    const int eY = bwd_exp(amax[AM_M * B + b], rn) + eV;
     if (stage == 0) {
         const int eG = bwd_exp(amax[AM_G * B + b], polar ? rn : 1.0), eB = bwd_exp(amax[AM_B * B + b], polar ? rn : 1.0);
         const int eU = bwd_exp_factor(amax[AM_U * B + b]);
-        put(ES_M, eM); put(ES_G, eG); put(ES_B, eB); put(ES_U, eU); put(ES_V, eV); put(ES_IM, -(eM + eV)); put(ES_IG, -eG);
-        put(ES_AU, eU + eG - 28); put(ES_BV, eV + eB - 28); put(ES_Y, eM + eV - 28); put(ES_Z, eM + eV + eG - 28);
+        put(ES_M, eM); put(ES_G, eG); put(ES_B, eB); put(ES_U, eU); put(ES_V, eV); put(ES_IM, -eY); put(ES_IG, -eG);
+        put(ES_AU, eU + eG - 28); put(ES_BV, eV + eB - 28); put(ES_Y, eM + eV - 28); put(ES_Z, eY + eG - 28);
         put(ES_T1, eB - 28); put(ES_EH, eB - 28); put(ES_WV, eG - 28);
     } else if (stage == 1) {
         const int eX = bwd_exp(amax[AM_X * B + b], 1.0);
-        put(ES_X, eX); put(ES_QP, eM + eV + eX - 28);
+        put(ES_X, eX); put(ES_QP, eY + eX - 28);
     } else {
         const int eQ = bwd_exp(amax[AM_Q * B + b], 1.0);
         put(ES_Q, eQ); put(ES_DA, eQ + eV - 28);

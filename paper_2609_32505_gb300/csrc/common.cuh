@@ -118,6 +118,15 @@ PSVD_DEV void umma_f16(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
         "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
         : "memory");
 }
+// the same with D = A B + 2^-kF16LoBits D (split_f16 below: the low halves carry that factor)
+constexpr int kF16LoBits = 11;
+PSVD_DEV void umma_f16_lo(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.eq.b32 p, 0, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p, %4;\n}\n" ::"r"(dtmem),
+        "l"(ad), "l"(bd), "r"(idesc), "n"(kF16LoBits)
+        : "memory");
+}
 // Arrive on `bar` once all previously issued MMAs of this thread have completed.
 PSVD_DEV void umma_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -153,15 +162,18 @@ PSVD_DEV void split_tf32(float x, float &hi, float &lo) {
     lo = tf32_round(x - hi);
 }
 
-// Split FP16: x * 2^e = hi + lo with FP16 halves, the 11 + 11 significant bits of the split TF32 at
-// half the bytes and twice the tensor rate.  The caller's power of two puts the operand's bound
-// below 2^16; elements down to 2^-18 of it keep both halves normal (|x - hi - lo| <= 2^-22 |x|),
-// smaller ones an error of 2^-40 of the bound.
+// Split FP16: x * 2^e = hi + 2^-11 lo with FP16 halves, the 11 + 11 significant bits of the split TF32 at
+// half the bytes and twice the tensor rate.  lo is the rest of hi times 2^11, so that it is as far from
+// the end of FP16's range as hi (stored as it is, it loses bits from 2^-16 of 1 on with e = 14, and
+// columns of 1e-6 beside columns of 1 came out with 1e-4 relative errors); the product kernel takes the factor
+// back out.  The caller's power of two puts the operand's bound below 2^16; elements down to 2^-30 of
+// that keep their 22 bits (|x - hi - 2^-11 lo| <= 2^-22 |x|), smaller ones an error of 2^-52 of it.
+constexpr float kF16Lo = 1 << kF16LoBits, kF16LoInv = 1.f / kF16Lo;
 PSVD_DEV void split_f16(float xs, __half &hi, __half &lo) {
     hi = __float2half_rn(xs);
-    lo = __float2half_rn(xs - __half2float(hi));
+    lo = __float2half_rn((xs - __half2float(hi)) * kF16Lo);
 }
-PSVD_DEV float join_f16(__half hi, __half lo) { return __half2float(hi) + __half2float(lo); }
+PSVD_DEV float join_f16(__half hi, __half lo) { return __fmaf_rn(__half2float(lo), kF16LoInv, __half2float(hi)); }
 
 PSVD_DEV float warp_sum(float v) {
 #pragma unroll

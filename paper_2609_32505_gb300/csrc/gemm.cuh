@@ -214,14 +214,14 @@ PSVD_DEV float warp_sum16(float (&a)[16]) {
     }
     return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
 }
-// 16 values -> packed FP16 halves of x * fs
+// 16 values -> packed FP16 halves of x * fs (split_f16)
 PSVD_DEV void split_f16x16(const float (&v)[16], float fs, uint32_t (&h)[8], uint32_t (&l)[8]) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const float x0 = v[2 * i] * fs, x1 = v[2 * i + 1] * fs;
         const __half2 hh = __floats2half2_rn(x0, x1);
         const float2 f = __half22float2(hh);
-        const __half2 ll = __floats2half2_rn(x0 - f.x, x1 - f.y);
+        const __half2 ll = __floats2half2_rn((x0 - f.x) * kF16Lo, (x1 - f.y) * kF16Lo);
         h[i] = *reinterpret_cast<const uint32_t *>(&hh);
         l[i] = *reinterpret_cast<const uint32_t *>(&ll);
     }
@@ -298,8 +298,11 @@ PSVD_DEV bool mma_tile_x3(MmaRing &r, int nkb, uint32_t tmem, uint64_t *acc_full
             mma(sdesc_step(alo, k), sdesc_step(bhi, k), k != 0);
             mma(sdesc_step(ahi, k), sdesc_step(blo, k), 1);
         }
+        // (the low halves of split FP16 carry 2^kF16LoBits, which the first hi*hi takes out of their sum)
+        if constexpr (kF16) umma_f16_lo(tacc, ahi, bhi, id);
+        else mma(ahi, bhi, 1);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) mma(sdesc_step(ahi, k), sdesc_step(bhi, k), 1);
+        for (int k = 1; k < 4; ++k) mma(sdesc_step(ahi, k), sdesc_step(bhi, k), 1);
         umma_commit(&r.empty[s0]);
         umma_commit(&r.empty[s1]);
         umma_commit(&acc_full[buf]);

@@ -162,8 +162,8 @@ struct EpiSubHalf {
         for (int i = 0; i < 8; ++i) {
             const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&h[i]));
             const float2 c = __half22float2(*reinterpret_cast<const __half2 *>(&l[i]));
-            v[2 * i] = (a.x + c.x) * inv - v[2 * i];
-            v[2 * i + 1] = (a.y + c.y) * inv - v[2 * i + 1];
+            v[2 * i] = __fmaf_rn(c.x, kF16LoInv, a.x) * inv - v[2 * i];
+            v[2 * i + 1] = __fmaf_rn(c.y, kF16LoInv, a.y) * inv - v[2 * i + 1];
         }
         split_f16x16(v, scale, h, l);
         st_v8(hi + o, h);
