@@ -358,7 +358,7 @@ static int g16(const __half *ahi, const __half *alo, int M, int K, long long lda
     memset(&s, 0, sizeof(s));
     s.M = M; s.N = N; s.K = K; s.prec_uniform = PREC_F16X3; s.err = err;
     s.f16_scale = 1.f;
-    s.f16_scale_b = scale;
+    s.scale_b = scale;
     return launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f) == cudaSuccess
                ? PSVD_OK : PSVD_ERR_CUDA;
 }

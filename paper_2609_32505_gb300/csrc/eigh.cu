@@ -1304,9 +1304,10 @@ __global__ void __launch_bounds__(2 * kWY) s_pair_kernel(const float *S, int ks,
 
 // sign convention + outputs: each row of V^T flipped so its largest-|.| entry is positive
 __global__ void eig_finalize_kernel(__half *VThi, __half *VTlo, long long ldn, int n, const double *lam, float *S,
-                                    float *VT, float *t32hi, float *t32lo) {
+                                    float *VT, float *t32hi, float *t32lo, const int *t32prec) {
     const int b = blockIdx.y, i = blockIdx.x;
     const long long row = (long long)b * n * ldn + (long long)i * ldn;
+    if (t32prec && t32prec[b] != PREC_TF32X3) t32hi = nullptr;
     __half *h = VThi + row, *l = VTlo + row;
     __shared__ float sv[32];
     __shared__ int si[32];
@@ -1368,7 +1369,8 @@ int eigh_groups(int B, int n) {
     return trd_groups(B, n);
 }
 
-int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t st, float *vt_hi, float *vt_lo) {
+int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t st, float *vt_hi, float *vt_lo,
+                 const int *vt_prec) {
     const int B = w.B, n = w.n;
     const long long ldn = w.ldn;
     PSVD_TRY(cudaMemsetAsync(w.bar, 0, sizeof(unsigned) * (size_t)w.groups * (std::max(trd_ctas_per_group(n), 15) + 1), st));
@@ -1580,7 +1582,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
         }
         if (first) PSVD_TRY_RC(single(0));
     }
-    eig_finalize_kernel<<<dim3(n, B), 128, 0, st>>>(w.VThi, w.VTlo, ldn, n, w.lam, S, VT, vt_hi, vt_lo);
+    eig_finalize_kernel<<<dim3(n, B), 128, 0, st>>>(w.VThi, w.VTlo, ldn, n, w.lam, S, VT, vt_hi, vt_lo, vt_prec);
     count_launch(1);
     PSVD_TRY(cudaGetLastError());
     return PSVD_OK;

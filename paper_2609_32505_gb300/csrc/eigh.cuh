@@ -96,8 +96,9 @@ int trd_chip(const float *Hs, EighWS &w, cudaStream_t st, bool *ran);
 // Eigendecomposition of the symmetric matrices Hs (B x n x n, FP32, full storage).
 // Writes eigenvalues descending to S (B x n, may be null) and V^T as split-FP16 halves in
 // ws.VThi / ws.VTlo (rows = eigenvectors, largest-|.| entry positive), V^T to VT (B x n x n, may be
-// null) and V^T as split TF32 to vt_hi / vt_lo (B x n x ldn, may be null).
+// null) and V^T as split TF32 to vt_hi / vt_lo (B x n x ldn, may be null), of the matrices whose vt_prec is
+// PREC_TF32X3 only if that is given.
 int eigh_forward(const float *Hs, float *S, float *VT, EighWS &ws, cudaStream_t st, float *vt_hi = nullptr,
-                 float *vt_lo = nullptr);
+                 float *vt_lo = nullptr, const int *vt_prec = nullptr);
 
 }  // namespace psvd

@@ -85,8 +85,8 @@ struct GemmShape {
                             // returns at once (written by an earlier kernel on the same stream)
     unsigned *ticket;       // nullptr, or a zeroed counter: the last CTA to finish runs epi.tail()
     unsigned *err;          // device error word
-    float f16_scale;        // PREC_F16X3: the product of the operands' inverse scales ...
-    const float *f16_scale_b;   // ... times this entry of the matrix (nullptr: 1)
+    float f16_scale;        // PREC_F16X3: the product of the operands' inverse scales
+    const float *scale_b;   // split precisions: another factor for each matrix (nullptr: 1)
     int prof_as;            // profiling class + 1 for the launch timing (0: by precision)
 };
 
@@ -432,7 +432,8 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
             const int be = b + jb.kc * shp.batch;     // epilogue's batch index (partial-sum slice)
             const int nph = nkb == 0 ? 0 : (prec >= PREC_TF32X3 ? nkb : 1);
             float fs = 1.f;                       // undoes the operands' powers of two (exact)
-            if (prec == PREC_F16X3) fs = shp.f16_scale * (shp.f16_scale_b ? shp.f16_scale_b[b] : 1.f);
+            if (prec == PREC_F16X3) fs = shp.f16_scale;
+            if (prec >= PREC_TF32X3 && shp.scale_b) fs *= shp.scale_b[b];
             float acc[128];
 #pragma unroll
             for (int c = 0; c < 128; ++c) acc[c] = 0.f;

@@ -16,8 +16,8 @@ cudaError_t l1_norms(const float *A, int B, int m, int n, float *rowsum, float *
                      cudaStream_t st);
 __global__ void __launch_bounds__(kNormThreads) norm_finalize_kernel(const float *rowsum, const float *colsum,
                                                                       const int *nonfinite, int m, int n,
-                                                                      float *scale, float *ascale, int *done,
-                                                                      int *status, int *fin);
+                                                                      float *scale, float *ascale, int *fine,
+                                                                      int *prec, int *done, int *status, int *fin);
 
 constexpr int kH = 64, kF = 8;
 constexpr int kP_W1 = 0, kP_b1 = kH * kF, kP_W2 = kP_b1 + kH, kP_b2 = kP_W2 + kH * kH, kP_W3 = kP_b2 + kH,
@@ -456,8 +456,8 @@ extern "C" int psvd_sketch_features(const float *A, const float *Z, int64_t s, f
     PSVD_TRY(cudaMemsetAsync(w.rowsum, 0, sizeof(float) * batch * m, st));
     PSVD_TRY(cudaMemsetAsync(w.nonfinite, 0, sizeof(int) * batch, st));
     PSVD_TRY(l1_norms(A, B, M, Nn, w.rowsum, w.colsum, w.nonfinite, st));
-    norm_finalize_kernel<<<B, kNormThreads, 0, st>>>(w.rowsum, w.colsum, w.nonfinite, M, Nn, w.scale, nullptr, w.done,
-                                                     w.status, w.fin);
+    norm_finalize_kernel<<<B, kNormThreads, 0, st>>>(w.rowsum, w.colsum, w.nonfinite, M, Nn, w.scale, nullptr, nullptr,
+                                                     nullptr, w.done, w.status, w.fin);
     const bool vec_mn = ((uintptr_t)A & 15) == 0 && ((m * n) & 3) == 0;
     const bool vec_n = ((uintptr_t)A & 15) == 0 && (n & 3) == 0;
     if (vec_mn) fro_part_kernel<true><<<dim3(kFroBlocks, B), 256, 0, st>>>(A, w.scale, (long long)m * n, w.fropart);

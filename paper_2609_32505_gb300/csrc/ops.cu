@@ -43,8 +43,8 @@ __global__ void prepare_kernel(const float *__restrict__ src, long long lds, lon
             dst.fhi[of] = h;
             dst.flo[of] = l;
         }
-        if (dst.hi && (p < 0 || p == PREC_TF32)) {
-            if (dst.lo) { float h, l; split_tf32(x, h, l); dst.hi[o] = h; dst.lo[o] = l; }
+        if (dst.hi && (p < 0 || p == PREC_TF32 || p == PREC_TF32X3)) {
+            if (dst.lo && p != PREC_TF32) { float h, l; split_tf32(x, h, l); dst.hi[o] = h; dst.lo[o] = l; }
             else dst.hi[o] = p == PREC_TF32 ? tf32_round(x) : x;
         }
         if (dst.h16 && (p < 0 || p == PREC_BF16)) dst.h16[o] = __float2bfloat16_rn(x);
@@ -72,24 +72,25 @@ PSVD_DEV void prepare_store8(const SplitOut &d, int p, int b, int r, int c, int 
                 if (i < nv) { d.fhi[of + i] = h[i]; d.flo[of + i] = l[i]; }
         }
     }
-    if (d.hi && (p < 0 || p == PREC_TF32)) {
+    if (d.hi && (p < 0 || p == PREC_TF32 || p == PREC_TF32X3)) {
+        const bool two = d.lo && p != PREC_TF32;
         float h[8], l[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            if (d.lo) split_tf32(x[i], h[i], l[i]);
+            if (two) split_tf32(x[i], h[i], l[i]);
             else h[i] = p == PREC_TF32 ? tf32_round(x[i]) : x[i];
         }
         if (nv == 8) {
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 reinterpret_cast<float4 *>(d.hi + o)[q] = make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
-                if (d.lo)
+                if (two)
                     reinterpret_cast<float4 *>(d.lo + o)[q] = make_float4(l[4 * q], l[4 * q + 1], l[4 * q + 2], l[4 * q + 3]);
             }
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-                if (i < nv) { d.hi[o + i] = h[i]; if (d.lo) d.lo[o + i] = l[i]; }
+                if (i < nv) { d.hi[o + i] = h[i]; if (two) d.lo[o + i] = l[i]; }
         }
     }
     if (d.h16 && (p < 0 || p == PREC_BF16)) {

@@ -118,12 +118,16 @@ cudaError_t l1_norms(const float *A, int B, int m, int n, float *rowsum, float *
 // (launched with kNormThreads threads; the slab sums of a column are loaded eight at a time)
 __global__ void __launch_bounds__(kNormThreads) norm_finalize_kernel(const float *rowsum, const float *colsum,
                                                                       const int *nonfinite, int m, int n,
-                                                                      float *scale, float *ascale, int *done,
-                                                                      int *status, int *fin) {
-    __shared__ float sm[2][32];
+                                                                      float *scale, float *ascale, int *fine,
+                                                                      int *prec, int *done, int *status, int *fin) {
+    __shared__ float sm[4][32];
     const int b = blockIdx.x;
-    float r = 0.f, c = 0.f;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) r = fmaxf(r, rowsum[(long long)b * m + i]);
+    float r = 0.f, c = 0.f, rl = INFINITY, cl = INFINITY;   // largest sums, and smallest of those above 0
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        const float x = rowsum[(long long)b * m + i];
+        r = fmaxf(r, x);
+        if (x > 0.f) rl = fminf(rl, x);
+    }
     const int S = l1_slabs(m);
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         float cs = 0.f;                              // slab partial sums, added in slab order
@@ -135,16 +139,22 @@ __global__ void __launch_bounds__(kNormThreads) norm_finalize_kernel(const float
             for (int u = 0; u < 8; ++u) cs += x[u];
         }
         c = fmaxf(c, cs);
+        if (cs > 0.f) cl = fminf(cl, cs);
     }
     r = warp_max(r);
     c = warp_max(c);
+    rl = -warp_max(-rl);
+    cl = -warp_max(-cl);
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-    if (l == 0) { sm[0][w] = r; sm[1][w] = c; }
+    if (l == 0) { sm[0][w] = r; sm[1][w] = c; sm[2][w] = rl; sm[3][w] = cl; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int i = 1; i < nw; ++i) { r = fmaxf(r, sm[0][i]); c = fmaxf(c, sm[1][i]); }
-        r = fmaxf(r, sm[0][0]);
-        c = fmaxf(c, sm[1][0]);
+        for (int i = 1; i < nw; ++i) {
+            r = fmaxf(r, sm[0][i]);
+            c = fmaxf(c, sm[1][i]);
+            rl = fminf(rl, sm[2][i]);
+            cl = fminf(cl, sm[3][i]);
+        }
         const double s = sqrt((double)r * (double)c);
         scale[b] = (float)s;
         // 2^-e with |M_ij| <= s < 2^e: the operand M 2^-e of H = W^T M (s is at least ||M||_2), and 2^e
@@ -152,6 +162,14 @@ __global__ void __launch_bounds__(kNormThreads) norm_finalize_kernel(const float
         if (ascale) {
             ascale[b] = ldexpf(1.f, -e);
             ascale[gridDim.x + b] = ldexpf(1.f, e);
+        }
+        // Rows or columns of X0 whose entries are on average below 2^-28 lose bits in FP16 halves (split_f16 with
+        // kF16X), and the iteration brings them up to the size of the others, errors included (columns of
+        // 1e-9 of the others: W off by 4e-5, in split TF32 1e-6): such a matrix takes split TF32.
+        if (fine) {
+            const double lim = s * 0x1p-28;
+            fine[b] = (double)rl < lim * n || (double)cl < lim * m ? PREC_TF32X3 : PREC_F16X3;
+            if (prec[b] == PREC_F16X3) prec[b] = fine[b];
         }
         if (nonfinite[b]) { done[b] = 1; status[b] = PSVD_ERR_NONFINITE; fin[b] = 0; }
         else if (s == 0.0) { done[b] = 1; status[b] = PSVD_OK; fin[b] = 0; }
@@ -177,22 +195,22 @@ struct CoefTable {
 // matrix (FP64), each applied to x / kPeDamp while the tracked interval is wider than
 // kPeWidth (undamped greedy cubics from a small bound lose accuracy: relative
 // reconstruction ~2e-4 at kappa = 1e6 in FP32 against ~3e-6 damped, for the same number of
-// steps), and the step budget before the conservative rerun; with gate_x3, a matrix whose
-// bound is below PSVD_MIXED_LB_MIN starts on the FP32-accurate (split-FP16) rung.
+// steps), and the step budget before the conservative rerun; with gate_fine, a matrix whose
+// bound is below PSVD_MIXED_LB_MIN starts on its FP32-accurate rung.
 // Damped (schedule PSVD_SCHED_PE, the Polar-Express-style comparison): the same damped cubics
 // from [l_b, 1] until a damped step stops shrinking the interval (width below 0.1 and less
 // than 10% gained: the damped fixed point near 1 - 1.5e-4, the plateau the ablation
 // describes), then undamped from there; no budget and no rerun.
 constexpr double kPeDamp = 1.01, kPeWidth = 1e-2;
 __global__ void schedule_fill_kernel(int B, int K, CoefTable tab, const float *lower, int learned, double tol,
-                                     int budget_opt, const int *active, float *coef, int *budget, int gate_x3,
-                                     int *prec, int pe = 0) {
+                                     int budget_opt, const int *active, float *coef, int *budget,
+                                     const int *gate_fine, int *prec, int pe = 0) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
     if (active && !active[b]) return;
     if (learned || pe) {
         double l = (double)lower[b];
-        if (learned && gate_x3 && !(l >= PSVD_MIXED_LB_MIN)) prec[b] = PREC_F16X3;
+        if (learned && gate_fine && !(l >= PSVD_MIXED_LB_MIN)) prec[b] = gate_fine[b];
         if (!(l > 1e-12)) l = 1e-12;
         if (l > 0.999) l = 0.999;
         double lo = l, hi = 1.0;
@@ -242,7 +260,8 @@ PSVD_DEV void store_prec(int p, long long o, float x, __nv_bfloat16 *p16, float 
     if (p == PREC_BF16) p16[o] = __float2bfloat16_rn(x);
     else phi[o] = tf32_round(x);
 }
-// the same with the split-FP16 rung: halves of x * fs at element of (stride of a batch entry doubled)
+// the same with the split-FP16 rung: halves of x * fs at element of (stride of a batch entry doubled); split TF32
+// is wide_piece's
 PSVD_DEV void store_rung(int p, long long o, long long of, float x, float fs, __nv_bfloat16 *p16, float *phi,
                          float *plo) {
     if (p == PREC_F16X3) {
@@ -253,6 +272,38 @@ PSVD_DEV void store_rung(int p, long long o, long long of, float x, float fs, __
     } else {
         store_prec(p, o, x, p16, phi);
     }
+}
+
+// The split-TF32 rung of matrices of a wide range: a warp's piece of 32 rows x 16 columns from (r0, c0) on, of
+// which nr x nc are inside.  Entries at or above the diagonal (column + off >= row, all if off is large)
+// become x = c3 v + (diagonal: c1) and are stored at rhi / rlo (the place of (r0, c0)) and, mirrored or transposed, at
+// chi / clo (that of (c0, r0)); returns this lane's part of sum (v - I)^2 over them, off-diagonal entries twice.
+// Out of line, and fed through shared memory: it is rare, and inlined into the eight pieces of a tile it made
+// the product kernels of every other matrix 10 to 17% slower (64 x 512: 1.87 -> 2.21 ms of Gram products).
+__device__ __noinline__ ff wide_piece(const float *v, float *rhi, float *rlo, long long ldr, float *chi, float *clo,
+                                      long long ldc, int nr, int nc, int off, float c1, float c3) {
+    const int lane = threadIdx.x & 31;
+    ff res = ff_zero();
+#pragma unroll 1
+    for (int k = 0; k < 16; ++k) {
+        const int r = 2 * k + (lane >> 4), c = lane & 15;
+        if (r >= nr || c >= nc || c + off < r) continue;
+        const bool diag = c + off == r;
+        const float g = v[r * kStageRow + c], d = diag ? g - 1.f : g;
+        res = ff_fma(res, diag ? d : 2.f * d, d);
+        split_tf32(c3 * g + (diag ? c1 : 0.f), rhi[r * ldr + c], rlo[r * ldr + c]);
+    }
+#pragma unroll 1
+    for (int c = 0; c < nc; ++c)
+        if (lane < nr && c + off > lane) split_tf32(c3 * v[lane * kStageRow + c], chi[c * ldc + lane], clo[c * ldc + lane]);
+    return res;
+}
+// the warp's values, lane = row, into its staging area
+PSVD_DEV void stage_piece(const float (&v)[16], float *sw) {
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sw[(threadIdx.x & 31) * kStageRow + i] = v[i];
+    __syncwarp();
 }
 
 // 16 values of one row in the format of rung p: along the row at element ro (roh for halves) when
@@ -287,14 +338,14 @@ PSVD_DEV void rung_row16(int p, const float (&v)[16], float fs, __nv_bfloat16 *r
 }
 
 // Per-matrix decision after the Gram of step k.
-// mixed: 0 every step split FP16; 1 TF32 until the residual drops below kTauTF32; 2 BF16
-// above kTauBF16 first.  The precision never decreases from one step to the next.
+// mixed: 0 every step FP32-accurate (fine[b]: split FP16, or split TF32 for matrices of a wide range); 1 TF32
+// until the residual drops below kTauTF32; 2 BF16 above kTauBF16 first.  The precision never decreases from one step to the next.
 struct DecideArgs {
     int k, B, n, mixed, learned, kcap;
     double tol;
     int *done, *fin, *status, *prec, *steps, *fallback, *notdone;
     const double *res;
-    const int *budget;
+    const int *budget, *fine;
     float *fres;
 };
 
@@ -313,9 +364,9 @@ PSVD_DEV void decide_matrix(const DecideArgs &d, int b) {
         d.done[b] = 1; d.fin[b] = k; d.status[b] = PSVD_NOT_CONVERGED; d.fres[b] = (float)r; d.fallback[b] = 1;
         return;
     }
-    int pn = PREC_F16X3;
+    int pn = d.fine[b];
     if (d.mixed) {
-        const int want = (d.mixed == 2 && r > kTauBF16) ? PREC_BF16 : (r > kTauTF32 ? PREC_TF32 : PREC_F16X3);
+        const int want = (d.mixed == 2 && r > kTauBF16) ? PREC_BF16 : (r > kTauTF32 ? PREC_TF32 : pn);
         pn = want > pk ? want : pk;
     }
     d.prec[(long long)(k + 1) * B + b] = pn;
@@ -341,8 +392,16 @@ struct EpiGram {
     static constexpr bool kElem = true, kTrans = true, kTail = true, kRow = true;
     PSVD_DEV bool row16(Acc &a, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
         if (r0 >= n || c0 >= n || c0 + 15 < r0) return true;       // outside, or left to the mirror's tile
-        if (c0 < r0 + 32) return false;                            // crosses the diagonal
         load(a, b);
+        if (a.p == PREC_TF32X3) {
+            stage_piece(v, sw);
+            const long long bo = (long long)b * n * ldp, rc = bo + (long long)r0 * ldp + c0, cr = bo + (long long)c0 * ldp + r0;
+            const ff s = wide_piece(sw, Phi + rc, Plo + rc, ldp, Phi + cr, Plo + cr, ldp, n - r0, min(16, n - c0), c0 - r0,
+                                    a.c1, a.c3);
+            a.r = ff_add(a.r, s);
+            return true;
+        }
+        if (c0 < r0 + 32) return false;                            // crosses the diagonal
         // entries past n are products of the zero fill
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -410,6 +469,13 @@ struct EpiApply {
     PSVD_DEV bool row16(Acc &a, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
         if (r0 >= m || c0 >= n) return true;
         if (a.p < 0) a.p = prec_next[b];
+        if (a.p == PREC_TF32X3) {
+            stage_piece(v, sw);
+            const long long rc = (long long)b * m * ldn + (long long)r0 * ldn + c0;
+            const long long cr = (long long)b * n * ldm + (long long)c0 * ldm + r0;
+            wide_piece(sw, Xhi + rc, Xlo + rc, ldn, XThi + cr, XTlo + cr, ldm, m - r0, min(16, n - c0), 1 << 20, 0.f, 1.f);
+            return true;
+        }
         // columns past n and rows past m are zeros, and land in the padding of the rows
         const int r = r0 + lane, ct = c0 + (lane >> 1);
         const long long bo = (long long)b * m * ldn, rc = (long long)r * ldn + c0;
@@ -446,8 +512,8 @@ struct EpiApply {
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 
-// W (user layout) from X_fin; leaves W and W^T as split-FP16 halves in ws.wf_hi() ... for the products
-// that follow (H, U).
+// W (user layout) from X_fin; leaves W and W^T for the products that follow (H, U): as split-FP16 halves in
+// ws.wf_hi() ..., or as split TF32 in ws.Xhi[0] ... where fine[b] says so.
 __global__ void polar_finalize_kernel(int m, int n, int B, const int *fin, const int *prec, const int *status,
                                       PolarWS ws, __half *wh, __half *wl, __half *wth, __half *wtl, float *W) {
     __shared__ float tile[32][33];
@@ -457,35 +523,56 @@ __global__ void polar_finalize_kernel(int m, int n, int B, const int *fin, const
     const int par = f & 1;
     const int p = prec[(long long)f * B + b];
     const bool nan_out = status[b] == PSVD_ERR_NONFINITE;
+    const bool wide = ws.fine[b] == PREC_TF32X3;
     const long long rbase = (long long)b * m * ws.ldn;
     const __half *hp = reinterpret_cast<const __half *>(ws.Xhi[par]) + 2 * rbase;
     const __half *lp = reinterpret_cast<const __half *>(ws.Xlo[par]) + 2 * rbase;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        float x = 0.f;
-        if (r < m && c < n) {
-            const long long rc = (long long)r * ws.ldn + c;
-            if (nan_out) x = __int_as_float(0x7fc00000);
-            else if (p == PREC_BF16) x = __bfloat162float(ws.X16[par][rbase + rc]);
-            else if (p == PREC_TF32) x = ws.Xhi[par][rbase + rc];
-            else x = join_f16(hp[rc], lp[rc]) * (1.f / kF16X);
-            if (W) W[(long long)b * m * n + (long long)r * n + c] = x;
-            __half h, l;
-            split_f16(x * kF16X, h, l);
-            wh[2 * rbase + rc] = h;
-            wl[2 * rbase + rc] = l;
-        }
-        tile[i][threadIdx.x] = x;
+    const int tx = threadIdx.x, ty = threadIdx.y, c = c0 + tx;
+    float x[4];                                    // rows ty + 8 q: all loads ahead of the stores
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = r0 + ty + 8 * q;
+        const long long rc = (long long)r * ws.ldn + c;
+        x[q] = 0.f;
+        if (r >= m || c >= n) continue;
+        if (nan_out) x[q] = __int_as_float(0x7fc00000);
+        else if (p == PREC_F16X3) x[q] = join_f16(hp[rc], lp[rc]) * (1.f / kF16X);
+        else if (p == PREC_BF16) x[q] = __bfloat162float(ws.X16[par][rbase + rc]);
+        else x[q] = ws.Xhi[par][rbase + rc] + (p == PREC_TF32X3 ? ws.Xlo[par][rbase + rc] : 0.f);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = r0 + ty + 8 * q;
+        tile[ty + 8 * q][tx] = x[q];
+        if (r < m && c < n && W) W[(long long)b * m * n + (long long)r * n + c] = x[q];
     }
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (c < n && r < m) {
-            __half h, l;
-            split_f16(tile[threadIdx.x][i] * kF16X, h, l);
-            const long long o = 2 * (long long)b * n * ws.ldm + (long long)c * ws.ldm + r;
-            wth[o] = h;
-            wtl[o] = l;
+    const long long tbase = (long long)b * n * ws.ldm;
+    if (wide) {
+        if (par == 0 && p == PREC_TF32X3) return;  // (already there)
+        for (int i = ty; i < 32; i += 8) {
+            const int r = r0 + i, ct = c0 + i, rt = r0 + tx;
+            if (r < m && c < n) {
+                const long long o = rbase + (long long)r * ws.ldn + c;
+                split_tf32(tile[i][tx], ws.Xhi[0][o], ws.Xlo[0][o]);
+            }
+            if (rt < m && ct < n) {
+                const long long o = tbase + (long long)ct * ws.ldm + rt;
+                split_tf32(tile[tx][i], ws.XThi[0][o], ws.XTlo[0][o]);
+            }
+        }
+        return;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = ty + 8 * q, r = r0 + i, ct = c0 + i, rt = r0 + tx;
+        if (r < m && c < n) {
+            const long long o = 2 * rbase + (long long)r * ws.ldn + c;
+            split_f16(x[q] * kF16X, wh[o], wl[o]);
+        }
+        if (rt < m && ct < n) {
+            const long long o = 2 * tbase + (long long)ct * ws.ldm + rt;
+            split_f16(tile[tx][i] * kF16X, wth[o], wtl[o]);
         }
     }
 }
@@ -556,6 +643,7 @@ static cudaError_t plan_steps(PolarWS &w, StepPlans &p) {
         {   // Gram: A = B = X^T (n x m, K = m), upper-triangle tiles
             MatView v16 = w.bf16 ? view_of16(w.XT16[par], n, m, w.ldm, (long long)n * w.ldm, B) : MatView();
             MatView vhi = view_of(w.XThi[par], n, m, w.ldm, (long long)n * w.ldm, B);
+            MatView vlo = view_of(w.XTlo[par], n, m, w.ldm, (long long)n * w.ldm, B);
             F16Views f;
             f.ah = f.bh = view_f16(as_half(w.XThi[par]), n, m, w.ldm, 2LL * n * w.ldm, B);
             f.al = f.bl = view_f16(as_half(w.XTlo[par]), n, m, w.ldm, 2LL * n * w.ldm, B);
@@ -563,14 +651,16 @@ static cudaError_t plan_steps(PolarWS &w, StepPlans &p) {
             memset(&s, 0, sizeof(s));
             s.M = n; s.N = n; s.K = m; s.sym = 1;
             s.f16_scale = 1.f / (kF16X * kF16X);
-            const MatView *t = w.mixed ? &vhi : nullptr, *t16 = w.bf16 ? &v16 : nullptr;
-            if (cudaError_t e = plan_gemm(p.gram[par], t16, t16, t, nullptr, t, nullptr, s, B, &f)) return e;
+            const MatView *t16 = w.bf16 ? &v16 : nullptr;
+            if (cudaError_t e = plan_gemm(p.gram[par], t16, t16, &vhi, &vlo, &vhi, &vlo, s, B, &f)) return e;
         }
         {   // Apply: A = X (m x n, K = n), B = P (n x n, symmetric)
             MatView a16 = w.bf16 ? view_of16(w.X16[par], m, n, w.ldn, (long long)m * w.ldn, B) : MatView();
             MatView ahi = view_of(w.Xhi[par], m, n, w.ldn, (long long)m * w.ldn, B);
+            MatView alo = view_of(w.Xlo[par], m, n, w.ldn, (long long)m * w.ldn, B);
             MatView b16 = w.bf16 ? view_of16(w.P16, n, n, w.ldn, (long long)n * w.ldn, B) : MatView();
             MatView bhi = view_of(w.Phi, n, n, w.ldn, (long long)n * w.ldn, B);
+            MatView blo = view_of(w.Plo, n, n, w.ldn, (long long)n * w.ldn, B);
             F16Views f;
             f.ah = view_f16(as_half(w.Xhi[par]), m, n, w.ldn, 2LL * m * w.ldn, B);
             f.al = view_f16(as_half(w.Xlo[par]), m, n, w.ldn, 2LL * m * w.ldn, B);
@@ -580,8 +670,8 @@ static cudaError_t plan_steps(PolarWS &w, StepPlans &p) {
             memset(&s, 0, sizeof(s));
             s.M = m; s.N = n; s.K = n;
             s.f16_scale = 1.f / (kF16X * kF16P);
-            if (cudaError_t e = plan_gemm(p.apply[par], w.bf16 ? &a16 : nullptr, w.bf16 ? &b16 : nullptr,
-                                          w.mixed ? &ahi : nullptr, nullptr, w.mixed ? &bhi : nullptr, nullptr, s, B, &f))
+            if (cudaError_t e = plan_gemm(p.apply[par], w.bf16 ? &a16 : nullptr, w.bf16 ? &b16 : nullptr, &ahi, &alo,
+                                          &bhi, &blo, s, B, &f))
                 return e;
         }
     }
@@ -607,7 +697,7 @@ static int launch_step(PolarWS &w, StepPlans &plans, int k, bool apply, double t
         EpiGram e;
         e.n = n; e.B = B;
         e.dec = DecideArgs{k, B, n, w.bf16 ? 2 : (w.mixed ? 1 : 0), learned ? 1 : 0, w.kcap, tol, w.done, w.fin,
-                           w.status, w.prec, w.steps, w.fallback, w.notdone, w.res, w.budget, fres};
+                           w.status, w.prec, w.steps, w.fallback, w.notdone, w.res, w.budget, w.fine, fres};
         e.coef = w.coef + (long long)k * B * 2;
         e.prec = w.prec + (long long)k * B;
         e.res = w.res + (long long)k * B;
@@ -647,10 +737,11 @@ static int run_iteration(PolarWS &w, int kmax, double tol, bool learned, float *
     return PSVD_OK;
 }
 
-__global__ void fallback_reset_kernel(int B, int prec0, const int *fallback, int *done, int *prec, int *count) {
+__global__ void fallback_reset_kernel(int B, int prec0, const int *fine, const int *fallback, int *done, int *prec,
+                                      int *count) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
-    if (fallback[b]) { done[b] = 0; prec[b] = prec0; atomicAdd(count, 1); }
+    if (fallback[b]) { done[b] = 0; prec[b] = prec0 == PREC_F16X3 ? fine[b] : prec0; atomicAdd(count, 1); }
     else done[b] = 1;
 }
 
@@ -665,9 +756,9 @@ static int prepare_x0(const float *A, PolarWS &w, cudaStream_t st, const int *sk
     SplitOut r, t;
     r.ld = w.ldn; r.bstride = (long long)m * w.ldn;
     t.ld = w.ldm; t.bstride = (long long)n * w.ldm;
-    // every matrix in the format of its first rung (the lo array only serves split FP16)
+    // every matrix in the format of its first rung
     if (w.bf16) { r.h16 = w.X16[0]; t.h16 = w.XT16[0]; }
-    r.hi = w.Xhi[0]; t.hi = w.XThi[0];
+    r.hi = w.Xhi[0]; r.lo = w.Xlo[0]; t.hi = w.XThi[0]; t.lo = w.XTlo[0];
     r.fhi = as_half(w.Xhi[0]); r.flo = as_half(w.Xlo[0]); r.fbstride = 2 * r.bstride;
     t.fhi = as_half(w.XThi[0]); t.flo = as_half(w.XTlo[0]); t.fbstride = 2 * t.bstride;
     r.fscale = t.fscale = kF16X;
@@ -695,8 +786,8 @@ int polar_forward(const float *A, float *W, float *H_out, bool want_h, PolarWS &
     polar_init_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, prec0, w.done, w.fin, w.status, w.prec, w.steps,
                                                         w.fallback);
     if (l1_norms(A, B, m, n, w.rowsum, w.colsum, w.nonfinite, st) != cudaSuccess) return PSVD_ERR_CUDA;
-    norm_finalize_kernel<<<B, kNormThreads, 0, st>>>(w.rowsum, w.colsum, w.nonfinite, m, n, w.scale, w.ascale, w.done,
-                                                      w.status, w.fin);
+    norm_finalize_kernel<<<B, kNormThreads, 0, st>>>(w.rowsum, w.colsum, w.nonfinite, m, n, w.scale, w.ascale, w.fine, w.prec,
+                                                      w.done, w.status, w.fin);
     count_launch(2);
     // coefficient tables: conservative CANS (Appendix B.8), classical NS, or learned bounds
     CoefTable tab;
@@ -705,17 +796,18 @@ int polar_forward(const float *A, float *W, float *H_out, bool want_h, PolarWS &
     std::vector<Cubic> sched = o.schedule == PSVD_SCHED_NS ? std::vector<Cubic>(1, Cubic{1.5, -0.5, 0.0}) : cons;
     tab.len = (int)sched.size();
     for (int i = 0; i < tab.len; ++i) { tab.c1[i] = (float)sched[i].c1; tab.c3[i] = (float)sched[i].c3; }
-    const int gate_x3 = learned && w.mixed && !w.bf16 ? 1 : 0;
+    const int *gate_fine = learned && w.mixed && !w.bf16 ? w.fine : nullptr;
     schedule_fill_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, w.kcap + 1, tab, o.lower_bound, learned ? 1 : 0,
-                                                          o.tol, o.budget, nullptr, w.coef, w.budget, gate_x3,
+                                                          o.tol, o.budget, nullptr, w.coef, w.budget, gate_fine,
                                                           w.prec, o.schedule == PSVD_SCHED_PE ? 1 : 0);
     count_launch(1);
     if (int rc = prepare_x0(A, w, st, nullptr)) return rc;   // zero matrices get X0 = 0
     if (want_h) {
         SplitOut at;
-        at.fhi = as_half(w.AThi); at.flo = as_half(w.ATlo); at.ld = w.ldm;
-        at.bstride = at.fbstride = (long long)n * w.ldm;
+        at.hi = w.AThi; at.lo = w.ATlo; at.fhi = as_half(w.AThi); at.flo = as_half(w.ATlo); at.ld = w.ldm;
+        at.bstride = (long long)n * w.ldm; at.fbstride = 2 * at.bstride;
         at.fscale = kF16X;
+        at.prec = w.fine;
         // M 2^-e: scale_ptr is divided by, so it gets the inverse, 2^e
         if (prepare_operand(A, n, (long long)m * n, B, m, n, true, 1.f, w.ascale + B, at, st)) return PSVD_ERR_CUDA;
     }
@@ -736,14 +828,14 @@ int polar_forward(const float *A, float *W, float *H_out, bool want_h, PolarWS &
         // conservative schedule.  Nothing is read back: the rerun's steps are launched for the
         // whole budget, gated on the number of rerun matrices (misc[0]) and then on the
         // per-step counts, so without a fallback every one of them returns at once.
-        fallback_reset_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, prec0, w.fallback, w.done, w.prec, w.misc);
+        fallback_reset_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, prec0, w.fine, w.fallback, w.done, w.prec, w.misc);
         count_launch(1);
         CoefTable ct;
         memset(&ct, 0, sizeof(ct));
         ct.len = (int)cons.size();
         for (int i = 0; i < ct.len; ++i) { ct.c1[i] = (float)cons[i].c1; ct.c3[i] = (float)cons[i].c3; }
         schedule_fill_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, w.kcap + 1, ct, nullptr, 0, o.tol, 0,
-                                                              w.fallback, w.coef, w.budget, 0, w.prec);
+                                                              w.fallback, w.coef, w.budget, nullptr, w.prec);
         count_launch(1);
         if (cudaMemsetAsync(w.res, 0, sizeof(double) * (size_t)(w.kcap + 2) * B, st) ||
             cudaMemsetAsync(w.notdone, 0, sizeof(int) * (size_t)(w.kcap + 2), st) ||
@@ -770,16 +862,20 @@ int polar_forward(const float *A, float *W, float *H_out, bool want_h, PolarWS &
         F16Views f;
         f.ah = view_f16(w.wtf_hi(), n, m, w.ldm, 2LL * n * w.ldm, B);
         f.al = view_f16(w.wtf_lo(), n, m, w.ldm, 2LL * n * w.ldm, B);
-        f.bh = view_f16(as_half(w.AThi), n, m, w.ldm, (long long)n * w.ldm, B);
-        f.bl = view_f16(as_half(w.ATlo), n, m, w.ldm, (long long)n * w.ldm, B);
+        f.bh = view_f16(as_half(w.AThi), n, m, w.ldm, 2LL * n * w.ldm, B);
+        f.bl = view_f16(as_half(w.ATlo), n, m, w.ldm, 2LL * n * w.ldm, B);
+        MatView ah = view_of(w.XThi[0], n, m, w.ldm, (long long)n * w.ldm, B);
+        MatView al = view_of(w.XTlo[0], n, m, w.ldm, (long long)n * w.ldm, B);
+        MatView bh = view_of(w.AThi, n, m, w.ldm, (long long)n * w.ldm, B);
+        MatView bl = view_of(w.ATlo, n, m, w.ldm, (long long)n * w.ldm, B);
         GemmShape s;
         memset(&s, 0, sizeof(s));
-        s.M = n; s.N = n; s.K = m; s.prec_uniform = PREC_F16X3; s.err = w.err;
+        s.M = n; s.N = n; s.K = m; s.prec = w.fine; s.err = w.err;
+        s.prof_as = PREC_TF32X3 + 1;       // timed with the FP32-accurate products
         s.f16_scale = 1.f / (kF16X * kF16X);
-        s.f16_scale_b = w.ascale + B;
+        s.scale_b = w.ascale + B;
         EpiStore e = epi_store_plain(w.Hraw, n, (long long)n * n, n, n);
-        if (launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f) != cudaSuccess)
-            return PSVD_ERR_CUDA;
+        if (launch_gemm(nullptr, nullptr, &ah, &al, &bh, &bl, s, B, e, st, &f) != cudaSuccess) return PSVD_ERR_CUDA;
         symmetrize_kernel<<<dim3((n + 31) / 32, (n + 31) / 32, B), dim3(32, 8), 0, st>>>(w.Hraw, n, w.Hsym, H_out);
         count_launch(1);
     }

@@ -12,7 +12,7 @@ namespace psvd {
 #define PSVD_TAU_TF32 2e-3
 #endif
 constexpr double kTauBF16 = PSVD_TAU_BF16;   // mixed path: leave BF16 once the residual is below this
-constexpr double kTauTF32 = PSVD_TAU_TF32;   // ... and TF32 once below this (split-FP16 polish afterwards)
+constexpr double kTauTF32 = PSVD_TAU_TF32;   // ... and TF32 once below this (FP32-accurate polish afterwards)
 
 struct PolarWS {
     int B = 0, m = 0, n = 0, kcap = 0;
@@ -24,14 +24,15 @@ struct PolarWS {
     float *Xhi[2] = {}, *Xlo[2] = {}, *XThi[2] = {}, *XTlo[2] = {};
     __nv_bfloat16 *P16 = nullptr;
     float *Phi = nullptr, *Plo = nullptr;
-    // (split-TF32 never occurs here: the FP32-accurate rung reads split-FP16 halves, as_half(Xhi), ...)
-    float *AThi = nullptr, *ATlo = nullptr;     // M^T split in FP16 halves (for H = W^T M)
+    // (the FP32-accurate rung of a matrix, fine[b], holds split-FP16 halves in them, as_half(Xhi), ..., or split TF32)
+    float *AThi = nullptr, *ATlo = nullptr;     // M^T split the same way (for H = W^T M)
     float *ascale = nullptr;                    // [2][B] power of two below 1/max|M|, and its inverse
     float *Hraw = nullptr;                      // W^T M before symmetrization
     float *Hsym = nullptr;                      // (W^T M)_sym, FP32 copy
     float *rowsum = nullptr, *colsum = nullptr, *scale = nullptr;
     // per-matrix state
     int *done = nullptr, *fin = nullptr, *status = nullptr, *prec = nullptr, *steps = nullptr;
+    int *fine = nullptr;          // [B] PREC_F16X3, or PREC_TF32X3 for a matrix with rows or columns of very small size
     int *budget = nullptr, *fallback = nullptr, *notdone = nullptr, *nonfinite = nullptr;
     double *res = nullptr;
     float *coef = nullptr, *fres = nullptr;
@@ -40,7 +41,8 @@ struct PolarWS {
     unsigned *err = nullptr;
 
     // The final W and W^T, as halves scaled by kF16X (batch stride 2 m ldn / 2 n ldm): the other half of
-    // the lo arrays' space, which no rung uses, so that the conversion is never in place.
+    // the lo arrays' space, which no rung of these matrices uses, so that the conversion is never in place.
+    // Matrices with fine[b] = PREC_TF32X3 have them as split TF32 in Xhi[0], Xlo[0], XThi[0], XTlo[0].
     __half *wf_hi() const { return reinterpret_cast<__half *>(Xlo[0]) + (long long)m * ldn; }
     __half *wf_lo() const { return reinterpret_cast<__half *>(Xlo[1]) + (long long)m * ldn; }
     __half *wtf_hi() const { return reinterpret_cast<__half *>(XTlo[0]) + (long long)n * ldm; }
@@ -74,13 +76,11 @@ struct PolarWS {
         colsum = cv.template take<float>(B64 * l1_slabs(m) * n);
         scale = cv.template take<float>(B64);
         ascale = cv.template take<float>(B64 * 2);
-        done = cv.template take<int>(B64);
-        fin = cv.template take<int>(B64);
-        status = cv.template take<int>(B64);
+        if (int *p = cv.template take<int>(B64 * 6)) {      // (one piece: the scratch of psvd_polar_fwd_noalloc is fixed)
+            done = p; fin = p + B64; status = p + 2 * B64; fine = p + 3 * B64; budget = p + 4 * B64; fallback = p + 5 * B64;
+        }
         prec = cv.template take<int>((long long)(kcap + 2) * B64);
         steps = cv.template take<int>(3 * B64);
-        budget = cv.template take<int>(B64);
-        fallback = cv.template take<int>(B64);
         notdone = cv.template take<int>(kcap + 2);
         nonfinite = cv.template take<int>(B64);
         res = cv.template take<double>((long long)(kcap + 2) * B64);
@@ -99,7 +99,7 @@ inline __half *as_half(float *p) { return reinterpret_cast<__half *>(p); }
 inline int polar_kcap(const psvd_opts &o) { return o.max_iter + (o.schedule == PSVD_SCHED_CANS ? o.pre_iters : 0); }
 
 // Runs the iteration of Algorithm 1 (normalize, schedule, iterate) for all matrices, then
-// writes W (user layout, may be null) and leaves W and W^T as split-FP16 halves (wf_hi(), ...).  If `want_h`, also computes Hsym = (W^T M)_sym (FP64
+// writes W (user layout, may be null) and leaves W and W^T split (wf_hi(), ... or Xhi[0], ... by fine[b]).  If `want_h`, also computes Hsym = (W^T M)_sym (FP64
 // averaging) and copies it to H_out (may be null).  Never synchronizes: the step budget is
 // launched whole and finished matrices are skipped on the device.  Fills info (device,
 // may be null).  With the learned schedule, matrices that miss tol within their budget

@@ -427,10 +427,10 @@ __global__ void x2_split_kernel(const float *X2, int n, long long ld, float *hi)
     hi[(long long)b * n * ld + (long long)i * ld + j] = tf32_round(X2[(long long)b * n * n + (long long)i * n + j]);
 }
 
-// (V E)^T = V^T - X V^T + h V^T (split FP16, the operand of U) and V^T + X V^T + h V^T, in FP32;
-// XV = X V^T (split-TF32 product), HV = h V^T (TF32 product), both n x n.
-__global__ void add_split_kernel(const float *vthi, const float *vtlo, const float *XV, const float *HV, int n,
-                                 long long ld, __half *VEt_hi, __half *VEt_lo, float *VT) {
+// (V E)^T = V^T - X V^T + h V^T, the operand of U (split FP16, or split TF32 over V^T where fine[b] says so), and
+// V^T + X V^T + h V^T, in FP32; XV = X V^T (split-TF32 product), HV = h V^T (TF32 product), both n x n.
+__global__ void add_split_kernel(float *vthi, float *vtlo, const float *XV, const float *HV, int n, long long ld,
+                                 const int *fine, __half *VEt_hi, __half *VEt_lo, float *VT) {
     const int b = blockIdx.z;
     const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
     if (i >= n || j >= n) return;
@@ -440,10 +440,14 @@ __global__ void add_split_kernel(const float *vthi, const float *vtlo, const flo
     const float xv = XV[p], hv = HV[p];
     const float ve = v + (hv - xv);
     const float vn = v + (hv + xv);
-    __half h, l;
-    split_f16(ve * kF16X, h, l);
-    VEt_hi[o] = h;
-    VEt_lo[o] = l;
+    if (fine[b] == PREC_TF32X3) {
+        split_tf32(ve, vthi[o], vtlo[o]);
+    } else {
+        __half h, l;
+        split_f16(ve * kF16X, h, l);
+        VEt_hi[o] = h;
+        VEt_lo[o] = l;
+    }
     VT[p] = vn;
 }
 
@@ -478,7 +482,7 @@ struct SvdWS {
     float *Khi = nullptr, *Klo = nullptr, *T1 = nullptr, *T1hi = nullptr, *T1lo = nullptr, *Kt = nullptr;
     float *X = nullptr, *Xneg = nullptr, *X2 = nullptr, *F = nullptr, *Ft = nullptr;
     __half *VEt = nullptr;       // (V E)^T, split FP16 (hi, then lo)
-    float *VT32hi = nullptr, *VT32lo = nullptr;      // V^T split TF32 (operand of the correction)
+    float *VT32hi = nullptr, *VT32lo = nullptr;      // V^T split TF32 (operand of the correction, and of U by pw.fine)
     unsigned *xmax = nullptr, *kmax = nullptr;
     int *cprec = nullptr;        // [2][B] precision of the correction products (corr_prec_kernel)
     int *mflag = nullptr;
@@ -509,6 +513,8 @@ struct SvdWS {
             qbar = cv.template take<unsigned>(4);
         }
         mflag = cv.template take<int>(B64);
+        VT32hi = cv.template take<float>(B64 * nn);
+        VT32lo = cv.template take<float>(B64 * nn);
         if (mixed) {
             Vhi = cv.template take<float>(B64 * nn);
             Vlo = cv.template take<float>(B64 * nn);
@@ -524,8 +530,6 @@ struct SvdWS {
             F = cv.template take<float>(B64 * nn);
             Ft = cv.template take<float>(B64 * nn);
             VEt = cv.template take<__half>(B64 * nn * 2);
-            VT32hi = cv.template take<float>(B64 * nn);
-            VT32lo = cv.template take<float>(B64 * nn);
             xmax = cv.template take<unsigned>(B64);
             kmax = cv.template take<unsigned>(B64);
             cprec = cv.template take<int>(B64 * 2);
@@ -575,9 +579,10 @@ int svd_forward(const float *A, float *U, float *Sout, float *VT, SvdWS &w, cons
     if (cudaMemsetAsync(w.any, 0, sizeof(int) * 4, st)) return PSVD_ERR_CUDA;
     // a learned schedule's misses are recomputed with the rest of the rerun (below), not here
     if (int rc = polar_forward(A, nullptr, nullptr, true, p, o, info, st, false)) return rc;
-    if (int rc = eigh_forward(p.Hsym, Sout, w.mixed ? nullptr : VT, w.ew, st, w.VT32hi, w.VT32lo)) return rc;
+    if (int rc = eigh_forward(p.Hsym, Sout, w.mixed ? nullptr : VT, w.ew, st, w.VT32hi, w.VT32lo,
+                              w.mixed ? nullptr : p.fine)) return rc;
     if (cudaMemcpyAsync(w.S, Sout, sizeof(float) * (size_t)B * n, cudaMemcpyDeviceToDevice, st)) return PSVD_ERR_CUDA;
-    const float *vthi = w.VT32hi, *vtlo = w.VT32lo;  // (mixed only) split TF32
+    float *vthi = w.VT32hi, *vtlo = w.VT32lo;        // split TF32 (plain: of the matrices with fine[b] = PREC_TF32X3)
     const __half *bu_hi = w.ew.VThi, *bu_lo = w.ew.VTlo;        // B operand of U = W V: rows of V^T
     dim3 g16((n + 15) / 16, (n + 15) / 16, B), b16(16, 16);
     if (w.mixed) {
@@ -620,7 +625,7 @@ int svd_forward(const float *A, float *U, float *Sout, float *VT, SvdWS &w, cons
         if (int rc = gemm3p(w.X, w.Ft, n, n, ld, nn, w.Vhi, w.Vlo, n, ld, nn, B, w.cprec + B, e4, p.err, st)) return rc;
         EpiStore e5 = epi_store_plain(w.Kt, n, (long long)n * n, n, n);
         if (int rc = gemm1(w.F, n, n, ld, nn, w.Vhi, n, ld, nn, B, e5, p.err, st)) return rc;
-        add_split_kernel<<<g16, b16, 0, st>>>(vthi, vtlo, w.T1, w.Kt, n, ld, VEt_hi, VEt_lo, VT);
+        add_split_kernel<<<g16, b16, 0, st>>>(vthi, vtlo, w.T1, w.Kt, n, ld, p.fine, VEt_hi, VEt_lo, VT);
         count_launch(1);
         bu_hi = VEt_hi;
         bu_lo = VEt_lo;
@@ -637,10 +642,13 @@ int svd_forward(const float *A, float *U, float *Sout, float *VT, SvdWS &w, cons
         f.bl = view_f16(bu_lo, n, n, ld, nn, B);
         GemmShape s;
         memset(&s, 0, sizeof(s));
-        s.M = m; s.N = n; s.K = n; s.prec_uniform = PREC_F16X3; s.err = p.err;
+        s.M = m; s.N = n; s.K = n; s.prec = p.fine; s.err = p.err;
         s.f16_scale = 1.f / (kF16X * kF16X);
-        if (launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f) != cudaSuccess)
-            return PSVD_ERR_CUDA;
+        s.prof_as = PREC_TF32X3 + 1;
+        MatView ah = view_of(p.Xhi[0], m, n, p.ldn, (long long)m * p.ldn, B);
+        MatView al = view_of(p.Xlo[0], m, n, p.ldn, (long long)m * p.ldn, B);
+        MatView bh = view_of(vthi, n, n, ld, nn, B), bl = view_of(vtlo, n, n, ld, nn, B);
+        if (launch_gemm(nullptr, nullptr, &ah, &al, &bh, &bl, s, B, e, st, &f) != cudaSuccess) return PSVD_ERR_CUDA;
     }
     qr_flag_kernel<<<B, 256, 0, st>>>(w.colss, n, o.eps_qr, w.learned ? p.fallback : nullptr, w.flag, w.any);
     count_launch(1);

@@ -27,8 +27,8 @@ def _full(m, n):
     return _orth(7, m, n) @ ((_orth(8, n, n) * np.linspace(1.0, 4.0, n)) @ _orth(9, n, n).T)
 
 
-@pytest.mark.parametrize("n", [24, 200])
-@pytest.mark.parametrize("t", [1e-3, 1e-5, 1e-7])
+@pytest.mark.parametrize("n", [24, 200, 257])
+@pytest.mark.parametrize("t", [1e-3, 1e-5, 1e-7, 1e-9])
 def test_polar_columns(n, t):
     """Half of the columns t times the size of the others: the columns of W, and the blocks of H."""
     import paper_2609_32505_gb300 as P
@@ -44,9 +44,8 @@ def test_polar_columns(n, t):
         assert _rel(h[c, c], h0[c, c]) <= 1e-5
 
 
-@pytest.mark.parametrize("m,n", [(400, 100), (260, 17)])
-@pytest.mark.parametrize("t", [1e-4, 1e-6])
-@pytest.mark.parametrize("preqr", [0, 1])
+@pytest.mark.parametrize("m,n", [(400, 100), (260, 17), (700, 272)])
+@pytest.mark.parametrize("t,preqr", [(1e-4, 0), (1e-6, 0), (1e-8, 0), (1e-12, 0), (1e-4, 1), (1e-6, 1)])
 def test_polar_and_svd_rows(m, n, t, preqr):
     """Half of the rows t times the size of the others: W, and U diag(s) V^T, in either half."""
     import paper_2609_32505_gb300 as P
@@ -62,6 +61,36 @@ def test_polar_and_svd_rows(m, n, t, preqr):
     for r in (slice(0, m // 2), slice(m // 2, m)):
         assert _rel(w[r], ref[r]) <= 1e-5
         assert _rel(((u * s) @ vt)[r], g[r]) <= 1e-5
+
+
+@pytest.mark.parametrize("schedule", ["cans", "learned"])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_polar_batch_of_ranges(precision, schedule):
+    """One batch with ordinary matrices between such of a wide range, every rung and the conservative rerun: the
+    ordinary ones have the bits that they have in a batch of their own, the others' W is right in their small parts."""
+    import paper_2609_32505_gb300 as P
+    m, n = 300, 130
+    a = np.stack([_full(m, n)] * 4)
+    a[1, :, :50] *= 1e-8
+    a[2, :, 7:90] *= 1e-6
+    a[3, 200:] *= 1e-10
+    A = torch.from_numpy(a.astype(np.float32)).cuda()
+    kw = {"precision": precision, "max_iter": 64}
+    if schedule == "learned":                     # far too high for matrices 1 and 2, which are then run again
+        kw.update(schedule=P.SCHED_LEARNED, lower_bound=torch.full((4,), 0.05, device="cuda"))
+    w, h, info = P.polar(A, P.make_opts(**kw), return_info=True)
+    assert all(i["status"] == 0 for i in info), info
+    if schedule == "learned":
+        kw["lower_bound"] = kw["lower_bound"][:1]
+    w0, h0 = P.polar(A[:1], P.make_opts(**kw))
+    assert torch.equal(w[0], w0[0]) and torch.equal(h[0], h0[0])
+    if precision:
+        return
+    w = w.cpu().double().numpy()
+    for b, part in [(1, np.s_[:, :50]), (2, np.s_[:, 7:90]), (3, np.s_[200:])]:
+        u, _, vt = np.linalg.svd(A[b].cpu().double().numpy(), full_matrices=False)
+        assert _rel(w[b], u @ vt) <= 1e-5
+        assert _rel(w[b][part], (u @ vt)[part]) <= 1e-5
 
 
 @pytest.mark.parametrize("t", [1.0, 1e-3, 1e-6, 1e-8])
