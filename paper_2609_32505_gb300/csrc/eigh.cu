@@ -1520,7 +1520,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
                 GemmShape s;
                 memset(&s, 0, sizeof(s));
                 s.M = n; s.N = Lr; s.K = nb; s.prec_uniform = PREC_F16X3; s.err = w.err;
-                EpiSubHalf e;
+                EpiSubHalf e{};
                 e.rows = n; e.cols = Lr; e.hi = w.VThi + r0; e.lo = w.VTlo + r0; e.ld = ldn;
                 e.bs = (long long)n * ldn; e.scale = kF16X; e.inv = 1.f / kF16X;
                 s.f16_scale = 1.f / (kF16S2 * kF16V);
@@ -1572,7 +1572,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
                 GemmShape s;
                 memset(&s, 0, sizeof(s));
                 s.M = n; s.N = Lr; s.K = W; s.prec_uniform = PREC_F16X3; s.err = w.err;
-                EpiSubHalf e;
+                EpiSubHalf e{};
                 e.rows = n; e.cols = Lr; e.hi = w.VThi + r0; e.lo = w.VTlo + r0; e.ld = ldn;
                 e.bs = (long long)n * ldn; e.scale = kF16X; e.inv = 1.f / kF16X;
                 s.f16_scale = 1.f / (kF16S2 * kF16V);

@@ -188,32 +188,58 @@ cudaError_t prepare_operand(const float *src, long long lds, long long bss, int 
     return e;
 }
 
+__global__ void fine_reset_kernel(int *fine, int B) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < B) fine[b] = PREC_F16X3;
+}
+cudaError_t fine_reset(int *fine, int B, cudaStream_t st) {
+    fine_reset_kernel<<<(B + 127) / 128, 128, 0, st>>>(fine, B);
+    count_launch(1);
+    return cudaGetLastError();
+}
+// One warp per row.  Entries x 2^14 are held to 22 bits down to 2^-28 (split_f16), so a row with a largest
+// entry above sqrt(n) 2^-28 has no more rounding error in halves than in split TF32.
+__global__ void __launch_bounds__(256) fine_rows_kernel(const float *A, int m, int n, const float *colscale,
+                                                        const int *skip, float lim, int *fine) {
+    const int b = blockIdx.y, lane = threadIdx.x & 31, r = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (r >= m || (skip && skip[b])) return;
+    const float *a = A + ((long long)b * m + r) * n, *cs = colscale ? colscale + (long long)b * n : nullptr;
+    float v = 0.f;
+#pragma unroll 8
+    for (int c = lane; c < n; c += 32) v = fmaxf(v, fabsf(a[c]) * (cs ? cs[c] : 1.f));
+    v = warp_max(v);
+    if (lane == 0 && v > 0.f && v < lim) fine[b] = PREC_TF32X3;
+}
+cudaError_t fine_rows(const float *A, int B, int m, int n, const float *colscale, const int *skip, int *fine,
+                      cudaStream_t st) {
+    fine_rows_kernel<<<dim3((m + 7) / 8, B), 256, 0, st>>>(A, m, n, colscale, skip, sqrtf((float)n) * 0x1p-28f, fine);
+    count_launch(1);
+    return cudaGetLastError();
+}
+
 // out = Q X for the preprocessed route (Q: B x M x N, X: B x N x N, both with orthonormal columns), operands
-// split FP16 in scratch carved from cv.  (4 x 14336 x 4096 x 4096: 3.8 ms, in split TF32 7.0 ms.)
+// split FP16 (split TF32 where rows of Q are very small) in scratch carved from cv.  (4 x 14336 x 4096 x 4096: 3.8 ms, in
+// split TF32 7.0 ms.)
 int orth_product(Carver &cv, const float *Q, const float *X, float *out, int B, int M, int N, cudaStream_t st) {
     const long long ld = pad_ld(N), qs = (long long)M * ld, xs = (long long)N * ld;
-    __half *qhi = cv.take<__half>((size_t)B * qs), *qlo = cv.take<__half>((size_t)B * qs);
-    __half *xhi = cv.take<__half>((size_t)B * xs), *xlo = cv.take<__half>((size_t)B * xs);
+    float *qhi = cv.take<float>((size_t)B * qs), *qlo = cv.take<float>((size_t)B * qs);
+    float *xhi = cv.take<float>((size_t)B * xs), *xlo = cv.take<float>((size_t)B * xs);
+    int *fine = cv.take<int>(B);
     unsigned *err = cv.take<unsigned>(4);
     if (cv.overflow) return PSVD_ERR_WORKSPACE;
-    SplitOut a, bt;
-    a.fhi = qhi; a.flo = qlo; a.ld = ld; a.bstride = a.fbstride = qs;
-    bt.fhi = xhi; bt.flo = xlo; bt.ld = ld; bt.bstride = bt.fbstride = xs;
-    a.fscale = bt.fscale = kF16X;
+    PSVD_TRY(fine_reset(fine, B, st));
+    PSVD_TRY(fine_rows(Q, B, M, N, nullptr, nullptr, fine, st));
+    SplitOut a = split_out(qhi, qlo, ld, qs, kF16X, fine), bt = split_out(xhi, xlo, ld, xs, kF16X, fine);
     PSVD_TRY(prepare_operand(Q, N, (long long)M * N, B, M, N, false, 1.f, nullptr, a, st));
     // B operand B[k][j] = X[j][k] (X transposed)
     PSVD_TRY(prepare_operand(X, N, (long long)N * N, B, N, N, true, 1.f, nullptr, bt, st));
-    F16Views f;
-    f.ah = view_f16(qhi, M, N, ld, qs, B);
-    f.al = view_f16(qlo, M, N, ld, qs, B);
-    f.bh = view_f16(xhi, N, N, ld, xs, B);
-    f.bl = view_f16(xlo, N, N, ld, xs, B);
     GemmShape s;
     memset(&s, 0, sizeof(s));
-    s.M = M; s.N = N; s.K = N; s.prec_uniform = PREC_F16X3; s.err = err;
+    s.M = M; s.N = N; s.K = N; s.prec = fine; s.err = err;
     s.f16_scale = 1.f / (kF16X * kF16X);
+    s.prof_as = PREC_TF32X3 + 1;
     EpiStore e = epi_store_plain(out, N, (long long)M * N, M, N);
-    PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
+    PSVD_TRY(launch_split(SplitView(qhi, qlo, 0, M, N, ld, qs, B), SplitView(xhi, xlo, 0, N, N, ld, xs, B), s, B, e, st));
     return PSVD_OK;
 }
 

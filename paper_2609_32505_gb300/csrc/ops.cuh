@@ -32,6 +32,15 @@ struct SplitOut {
     long long ld = 0, bstride = 0, fbstride = 0;
 };
 
+// Both split formats of arrays with room for floats (batch stride bs floats), by prec[b].
+inline SplitOut split_out(float *hi, float *lo, long long ld, long long bs, float fscale, const int *prec) {
+    SplitOut s;
+    s.hi = hi; s.lo = lo; s.fhi = reinterpret_cast<__half *>(hi); s.flo = reinterpret_cast<__half *>(lo);
+    s.ld = ld; s.bstride = bs; s.fbstride = 2 * bs;
+    s.fscale = fscale; s.prec = prec;
+    return s;
+}
+
 // Powers of two that bring split-FP16 operands below 2^16: polar iterates (singular values <= 2 at
 // every step of every schedule) and orthonormal factors; the step polynomial c1 I + c3 G
 // (entries <= 5.2: c1 = 3 sqrt(3) on [0, 1]); Householder vectors (entries <= 1); the back-transform's S2 = S T^T.
@@ -58,6 +67,49 @@ inline MatView view_f16(const __half *p, int rows, int cols, long long ld, long 
     MatView v; v.ptr = p; v.rows = rows; v.cols = cols; v.ld = ld; v.bstride = bs; v.batch = batch; v.f16 = true;
     return v;
 }
+
+// A split array whose matrices are each in one of the two split formats (fine[b] = PREC_F16X3 or PREC_TF32X3) has
+// room for floats; halves lie at the start of their matrix's space, so their batch stride is twice that of floats.
+__host__ __device__ inline __half *as_half(float *p) { return reinterpret_cast<__half *>(p); }
+__host__ __device__ inline const __half *as_half(const float *p) { return reinterpret_cast<const __half *>(p); }
+// element o of the matrix that starts at float bo: x * fs as halves, or x as it is
+PSVD_DEV void split_store(bool wide, float *hi, float *lo, long long bo, long long o, float x, float fs) {
+    if (wide) {
+        float h, l;
+        split_tf32(x, h, l);
+        hi[bo + o] = h;
+        lo[bo + o] = l;
+    } else {
+        __half h, l;
+        split_f16(x * fs, h, l);
+        as_half(hi)[2 * bo + o] = h;
+        as_half(lo)[2 * bo + o] = l;
+    }
+}
+PSVD_DEV float split_load(bool wide, const float *hi, const float *lo, long long bo, long long o, float inv) {
+    return wide ? hi[bo + o] + lo[bo + o] : join_f16(as_half(hi)[2 * bo + o], as_half(lo)[2 * bo + o]) * inv;
+}
+// the two pairs of views of a split array, `off` elements into every matrix
+struct SplitView {
+    MatView h, l, fh, fl;
+    SplitView(const float *hi, const float *lo, long long off, int rows, int cols, long long ld, long long bs, int batch)
+        : h(view_f16(as_half(hi) + off, rows, cols, ld, 2 * bs, batch)),
+          l(view_f16(as_half(lo) + off, rows, cols, ld, 2 * bs, batch)),
+          fh(view_of(hi + off, rows, cols, ld, bs, batch)), fl(view_of(lo + off, rows, cols, ld, bs, batch)) {}
+};
+// product of two of them, s.prec = fine
+template <class Epi>
+cudaError_t launch_split(const SplitView &a, const SplitView &b, const GemmShape &s, int batch, const Epi &e,
+                         cudaStream_t st) {
+    const F16Views f{a.h, a.l, b.h, b.l};
+    return launch_gemm(nullptr, nullptr, &a.fh, &a.fl, &b.fh, &b.fl, s, batch, e, st, &f);
+}
+
+// fine[b] = PREC_F16X3 for all b; then PREC_TF32X3 for matrices with a nonzero row of A (B x m x n, columns times
+// colscale) whose entries are so small that FP16 halves of them, bound 1, lose bits.
+cudaError_t fine_reset(int *fine, int B, cudaStream_t st);
+cudaError_t fine_rows(const float *A, int B, int m, int n, const float *colscale, const int *skip, int *fine,
+                      cudaStream_t st);
 
 // Generic epilogue: D = alpha * acc (+ beta * C) stored row-major, transposed,
 // and/or split into TF32 hi/lo halves (row-major or transposed).
@@ -142,16 +194,20 @@ struct EpiStore {
 };
 
 // In place: X[r][c] -= acc for a matrix kept as FP16 halves of x * scale (the eigensolver's back-transform,
-// the QR's trailing updates).
+// the QR's trailing updates), or as split TF32 at fhi / flo where fine[b] says so.
 struct EpiSubHalf {
     int rows, cols;
     __half *hi, *lo;
     long long ld, bs;
     float scale, inv;
+    const int *fine;              // null: halves
+    float *fhi, *flo;
+    long long fbs;
     struct Acc {};
     static constexpr bool kElem = true, kRow = true;
     PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
         if (r0 >= rows || c0 >= cols) return true;
+        if (fine && fine[b] == PREC_TF32X3) return false;
         if (c0 + 16 > cols || (((uintptr_t)hi | (uintptr_t)lo) & 31) || ((ld | bs) & 15)) return false;
         if (r0 + lane >= rows) return true;
         const long long o = b * bs + (long long)(r0 + lane) * ld + c0;
@@ -173,6 +229,11 @@ struct EpiSubHalf {
     PSVD_DEV bool staged() const { return true; }
     PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
         if (r >= rows || c >= cols) return;
+        if (fine && fine[b] == PREC_TF32X3) {
+            const long long o = b * fbs + (long long)r * ld + c;
+            split_tf32((fhi[o] + flo[o]) - v, fhi[o], flo[o]);
+            return;
+        }
         const long long o = b * bs + (long long)r * ld + c;
         __half h, l;
         split_f16((join_f16(hi[o], lo[o]) * inv - v) * scale, h, l);

@@ -260,18 +260,11 @@ PSVD_DEV void store_prec(int p, long long o, float x, __nv_bfloat16 *p16, float 
     if (p == PREC_BF16) p16[o] = __float2bfloat16_rn(x);
     else phi[o] = tf32_round(x);
 }
-// the same with the split-FP16 rung: halves of x * fs at element of (stride of a batch entry doubled); split TF32
-// is wide_piece's
-PSVD_DEV void store_rung(int p, long long o, long long of, float x, float fs, __nv_bfloat16 *p16, float *phi,
+// the same with the split-FP16 rung (split TF32 is wide_piece's); bo: start of the matrix
+PSVD_DEV void store_rung(int p, long long bo, long long o, float x, float fs, __nv_bfloat16 *p16, float *phi,
                          float *plo) {
-    if (p == PREC_F16X3) {
-        __half h, l;
-        split_f16(x * fs, h, l);
-        reinterpret_cast<__half *>(phi)[of] = h;
-        reinterpret_cast<__half *>(plo)[of] = l;
-    } else {
-        store_prec(p, o, x, p16, phi);
-    }
+    if (p == PREC_F16X3) split_store(false, phi, plo, bo, o, x, fs);
+    else store_prec(p, bo + o, x, p16, phi);
 }
 
 // The split-TF32 rung of matrices of a wide range: a warp's piece of 32 rows x 16 columns from (r0, c0) on, of
@@ -430,7 +423,7 @@ struct EpiGram {
         a.r = ff_fma(a.r, r == c ? d : 2.f * d, d);
         const float pv = a.c3 * g + (r == c ? a.c1 : 0.f);
         const long long bo = (long long)b * n * ldp, rc = (long long)r * ldp + c;
-        store_rung(a.p, bo + rc, 2 * bo + rc, pv, kF16P, P16, Phi, Plo);
+        store_rung(a.p, bo, rc, pv, kF16P, P16, Phi, Plo);
     }
     PSVD_DEV void trans(Acc &a, int b, int r, int c0, float (&v)[16]) const {
         if (r >= n) return;
@@ -442,7 +435,7 @@ struct EpiGram {
             if (c >= n) break;
             if (c <= r) continue;
             const long long rc = (long long)c * ldp + r;
-            store_rung(a.p, bo + rc, 2 * bo + rc, a.c3 * v[i], kF16P, P16, Phi, Plo);
+            store_rung(a.p, bo, rc, a.c3 * v[i], kF16P, P16, Phi, Plo);
         }
     }
     PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
@@ -490,7 +483,7 @@ struct EpiApply {
         if (r >= m || c >= n) return;
         if (a.p < 0) a.p = prec_next[b];
         const long long bo = (long long)b * m * ldn, rc = (long long)r * ldn + c;
-        store_rung(a.p, bo + rc, 2 * bo + rc, x, kF16X, X16, Xhi, Xlo);
+        store_rung(a.p, bo, rc, x, kF16X, X16, Xhi, Xlo);
     }
     PSVD_DEV void trans(Acc &a, int b, int r, int c0, float (&v)[16]) const {
         if (r >= m) return;
@@ -501,7 +494,7 @@ struct EpiApply {
             const int c = c0 + i;
             if (c >= n) break;
             const long long rc = (long long)c * ldm + r;
-            store_rung(a.p, bo + rc, 2 * bo + rc, v[i], kF16X, XT16, XThi, XTlo);
+            store_rung(a.p, bo, rc, v[i], kF16X, XT16, XThi, XTlo);
         }
     }
     PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
@@ -753,16 +746,10 @@ __global__ void set_all_done_kernel(int B, int *done) {
 
 static int prepare_x0(const float *A, PolarWS &w, cudaStream_t st, const int *skip) {
     const int B = w.B, m = w.m, n = w.n;
-    SplitOut r, t;
-    r.ld = w.ldn; r.bstride = (long long)m * w.ldn;
-    t.ld = w.ldm; t.bstride = (long long)n * w.ldm;
     // every matrix in the format of its first rung
+    SplitOut r = split_out(w.Xhi[0], w.Xlo[0], w.ldn, (long long)m * w.ldn, kF16X, w.prec);
+    SplitOut t = split_out(w.XThi[0], w.XTlo[0], w.ldm, (long long)n * w.ldm, kF16X, w.prec);
     if (w.bf16) { r.h16 = w.X16[0]; t.h16 = w.XT16[0]; }
-    r.hi = w.Xhi[0]; r.lo = w.Xlo[0]; t.hi = w.XThi[0]; t.lo = w.XTlo[0];
-    r.fhi = as_half(w.Xhi[0]); r.flo = as_half(w.Xlo[0]); r.fbstride = 2 * r.bstride;
-    t.fhi = as_half(w.XThi[0]); t.flo = as_half(w.XTlo[0]); t.fbstride = 2 * t.bstride;
-    r.fscale = t.fscale = kF16X;
-    r.prec = t.prec = w.prec;
     if (prepare_operand(A, n, (long long)m * n, B, m, n, false, 1.f, w.scale, r, st, skip) ||
         prepare_operand(A, n, (long long)m * n, B, m, n, true, 1.f, w.scale, t, st, skip))
         return PSVD_ERR_CUDA;
@@ -803,11 +790,7 @@ int polar_forward(const float *A, float *W, float *H_out, bool want_h, PolarWS &
     count_launch(1);
     if (int rc = prepare_x0(A, w, st, nullptr)) return rc;   // zero matrices get X0 = 0
     if (want_h) {
-        SplitOut at;
-        at.hi = w.AThi; at.lo = w.ATlo; at.fhi = as_half(w.AThi); at.flo = as_half(w.ATlo); at.ld = w.ldm;
-        at.bstride = (long long)n * w.ldm; at.fbstride = 2 * at.bstride;
-        at.fscale = kF16X;
-        at.prec = w.fine;
+        const SplitOut at = split_out(w.AThi, w.ATlo, w.ldm, (long long)n * w.ldm, kF16X, w.fine);
         // M 2^-e: scale_ptr is divided by, so it gets the inverse, 2^e
         if (prepare_operand(A, n, (long long)m * n, B, m, n, true, 1.f, w.ascale + B, at, st)) return PSVD_ERR_CUDA;
     }
@@ -936,7 +919,7 @@ struct PolarPreqr {
         QrWS qw;
         qw.carve(q, (int)B, (int)m, (int)n);
         const long long ld = pad_ld(n);
-        const size_t ops = (size_t)(2 * B * m * ld + 2 * B * n * ld) * sizeof(__half) + 2048;
+        const size_t ops = (size_t)(2 * B * m * ld + 2 * B * n * ld) * sizeof(float) + 4096 + 4 * (size_t)B;
         need = head + std::max(std::max(q.used + 256, polar_direct_bytes(B, n, n, o)), ops);
         rest = ws ? static_cast<char *>(ws) + head : nullptr;
         rest_bytes = ws_bytes > head ? ws_bytes - head : 0;

@@ -92,10 +92,6 @@ struct PolarWS {
     }
 };
 
-// Split-FP16 halves of the FP32-accurate rung live in the memory of the float arrays: matrix b starts
-// where its float matrix does and its halves fill the first half of that space.
-inline __half *as_half(float *p) { return reinterpret_cast<__half *>(p); }
-
 inline int polar_kcap(const psvd_opts &o) { return o.max_iter + (o.schedule == PSVD_SCHED_CANS ? o.pre_iters : 0); }
 
 // Runs the iteration of Algorithm 1 (normalize, schedule, iterate) for all matrices, then

@@ -3,7 +3,7 @@
 //
 // Every column is scaled by its own power of two to a norm <= 1 (A D = Q (R D), exactly, so the scales only come
 // back on R's columns, and a small column beside large ones keeps its accuracy) and the matrix kept transposed
-// and split into FP16 hi/lo halves (UT: row j = column j).  Panels of nb columns are factored by one thread-block
+// and split into FP16 hi/lo halves (UT: row j = column j), or, with rows of very small size, into split TF32.  Panels of nb columns are factored by one thread-block
 // cluster per matrix: each of its CTAs holds a slab of the panel's rows in registers, and the
 // per-column dot products (the norm below the diagonal and the projections of the later panel
 // columns) are summed across the cluster through distributed shared memory -- one cluster barrier
@@ -37,10 +37,39 @@ bool qr_shape(int m, int *nb) {
     return m <= 23024;
 }
 
+// four consecutive elements of a split array
+PSVD_DEV void split_load4(bool wide, const float *hi, const float *lo, long long bo, long long o, float inv, float (&x)[4]) {
+    if (wide) {
+        const float4 h = *reinterpret_cast<const float4 *>(hi + bo + o), l = *reinterpret_cast<const float4 *>(lo + bo + o);
+        x[0] = h.x + l.x; x[1] = h.y + l.y; x[2] = h.z + l.z; x[3] = h.w + l.w;
+    } else {
+        __align__(8) __half h[4], l[4];
+        *reinterpret_cast<uint2 *>(h) = *reinterpret_cast<const uint2 *>(as_half(hi) + 2 * bo + o);
+        *reinterpret_cast<uint2 *>(l) = *reinterpret_cast<const uint2 *>(as_half(lo) + 2 * bo + o);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = join_f16(h[e], l[e]) * inv;
+    }
+}
+PSVD_DEV void split_store4(bool wide, float *hi, float *lo, long long bo, long long o, const float (&x)[4], float fs) {
+    if (wide) {
+        float h[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) split_tf32(x[e], h[e], l[e]);
+        *reinterpret_cast<float4 *>(hi + bo + o) = make_float4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<float4 *>(lo + bo + o) = make_float4(l[0], l[1], l[2], l[3]);
+    } else {
+        __align__(8) __half h[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) split_f16(x[e] * fs, h[e], l[e]);
+        *reinterpret_cast<uint2 *>(as_half(hi) + 2 * bo + o) = *reinterpret_cast<const uint2 *>(h);
+        *reinterpret_cast<uint2 *>(as_half(lo) + 2 * bo + o) = *reinterpret_cast<const uint2 *>(l);
+    }
+}
+
 struct PanelArgs {
-    __half *UThi, *UTlo, *YThi, *YTlo, *Yhi, *Ylo;
+    float *UThi, *UTlo, *YThi, *YTlo, *Yhi, *Ylo;    // (split arrays, formats by fine)
     float *tau, *beta, *Tm;
-    const int *skip;
+    const int *skip, *fine;
     int m, n, j0, pw, panel, npan, cl;
     long long ldm, ldn;
 };
@@ -91,6 +120,7 @@ __global__ void __launch_bounds__(kQrThreads, 1) qr_panel_kernel(PanelArgs P) {
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int r0 = j0 + rank * S;                    // multiple of 4
     const long long ubase = (long long)b * n * P.ldm;
+    const bool wide = P.fine[b] == PREC_TF32X3;
 
     float a[C][RPL];
 #pragma unroll
@@ -98,15 +128,10 @@ __global__ void __launch_bounds__(kQrThreads, 1) qr_panel_kernel(PanelArgs P) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const int c = k * kQrWarps + w, r = r0 + 128 * i + 4 * lane;
-            __align__(8) __half h[4], l[4];
-            *reinterpret_cast<uint2 *>(h) = *reinterpret_cast<uint2 *>(l) = make_uint2(0u, 0u);
-            if (c < pw && r < m) {                   // (the padding of a row takes part as zeros)
-                const long long o = ubase + (long long)(j0 + c) * P.ldm + r;
-                *reinterpret_cast<uint2 *>(h) = *reinterpret_cast<const uint2 *>(P.UThi + o);
-                *reinterpret_cast<uint2 *>(l) = *reinterpret_cast<const uint2 *>(P.UTlo + o);
-            }
+            float x[4] = {0.f, 0.f, 0.f, 0.f};
+            if (c < pw && r < m) split_load4(wide, P.UThi, P.UTlo, ubase, (long long)(j0 + c) * P.ldm + r, 1.f / kF16X, x);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) a[k][4 * i + e] = r + e < m ? join_f16(h[e], l[e]) * (1.f / kF16X) : 0.f;
+            for (int e = 0; e < 4; ++e) a[k][4 * i + e] = r + e < m ? x[e] : 0.f;   // (the padding of a row takes part as zeros)
         }
     // column c (this warp's index k) to shared memory, zero in rows <= c of CTA 0
     auto publish = [&](const float (&col)[RPL], int c) {
@@ -255,41 +280,37 @@ __global__ void __launch_bounds__(kQrThreads, 1) qr_panel_kernel(PanelArgs P) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const int rl = 128 * i + 4 * lane, r = r0 + rl;
-            __align__(8) __half uh[4], ul[4], yh[4], yl[4];
+            float u[4], y[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float v = a[k][4 * i + e];
+                u[e] = a[k][4 * i + e];
                 const int d = r + e - (j0 + c);
-                const float y = d < 0 ? 0.f : (d == 0 ? 1.f : v);
-                split_f16(v * kF16X, uh[e], ul[e]);
-                split_f16(y * kF16V, yh[e], yl[e]);
-                sm.slab[c][rl + e] = y;
+                y[e] = d < 0 ? 0.f : (d == 0 ? 1.f : u[e]);
+                sm.slab[c][rl + e] = y[e];
             }
             if (c < pw && r < m) {                   // rows of UT and YT are padded to multiples of 32
-                const long long o = ubase + (long long)(j0 + c) * P.ldm + r;
-                *reinterpret_cast<uint2 *>(P.UThi + o) = *reinterpret_cast<const uint2 *>(uh);
-                *reinterpret_cast<uint2 *>(P.UTlo + o) = *reinterpret_cast<const uint2 *>(ul);
-                *reinterpret_cast<uint2 *>(P.YThi + o) = *reinterpret_cast<const uint2 *>(yh);
-                *reinterpret_cast<uint2 *>(P.YTlo + o) = *reinterpret_cast<const uint2 *>(yl);
+                const long long o = (long long)(j0 + c) * P.ldm + r;
+                split_store4(wide, P.UThi, P.UTlo, ubase, o, u, kF16X);
+                split_store4(wide, P.YThi, P.YTlo, ubase, o, y, kF16V);
             }
         }
     }
     __syncthreads();
-    const long long ybase = (long long)b * m * P.ldn + j0;
+    const long long ybase = (long long)b * m * P.ldn;
     {
         const int c = 2 * (tid % (NB / 2)), nr = min(S, m - r0);
         for (int rl = tid / (NB / 2); rl < nr; rl += kQrThreads / (NB / 2)) {
             if (c >= pw) continue;
-            __half h0, l0, h1, l1;
-            split_f16(sm.slab[c][rl] * kF16V, h0, l0);
-            split_f16(sm.slab[c + 1][rl] * kF16V, h1, l1);
-            const long long o = ybase + (long long)(r0 + rl) * P.ldn + c;
-            if (c + 1 < pw) {
-                *reinterpret_cast<__half2 *>(P.Yhi + o) = __halves2half2(h0, h1);
-                *reinterpret_cast<__half2 *>(P.Ylo + o) = __halves2half2(l0, l1);
+            const long long o = (long long)(r0 + rl) * P.ldn + j0 + c;
+            if (!wide && c + 1 < pw) {
+                __half h0, l0, h1, l1;
+                split_f16(sm.slab[c][rl] * kF16V, h0, l0);
+                split_f16(sm.slab[c + 1][rl] * kF16V, h1, l1);
+                *reinterpret_cast<__half2 *>(as_half(P.Yhi) + 2 * ybase + o) = __halves2half2(h0, h1);
+                *reinterpret_cast<__half2 *>(as_half(P.Ylo) + 2 * ybase + o) = __halves2half2(l0, l1);
             } else {
-                P.Yhi[o] = h0;
-                P.Ylo[o] = l0;
+                split_store(wide, P.Yhi, P.Ylo, ybase, o, sm.slab[c][rl], kF16V);
+                if (c + 1 < pw) split_store(wide, P.Yhi, P.Ylo, ybase, o + 1, sm.slab[c + 1][rl], kF16V);
             }
         }
     }
@@ -298,12 +319,8 @@ __global__ void __launch_bounds__(kQrThreads, 1) qr_panel_kernel(PanelArgs P) {
     if (rank == CL - 1)
         for (int t = tid; t < (j0 - s0) * pw; t += blockDim.x) {
             const int rr = t / pw, c = t - rr * pw;
-            const __half z = __float2half_rn(0.f);
-            P.Yhi[ybase + (long long)(s0 + rr) * P.ldn + c] = z;
-            P.Ylo[ybase + (long long)(s0 + rr) * P.ldn + c] = z;
-            const long long o = ubase + (long long)(j0 + c) * P.ldm + s0 + rr;
-            P.YThi[o] = z;
-            P.YTlo[o] = z;
+            split_store(wide, P.Yhi, P.Ylo, ybase, (long long)(s0 + rr) * P.ldn + j0 + c, 0.f, 1.f);
+            split_store(wide, P.YThi, P.YTlo, ubase, (long long)(j0 + c) * P.ldm + s0 + rr, 0.f, 1.f);
         }
     if (rank != 0 || 4 * w >= NB) return;
     // T[c][c] = tau_c, T[:c, c] = -tau_c T[:c, :c] G[:c, c].  Row i needs nothing of the other rows: 8 lanes
@@ -371,8 +388,8 @@ static int qr_launch_panel(PanelArgs &a, int B, cudaStream_t st) {
 constexpr int kTaCols = 32, kTaWarps = 8;
 __global__ void __launch_bounds__(32 * kTaWarps) qr_tapply_kernel(const float *Wp, int ks, int B, int nb, int pw,
                                                                   int n, int ldw, int ncol, const float *Tm, int npan,
-                                                                  int panel, const int *skip, __half *W2hi,
-                                                                  __half *W2lo) {
+                                                                  int panel, const int *skip, const int *fine,
+                                                                  float *W2hi, float *W2lo) {
     __shared__ float Ts[64 * 65];                   // T^T, rows padded
     __shared__ float ws[64][kTaCols + 1];           // W[l][c] for the block's columns
     const int b = blockIdx.y;
@@ -395,27 +412,25 @@ __global__ void __launch_bounds__(32 * kTaWarps) qr_tapply_kernel(const float *W
         float sum = 0.f;
         for (int l = 0; l < pw; ++l) sum += Ts[i * 65 + l] * ws[l][lane];
         if (c >= ncol) continue;
-        __half h, lo;
-        split_f16(sum * kF16S2, h, lo);
-        const long long o = ((long long)b * n + c) * kWY + i;
-        W2hi[o] = h;
-        W2lo[o] = lo;
+        split_store(fine[b] == PREC_TF32X3, W2hi, W2lo, (long long)b * n * kWY, (long long)c * kWY + i, sum, kF16S2);
     }
 }
 
 // S2 = S T (trans = 0) or S T^T (trans = 1) of a block of kWY columns, S (ncol x kWY) the sum of ks K-split
-// slices in slice order, S2 split into FP16 halves.  One block of 2 kWY threads per kQsRows rows: op(T)^T
+// slices in slice order, S2 split.  One block of 2 kWY threads per kQsRows rows: op(T)^T
 // staged with rows padded to kQsLd floats (thread j of a half reads row j as float4), the rows of S
 // as float4 broadcasts.  T is zero outside its triangle and past the block's width.
 constexpr int kQsRows = 32, kQsLd = kWY + 4;
 constexpr size_t kQsSmem = sizeof(float) * ((size_t)kWY * kQsLd + (size_t)kQsRows * kWY);
 __global__ void __launch_bounds__(2 * kWY) qr_stapply_kernel(const float *Sp, int ks, int B, int n, int ncol, int ws,
                                                              const float *Ts, int nsup, int sup, int trans,
-                                                             const int *skip, __half *W2hi, __half *W2lo) {
+                                                             const int *skip, const int *fine, float *W2hi,
+                                                             float *W2lo) {
     extern __shared__ __align__(16) float qsm2[];
     float *Ms = qsm2, *sr = qsm2 + kWY * kQsLd;
     const int b = blockIdx.y, t = threadIdx.x, i0 = blockIdx.x * kQsRows;
     if (skip[b]) return;
+    const bool wide = fine[b] == PREC_TF32X3;
     const float *T = Ts + ((long long)b * nsup + sup) * kWY * kWY;
     for (int e = t; e < kWY * kWY; e += 2 * kWY) {
         const int r = e / kWY, c = e % kWY;
@@ -450,11 +465,7 @@ __global__ void __launch_bounds__(2 * kWY) qr_stapply_kernel(const float *Sp, in
     for (int r = 0; r < kH; ++r) {
         const int i = i0 + rh + r;
         if (i >= ncol) break;
-        __half h, lo;
-        split_f16(acc[r] * kF16S2, h, lo);
-        const long long o = ((long long)b * n + i) * kWY + j;
-        W2hi[o] = h;
-        W2lo[o] = lo;
+        split_store(wide, W2hi, W2lo, (long long)b * n * kWY, (long long)i * kWY + j, acc[r], kF16S2);
     }
 }
 
@@ -491,38 +502,39 @@ __global__ void qr_scale_kernel(const unsigned *amax, long long cols, int m, flo
     iscale[c] = ldexpf(1.f, -e);
 }
 
-__global__ void qr_skip_kernel(const int *flag, int B, int *skip) {
+__global__ void qr_skip_kernel(const int *flag, int B, int *skip, int *fine) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < B) skip[b] = flag ? (flag[b] ? 0 : 1) : 0;
+    if (b >= B) return;
+    skip[b] = flag ? (flag[b] ? 0 : 1) : 0;
+    fine[b] = PREC_F16X3;
 }
 
 // Q^T = [I 0] (split: hi = identity, lo = 0) for the factored matrices
-__global__ void qr_qinit_kernel(int n, int m, long long ldm, const int *skip, __half *QThi, __half *QTlo) {
+__global__ void qr_qinit_kernel(int n, int m, long long ldm, const int *skip, const int *fine, float *QThi, float *QTlo) {
     const int b = blockIdx.z;
     if (skip[b]) return;
     const int c = blockIdx.y, r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= m) return;
-    const long long o = ((long long)b * n + c) * ldm + r;
-    QThi[o] = __float2half_rn(r == c ? kF16X : 0.f);
-    QTlo[o] = __float2half_rn(0.f);
+    split_store(fine[b] == PREC_TF32X3, QThi, QTlo, (long long)b * n * ldm, (long long)c * ldm + r, r == c ? 1.f : 0.f, kF16X);
 }
 
 // Q[r][c] = sign(beta_c) Q^T[c][r] (transposed through a shared tile) and, if R is given,
 // R[r][c] = 2^e_c sign(beta_r) (r < c ? UT[c][r] : r == c ? beta_c : 0).
-__global__ void qr_store_kernel(const __half *QThi, const __half *QTlo, const __half *UThi, const __half *UTlo,
+__global__ void qr_store_kernel(const float *QThi, const float *QTlo, const float *UThi, const float *UTlo,
                                 const float *beta, const float *scale, int m, int n, long long ldm, const int *skip,
-                                float *Q, float *R) {
+                                const int *fine, float *Q, float *R) {
     __shared__ float tile[32][33];
     const int b = blockIdx.z;
     if (skip[b]) return;
     const int c0 = blockIdx.y * 32, r0 = blockIdx.x * 32;   // c: column of Q (row of Q^T)
     const float *bb = beta + (long long)b * n;
+    const bool wide = fine[b] == PREC_TF32X3;
+    const long long ub = (long long)b * n * ldm;
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
         const int c = c0 + i, r = r0 + threadIdx.x;
         float v = 0.f;
         if (c < n && r < m) {
-            const long long o = ((long long)b * n + c) * ldm + r;
-            v = (bb[c] < 0.f ? -1.f : 1.f) * (join_f16(QThi[o], QTlo[o]) * (1.f / kF16X));
+            v = (bb[c] < 0.f ? -1.f : 1.f) * split_load(wide, QThi, QTlo, ub, (long long)c * ldm + r, 1.f / kF16X);
         }
         tile[i][threadIdx.x] = v;
     }
@@ -538,8 +550,7 @@ __global__ void qr_store_kernel(const __half *QThi, const __half *QTlo, const __
         const int c = c0 + i, r = r0 + threadIdx.x;
         float v = 0.f;
         if (c < n && r < n) {
-            const long long o = ((long long)b * n + c) * ldm + r;
-            v = r < c ? join_f16(UThi[o], UTlo[o]) * (1.f / kF16X) : (r == c ? fabsf(bb[c]) : 0.f);
+            v = r < c ? split_load(wide, UThi, UTlo, ub, (long long)c * ldm + r, 1.f / kF16X) : (r == c ? fabsf(bb[c]) : 0.f);
             if (r < c && bb[r] < 0.f) v = -v;
             v *= scale[(long long)b * n + c];
         }
@@ -552,23 +563,29 @@ __global__ void qr_store_kernel(const __half *QThi, const __half *QTlo, const __
     }
 }
 
-// X^T[c][j0 + r] -= sum_i W2^T[c][i] Y[j0 + r][j0 + i] for rows c0 .. c0 + ncol - 1 of X^T and the pw reflectors
-// from j0 on, W2^T in w.W2hi / w.W2lo.
-static int qr_update(QrWS &w, int j0, int pw, int c0, int ncol, __half *Xhi, __half *Xlo, cudaStream_t st) {
-    const int B = w.B, m = w.m, n = w.n, K = m - j0;
-    F16Views f;
-    f.ah = view_f16(w.W2hi, ncol, pw, kWY, (long long)n * kWY, B);
-    f.al = view_f16(w.W2lo, ncol, pw, kWY, (long long)n * kWY, B);
-    f.bh = view_f16(w.Yhi + (long long)j0 * w.ldn + j0, K, pw, w.ldn, (long long)m * w.ldn, B);
-    f.bl = view_f16(w.Ylo + (long long)j0 * w.ldn + j0, K, pw, w.ldn, (long long)m * w.ldn, B);
+// a product of split arrays whose halves carry `scale`
+static GemmShape qr_shape_of(const QrWS &w, int M, int N, int K, float scale) {
     GemmShape s;
     memset(&s, 0, sizeof(s));
-    s.M = ncol; s.N = K; s.K = pw; s.prec_uniform = PREC_F16X3; s.skip = w.skip; s.err = w.err;
-    s.f16_scale = 1.f / (kF16S2 * kF16V);
+    s.M = M; s.N = N; s.K = K; s.prec = w.fine; s.skip = w.skip; s.err = w.err;
+    s.f16_scale = 1.f / scale;
+    s.prof_as = PREC_TF32X3 + 1;
+    return s;
+}
+
+// X^T[c][j0 + r] -= sum_i W2^T[c][i] Y[j0 + r][j0 + i] for rows c0 .. c0 + ncol - 1 of X^T and the pw reflectors
+// from j0 on, W2^T in w.W2hi / w.W2lo.
+static int qr_update(QrWS &w, int j0, int pw, int c0, int ncol, float *Xhi, float *Xlo, cudaStream_t st) {
+    const int B = w.B, m = w.m, n = w.n, K = m - j0;
+    GemmShape s = qr_shape_of(w, ncol, K, pw, kF16S2 * kF16V);
+    const long long off = (long long)c0 * w.ldm + j0;
     EpiSubHalf e;
-    e.rows = ncol; e.cols = K; e.hi = Xhi + (long long)c0 * w.ldm + j0; e.lo = Xlo + (long long)c0 * w.ldm + j0;
-    e.ld = w.ldm; e.bs = (long long)n * w.ldm; e.scale = kF16X; e.inv = 1.f / kF16X;
-    PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
+    e.rows = ncol; e.cols = K; e.ld = w.ldm; e.scale = kF16X; e.inv = 1.f / kF16X;
+    e.fine = w.fine; e.fhi = Xhi + off; e.flo = Xlo + off; e.fbs = (long long)n * w.ldm;
+    e.hi = as_half(Xhi) + off; e.lo = as_half(Xlo) + off; e.bs = 2 * e.fbs;
+    PSVD_TRY(launch_split(SplitView(w.W2hi, w.W2lo, 0, ncol, pw, kWY, (long long)n * kWY, B),
+                          SplitView(w.Yhi, w.Ylo, (long long)j0 * w.ldn + j0, K, pw, w.ldn, (long long)m * w.ldn, B), s, B,
+                          e, st));
     return PSVD_OK;
 }
 
@@ -578,20 +595,13 @@ static int qr_apply_panel(QrWS &w, int j0, int pw, int panel, int c0, int ncol, 
     const int K = m - j0;
     const long long nm = (long long)n * w.ldm;
     // W = Y^T X: A = Y^T rows of the panel (pw x K), B = X^T rows (ncol x K), split over K
-    F16Views f;
-    f.ah = view_f16(w.YThi + (long long)j0 * w.ldm + j0, pw, K, w.ldm, nm, B);
-    f.al = view_f16(w.YTlo + (long long)j0 * w.ldm + j0, pw, K, w.ldm, nm, B);
-    f.bh = view_f16(w.UThi + (long long)c0 * w.ldm + j0, ncol, K, w.ldm, nm, B);
-    f.bl = view_f16(w.UTlo + (long long)c0 * w.ldm + j0, ncol, K, w.ldm, nm, B);
-    GemmShape s;
-    memset(&s, 0, sizeof(s));
-    s.M = pw; s.N = ncol; s.K = K; s.prec_uniform = PREC_F16X3; s.skip = w.skip; s.err = w.err;
-    s.f16_scale = 1.f / (kF16V * kF16X);
+    GemmShape s = qr_shape_of(w, pw, ncol, K, kF16V * kF16X);
     s.ksplit = std::max(1, std::min(std::min(w.ks, (num_sms() + B - 1) / B), (K + 127) / 128));
     EpiStore e = epi_store_plain(w.Wp, ldw, (long long)nb * ldw, pw, ncol);
-    PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
+    PSVD_TRY(launch_split(SplitView(w.YThi, w.YTlo, (long long)j0 * w.ldm + j0, pw, K, w.ldm, nm, B),
+                          SplitView(w.UThi, w.UTlo, (long long)c0 * w.ldm + j0, ncol, K, w.ldm, nm, B), s, B, e, st));
     qr_tapply_kernel<<<dim3((ncol + kTaCols - 1) / kTaCols, B), 32 * kTaWarps, 0, st>>>(
-        w.Wp, s.ksplit, B, nb, pw, n, ldw, ncol, w.Tm, w.npan, panel, w.skip, w.W2hi, w.W2lo);
+        w.Wp, s.ksplit, B, nb, pw, n, ldw, ncol, w.Tm, w.npan, panel, w.skip, w.fine, w.W2hi, w.W2lo);
     count_launch(1);
     PSVD_TRY(cudaGetLastError());
     return qr_update(w, j0, pw, c0, ncol, w.UThi, w.UTlo, st);
@@ -601,42 +611,30 @@ static int qr_apply_panel(QrWS &w, int j0, int pw, int panel, int c0, int ncol, 
 static int qr_block_t(QrWS &w, int j0, int ws, int sup, cudaStream_t st) {
     const int B = w.B, K = w.m - j0;
     const long long nm = (long long)w.n * w.ldm, gbs = (long long)w.n * kWY;
-    F16Views f;
-    f.ah = f.bh = view_f16(w.YThi + (long long)j0 * w.ldm + j0, ws, K, w.ldm, nm, B);
-    f.al = f.bl = view_f16(w.YTlo + (long long)j0 * w.ldm + j0, ws, K, w.ldm, nm, B);
-    GemmShape s;
-    memset(&s, 0, sizeof(s));
-    s.M = ws; s.N = ws; s.K = K; s.prec_uniform = PREC_F16X3; s.skip = w.skip; s.err = w.err;
-    s.f16_scale = 1.f / (kF16V * kF16V);
+    GemmShape s = qr_shape_of(w, ws, ws, K, kF16V * kF16V);
     // one tile with all of K: split (4 matrices of 14336 rows 185 -> 29 us, and 38 -> 64 in the T kernel that adds the slices)
     s.ksplit = std::max(1, std::min(kQrSplit, (K + 255) / 256));
     EpiStore e = epi_store_plain(w.Sp, kWY, gbs, ws, ws);
-    PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
+    const SplitView y(w.YThi, w.YTlo, (long long)j0 * w.ldm + j0, ws, K, w.ldm, nm, B);
+    PSVD_TRY(launch_split(y, y, s, B, e, st));
     return larft_blocks(w.Sp, s.ksplit, gbs, w.tau, w.n, w.n, w.nsup, sup, 1, B, w.Ts, st);
 }
 
 // The reflectors of a whole block on rows c0 .. c0 + ncol - 1 of X^T: trans = 0 in the factorization
 // (X <- (I - Y T Y^T)^T X), 1 in the accumulation of Q (X <- (I - Y T Y^T) X).
-static int qr_apply_block(QrWS &w, int j0, int ws, int sup, int c0, int ncol, __half *Xhi, __half *Xlo, int trans,
+static int qr_apply_block(QrWS &w, int j0, int ws, int sup, int c0, int ncol, float *Xhi, float *Xlo, int trans,
                           cudaStream_t st) {
     const int B = w.B, n = w.n, K = w.m - j0;
     const long long nm = (long long)n * w.ldm;
-    F16Views f;
-    f.ah = view_f16(Xhi + (long long)c0 * w.ldm + j0, ncol, K, w.ldm, nm, B);
-    f.al = view_f16(Xlo + (long long)c0 * w.ldm + j0, ncol, K, w.ldm, nm, B);
-    f.bh = view_f16(w.YThi + (long long)j0 * w.ldm + j0, ws, K, w.ldm, nm, B);
-    f.bl = view_f16(w.YTlo + (long long)j0 * w.ldm + j0, ws, K, w.ldm, nm, B);
-    GemmShape s;
-    memset(&s, 0, sizeof(s));
-    s.M = ncol; s.N = ws; s.K = K; s.prec_uniform = PREC_F16X3; s.skip = w.skip; s.err = w.err;
-    s.f16_scale = 1.f / (kF16X * kF16V);
+    GemmShape s = qr_shape_of(w, ncol, ws, K, kF16X * kF16V);
     const int tiles = ((ncol + kBM - 1) / kBM) * B;
     s.ksplit = std::max(1, std::min(std::min(kQrSplit, (num_sms() + tiles - 1) / tiles), (K + 255) / 256));
     EpiStore e = epi_store_plain(w.Sp, kWY, (long long)n * kWY, ncol, ws);
-    PSVD_TRY(launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f));
+    PSVD_TRY(launch_split(SplitView(Xhi, Xlo, (long long)c0 * w.ldm + j0, ncol, K, w.ldm, nm, B),
+                          SplitView(w.YThi, w.YTlo, (long long)j0 * w.ldm + j0, ws, K, w.ldm, nm, B), s, B, e, st));
     PSVD_TRY(cudaFuncSetAttribute(qr_stapply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQsSmem));
     qr_stapply_kernel<<<dim3((ncol + kQsRows - 1) / kQsRows, B), 2 * kWY, kQsSmem, st>>>(
-        w.Sp, s.ksplit, B, n, ncol, ws, w.Ts, w.nsup, sup, trans, w.skip, w.W2hi, w.W2lo);
+        w.Sp, s.ksplit, B, n, ncol, ws, w.Ts, w.nsup, sup, trans, w.skip, w.fine, w.W2hi, w.W2lo);
     count_launch(1);
     PSVD_TRY(cudaGetLastError());
     return qr_update(w, j0, ws, c0, ncol, Xhi, Xlo, st);
@@ -645,15 +643,15 @@ static int qr_apply_block(QrWS &w, int j0, int ws, int sup, int c0, int ncol, __
 int qr_factor(const float *A, float *Q, float *R, const int *flag, QrWS &w, cudaStream_t st) {
     const int B = w.B, m = w.m, n = w.n, nb = w.nb;
     const long long nm = (long long)n * w.ldm;
-    qr_skip_kernel<<<(B + 127) / 128, 128, 0, st>>>(flag, B, w.skip);
+    qr_skip_kernel<<<(B + 127) / 128, 128, 0, st>>>(flag, B, w.skip, w.fine);
     const long long mn = (long long)m * n, bn = (long long)B * n;
     PSVD_TRY(cudaMemsetAsync(w.amax, 0, sizeof(unsigned) * (size_t)bn, st));
     qr_colmax_kernel<<<dim3((n + 31) / 32, (m + kCmRows - 1) / kCmRows, B), 256, 0, st>>>(A, m, n, w.skip, w.amax);
     qr_scale_kernel<<<(unsigned)((bn + 127) / 128), 128, 0, st>>>(w.amax, bn, m, w.scale, w.iscale);
     count_launch(3);
     {
-        SplitOut t;
-        t.fhi = w.UThi; t.flo = w.UTlo; t.ld = w.ldm; t.bstride = t.fbstride = nm; t.fscale = kF16X;
+        PSVD_TRY(fine_rows(A, B, m, n, w.iscale, w.skip, w.fine, st));
+        SplitOut t = split_out(w.UThi, w.UTlo, w.ldm, nm, kF16X, w.fine);
         t.colscale = w.iscale;
         PSVD_TRY(prepare_operand(A, n, mn, B, m, n, true, 1.f, nullptr, t, st, w.skip));
     }
@@ -663,7 +661,7 @@ int qr_factor(const float *A, float *Q, float *R, const int *flag, QrWS &w, cuda
             const int pw = std::min(nb, s1 - j0), p = j0 / nb;
             PanelArgs a;
             a.UThi = w.UThi; a.UTlo = w.UTlo; a.YThi = w.YThi; a.YTlo = w.YTlo; a.Yhi = w.Yhi; a.Ylo = w.Ylo;
-            a.tau = w.tau; a.beta = w.beta; a.Tm = w.Tm; a.skip = w.skip;
+            a.tau = w.tau; a.beta = w.beta; a.Tm = w.Tm; a.skip = w.skip; a.fine = w.fine;
             a.m = m; a.n = n; a.j0 = j0; a.pw = pw; a.panel = p; a.npan = w.npan;
             a.ldm = w.ldm; a.ldn = w.ldn;
             const int rows = m - j0;
@@ -676,7 +674,7 @@ int qr_factor(const float *A, float *Q, float *R, const int *flag, QrWS &w, cuda
     }
     {
         dim3 g((m + 127) / 128, n, B);
-        qr_qinit_kernel<<<g, 128, 0, st>>>(n, m, w.ldm, w.skip, w.QThi, w.QTlo);
+        qr_qinit_kernel<<<g, 128, 0, st>>>(n, m, w.ldm, w.skip, w.fine, w.QThi, w.QTlo);
         count_launch(1);
         PSVD_TRY(cudaGetLastError());
     }
@@ -686,7 +684,8 @@ int qr_factor(const float *A, float *Q, float *R, const int *flag, QrWS &w, cuda
     }
     {
         dim3 g((m + 31) / 32, (n + 31) / 32, B), blk(32, 8);
-        qr_store_kernel<<<g, blk, 0, st>>>(w.QThi, w.QTlo, w.UThi, w.UTlo, w.beta, w.scale, m, n, w.ldm, w.skip, Q, R);
+        qr_store_kernel<<<g, blk, 0, st>>>(w.QThi, w.QTlo, w.UThi, w.UTlo, w.beta, w.scale, m, n, w.ldm, w.skip, w.fine,
+                                            Q, R);
         count_launch(1);
         PSVD_TRY(cudaGetLastError());
     }

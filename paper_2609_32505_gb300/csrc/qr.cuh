@@ -12,22 +12,23 @@ bool qr_shape(int m, int *nb);
 constexpr int kQrSplit = 8;   // largest K split of the X^T Y products of a block
 
 // The columns are normalized by powers of two (norms <= 1), so every array below is bounded and kept as
-// split-FP16 halves.
+// split-FP16 halves; matrices with very small rows (fine[b]) as split TF32 in the same memory.
 struct QrWS {
     int B = 0, m = 0, n = 0, nb = 0, npan = 0, nsup = 0, ks = 1;
     long long ldm = 0, ldn = 0;
-    __half *UThi = nullptr, *UTlo = nullptr;   // [B][n][ldm] the matrix transposed, being factored (kF16X)
-    __half *YThi = nullptr, *YTlo = nullptr;   // [B][n][ldm] reflector j as row j (1 at j, 0 above) (kF16V)
-    __half *Yhi = nullptr, *Ylo = nullptr;     // [B][m][ldn] the same reflectors as columns (kF16V)
-    __half *QThi = nullptr, *QTlo = nullptr;   // [B][n][ldm] Q^T being accumulated (kF16X)
+    float *UThi = nullptr, *UTlo = nullptr;   // [B][n][ldm] the matrix transposed, being factored (kF16X)
+    float *YThi = nullptr, *YTlo = nullptr;   // [B][n][ldm] reflector j as row j (1 at j, 0 above) (kF16V)
+    float *Yhi = nullptr, *Ylo = nullptr;     // [B][m][ldn] the same reflectors as columns (kF16V)
+    float *QThi = nullptr, *QTlo = nullptr;   // [B][n][ldm] Q^T being accumulated (kF16X)
     float *tau = nullptr, *beta = nullptr;     // [B][n]
     float *Tm = nullptr;                       // [B][npan][nb][nb] compact-WY T of every panel
     float *Wp = nullptr;                       // [ks][B][nb][n] partial Y^T X of a panel (K split)
-    __half *W2hi = nullptr, *W2lo = nullptr;   // [B][n][kWY] (op(T) Y^T X)^T (kF16S2)
+    float *W2hi = nullptr, *W2lo = nullptr;   // [B][n][kWY] (op(T) Y^T X)^T (kF16S2)
     float *Ts = nullptr;                       // [B][nsup][kWY][kWY] T of blocks of kWY columns
     float *Sp = nullptr;                       // [kQrSplit][B][n][kWY] partial X^T Y, or Y^T Y, of a block
     unsigned *amax = nullptr;                  // [B][n] max |a| of every column (float bits)
     float *scale = nullptr, *iscale = nullptr; // [B][n] 2^e and 2^-e of every column
+    int *fine = nullptr;                       // [B] PREC_F16X3 or PREC_TF32X3
     int *skip = nullptr;                       // [B] 1 = matrix not factored (flag[b] == 0)
     unsigned *err = nullptr;
 
@@ -40,20 +41,21 @@ struct QrWS {
         ldm = pad_ld(m); ldn = pad_ld(n);
         ks = 16;
         const long long B64 = B, nm = (long long)n * ldm;
-        UThi = cv.template take<__half>(B64 * nm); UTlo = cv.template take<__half>(B64 * nm);
-        YThi = cv.template take<__half>(B64 * nm); YTlo = cv.template take<__half>(B64 * nm);
-        Yhi = cv.template take<__half>(B64 * m * ldn); Ylo = cv.template take<__half>(B64 * m * ldn);
-        QThi = cv.template take<__half>(B64 * nm); QTlo = cv.template take<__half>(B64 * nm);
+        UThi = cv.template take<float>(B64 * nm); UTlo = cv.template take<float>(B64 * nm);
+        YThi = cv.template take<float>(B64 * nm); YTlo = cv.template take<float>(B64 * nm);
+        Yhi = cv.template take<float>(B64 * m * ldn); Ylo = cv.template take<float>(B64 * m * ldn);
+        QThi = cv.template take<float>(B64 * nm); QTlo = cv.template take<float>(B64 * nm);
         tau = cv.template take<float>(B64 * n); beta = cv.template take<float>(B64 * n);
         Tm = cv.template take<float>(B64 * npan * nb * nb);
         Wp = cv.template take<float>((long long)ks * B64 * nb * std::min(n, kWY));
-        W2hi = cv.template take<__half>(B64 * n * kWY); W2lo = cv.template take<__half>(B64 * n * kWY);
+        W2hi = cv.template take<float>(B64 * n * kWY); W2lo = cv.template take<float>(B64 * n * kWY);
         Ts = cv.template take<float>(B64 * nsup * kWY * kWY);
         Sp = cv.template take<float>((long long)kQrSplit * B64 * n * kWY);
         amax = cv.template take<unsigned>(B64 * n);
         scale = cv.template take<float>(B64 * n);
         iscale = cv.template take<float>(B64 * n);
         skip = cv.template take<int>(B64);
+        fine = cv.template take<int>(B64);
         err = cv.template take<unsigned>(4);
     }
 };

@@ -852,7 +852,7 @@ struct PreqrLayout {
         QrWS qw;
         qw.carve(q, (int)B, (int)m, (int)n);
         const long long ld = pad_ld(n);
-        const size_t ops = (size_t)(2 * B * m * ld + 2 * B * n * ld) * sizeof(__half) + 2048;
+        const size_t ops = (size_t)(2 * B * m * ld + 2 * B * n * ld) * sizeof(float) + 4096 + 4 * (size_t)B;
         const size_t region = std::max(std::max(q.used + 256, svd_direct_bytes(B, n, n, sq)), ops);
         need = head + region;
         rest = ws ? static_cast<char *>(ws) + head : nullptr;
