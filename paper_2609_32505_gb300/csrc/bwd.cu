@@ -24,6 +24,8 @@ namespace psvd {
 // V, the largest column norm (both 1 for orthonormal factors, whatever else a caller hands over stays in
 // range); Y = M V, T1 = V^T sym(Hbar) and Wbar V are bounded by sqrt(n) times the largest entry of the one
 // and the column norm of the other; X and Q are written in FP32 with their largest entries recorded, then split.
+// A matrix M with rows or columns so small that halves of them lose bits has all its operands in split TF32
+// (fine[b]; the same memory): the rows of the gradient are of the sizes of M's.
 enum BwdMax { AM_M = 0, AM_G, AM_B, AM_U, AM_V, AM_IN, AM_X = AM_IN, AM_Q, AM_N };   // slots of amax; inputs first
 enum BwdScale {                                                        // slots of es, each [B]
     ES_M = 0, ES_G, ES_B, ES_U, ES_V, ES_X, ES_Q,      // 2^e (operands are divided by it)
@@ -35,25 +37,27 @@ enum BwdScale {                                                        // slots 
 struct BwdWS {
     int B = 0, m = 0, n = 0;
     long long ldn = 0, ldm = 0;
-    __half *UThi = nullptr, *UTlo = nullptr;      // U^T (n x m)
-    __half *GThi = nullptr, *GTlo = nullptr;      // Ubar^T or (Wbar V)^T (n x m)
+    float *UThi = nullptr, *UTlo = nullptr;      // U^T (n x m)
+    float *GThi = nullptr, *GTlo = nullptr;      // Ubar^T or (Wbar V)^T (n x m)
     float *G = nullptr;                           // Wbar V row-major FP32 (m x n) for the epilogue (polar)
-    __half *Mhi = nullptr, *Mlo = nullptr;        // M (m x n)
-    __half *VThi = nullptr, *VTlo = nullptr;      // V^T (n x n)
-    __half *Vhi = nullptr, *Vlo = nullptr;        // V (n x n)
-    __half *dVThi = nullptr, *dVTlo = nullptr;    // Vbar^T (n x n) or sym(Hbar) (polar)
-    __half *Yhi = nullptr, *Ylo = nullptr;        // Y = M V (m x n)
-    __half *YThi = nullptr, *YTlo = nullptr;      // Y^T (n x m)
+    float *Mhi = nullptr, *Mlo = nullptr;        // M (m x n)
+    float *VThi = nullptr, *VTlo = nullptr;      // V^T (n x n)
+    float *Vhi = nullptr, *Vlo = nullptr;        // V (n x n)
+    float *dVThi = nullptr, *dVTlo = nullptr;    // Vbar^T (n x n) or sym(Hbar) (polar)
+    float *Yhi = nullptr, *Ylo = nullptr;        // Y = M V (m x n)
+    float *YThi = nullptr, *YTlo = nullptr;      // Y^T (n x m)
     float *AU = nullptr, *BV = nullptr, *Z = nullptr;   // n x n FP32
     float *X = nullptr;                           // V^T X V (n x n)
-    __half *Xhi = nullptr, *Xlo = nullptr;
+    float *Xhi = nullptr, *Xlo = nullptr;
     float *Q = nullptr;                           // (m x n)
-    __half *Qhi = nullptr, *Qlo = nullptr;
-    __half *Wbhi = nullptr, *Wblo = nullptr;      // Wbar (m x n), polar only
+    float *Qhi = nullptr, *Qlo = nullptr;
+    float *Wbhi = nullptr, *Wblo = nullptr;      // Wbar (m x n), polar only
     float *S = nullptr;                           // sigma FP32 (polar: eigenvalues of H)
     float *T1 = nullptr;                          // polar: V^T, then V^T Hbar
-    __half *T1hi = nullptr, *T1lo = nullptr;
+    float *T1hi = nullptr, *T1lo = nullptr;
     unsigned *amax = nullptr;                     // [AM_N][B]
+    unsigned *ext = nullptr;                      // [B][m + n] largest entries of M's rows and columns
+    int *fine = nullptr;                          // [B] PREC_F16X3 or PREC_TF32X3
     float *es = nullptr;                          // [ES_N][B]
     unsigned *err = nullptr;
     EighWS ew;
@@ -65,9 +69,9 @@ struct BwdWS {
         B = B_; m = m_; n = n_; polar = polar_;
         ldn = pad_ld(n); ldm = pad_ld(m);
         const long long B64 = B, mn = (long long)m * ldn, nm = (long long)n * ldm, nn = (long long)n * ldn;
-        auto pair = [&](__half *&hi, __half *&lo, long long k) {
-            hi = cv.template take<__half>(B64 * k);
-            lo = cv.template take<__half>(B64 * k);
+        auto pair = [&](float *&hi, float *&lo, long long k) {
+            hi = cv.template take<float>(B64 * k);
+            lo = cv.template take<float>(B64 * k);
         };
         pair(UThi, UTlo, nm); pair(GThi, GTlo, nm); pair(Mhi, Mlo, mn); pair(VThi, VTlo, nn); pair(Vhi, Vlo, nn);
         pair(dVThi, dVTlo, nn); pair(Yhi, Ylo, mn); pair(YThi, YTlo, nm); pair(Xhi, Xlo, nn); pair(Qhi, Qlo, mn);
@@ -75,7 +79,9 @@ struct BwdWS {
         Z = cv.template take<float>(B64 * n * n);
         X = cv.template take<float>(B64 * n * n); Q = cv.template take<float>(B64 * m * n);
         S = cv.template take<float>(B64 * n);
-        amax = cv.template take<unsigned>(B64 * AM_N);
+        amax = cv.template take<unsigned>(B64 * (AM_N + m + n));
+        ext = amax + B64 * AM_N;
+        fine = cv.template take<int>(B64);
         es = cv.template take<float>(B64 * ES_N);
         err = cv.template take<unsigned>(4);
         if (polar) {
@@ -99,9 +105,7 @@ PSVD_DEV int bwd_exp_factor(unsigned amax) {
     return v > 2.f && v < INFINITY ? ilogbf(v) : 0;
 }
 // stage 0: the scales of the inputs; 1: of X; 2: of Q
-__global__ void bwd_scale_kernel(const unsigned *amax, int B, int n, int stage, int polar, float *es) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
+PSVD_DEV void bwd_scale(const unsigned *amax, int B, int b, int n, int stage, int polar, float *es) {
     auto put = [&](int slot, int e) { es[(long long)slot * B + b] = ldexpf(1.f, e); };
     const double rn = sqrt((double)n);
     const int eM = bwd_exp(amax[AM_M * B + b], 1.0), eV = bwd_exp_factor(amax[AM_V * B + b]);
@@ -121,17 +125,65 @@ __global__ void bwd_scale_kernel(const unsigned *amax, int B, int n, int stage, 
     }
 }
 
+__global__ void bwd_scale_kernel(const unsigned *amax, int B, int n, int stage, float *es) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < B) bwd_scale(amax, B, b, n, stage, 0, es);
+}
+// stage 0, and fine[b]: halves of M / 2^eM hold 22 bits down to 2^-28, so a row with a largest entry above sqrt(n)
+// 2^(eM - 28), or a column above sqrt(m) 2^(eM - 28), has no more rounding error in them than in split TF32
+__global__ void __launch_bounds__(256) bwd_fine_kernel(const unsigned *amax, const unsigned *ext, int B, int m, int n,
+                                                       int polar, float *es, int *fine) {
+    const int b = blockIdx.x;
+    const float lim = ldexpf(1.f, bwd_exp(amax[AM_M * B + b], 1.0)) * 0x1p-28f;
+    const float lr = sqrtf((float)n) * lim, lc = sqrtf((float)m) * lim;
+    bool small = false;
+    for (int i = threadIdx.x; i < m + n; i += blockDim.x) {
+        const float v = __uint_as_float(ext[(long long)b * (m + n) + i]);
+        small |= v > 0.f && v < (i < m ? lr : lc);
+    }
+    small = __syncthreads_or(small);
+    if (threadIdx.x) return;
+    fine[b] = small ? PREC_TF32X3 : PREC_F16X3;
+    bwd_scale(amax, B, b, n, 0, polar, es);
+}
+
 // The AM_ slots of the inputs, one launch for all of them (grid.z = slot): entries, or for V^T the 2-norm
-// of its rows, a warp at a time.
+// of its rows, a warp at a time.  For M also the largest entries of its rows and columns, by tiles of 32 x 128 a
+// warp (ext).
 struct BwdMaxIn { const float *x[AM_IN]; long long len[AM_IN]; };
-__global__ void __launch_bounds__(256) bwd_max_kernel(BwdMaxIn in, int B, int n, unsigned *amax) {
+__global__ void __launch_bounds__(256) bwd_max_kernel(BwdMaxIn in, int B, int m, int n, unsigned *amax, unsigned *ext) {
     __shared__ unsigned red[8];
     const int b = blockIdx.y, slot = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (!in.x[slot]) return;
     const long long len = in.len[slot];
     const float *a = in.x[slot] + b * len;
     unsigned v = 0;
-    if (slot == AM_V) {
+    if (slot == AM_M) {
+        const int tn = (n + 127) / 128, tiles = tn * ((m + 31) / 32);
+        for (int t = blockIdx.x * 8 + warp; t < tiles; t += gridDim.x * 8) {
+            const int r0 = t / tn * 32, c0 = t % tn * 128 + lane, nr = min(32, m - r0);
+            unsigned cm[4] = {0u, 0u, 0u, 0u}, rm = 0u;
+#pragma unroll 8
+            for (int r = 0; r < nr; ++r) {
+                unsigned x = 0u;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (c0 + 32 * q < n) {
+                        const unsigned y = __float_as_uint(fabsf(a[(long long)(r0 + r) * n + c0 + 32 * q]));
+                        cm[q] = max(cm[q], y);
+                        x = max(x, y);
+                    }
+                x = __reduce_max_sync(0xffffffffu, x);
+                if (lane == r) rm = x;
+            }
+            unsigned *e = ext + (long long)b * (m + n);
+            if (lane < nr) atomicMax(&e[r0 + lane], rm);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (c0 + 32 * q < n) atomicMax(&e[m + c0 + 32 * q], cm[q]);
+            v = max(v, rm);
+        }
+    } else if (slot == AM_V) {
         for (int r = blockIdx.x * 8 + warp; r < n; r += gridDim.x * 8) {
             float s = 0.f;
 #pragma unroll 8
@@ -319,17 +371,15 @@ struct EpiQ {
     }
 };
 
-// sym(H) / scale as FP16 halves
-__global__ void sym_split_kernel(const float *H, const float *scale, int n, __half *hi, __half *lo, long long ld) {
+// sym(H) / scale, split
+__global__ void sym_split_kernel(const float *H, const float *scale, const int *fine, int n, float *hi, float *lo,
+                                 long long ld) {
     const int b = blockIdx.z;
     const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
     if (i >= n || j >= n) return;
     const float *h = H + (long long)b * n * n;
     const float x = 0.5f * (h[(long long)i * n + j] + h[(long long)j * n + i]);
-    __half a, c;
-    split_f16(x / scale[b] * kF16X, a, c);
-    hi[(long long)b * n * ld + (long long)i * ld + j] = a;
-    lo[(long long)b * n * ld + (long long)i * ld + j] = c;
+    split_store(fine[b] == PREC_TF32X3, hi, lo, (long long)b * n * ld, (long long)i * ld + j, x / scale[b], kF16X);
 }
 
 // split TF32 (the EVD backward, whose factors E and Z have no bound known in advance)
@@ -344,23 +394,20 @@ static int g3(const float *ahi, const float *alo, int M, int K, long long lda, l
     s.M = M; s.N = N; s.K = K; s.prec_uniform = PREC_TF32X3; s.err = err;
     return launch_gemm(nullptr, nullptr, &vah, &val, &vbh, &vbl, s, B, e, st) == cudaSuccess ? PSVD_OK : PSVD_ERR_CUDA;
 }
-// split FP16, scaled by scale[b]
+// split arrays in the formats of w.fine, scaled by es slot `scale` (which has the halves' 2^-28 in it)
 template <class Epi>
-static int g16(const __half *ahi, const __half *alo, int M, int K, long long lda, long long bsa, const __half *bhi,
-               const __half *blo, int N, long long ldb, long long bsb, int B, const float *scale, const Epi &e,
-               unsigned *err, cudaStream_t st) {
-    F16Views f;
-    f.ah = view_f16(ahi, M, K, lda, bsa, B);
-    f.al = view_f16(alo, M, K, lda, bsa, B);
-    f.bh = view_f16(bhi, N, K, ldb, bsb, B);
-    f.bl = view_f16(blo, N, K, ldb, bsb, B);
+static int g16(const float *ahi, const float *alo, int M, int K, long long lda, long long bsa, const float *bhi,
+               const float *blo, int N, long long ldb, long long bsb, const BwdWS &w, int scale, const Epi &e,
+               cudaStream_t st) {
     GemmShape s;
     memset(&s, 0, sizeof(s));
-    s.M = M; s.N = N; s.K = K; s.prec_uniform = PREC_F16X3; s.err = err;
+    s.M = M; s.N = N; s.K = K; s.prec = w.fine; s.err = w.err;
     s.f16_scale = 1.f;
-    s.scale_b = scale;
-    return launch_gemm(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s, B, e, st, &f) == cudaSuccess
-               ? PSVD_OK : PSVD_ERR_CUDA;
+    s.tf32_scale = kF16X * kF16X;
+    s.scale_b = w.esp(scale);
+    s.prof_as = PREC_TF32X3 + 1;
+    return launch_split(SplitView(ahi, alo, 0, M, K, lda, bsa, w.B), SplitView(bhi, blo, 0, N, K, ldb, bsb, w.B), s, w.B, e,
+                        st) == cudaSuccess ? PSVD_OK : PSVD_ERR_CUDA;
 }
 
 static SplitOut so(float *hi, float *lo, long long ld, long long bs) {
@@ -368,22 +415,16 @@ static SplitOut so(float *hi, float *lo, long long ld, long long bs) {
     s.hi = hi; s.lo = lo; s.ld = ld; s.bstride = bs;
     return s;
 }
-static SplitOut so16(__half *hi, __half *lo, long long ld, long long bs) {
-    SplitOut s;
-    s.fhi = hi; s.flo = lo; s.fscale = kF16X; s.ld = ld; s.bstride = s.fbstride = bs;
-    return s;
-}
-
 // Largest entries of the inputs (null: none) and the scales that follow from them.
 static int bwd_scales(BwdWS &w, const float *A, const float *G, const float *Bm, const float *U, const float *VT,
                       cudaStream_t st) {
     const int B = w.B, m = w.m, n = w.n;
     const long long mn = (long long)m * n, nn = (long long)n * n;
-    PSVD_TRY(cudaMemsetAsync(w.amax, 0, sizeof(unsigned) * (size_t)B * AM_N, st));
+    PSVD_TRY(cudaMemsetAsync(w.amax, 0, sizeof(unsigned) * (size_t)B * (AM_N + m + n), st));
     const BwdMaxIn in = {{A, G, Bm, U, VT}, {mn, mn, nn, mn, nn}};
     const long long per = std::max(1, 8 * num_sms() / std::min(B, 8));
-    bwd_max_kernel<<<dim3((unsigned)std::min<long long>((mn + 4095) / 4096, per), B, AM_IN), 256, 0, st>>>(in, B, n, w.amax);
-    bwd_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, n, 0, w.polar ? 1 : 0, w.es);
+    bwd_max_kernel<<<dim3((unsigned)std::min<long long>((mn + 4095) / 4096, per), B, AM_IN), 256, 0, st>>>(in, B, m, n, w.amax, w.ext);
+    bwd_fine_kernel<<<B, 256, 0, st>>>(w.amax, w.ext, B, m, n, w.polar ? 1 : 0, w.es, w.fine);
     count_launch(2);
     PSVD_TRY(cudaGetLastError());
     return PSVD_OK;
@@ -397,33 +438,33 @@ static int bwd_tail(BwdWS &w, const float *G, const float *EH, const float *AU, 
     {   // Y = M V : B operand B[j][k] = V[k][j] = V^T[j][k]
         EpiHalf e;
         memset(&e, 0, sizeof(e));
-        e.rows = m; e.cols = n; e.inv = w.esp(ES_IM);
+        e.rows = m; e.cols = n; e.inv = w.esp(ES_IM); e.fine = w.fine;
         e.hi = w.Yhi; e.lo = w.Ylo; e.ldh = ldn; e.bsh = mn;
         e.hi_t = w.YThi; e.lo_t = w.YTlo; e.ldht = ldm; e.bsht = nm;
-        PSVD_TRY_RC(g16(w.Mhi, w.Mlo, m, n, ldn, mn, w.VThi, w.VTlo, n, ldn, nn, B, w.esp(ES_Y), e, w.err, st));
+        PSVD_TRY_RC(g16(w.Mhi, w.Mlo, m, n, ldn, mn, w.VThi, w.VTlo, n, ldn, nn, w, ES_Y, e, st));
     }
     if (G) {   // Z = Y^T G
         EpiStore e = epi_store_plain(w.Z, n, (long long)n * n, n, n);
-        PSVD_TRY_RC(g16(w.YThi, w.YTlo, n, m, ldm, nm, w.GThi, w.GTlo, n, ldm, nm, B, w.esp(ES_Z), e, w.err, st));
+        PSVD_TRY_RC(g16(w.YThi, w.YTlo, n, m, ldm, nm, w.GThi, w.GTlo, n, ldm, nm, w, ES_Z, e, st));
     }
     const unsigned nt = (n + 31) / 32;
     bwd_core_kernel<<<dim3(nt, nt, B), dim3(32, 8), 0, st>>>(AU, BV, G ? w.Z : nullptr, EH, w.S, dS, n, eps, kreg, 1e-6f,
                                                             w.X, w.amax + AM_X * B);
-    bwd_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, n, 1, 0, w.es);
+    bwd_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, n, 1, w.es);
     count_launch(2);
-    PSVD_TRY(prepare_operand(w.X, n, (long long)n * n, B, n, n, false, 1.f, w.esp(ES_X), so16(w.Xhi, w.Xlo, ldn, nn), st));
+    PSVD_TRY(prepare_operand(w.X, n, (long long)n * n, B, n, n, false, 1.f, w.esp(ES_X), split_out(w.Xhi, w.Xlo, ldn, nn, kF16X, w.fine), st));
     {   // Q = G D_R + 2 Y (V^T X V)  (B operand = V^T X V, symmetric)
         EpiQ e;
         e.m = m; e.n = n; e.G = G; e.S = w.S; e.sqrt_eps = sqrtf(eps); e.exact = kreg == 2;
         e.Q = w.Q; e.qmax = w.amax + AM_Q * B;
-        PSVD_TRY_RC(g16(w.Yhi, w.Ylo, m, n, ldn, mn, w.Xhi, w.Xlo, n, ldn, nn, B, w.esp(ES_QP), e, w.err, st));
+        PSVD_TRY_RC(g16(w.Yhi, w.Ylo, m, n, ldn, mn, w.Xhi, w.Xlo, n, ldn, nn, w, ES_QP, e, st));
     }
-    bwd_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, n, 2, 0, w.es);
+    bwd_scale_kernel<<<(B + 127) / 128, 128, 0, st>>>(w.amax, B, n, 2, w.es);
     count_launch(1);
-    PSVD_TRY(prepare_operand(w.Q, n, (long long)m * n, B, m, n, false, 1.f, w.esp(ES_Q), so16(w.Qhi, w.Qlo, ldn, mn), st));
+    PSVD_TRY(prepare_operand(w.Q, n, (long long)m * n, B, m, n, false, 1.f, w.esp(ES_Q), split_out(w.Qhi, w.Qlo, ldn, mn, kF16X, w.fine), st));
     {   // dA = Q V^T : B operand B[j][k] = V^T[k][j] = V[j][k]
         EpiStore e = epi_store_plain(dA, n, (long long)m * n, m, n);
-        PSVD_TRY_RC(g16(w.Qhi, w.Qlo, m, n, ldn, mn, w.Vhi, w.Vlo, n, ldn, nn, B, w.esp(ES_DA), e, w.err, st));
+        PSVD_TRY_RC(g16(w.Qhi, w.Qlo, m, n, ldn, mn, w.Vhi, w.Vlo, n, ldn, nn, w, ES_DA, e, st));
     }
     return cudaGetLastError() == cudaSuccess ? PSVD_OK : PSVD_ERR_CUDA;
 }
@@ -436,19 +477,19 @@ int svd_backward(const float *A, const float *U, const float *S, const float *VT
     const float feps = kreg == 2 ? 0.f : (float)eps;
     PSVD_TRY(cudaMemcpyAsync(w.S, S, sizeof(float) * (size_t)B * n, cudaMemcpyDeviceToDevice, st));
     PSVD_TRY_RC(bwd_scales(w, A, dU, dVT, dU ? U : nullptr, VT, st));
-    PSVD_TRY(prepare_operand(A, n, umn, B, m, n, false, 1.f, w.esp(ES_M), so16(w.Mhi, w.Mlo, ldn, mn), st));
-    PSVD_TRY(prepare_operand(VT, n, unn, B, n, n, false, 1.f, w.esp(ES_V), so16(w.VThi, w.VTlo, ldn, nn), st));
-    PSVD_TRY(prepare_operand(VT, n, unn, B, n, n, true, 1.f, w.esp(ES_V), so16(w.Vhi, w.Vlo, ldn, nn), st));
+    PSVD_TRY(prepare_operand(A, n, umn, B, m, n, false, 1.f, w.esp(ES_M), split_out(w.Mhi, w.Mlo, ldn, mn, kF16X, w.fine), st));
+    PSVD_TRY(prepare_operand(VT, n, unn, B, n, n, false, 1.f, w.esp(ES_V), split_out(w.VThi, w.VTlo, ldn, nn, kF16X, w.fine), st));
+    PSVD_TRY(prepare_operand(VT, n, unn, B, n, n, true, 1.f, w.esp(ES_V), split_out(w.Vhi, w.Vlo, ldn, nn, kF16X, w.fine), st));
     if (dU) {
-        PSVD_TRY(prepare_operand(U, n, umn, B, m, n, true, 1.f, w.esp(ES_U), so16(w.UThi, w.UTlo, ldm, nm), st));
-        PSVD_TRY(prepare_operand(dU, n, umn, B, m, n, true, 1.f, w.esp(ES_G), so16(w.GThi, w.GTlo, ldm, nm), st));
+        PSVD_TRY(prepare_operand(U, n, umn, B, m, n, true, 1.f, w.esp(ES_U), split_out(w.UThi, w.UTlo, ldm, nm, kF16X, w.fine), st));
+        PSVD_TRY(prepare_operand(dU, n, umn, B, m, n, true, 1.f, w.esp(ES_G), split_out(w.GThi, w.GTlo, ldm, nm, kF16X, w.fine), st));
         EpiStore e = epi_store_plain(w.AU, n, unn, n, n);       // A_U = U^T Ubar
-        PSVD_TRY_RC(g16(w.UThi, w.UTlo, n, m, ldm, nm, w.GThi, w.GTlo, n, ldm, nm, B, w.esp(ES_AU), e, w.err, st));
+        PSVD_TRY_RC(g16(w.UThi, w.UTlo, n, m, ldm, nm, w.GThi, w.GTlo, n, ldm, nm, w, ES_AU, e, st));
     }
     if (dVT) {
-        PSVD_TRY(prepare_operand(dVT, n, unn, B, n, n, false, 1.f, w.esp(ES_B), so16(w.dVThi, w.dVTlo, ldn, nn), st));
+        PSVD_TRY(prepare_operand(dVT, n, unn, B, n, n, false, 1.f, w.esp(ES_B), split_out(w.dVThi, w.dVTlo, ldn, nn, kF16X, w.fine), st));
         EpiStore e = epi_store_plain(w.BV, n, unn, n, n);       // B_V = V^T Vbar
-        PSVD_TRY_RC(g16(w.VThi, w.VTlo, n, n, ldn, nn, w.dVThi, w.dVTlo, n, ldn, nn, B, w.esp(ES_BV), e, w.err, st));
+        PSVD_TRY_RC(g16(w.VThi, w.VTlo, n, n, ldn, nn, w.dVThi, w.dVTlo, n, ldn, nn, w, ES_BV, e, st));
     }
     return bwd_tail(w, dU, nullptr, dU ? w.AU : nullptr, dVT ? w.BV : nullptr, dS, feps, kreg, dA, st);
 }
@@ -461,33 +502,33 @@ int polar_backward(const float *A, const float *H, const float *dW, const float 
     // EVD of H (symmetrized by the eigensolver's reads of the full matrix); V^T plain in T1
     PSVD_TRY_RC(eigh_forward(H, w.S, w.T1, w.ew, st));
     PSVD_TRY_RC(bwd_scales(w, A, dW, dH, nullptr, nullptr, st));
-    PSVD_TRY(prepare_operand(A, n, umn, B, m, n, false, 1.f, w.esp(ES_M), so16(w.Mhi, w.Mlo, ldn, mn), st));
-    PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, false, 1.f, nullptr, so16(w.VThi, w.VTlo, ldn, nn), st));
-    PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, true, 1.f, nullptr, so16(w.Vhi, w.Vlo, ldn, nn), st));
+    PSVD_TRY(prepare_operand(A, n, umn, B, m, n, false, 1.f, w.esp(ES_M), split_out(w.Mhi, w.Mlo, ldn, mn, kF16X, w.fine), st));
+    PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, false, 1.f, nullptr, split_out(w.VThi, w.VTlo, ldn, nn, kF16X, w.fine), st));
+    PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, true, 1.f, nullptr, split_out(w.Vhi, w.Vlo, ldn, nn, kF16X, w.fine), st));
     const float *EH = w.BV;
     if (dH) {
         dim3 g16x((n + 15) / 16, (n + 15) / 16, B), b16(16, 16);
-        sym_split_kernel<<<g16x, b16, 0, st>>>(dH, w.esp(ES_B), n, w.dVThi, w.dVTlo, ldn);    // sym(Hbar)
+        sym_split_kernel<<<g16x, b16, 0, st>>>(dH, w.esp(ES_B), w.fine, n, w.dVThi, w.dVTlo, ldn);    // sym(Hbar)
         count_launch(1);
         // T1 = V^T sym(Hbar)  (B operand B[j][k] = Hs[k][j] = Hs[j][k])
         EpiStore e = epi_store_plain(w.T1, n, unn, n, n);
-        PSVD_TRY_RC(g16(w.VThi, w.VTlo, n, n, ldn, nn, w.dVThi, w.dVTlo, n, ldn, nn, B, w.esp(ES_T1), e, w.err, st));
-        PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, false, 1.f, w.esp(ES_B), so16(w.T1hi, w.T1lo, ldn, nn), st));
+        PSVD_TRY_RC(g16(w.VThi, w.VTlo, n, n, ldn, nn, w.dVThi, w.dVTlo, n, ldn, nn, w, ES_T1, e, st));
+        PSVD_TRY(prepare_operand(w.T1, n, unn, B, n, n, false, 1.f, w.esp(ES_B), split_out(w.T1hi, w.T1lo, ldn, nn, kF16X, w.fine), st));
         // E_H = T1 V  (B operand B[j][k] = V[k][j] = V^T[j][k])
         EpiStore e2 = epi_store_plain(w.BV, n, unn, n, n);
-        PSVD_TRY_RC(g16(w.T1hi, w.T1lo, n, n, ldn, nn, w.VThi, w.VTlo, n, ldn, nn, B, w.esp(ES_EH), e2, w.err, st));
+        PSVD_TRY_RC(g16(w.T1hi, w.T1lo, n, n, ldn, nn, w.VThi, w.VTlo, n, ldn, nn, w, ES_EH, e2, st));
     } else {
         PSVD_TRY(cudaMemsetAsync(w.BV, 0, sizeof(float) * (size_t)B * n * n, st));
     }
     if (dW) {
         // G = Wbar V (row-major FP32 for the epilogue, and transposed halves for Z)
-        PSVD_TRY(prepare_operand(dW, n, umn, B, m, n, false, 1.f, w.esp(ES_G), so16(w.Wbhi, w.Wblo, ldn, mn), st));
+        PSVD_TRY(prepare_operand(dW, n, umn, B, m, n, false, 1.f, w.esp(ES_G), split_out(w.Wbhi, w.Wblo, ldn, mn, kF16X, w.fine), st));
         EpiHalf e;
         memset(&e, 0, sizeof(e));
-        e.rows = m; e.cols = n; e.inv = w.esp(ES_IG);
+        e.rows = m; e.cols = n; e.inv = w.esp(ES_IG); e.fine = w.fine;
         e.out = w.G; e.ld = n; e.bs = umn;
         e.hi_t = w.GThi; e.lo_t = w.GTlo; e.ldht = ldm; e.bsht = nm;
-        PSVD_TRY_RC(g16(w.Wbhi, w.Wblo, m, n, ldn, mn, w.VThi, w.VTlo, n, ldn, nn, B, w.esp(ES_WV), e, w.err, st));
+        PSVD_TRY_RC(g16(w.Wbhi, w.Wblo, m, n, ldn, mn, w.VThi, w.VTlo, n, ldn, nn, w, ES_WV, e, st));
     }
     return bwd_tail(w, dW ? w.G : nullptr, EH, nullptr, nullptr, nullptr, (float)eps, eps == 0.0 ? 2 : 0, dA, st);
 }

@@ -86,6 +86,7 @@ struct GemmShape {
     unsigned *ticket;       // nullptr, or a zeroed counter: the last CTA to finish runs epi.tail()
     unsigned *err;          // device error word
     float f16_scale;        // PREC_F16X3: the product of the operands' inverse scales
+    float tf32_scale;       // PREC_TF32X3: the same (0: 1)
     const float *scale_b;   // split precisions: another factor for each matrix (nullptr: 1)
     int prof_as;            // profiling class + 1 for the launch timing (0: by precision)
 };
@@ -433,6 +434,7 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
             const int nph = nkb == 0 ? 0 : (prec >= PREC_TF32X3 ? nkb : 1);
             float fs = 1.f;                       // undoes the operands' powers of two (exact)
             if (prec == PREC_F16X3) fs = shp.f16_scale;
+            if (prec == PREC_TF32X3 && shp.tf32_scale != 0.f) fs = shp.tf32_scale;
             if (prec >= PREC_TF32X3 && shp.scale_b) fs *= shp.scale_b[b];
             float acc[128];
 #pragma unroll

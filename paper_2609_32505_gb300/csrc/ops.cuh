@@ -275,21 +275,23 @@ PSVD_DEV void f16_row16(const float (&v)[16], float fs, __half *rhi, __half *rlo
     }
 }
 
-// Split-FP16 output of v * inv[b] * kF16X, row-major (hi, may be null) and transposed (hi_t), optionally with
-// the plain values (out).
+// Split output of v * inv[b] in the format fine[b] (halves times kF16X), row-major (hi, may be null) and
+// transposed (hi_t), optionally with the plain values (out).
 struct EpiHalf {
     int rows, cols;
     const float *inv;
+    const int *fine;
     float *out;
     long long ld, bs;
-    __half *hi, *lo;
+    float *hi, *lo;
     long long ldh, bsh;
-    __half *hi_t, *lo_t;
+    float *hi_t, *lo_t;
     long long ldht, bsht;
     struct Acc {};
     static constexpr bool kRow = true;
     PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
         if (r0 >= rows || c0 >= cols) return true;
+        if (fine[b] == PREC_TF32X3) return false;
         if (c0 + 16 > cols || (out && ((((uintptr_t)out & 31) != 0) || ((ld | bs) & 7) != 0))) return false;
         const int r = r0 + lane, ct = c0 + (lane >> 1);
         if (out && r < rows) {
@@ -298,25 +300,24 @@ struct EpiHalf {
             for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(v[i]);
             st_v8x2(out + b * bs + (long long)r * ld + c0, w);
         }
-        const long long o = b * bsh + (long long)r * ldh + c0;
-        const long long t = b * bsht + (long long)ct * ldht + r0 + 16 * (lane & 1);    // (padding past `rows`: zeros)
-        f16_row16(v, inv[b] * kF16X, hi + o, lo + o, hi && r < rows, hi_t + t, lo_t + t, true, sw);
+        const long long o = 2 * b * bsh + (long long)r * ldh + c0;
+        const long long t = 2 * b * bsht + (long long)ct * ldht + r0 + 16 * (lane & 1);    // (padding past `rows`: zeros)
+        f16_row16(v, inv[b] * kF16X, as_half(hi) + o, as_half(lo) + o, hi && r < rows, as_half(hi_t) + t, as_half(lo_t) + t,
+                  true, sw);
         return true;
     }
     PSVD_DEV void begin(Acc &) const {}
     PSVD_DEV void chunk(Acc &, int b, int r, int c0, int, int, float (&v)[16]) const {
         if (r >= rows) return;
-        const float fs = inv[b] * kF16X;
+        const bool wide = fine[b] == PREC_TF32X3;
+        const float iv = inv[b];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int c = c0 + i;
             if (c >= cols) break;
             if (out) out[b * bs + (long long)r * ld + c] = v[i];
-            __half h, l;
-            split_f16(v[i] * fs, h, l);
-            if (hi) { hi[b * bsh + (long long)r * ldh + c] = h; lo[b * bsh + (long long)r * ldh + c] = l; }
-            hi_t[b * bsht + (long long)c * ldht + r] = h;
-            lo_t[b * bsht + (long long)c * ldht + r] = l;
+            if (hi) split_store(wide, hi, lo, b * bsh, (long long)r * ldh + c, v[i] * iv, kF16X);
+            split_store(wide, hi_t, lo_t, b * bsht, (long long)c * ldht + r, v[i] * iv, kF16X);
         }
     }
     PSVD_DEV bool staged() const { return false; }

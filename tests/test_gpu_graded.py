@@ -94,8 +94,8 @@ def test_polar_batch_of_ranges(precision, schedule):
         assert _rel(w[b][part], (u @ vt)[part]) <= 1e-5
 
 
-@pytest.mark.parametrize("t", [1.0, 1e-3, 1e-6, 1e-8])
-@pytest.mark.parametrize("m,n", [(200, 100), (300, 33)])
+@pytest.mark.parametrize("t", [1.0, 1e-3, 1e-6, 1e-8, 1e-12, 1e-18])
+@pytest.mark.parametrize("m,n", [(200, 100), (300, 33), (700, 272)])
 @pytest.mark.parametrize("grads", ["s", "all"])
 def test_svd_backward_rows(m, n, t, grads):
     """The gradient of either half of the rows, by the formula of the backward in FP64 on the same inputs.  With
@@ -129,6 +129,36 @@ def test_svd_backward_rows(m, n, t, grads):
     ref = (dU * D[None, :] + 2 * Y @ X) @ VT
     for r in (slice(0, m // 2), slice(m // 2, m)):
         assert _rel(da[r], ref[r]) <= 2e-5
+
+
+@pytest.mark.parametrize("t", [1e-3, 1e-12])
+@pytest.mark.parametrize("m,n", [(300, 40), (700, 272)])
+def test_polar_backward_rows(m, n, t):
+    """The same for the backward of W and H, next to a matrix of one size, whose bits do not depend on its neighbour."""
+    import paper_2609_32505_gb300 as P
+    g = np.random.default_rng(m)
+    a = np.stack([_full(m, n)] * 2)
+    d = np.where(np.arange(m) < m // 2, 1.0, t)[:, None]
+    a[1] *= d
+    a = a.astype(np.float32)
+    dw, dh = g.standard_normal((2, m, n)), g.standard_normal((2, n, n))
+    dw[1] /= d
+    dw, dh = dw.astype(np.float32), dh.astype(np.float32)
+    cu = lambda x: torch.from_numpy(x).cuda()
+    w, h = P.polar(cu(a))
+    da = P.polar_bwd(cu(a), w, h, cu(dw), cu(dh))
+    assert torch.equal(da[0], P.polar_bwd(cu(a[:1]), w[:1], h[:1], cu(dw[:1]), cu(dh[:1]))[0])
+    A, dW, dH, H = a[1].astype(np.float64), dw[1].astype(np.float64), dh[1].astype(np.float64), h[1].cpu().double().numpy()
+    eps = 1e-8
+    s, v = np.linalg.eigh(H)
+    r = (v * (s / (s * s + eps ** 0.5))) @ v.T
+    sym = lambda x: 0.5 * (x + x.T)
+    c = sym(sym(dH) - r @ (A.T @ dW) @ r)
+    tt = s[:, None] + s[None, :]
+    x = v @ ((tt / (tt * tt + eps ** 0.25)) * (v.T @ c @ v)) @ v.T
+    ref, da = dW @ r + 2.0 * A @ x, da[1].cpu().double().numpy()
+    for rows in (slice(0, m // 2), slice(m // 2, m)):
+        assert _rel(da[rows], ref[rows]) <= 2e-5
 
 
 @pytest.mark.parametrize("m,n", [(300, 40), (257, 257), (2100, 130), (9000, 66)])
