@@ -143,7 +143,10 @@ typedef struct psvd_info {
  * in psvd_info shows that the gate applied. */
 #define PSVD_MIXED_LB_MIN 5e-5
 
-/* ---- workspace queries ---------------------------------------------------- */
+/* ---- workspace queries ----------------------------------------------------
+ * Bytes of scratch of one call.  Calls with an eigendecomposition (svd_fwd, polar_bwd, eigh) hold, besides arrays of the
+ * batch's size, inverse iteration's scratch of as many matrices as fit 3 GB, one at least (740 MB for n = 4096,
+ * 11.8 GB for 16384). */
 size_t psvd_polar_workspace_bytes(int64_t batch, int64_t m, int64_t n, const psvd_opts *opts);
 size_t psvd_svd_workspace_bytes(int64_t batch, int64_t m, int64_t n, const psvd_opts *opts);
 size_t psvd_svd_bwd_workspace_bytes(int64_t batch, int64_t m, int64_t n);

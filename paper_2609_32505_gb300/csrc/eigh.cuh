@@ -12,6 +12,16 @@ constexpr int kBtSplit = 8; // largest K split of the back-transform's V^T Y pro
 constexpr int kIvJ = 8;     // rows per stage of inverse iteration's ring
 // rows of its arrays: half the matrix from either end, and what the last stage reads past it
 inline int iv_rows(int n) { return (int)round_up((n - 1) / 2 + kIvJ + 1, 2); }
+// doubles of one of them for a matrix: 16 vectors per warp, two lanes each
+inline long long iv_doubles(int n) { return (long long)((n + 15) / 16) * iv_rows(n) * 32; }
+// Matrices whose vectors are worked on at once: as many as fit 3 GB (five such arrays and the FP32 vectors), one at
+// least.  Four matrices of 4096 fit; one at a time leaves most of the chip idle.  (A matrix of 16384 takes 11.8 GB;
+// counted as 44 bytes an entry, without the padding to whole warps and stages, 65535 matrices of 33 took 6.4 GB.)
+constexpr long long kIvBytes = 3000000000LL;
+inline int iv_matrices(int B, int n) {
+    const long long per = 5 * 8 * iv_doubles(n) + 4LL * n * n;
+    return (int)std::max<long long>(1, std::min<long long>(B, kIvBytes / per));
+}
 
 struct EighWS {
     int B = 0, n = 0, nblk = 0, chunk = 0, nrp = 0;   // nrp: rows of Vh, padded to kWY
@@ -48,9 +58,7 @@ struct EighWS {
         nblk = n > 2 ? (n - 2 + kWY - 1) / kWY : 0;
         nrp = (int)round_up(n < 1 ? 1 : n, kWY);
         const long long B64 = B, nn = (long long)n * ldn, np = (long long)nrp * ldn;
-        // inverse-iteration scratch holds whole matrices: n vectors x n entries each, 44 bytes an entry; 2.9 GB
-        // at most (matrices of 4096 in fours; one at a time leaves most of the chip idle)
-        chunk = n * (int)std::max<long long>(1, std::min<long long>(B64, (1LL << 26) / ((long long)n * n)));
+        chunk = n * iv_matrices(B, n);
         Aw = cv.template take<float>(B64 * n * ldn);
         Vh = cv.template take<float>(B64 * np);
         tau = cv.template take<float>(B64 * n);
@@ -79,7 +87,7 @@ struct EighWS {
         Gm = cv.template take<float>(B64 * nrp * kWY);
         Gab = cv.template take<float>(B64 * nrp * kWY);
         xf = cv.template take<float>((long long)n * chunk);
-        const long long iv = (long long)(chunk / n) * ((n + 15) / 16) * iv_rows(n) * 32;   // 16 vectors per warp
+        const long long iv = (chunk / n) * iv_doubles(n);
         xs = cv.template take<double>(iv);
         lm = cv.template take<double>(iv);
         u = cv.template take<double>(3 * iv);
