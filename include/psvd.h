@@ -94,8 +94,8 @@ typedef struct psvd_opts {
                              U = Q U_R (svd_fwd) or W = Q W_R, H = H_R (polar_fwd) -- the QR
                              preprocessing of rectangular inputs of Section 4.1.  A learned
                              schedule's lower bounds then refer to R.  0 (default): the
-                             method runs on M itself.  Needs m <= 23040; psvd_polar_fwd_noalloc
-                             rejects it.                                                      */
+                             method runs on M itself.  Without effect for m > 23024 (psvd_qr's limit);
+                             psvd_polar_fwd_noalloc rejects it.                               */
 } psvd_opts;
 
 /* Fills *o with the defaults above (host pointer). */
@@ -307,8 +307,9 @@ int psvd_mlp_calibrate(const float *params, const float *F, const float *target,
  * psvd_qr -- thin QR A = Q R of a batch of m x n matrices (m >= n), diag(R) >= 0, by blocked
  *   Householder: panels of 64 (or 32) columns factored by one thread-block cluster per
  *   matrix, trailing updates and the accumulation of Q in compact-WY form on the tcgen05
- *   product kernel (split FP16, the matrix scaled by a power of two).  A: batch x m x n (read); Q: batch x m x n out (may alias A);
- *   R: batch x n x n out, upper triangular (may be NULL).  m <= 23024. */
+ *   product kernel (split operands, every column scaled by its own power of two: a column's accuracy
+ *   does not depend on the other columns' sizes).  A: batch x m x n (read); Q: batch x m x n out (may
+ *   alias A); R: batch x n x n out, upper triangular (may be NULL).  m <= 23024; above that PSVD_ERR_ARG. */
 size_t psvd_qr_workspace_bytes(int64_t batch, int64_t m, int64_t n);
 int psvd_qr(const float *A, float *Q, float *R, int64_t batch, int64_t m, int64_t n, void *ws,
             size_t ws_bytes, void *stream);

@@ -30,11 +30,13 @@ constexpr int kQrWarps = 16, kQrThreads = 32 * kQrWarps;
 constexpr int kQrMaxCl = 16;
 constexpr int kQrRows8 = 2048;            // panels of 64 columns up to here: 256 rows per CTA
 
-// The panel is 64 columns wide up to 8192 rows and 32 above, so that a CTA's rows fit its registers with
-// at most 16 CTAs per matrix; 23024 rows at most.
+// Panels are 64 columns wide as far as 16 CTAs hold 512 of their rows each in registers, and 32 above (1536 rows each).
+// kQrMaxRows is the interface's limit (psvd.h), within that.
+constexpr int kQrRows64 = kQrMaxCl * 512, kQrRows32 = kQrMaxCl * 1536;
+static_assert(kQrMaxRows <= kQrRows32, "panel registers");
 bool qr_shape(int m, int *nb) {
-    *nb = m <= 8192 ? 64 : 32;
-    return m <= 23024;
+    *nb = m <= kQrRows64 ? 64 : 32;
+    return m <= kQrMaxRows;
 }
 
 // four consecutive elements of a split array

@@ -6,7 +6,8 @@
 
 namespace psvd {
 
-// Panel width nb (64 or 32) for m rows; false when m is too large for the cluster panel.
+constexpr int kQrMaxRows = 23024;
+// Panel width nb (64 or 32) for m rows; false above kQrMaxRows.
 bool qr_shape(int m, int *nb);
 
 constexpr int kQrSplit = 8;   // largest K split of the X^T Y products of a block
