@@ -324,7 +324,6 @@ struct EpiQ {
     float *Q;
     unsigned *qmax;
     struct Acc { unsigned mx; };
-    static constexpr bool kRow = true;
     PSVD_DEV bool row16(Acc &a, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
         if (r0 >= m || c0 >= n) return true;
         if (c0 + 16 > n || (n & 7) || ((uintptr_t)Q & 31) || (G && ((uintptr_t)G & 31))) return false;
@@ -350,9 +349,8 @@ struct EpiQ {
         if (r < m) st_v8x2(Q + o, w);
         return true;
     }
-    PSVD_DEV bool staged() const { return false; }
     PSVD_DEV void begin(Acc &a) const { a.mx = 0u; }
-    PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
+    PSVD_DEV void chunk(Acc &a, int b, int r, int c0, float (&v)[16]) const {
         if (r >= m) return;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -606,7 +604,7 @@ int eigh_backward(const float *S, const float *VT, const float *dS, const float 
     {   // Z = V E (E symmetric, so the B operand B[k][j] = E[j][k] is E itself)
         EpiStore e;
         memset(&e, 0, sizeof(e));
-        e.rows = n; e.cols = n; e.alpha = 1.f;
+        e.rows = n; e.cols = n;
         e.hi = w.Zhi; e.lo = w.Zlo; e.ldh = ldn; e.bsh = nn;
         PSVD_TRY_RC(g3(w.Vhi, w.Vlo, n, n, ldn, nn, w.Ehi, w.Elo, n, ldn, nn, B, e, w.err, st));
     }

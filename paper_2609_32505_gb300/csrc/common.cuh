@@ -235,41 +235,6 @@ PSVD_DEV void counter_barrier(unsigned *ctr, unsigned target, unsigned *err, uin
     __syncthreads();
 }
 
-// Flag barrier over `g` co-resident CTAs: CTA c publishes arrive[c] = gen; CTA 0 polls all
-// arrival flags in parallel and publishes release = gen, which every other CTA polls.
-// Every wait is bounded and stops at once when the error word is raised elsewhere.
-PSVD_DEV void flag_barrier(unsigned *arrive, unsigned *release, int cig, int g, unsigned gen, unsigned *err) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        *(volatile unsigned *)&arrive[cig] = gen;
-    }
-    if (cig == 0) {
-        for (int c = threadIdx.x; c < g; c += blockDim.x) {
-            for (uint32_t i = 0;; ++i) {
-                if (*(volatile unsigned *)&arrive[c] >= gen) break;
-                if (*(volatile unsigned *)err) break;
-                if (i > kBarrierSpin) { atomicOr(err, DEV_ERR_TIMEOUT); break; }
-                __nanosleep(20);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            *(volatile unsigned *)release = gen;
-        }
-    } else if (threadIdx.x == 0) {
-        for (uint32_t i = 0;; ++i) {
-            if (*(volatile unsigned *)release >= gen) break;
-            if (*(volatile unsigned *)err) break;
-            if (i > kBarrierSpin) { atomicOr(err, DEV_ERR_TIMEOUT); break; }
-            __nanosleep(20);
-        }
-    }
-    __threadfence();
-    __syncthreads();
-}
-
 // ---------------------------------------------------------------- float-float sums
 // Compensated FP32 accumulation (Knuth's TwoSum and the FMA-based exact product,
 // written with the _rn intrinsics so that no add is contracted into an FMA): the
@@ -336,27 +301,6 @@ PSVD_DEV float block_sum_ff(ff v, float *red) {
     ff t = l < nw ? ff{red[l], red[32 + l]} : ff_zero();
     t = warp_sum(t);
     return __fadd_rn(t.hi, t.lo);
-}
-
-// Flag barrier over `g` co-resident CTAs in which every CTA polls every arrival
-// flag (no release hop): CTA c publishes arrive[c] = gen, then its threads wait
-// until all g flags have reached gen.  Bounded like flag_barrier.
-PSVD_DEV void flag_barrier_all(unsigned *arrive, int cig, int g, unsigned gen, unsigned *err) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        *(volatile unsigned *)&arrive[cig] = gen;
-    }
-    for (int c = threadIdx.x; c < g; c += blockDim.x) {
-        for (uint32_t i = 0;; ++i) {
-            if (*(volatile unsigned *)&arrive[c] >= gen) break;
-            if (*(volatile unsigned *)err) break;
-            if (i > kBarrierSpin) { atomicOr(err, DEV_ERR_TIMEOUT); break; }
-            __nanosleep(20);
-        }
-    }
-    __threadfence();
-    __syncthreads();
 }
 
 PSVD_DEV double block_sum(double v, double *red) {

@@ -36,9 +36,6 @@ namespace psvd {
 #ifndef PSVD_TRD_ROWDIV
 #define PSVD_TRD_ROWDIV 24
 #endif
-#ifndef PSVD_TRD_BARRIER
-#define PSVD_TRD_BARRIER 3      // 0: release flag, 1: every CTA polls every flag, 2: arrival counter,
-#endif                          // 3: arrival counter with release/acquire operations
 #ifndef PSVD_TRD_SLEEP
 #define PSVD_TRD_SLEEP 40
 #endif
@@ -183,17 +180,8 @@ __global__ void __launch_bounds__(kTrdThreads, PSVD_TRD_MINB) sytrd_kernel(TrdPa
     // about n / g rows spread over the whole matrix and loses them at the same rate
     const int gw = warp * P.g + cig, GW = P.g * nwarp;
     unsigned *rel = P.bar + (long long)grp * (P.g + 1);
-    unsigned *arr = rel + 1;
     unsigned nbar = 0;
-#if PSVD_TRD_BARRIER == 1
-#define TRD_BARRIER() flag_barrier_all(arr, cig, P.g, ++nbar, P.err)
-#elif PSVD_TRD_BARRIER == 2
-#define TRD_BARRIER() group_barrier(rel, (unsigned)P.g * (++nbar), P.err, P.spin)
-#elif PSVD_TRD_BARRIER == 3
 #define TRD_BARRIER() counter_barrier<PSVD_TRD_SLEEP>(rel, (unsigned)P.g * (++nbar), P.err, P.spin)
-#else
-#define TRD_BARRIER() flag_barrier(arr, rel, cig, P.g, ++nbar, P.err)
-#endif
     for (int b = grp; b < P.B; b += P.groups) {
         const float *Hb = P.H + (long long)b * n * n;
         float *A = P.Aw + (long long)b * n * ln;

@@ -140,8 +140,7 @@ PSVD_DEV TileJob tile_job(const GemmShape &s, int t, int tpm) {
     return j;
 }
 
-// Epilogues that define a per-element elem(acc, b, r, c, v) and a runtime staged() get
-// their values through a per-warp shared-memory transpose, so that each store instruction
+// Epilogues that define a per-element elem(acc, b, r, c, v) get their values through a per-warp shared-memory transpose, so that each store instruction
 // of a warp covers two rows x 16 consecutive columns instead of 32 rows x 1 column.
 template <class E, class = void> struct EpiHasElem : std::false_type {};
 template <class E> struct EpiHasElem<E, std::void_t<decltype(E::kElem)>> : std::integral_constant<bool, E::kElem> {};
@@ -156,14 +155,15 @@ template <class E> struct EpiHasTrans<E, std::void_t<decltype(E::kTrans)>> : std
 template <class E, class = void> struct EpiHasTail : std::false_type {};
 template <class E> struct EpiHasTail<E, std::void_t<decltype(E::kTail)>> : std::integral_constant<bool, E::kTail> {};
 
-// Epilogues with row16(acc, b, r0, lane, c0, v, sw) get the 16 columns c0 .. c0 + 15 of the thread's row
+// row16(acc, b, r0, lane, c0, v, sw) of every epilogue gets the 16 columns c0 .. c0 + 15 of the thread's row
 // r0 + lane as they are and store them in 32-byte pieces: along the row directly (a whole sector per
 // lane), transposed through the warp's shared memory `sw` (warp_transpose16).  It returns false
 // (uniformly) for pieces it does not handle -- ragged edges, the diagonal, unaligned outputs -- which
-// then take the element-wise paths above.  (Element by element a polar step's tile cost ~17,000
+// then take the element-wise paths above, or chunk(acc, b, r, c0, v) on the thread's own row where there is no
+// elem; kTotal: it handles every piece.  (Element by element a polar step's tile cost ~17,000
 // instructions per warp, about half the time of a 4096^3 split product: 474 -> 310 us with the pieces.)
-template <class E, class = void> struct EpiHasRow : std::false_type {};
-template <class E> struct EpiHasRow<E, std::void_t<decltype(E::kRow)>> : std::integral_constant<bool, E::kRow> {};
+template <class E, class = void> struct EpiIsTotal : std::false_type {};
+template <class E> struct EpiIsTotal<E, std::void_t<decltype(E::kTotal)>> : std::integral_constant<bool, E::kTotal> {};
 
 // 32 bytes at a 32-byte aligned address
 PSVD_DEV void st_v8(void *p, const uint32_t (&r)[8]) {
@@ -199,6 +199,13 @@ PSVD_DEV void warp_transpose16(float *sw, const uint32_t (&w)[16], uint32_t (&o)
         const uint4 x = q[i];
         o[4 * i] = x.x; o[4 * i + 1] = x.y; o[4 * i + 2] = x.z; o[4 * i + 3] = x.w;
     }
+}
+// the warp's values, lane = row, into its staging area (rows of kStageRow)
+PSVD_DEV void stage_piece(const float (&v)[16], float *sw) {
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sw[(threadIdx.x & 31) * kStageRow + i] = v[i];
+    __syncwarp();
 }
 // Sums of 16 per-lane values over the warp: lane l returns the sum of value l >> 1.
 PSVD_DEV float warp_sum16(float (&a)[16]) {
@@ -466,8 +473,6 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
             const int cbase = tj * bn + half * ncols;
             typename Epi::Acc ea;
             epi.begin(ea);
-            bool staged = false;
-            if constexpr (EpiHasElem<Epi>::value) staged = epi.staged();
             float *sw = stage + warp * kStageWarp;
             const int r0 = ti * kBM + quad * 32, rr0 = lane >> 4, cc = lane & 15;
 #pragma unroll
@@ -476,17 +481,9 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
                 float v[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] = acc[c + i];
-                if constexpr (EpiHasRow<Epi>::value)
-                    if (epi.row16(ea, be, r0, lane, cbase + c, v, sw)) continue;
-                if (!staged) {
-                    epi.chunk(ea, be, r, cbase + c, ti, tj, v);
-                    continue;
-                }
+                if (epi.row16(ea, be, r0, lane, cbase + c, v, sw)) continue;
                 if constexpr (EpiHasElem<Epi>::value) {
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) sw[lane * kStageRow + i] = v[i];
-                    __syncwarp();
+                    stage_piece(v, sw);
 #pragma unroll 1
                     for (int k = 0; k < 16; ++k) {
                         const int rr = 2 * k + rr0;
@@ -494,6 +491,8 @@ gemm_tn_kernel(const __grid_constant__ GemmMaps maps, const GemmShape shp, Epi e
                     }
                     __syncwarp();
                     if constexpr (EpiHasTrans<Epi>::value) epi.trans(ea, be, r, cbase + c, v);
+                } else if constexpr (!EpiIsTotal<Epi>::value) {
+                    epi.chunk(ea, be, r, cbase + c, v);
                 }
             }
             epi.finish(ea, be, ti, tj);

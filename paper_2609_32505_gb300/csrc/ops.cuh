@@ -111,85 +111,46 @@ cudaError_t fine_reset(int *fine, int B, cudaStream_t st);
 cudaError_t fine_rows(const float *A, int B, int m, int n, const float *colscale, const int *skip, int *fine,
                       cudaStream_t st);
 
-// Generic epilogue: D = alpha * acc (+ beta * C) stored row-major, transposed,
-// and/or split into TF32 hi/lo halves (row-major or transposed).
+// D = acc, row-major, plain (out, may be null) and/or split TF32 (hi and lo, may be null).
 struct EpiStore {
     int rows, cols;
-    float alpha;
-    const float *cin; long long ldc, bsc; float beta;      // optional addend
-    float *out; long long ld, bs;                          // optional plain store
-    float *out_t; long long ldt, bst;                      // optional transposed store
-    float *hi, *lo; long long ldh, bsh;                    // optional split store
-    float *hi_t, *lo_t; long long ldht, bsht;              // optional split transposed store
+    float *out; long long ld, bs;
+    float *hi, *lo; long long ldh, bsh;
     struct Acc {};
-    static constexpr bool kElem = true, kRow = true;
-    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
+    static constexpr bool kElem = true;
+    PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
         if (r0 >= rows || c0 >= cols) return true;
-        if (cin || out_t || c0 + 16 > cols) return false;
-        if (out && ((((uintptr_t)out & 31) != 0) || ((ld | bs) & 7) != 0)) return false;
+        if (c0 + 16 > cols || (out && ((((uintptr_t)out & 31) != 0) || ((ld | bs) & 7) != 0))) return false;
         const int r = r0 + lane;
+        if (r >= rows) return true;
         uint32_t h[16], l[16];
+        if (out) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) h[i] = __float_as_uint(alpha * v[i]);
-        if (out && r < rows) st_v8x2(out + b * bs + (long long)r * ld + c0, h);
-        if (!hi && !hi_t) return true;
+            for (int i = 0; i < 16; ++i) h[i] = __float_as_uint(v[i]);
+            st_v8x2(out + b * bs + (long long)r * ld + c0, h);
+        }
+        if (!hi) return true;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             float a, c;
-            split_tf32(__uint_as_float(h[i]), a, c);
+            split_tf32(v[i], a, c);
             h[i] = __float_as_uint(a);
             l[i] = __float_as_uint(c);
         }
-        if (hi && r < rows) {
-            const long long o = b * bsh + (long long)r * ldh + c0;
-            st_v8x2(hi + o, h);
-            if (lo) st_v8x2(lo + o, l);
-        }
-        if (hi_t) {                       // rows past `rows` are zeros of the padding
-            const long long o = b * bsht + (long long)(c0 + (lane >> 1)) * ldht + r0 + 16 * (lane & 1);
-            uint32_t t[16];
-            warp_transpose16(sw, h, t);
-            st_v8x2(hi_t + o, t);
-            if (lo_t) {
-                warp_transpose16(sw, l, t);
-                st_v8x2(lo_t + o, t);
-            }
-        }
+        const long long o = b * bsh + (long long)r * ldh + c0;
+        st_v8x2(hi + o, h);
+        st_v8x2(lo + o, l);
         return true;
     }
-    // staged (coalesced) element path when nothing is stored transposed
-    PSVD_DEV bool staged() const { return !out_t && !hi_t; }
     PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
         if (r >= rows || c >= cols) return;
-        float x = alpha * v;
-        if (cin) x += beta * cin[b * bsc + (long long)r * ldc + c];
-        if (out) out[b * bs + (long long)r * ld + c] = x;
+        if (out) out[b * bs + (long long)r * ld + c] = v;
         if (hi) {
-            float h, l;
-            split_tf32(x, h, l);
-            hi[b * bsh + (long long)r * ldh + c] = h;
-            if (lo) lo[b * bsh + (long long)r * ldh + c] = l;
+            const long long o = b * bsh + (long long)r * ldh + c;
+            split_tf32(v, hi[o], lo[o]);
         }
     }
     PSVD_DEV void begin(Acc &) const {}
-    PSVD_DEV void chunk(Acc &, int b, int r, int c0, int, int, float (&v)[16]) const {
-        if (r >= rows) return;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = c0 + i;
-            if (c >= cols) break;
-            float x = alpha * v[i];
-            if (cin) x += beta * cin[b * bsc + (long long)r * ldc + c];
-            if (out) out[b * bs + (long long)r * ld + c] = x;
-            if (out_t) out_t[b * bst + (long long)c * ldt + r] = x;
-            if (hi || hi_t) {
-                float h, l;
-                split_tf32(x, h, l);
-                if (hi) { hi[b * bsh + (long long)r * ldh + c] = h; if (lo) lo[b * bsh + (long long)r * ldh + c] = l; }
-                if (hi_t) { hi_t[b * bsht + (long long)c * ldht + r] = h; if (lo_t) lo_t[b * bsht + (long long)c * ldht + r] = l; }
-            }
-        }
-    }
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 
@@ -204,7 +165,7 @@ struct EpiSubHalf {
     float *fhi, *flo;
     long long fbs;
     struct Acc {};
-    static constexpr bool kElem = true, kRow = true;
+    static constexpr bool kElem = true;
     PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
         if (r0 >= rows || c0 >= cols) return true;
         if (fine && fine[b] == PREC_TF32X3) return false;
@@ -226,7 +187,6 @@ struct EpiSubHalf {
         st_v8(lo + o, l);
         return true;
     }
-    PSVD_DEV bool staged() const { return true; }
     PSVD_DEV void elem(Acc &, int b, int r, int c, float v) const {
         if (r >= rows || c >= cols) return;
         if (fine && fine[b] == PREC_TF32X3) {
@@ -241,10 +201,6 @@ struct EpiSubHalf {
         lo[o] = l;
     }
     PSVD_DEV void begin(Acc &) const {}
-    PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) elem(a, b, r, c0 + i, v[i]);
-    }
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 
@@ -288,7 +244,6 @@ struct EpiHalf {
     float *hi_t, *lo_t;
     long long ldht, bsht;
     struct Acc {};
-    static constexpr bool kRow = true;
     PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
         if (r0 >= rows || c0 >= cols) return true;
         if (fine[b] == PREC_TF32X3) return false;
@@ -307,7 +262,7 @@ struct EpiHalf {
         return true;
     }
     PSVD_DEV void begin(Acc &) const {}
-    PSVD_DEV void chunk(Acc &, int b, int r, int c0, int, int, float (&v)[16]) const {
+    PSVD_DEV void chunk(Acc &, int b, int r, int c0, float (&v)[16]) const {
         if (r >= rows) return;
         const bool wide = fine[b] == PREC_TF32X3;
         const float iv = inv[b];
@@ -320,7 +275,6 @@ struct EpiHalf {
             split_store(wide, hi_t, lo_t, b * bsht, (long long)c * ldht + r, v[i] * iv, kF16X);
         }
     }
-    PSVD_DEV bool staged() const { return false; }
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 
@@ -329,7 +283,7 @@ int orth_product(Carver &cv, const float *Q, const float *X, float *out, int B, 
 inline EpiStore epi_store_plain(float *out, long long ld, long long bs, int rows, int cols) {
     EpiStore e;
     memset(&e, 0, sizeof(e));
-    e.rows = rows; e.cols = cols; e.alpha = 1.f;
+    e.rows = rows; e.cols = cols;
     e.out = out; e.ld = ld; e.bs = bs;
     return e;
 }

@@ -291,14 +291,6 @@ __device__ __noinline__ ff wide_piece(const float *v, float *rhi, float *rlo, lo
         if (lane < nr && c + off > lane) split_tf32(c3 * v[lane * kStageRow + c], chi[c * ldc + lane], clo[c * ldc + lane]);
     return res;
 }
-// the warp's values, lane = row, into its staging area
-PSVD_DEV void stage_piece(const float (&v)[16], float *sw) {
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) sw[(threadIdx.x & 31) * kStageRow + i] = v[i];
-    __syncwarp();
-}
-
 // 16 values of one row in the format of rung p: along the row at element ro (roh for halves) when
 // `rowv`, and transposed (this lane's 16 rows of column c0 + lane / 2) at element co (coh) when `colv`.
 PSVD_DEV void rung_row16(int p, const float (&v)[16], float fs, __nv_bfloat16 *r16, float *rhi, float *rlo,
@@ -382,7 +374,7 @@ struct EpiGram {
     float *Phi, *Plo;
     long long ldp;
     struct Acc { ff r; int p; float c1, c3; };     // ||G - I||^2 partial, float-float (FP32 pipe)
-    static constexpr bool kElem = true, kTrans = true, kTail = true, kRow = true;
+    static constexpr bool kElem = true, kTrans = true, kTail = true;
     PSVD_DEV bool row16(Acc &a, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
         if (r0 >= n || c0 >= n || c0 + 15 < r0) return true;       // outside, or left to the mirror's tile
         load(a, b);
@@ -408,7 +400,6 @@ struct EpiGram {
                    ct < n, sw);
         return true;
     }
-    PSVD_DEV bool staged() const { return true; }
     PSVD_DEV void tail() const {
         for (int b = threadIdx.x; b < dec.B; b += blockDim.x) decide_matrix(dec, b);
     }
@@ -438,11 +429,6 @@ struct EpiGram {
             store_rung(a.p, bo, rc, a.c3 * v[i], kF16P, P16, Phi, Plo);
         }
     }
-    PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) elem(a, b, r, c0 + i, v[i]);
-        trans(a, b, r, c0, v);
-    }
     PSVD_DEV void finish(Acc &a, int b, int, int) const {
         const double s = warp_sum((double)a.r.hi + (double)a.r.lo);
         if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(&res[b], s);
@@ -458,7 +444,7 @@ struct EpiApply {
     float *Xhi, *Xlo, *XThi, *XTlo;
     long long ldn, ldm;
     struct Acc { int p; };
-    static constexpr bool kElem = true, kTrans = true, kRow = true;
+    static constexpr bool kTotal = true;
     PSVD_DEV bool row16(Acc &a, int b, int r0, int lane, int c0, float (&v)[16], float *sw) const {
         if (r0 >= m || c0 >= n) return true;
         if (a.p < 0) a.p = prec_next[b];
@@ -477,31 +463,7 @@ struct EpiApply {
                    ct < n, sw);
         return true;
     }
-    PSVD_DEV bool staged() const { return true; }
     PSVD_DEV void begin(Acc &a) const { a.p = -1; }
-    PSVD_DEV void elem(Acc &a, int b, int r, int c, float x) const {
-        if (r >= m || c >= n) return;
-        if (a.p < 0) a.p = prec_next[b];
-        const long long bo = (long long)b * m * ldn, rc = (long long)r * ldn + c;
-        store_rung(a.p, bo, rc, x, kF16X, X16, Xhi, Xlo);
-    }
-    PSVD_DEV void trans(Acc &a, int b, int r, int c0, float (&v)[16]) const {
-        if (r >= m) return;
-        if (a.p < 0) a.p = prec_next[b];
-        const long long bo = (long long)b * n * ldm;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = c0 + i;
-            if (c >= n) break;
-            const long long rc = (long long)c * ldm + r;
-            store_rung(a.p, bo, rc, v[i], kF16X, XT16, XThi, XTlo);
-        }
-    }
-    PSVD_DEV void chunk(Acc &a, int b, int r, int c0, int, int, float (&v)[16]) const {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) elem(a, b, r, c0 + i, v[i]);
-        trans(a, b, r, c0, v);
-    }
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
 

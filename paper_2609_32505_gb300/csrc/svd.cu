@@ -26,7 +26,6 @@ struct EpiColNorm {
     float *U;
     float *colss;   // [B][n]
     struct Acc {};
-    static constexpr bool kRow = true;
     PSVD_DEV bool row16(Acc &, int b, int r0, int lane, int c0, float (&v)[16], float *) const {
         if (r0 >= m || c0 >= n) return true;
         if (c0 + 16 > n || (n & 7) || ((uintptr_t)U & 31)) return false;
@@ -40,9 +39,8 @@ struct EpiColNorm {
         if (!(lane & 1) && s != 0.f) atomicAdd(&colss[(long long)b * n + c0 + (lane >> 1)], s);
         return true;
     }
-    PSVD_DEV bool staged() const { return false; }
     PSVD_DEV void begin(Acc &) const {}
-    PSVD_DEV void chunk(Acc &, int b, int r, int c0, int, int, float (&v)[16]) const {
+    PSVD_DEV void chunk(Acc &, int b, int r, int c0, float (&v)[16]) const {
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int c = c0 + i;
