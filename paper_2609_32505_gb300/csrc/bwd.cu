@@ -11,7 +11,7 @@
 // G = Wbar V in place of Ubar.  Six products on the split-FP16 tcgen05 kernel plus
 // one elementwise kernel that holds every mask (K_eps, T_eps, D_R).  The products are bound by the tensor
 // cores: at 4096 x 4096 each takes 345 us in split FP16 (0.40 PFLOP/s of FP32-accurate work, three FP16
-// products each) and took 700 us in split TF32; the whole backward 4.10 -> 2.40 ms, its error against
+// products each) and took 700 us in split TF32; the whole backward 4.10 -> 2.43 ms, its error against
 // 64 bits unchanged at 2.2e-6.
 #include <cmath>
 #include <cstring>
@@ -80,7 +80,7 @@ struct BwdWS {
         X = cv.template take<float>(B64 * n * n); Q = cv.template take<float>(B64 * m * n);
         S = cv.template take<float>(B64 * n);
         amax = cv.template take<unsigned>(B64 * (AM_N + m + n));
-        ext = amax + B64 * AM_N;
+        ext = amax ? amax + B64 * AM_N : nullptr;
         fine = cv.template take<int>(B64);
         es = cv.template take<float>(B64 * ES_N);
         err = cv.template take<unsigned>(4);
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256) bwd_fine_kernel(const unsigned *amax, con
 }
 
 // The AM_ slots of the inputs, one launch for all of them (grid.z = slot): entries, or for V^T the 2-norm
-// of its rows, a warp at a time.  For M also the largest entries of its rows and columns, by tiles of 32 x 128 a
+// of its rows, a warp at a time.  For M also the largest entries of its rows and columns, by tiles of 8 x 128 a
 // warp (ext).
 struct BwdMaxIn { const float *x[AM_IN]; long long len[AM_IN]; };
 __global__ void __launch_bounds__(256) bwd_max_kernel(BwdMaxIn in, int B, int m, int n, unsigned *amax, unsigned *ext) {
@@ -159,25 +159,26 @@ __global__ void __launch_bounds__(256) bwd_max_kernel(BwdMaxIn in, int B, int m,
     const float *a = in.x[slot] + b * len;
     unsigned v = 0;
     if (slot == AM_M) {
-        const int tn = (n + 127) / 128, tiles = tn * ((m + 31) / 32);
+        const int tn = (n + 127) / 128, tiles = tn * ((m + 7) / 8);
         for (int t = blockIdx.x * 8 + warp; t < tiles; t += gridDim.x * 8) {
-            const int r0 = t / tn * 32, c0 = t % tn * 128 + lane, nr = min(32, m - r0);
-            unsigned cm[4] = {0u, 0u, 0u, 0u}, rm = 0u;
-#pragma unroll 8
-            for (int r = 0; r < nr; ++r) {
-                unsigned x = 0u;
+            const int r0 = t / tn * 8, c0 = t % tn * 128 + lane;
+            unsigned y[8][4];                      // all loads ahead of the reductions
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    if (c0 + 32 * q < n) {
-                        const unsigned y = __float_as_uint(fabsf(a[(long long)(r0 + r) * n + c0 + 32 * q]));
-                        cm[q] = max(cm[q], y);
-                        x = max(x, y);
-                    }
-                x = __reduce_max_sync(0xffffffffu, x);
+                    y[r][q] = r0 + r < m && c0 + 32 * q < n
+                                  ? __float_as_uint(fabsf(a[(long long)(r0 + r) * n + c0 + 32 * q])) : 0u;
+            unsigned cm[4] = {0u, 0u, 0u, 0u}, rm = 0u;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cm[q] = max(cm[q], y[r][q]);
+                const unsigned x = __reduce_max_sync(0xffffffffu, max(max(y[r][0], y[r][1]), max(y[r][2], y[r][3])));
                 if (lane == r) rm = x;
             }
             unsigned *e = ext + (long long)b * (m + n);
-            if (lane < nr) atomicMax(&e[r0 + lane], rm);
+            if (lane < 8 && r0 + lane < m) atomicMax(&e[r0 + lane], rm);
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 if (c0 + 32 * q < n) atomicMax(&e[m + c0 + 32 * q], cm[q]);

@@ -264,16 +264,19 @@ struct EpiHalf {
     PSVD_DEV void begin(Acc &) const {}
     PSVD_DEV void chunk(Acc &, int b, int r, int c0, float (&v)[16]) const {
         if (r >= rows) return;
-        const bool wide = fine[b] == PREC_TF32X3;
         const float iv = inv[b];
+        auto store = [&](auto wide) {              // (the format decided once, not per value)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = c0 + i;
-            if (c >= cols) break;
-            if (out) out[b * bs + (long long)r * ld + c] = v[i];
-            if (hi) split_store(wide, hi, lo, b * bsh, (long long)r * ldh + c, v[i] * iv, kF16X);
-            split_store(wide, hi_t, lo_t, b * bsht, (long long)c * ldht + r, v[i] * iv, kF16X);
-        }
+            for (int i = 0; i < 16; ++i) {
+                const int c = c0 + i;
+                if (c >= cols) break;
+                if (out) out[b * bs + (long long)r * ld + c] = v[i];
+                if (hi) split_store(wide, hi, lo, b * bsh, (long long)r * ldh + c, v[i] * iv, kF16X);
+                split_store(wide, hi_t, lo_t, b * bsht, (long long)c * ldht + r, v[i] * iv, kF16X);
+            }
+        };
+        if (fine[b] == PREC_TF32X3) store(std::true_type{});
+        else store(std::false_type{});
     }
     PSVD_DEV void finish(Acc &, int, int, int) const {}
 };
