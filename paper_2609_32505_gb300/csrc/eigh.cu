@@ -1377,7 +1377,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
         P.ldn = ldn;
         P.spin = barrier_spin();
         const size_t smem = sizeof(float) * 3 * (size_t)ldn;
-        PSVD_TRY(cudaFuncSetAttribute(sytrd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        PSVD_TRY(cudaFuncSetAttribute(sytrd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 12 * kEighMaxN));
         int occ = 0;
         PSVD_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sytrd_kernel, kTrdThreads, smem));
         if (occ * num_sms() < P.groups * P.g) return cuda_fail(cudaErrorCooperativeLaunchTooLarge, __FILE__, __LINE__);
@@ -1399,7 +1399,7 @@ int eigh_forward(const float *Hs, float *S, float *VT, EighWS &w, cudaStream_t s
         const int rows = iv_rows(n);
         auto run = [&](auto lanes) -> cudaError_t {
             constexpr int kL = decltype(lanes)::value;
-            cudaError_t e = cudaFuncSetAttribute(tri_bisect_kernel<kL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = cudaFuncSetAttribute(tri_bisect_kernel<kL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kEighMaxN);
             if (e != cudaSuccess) return e;
             tri_bisect_kernel<kL><<<g, 256, smem, st>>>(w.d, w.e, n, w.lam, tn);
             sturm_prep_kernel<<<dim3((std::max(n, rows) + 255) / 256, B), 256, 0, st>>>(w.d, w.e, tn, n, rows, w.sturm,
@@ -1590,7 +1590,7 @@ extern "C" size_t psvd_eigh_workspace_bytes(int64_t batch, int64_t n) {
 
 extern "C" int psvd_eigh(const float *Hs, float *S, float *VT, int64_t batch, int64_t n, void *ws, size_t ws_bytes,
                          void *stream) {
-    if (!Hs || (!S && !VT) || batch <= 0 || n <= 0 || n > 16384 || batch > 65535) return PSVD_ERR_ARG;
+    if (!Hs || (!S && !VT) || batch <= 0 || n <= 0 || n > kEighMaxN || batch > 65535) return PSVD_ERR_ARG;
     if (int e = check_device()) return e;
     if (ws_bytes < psvd_eigh_workspace_bytes(batch, n)) return PSVD_ERR_WORKSPACE;
     Carver cv(ws, ws_bytes);

@@ -6,6 +6,10 @@
 
 namespace psvd {
 
+// Largest n.  The kernels whose shared memory goes with n have their limit set for this one: the limit is the
+// function's, for all threads, and a call that set it for its own n could lower it between another thread's setting
+// and launch.
+constexpr int kEighMaxN = 16384;
 constexpr int kTrdChipMin = 3, kTrdChipMax = 4096;   // sizes whose tridiagonalization runs on chip (trd.cu)
 constexpr int kBtSplit = 8; // largest K split of the back-transform's V^T Y products
 
