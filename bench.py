@@ -4,7 +4,7 @@ geometric spectrum, the square-matrix setting of Section 4.1 / Tables 1-2), FP32
 One step = psvd_svd_fwd (Algorithm 1) + psvd_svd_bwd (Algorithm 4, eps = 1e-8) of the
 loss <G_U, U> + <g_S, sigma> + <G_V, V> with seeded N(0,1) weights.  The headline
 `value` is the mixed-precision path (BF16 -> TF32 -> split-FP16 polish, eigenbasis
-correction); the plain FP32-accurate path (split FP16 throughout) is timed beside it.
+correction); the plain FP32-accurate path (split FP16 throughout) is timed beside it, and is as fast.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -363,11 +363,12 @@ def main():
                 "traffic": None,
                 "kernel": "trd_chip_kernel (Householder tridiagonalization of H, eigensolver stage 1; all its launches)",
                 "algorithmic_bytes": trd["work"], "ms": trd["ms"], "share_of_step": trd["ms"] / ms_mixed,
-                "peak_src": "SMs x 128 B/clock x 2.07 GHz (shared memory)",
-                "l2_peak": l2_gbs,
+                "peak_src": "nominal, not measured: SMs x 128 B/clock x 2.07 GHz (shared-memory port)",
+                "l2_peak": l2_gbs, "frac_of_l2_peak": trd_gbs / l2_gbs,
                 "note": (f"every step reads and writes the trailing matrix, 8 sum (n-k-2)^2 bytes, held in the SMs' "
                          f"registers, shared and tensor memory; streamed through L2 the measured read-modify-write "
-                         f"peak would be {l2_gbs:.0f} GB/s; in flops (4/3 n^3) "
+                         f"peak would be {l2_gbs:.0f} GB/s; by the counters neither the port nor a pipe is the "
+                         f"limit, the warps of a block wait for each other at its barriers; in flops (4/3 n^3) "
                          f"{trd_flops / (trd['ms'] * 1e-3) / 1e12 if trd['ms'] > 0 else 0:.2f} TFLOP/s; one exchange "
                          f"between all SMs per reflector (~1.5 us) is the other half of the time"),
                 "polar_chain": {"bound": "tensor", "achieved": chain_tf, "unit": "TFLOP/s",

@@ -50,11 +50,20 @@ extern "C" {
 #define PSVD_ERR_UNSUPPORTED   -6   /* device is not sm_103 / sm_100 class            */
 
 /* ---- options ----------------------------------------------------------- */
-#define PSVD_PREC_FP32       0   /* every product FP32-accurate (operands split into FP16
-                                    halves hi + lo and scaled by powers of two, three products) */
+/* Operands of FP32-accurate products are split in two halves, 22 bits of every entry, and multiplied in three
+ * products: FP16 halves scaled by powers of two, or TF32 halves for a matrix that has rows or columns so small beside
+ * the rest that FP16 halves would lose bits of them (decided per matrix on the device, about half the speed; rows and
+ * columns of A in qr, polar_fwd, svd_fwd and the backwards).  Entries that are small within their row and column,
+ * or in a caller's U and gradients, keep 22 bits down to 2^-28 of the largest of their array, and 2^-50 of that
+ * below. */
+#define PSVD_PREC_FP32       0   /* every product FP32-accurate                              */
 #define PSVD_PREC_MIXED      1   /* TF32 steps -> FP32-accurate polish, switched per matrix from the
                                     measured orthogonality residual; with the learned
-                                    schedule, bounds below PSVD_MIXED_LB_MIN start there */
+                                    schedule, bounds below PSVD_MIXED_LB_MIN start there.
+                                    Not faster than mode 0 in what was measured: forward and
+                                    backward of 4096 x 4096, kappa = 10, 36.8 ms against 36.4;
+                                    8 of 4096 x 1024 14.8 against 14.7 with preqr, 22.5
+                                    (all recomputed) against 11.6 without                    */
 #define PSVD_PREC_MIXED_BF16 2   /* BF16 early steps -> TF32 -> the same polish; the BF16
                                     rounding leaves a rotation that the eigenbasis correction
                                     undoes only to first order (reconstruction ~1e-5 at
@@ -196,7 +205,7 @@ int psvd_svd_fwd(const float *A, float *U, float *S, float *VT, int64_t batch, i
                  psvd_info *info, void *stream);
 
 /* psvd_eigh -- symmetric EVD H = V diag(S) V^T (the EVD of Algorithm 1) of a batch of
- *   n x n symmetric matrices (only the upper triangle is read).  S descending,
+ *   n x n symmetric matrices (full storage).  S descending,
  *   VT rows = eigenvectors with the sign convention above. */
 int psvd_eigh(const float *Hs, float *S, float *VT, int64_t batch, int64_t n,
               void *ws, size_t ws_bytes, void *stream);
@@ -227,6 +236,7 @@ int psvd_eigh_dc(const float *Hs, float *S, float *VT, int64_t batch, int64_t n,
  *   kreg_mode selects K_eps: 0 = (s_i-s_j)/((s_i-s_j)^2 + eps^(1/2)) as in Algorithm 4,
  *   1 = (s_i-s_j)/((s_i-s_j)^2 + eps^2) as in Section 5.2, 2 = exact 1/(s_i-s_j) with
  *   ties (|s_i-s_j| <= 1e-6 s_max) masked and eps = 0 in R and T.
+ *   The rows of dA are as accurate, each relative to itself, as M's rows are given, whatever their sizes.
  *   dA: batch x m x n out. */
 int psvd_svd_bwd(const float *A, const float *U, const float *S, const float *VT,
                  const float *dU, const float *dS, const float *dVT, float *dA,

@@ -19,7 +19,8 @@
 //   PREC_TF32X3 : 32 fp32 of K, two units per k-block (hi parts, lo parts);
 //                 hi*hi + hi*lo + lo*hi (split-TF32, FP32-accurate products)
 //   PREC_F16X3  : 64 fp16 of K, two units per k-block: the same three products of split FP16 halves
-//                 (operands scaled by powers of two, undone by GemmShape::f16_scale).  An FP16 MMA
+//                 (operands scaled by powers of two, undone by GemmShape::f16_scale; the low halves by
+//                 2^kF16LoBits more, undone by the first hi*hi of a k-block).  An FP16 MMA
 //                 covers twice the K of a TF32 one in the same time and its operands are half the
 //                 bytes (a 4096^3 polar step product: 780 us in split TF32, 474 us with the
 //                 same epilogue)

@@ -106,7 +106,7 @@ struct PanelSmem {
 // A panel is a chain of pw such columns, so its time is latency: with the panel in shared memory (5 block
 // barriers per column, every multiply-add fed from shared memory, the Gram matrix and T formed
 // afterwards) a column took 2.9 us at 256 rows, 6.2 at 4096 (8 matrices) and 7.4 at 14336 (4 matrices); it
-// takes 1.4, 2.6 and 3.0 us, everything included.
+// takes 1.4, 2.7 and 3.2 us, everything included.
 template <int RPL, int C>
 __global__ void __launch_bounds__(kQrThreads, 1) qr_panel_kernel(PanelArgs P) {
     using Sm = PanelSmem<RPL, C>;
