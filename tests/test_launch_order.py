@@ -36,6 +36,19 @@ def test_epilogues_do_not_read_through_the_read_only_path():
         assert "global.nc" not in text and "__ldg" not in text, name
 
 
+def test_shared_memory_limits_do_not_depend_on_the_call():
+    # the limit is the function's, for every thread: a value that goes with the call's sizes could be lowered by another
+    # thread between a call's setting and its launch
+    seen = 0
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        text = _code(path)
+        for m in re.finditer(r"cudaFuncAttributeMaxDynamicSharedMemorySize,([^;]*?)\)\s*[;)]", text):
+            names = set(re.findall(r"[A-Za-z_][A-Za-z_0-9.]*", m.group(1))) - {"int", "sizeof", "Sm"}
+            assert all(re.fullmatch(r"k[A-Z]\w*", x) for x in names), (path, m.group(0))
+            seen += 1
+    assert seen >= 10
+
+
 @pytest.mark.gpu
 def test_captured_rerun_matches_stream():
     # a learned schedule whose bounds are far off for one matrix: its rerun resets the counters that the
